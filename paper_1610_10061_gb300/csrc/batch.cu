@@ -27,21 +27,30 @@ pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std
         return PM_ERR_INVALID_ARG;
     out = pm_multi_plan();
     out.groups = G;
-    out.warps = warps;
     const pm_instance *i0 = insts[0];
-    for (const pm_instance *in : insts)
-        out.smem = std::max(out.smem, tile_bytes(in->W, G));
+    double depth = 0.0;
+    int64_t units = 0;  // units of 1024 pairs
+    for (int k = 0; k < K; ++k) {
+        const pm_instance *in = insts[k];
+        out.Wmax = std::max(out.Wmax, in->W);
+        depth = std::max(depth, pm_walk_depth(in->m, in->p, in->L));
+        units += pm_ceil_div(pops[k], 32) * pm_ceil_div(in->n, 32);
+    }
     const size_t budget = i0->smem_optin > 4096 ? i0->smem_optin - 4096 : 0;
-    if (out.smem > budget)
+    if (tile_bytes(out.Wmax, G) > budget)
         return PM_ERR_UNSUPPORTED;
+    if (pm_sliced_pays(i0, units))
+        pm_walk_shape(i0, out.Wmax, G, depth, warps, out.nb);
+    out.warps = warps;
     int slots_per_sm = 0;
     // resident CTAs per SM for this shape and shared memory
     {
-        const int by_smem = (int)std::max<size_t>(1, i0->smem_optin / std::max<size_t>(out.smem + 2048, 1));
+        const int by_smem = (int)std::max<size_t>(
+            1, i0->smem_optin / (pm_scan_smem(out.Wmax, G, warps, out.nb) + 3072));
         const int by_threads = std::max(1, 2048 / (warps * 32));
         slots_per_sm = std::max(1, std::min(by_smem, by_threads));
-        // register limit: ~56 registers per thread
-        const int by_regs = std::max(1, 65536 / (warps * 32 * 56));
+        // register limit: 128 registers per thread in the bit-sliced walk, ~56 in the client walk
+        const int by_regs = std::max(1, 65536 / (warps * 32 * (out.nb ? 128 : 56)));
         slots_per_sm = std::min(slots_per_sm, by_regs);
     }
     const int64_t slots = (int64_t)i0->sm_count * slots_per_sm;
@@ -51,7 +60,7 @@ pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std
     for (int k = 0; k < K; ++k) {
         const pm_instance *in = insts[k];
         const double tiles = (double)pm_ceil_div(pops[k], 32 * G);
-        const double steps = 1.0 + 5.4 * (double)(in->m + 1) / (double)(in->p + 1) / 32.0;
+        const double steps = 1.5 + pm_walk_depth(in->m, in->p, in->L) / 32.0;
         work[k] = tiles * (double)in->n * steps;
         total += work[k];
     }
@@ -75,10 +84,12 @@ pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std
         pr.tiles = std::max<int64_t>(1, pm_ceil_div(pops[k], 32 * G));
         const double want_items = total > 0 ? target_items * work[k] / total : 1.0;
         int64_t splits = (int64_t)std::ceil(want_items / (double)pr.tiles);
-        splits = std::max<int64_t>(1, std::min<int64_t>(splits, std::max<int64_t>(1, in->n / warps)));
+        const int64_t per_warp = out.nb ? 32 / G : 1;  // clients a warp takes at once
+        splits = std::max<int64_t>(1, std::min<int64_t>(splits, pm_ceil_div(in->n, warps * per_warp)));
         pr.splits = splits;
         pr.cps = pm_ceil_div(in->n, splits);
         pr.packed = pm_packed_reduction_ok(in, splits) ? 1 : 0;
+        pr.flush_units = pm_flush_units(in->max_d, G);
         pr.ind_base = ind;
         pr.out_base = 0;  // set by the caller for packed outputs
         pr.word_base = words;
@@ -108,6 +119,7 @@ pm_multi_plan pm_plan_from_single(const pm_instance *inst, const pm_eval_plan &p
     pm_multi_plan mp;
     mp.groups = plan.groups;
     mp.warps = plan.warps;
+    mp.nb = plan.nb;
     mp.grid = plan.grid;
     mp.probs.push_back(pm_single_prob(inst, plan, pop));
     mp.items = plan.tiles * plan.splits;
@@ -116,7 +128,7 @@ pm_multi_plan pm_plan_from_single(const pm_instance *inst, const pm_eval_plan &p
     mp.ind_total = pm_round_up(std::max<int64_t>(pop, 1), 32);
     mp.words_total = pop * inst->W;
     mp.cols_total = plan.groups ? plan.tiles * inst->W * 32 * plan.groups : 0;
-    mp.smem = plan.groups ? tile_bytes(inst->W, plan.groups) : 0;
+    mp.Wmax = inst->W;
     return mp;
 }
 
@@ -124,6 +136,8 @@ void pm_scan_launch_from(const pm_multi_plan &mp, const pm_prob *probs_dev, pm_s
 {
     L.groups = mp.groups;
     L.warps = mp.warps;
+    L.nb = mp.nb;
+    L.Wmax = mp.Wmax;
     L.grid = mp.grid;
     L.K = (int)mp.probs.size();
     L.one = mp.probs[0];
@@ -143,6 +157,7 @@ struct pm_batch {
     std::vector<int64_t> plan_pops;
     pm_multi_plan plan;
     bool have_plan = false;
+    int plan_G = 0, plan_warps = 0;  // the shape asked for (the plan may use fewer warps)
     std::vector<int64_t> tuned_pops;
     int tuned_G = 0, tuned_warps = 0, tuned_ips = 0;
     pm_dbuf probs, accum, tickets, columns, err, stage_masks, stage_costs;
@@ -170,6 +185,8 @@ static pm_status batch_plan(pm_batch *b, const std::vector<int64_t> &pops, int G
         PM_CUDA(cudaMemsetAsync(b->tickets.ptr, 0, b->tickets.bytes, s));
     PM_TRY(b->columns.reserve(std::max<size_t>((size_t)mp.cols_total * 4, 256)));
     b->plan = mp;
+    b->plan_G = G;
+    b->plan_warps = warps;
     b->plan_pops = pops;
     b->have_plan = true;
     return PM_OK;
@@ -232,7 +249,7 @@ static pm_status batch_eval_impl(pm_batch *b, const uint32_t *masks, const std::
     } else {
         default_shape(b, G, warps, ips);
     }
-    if (!b->have_plan || b->plan_pops != pops || b->plan.groups != G || b->plan.warps != warps)
+    if (!b->have_plan || b->plan_pops != pops || b->plan_G != G || b->plan_warps != warps)
         PM_TRY(batch_plan(b, pops, G, warps, ips, s));
     PM_TRY(b->err.reserve(256));
     pm_scan_launch L;
@@ -244,7 +261,7 @@ static pm_status batch_eval_impl(pm_batch *b, const uint32_t *masks, const std::
     L.err = static_cast<int *>(b->err.ptr);
     pm_accept_args acc;
     // the epilogue writes costs[out_base + t]; masks rows start at word_base (packed, as the caller lays them out)
-    return pm_launch_scan(L, acc, costs, b->plan.smem, s);
+    return pm_launch_scan(L, acc, costs, s);
 }
 
 extern "C" pm_status pm_batch_eval(pm_batch *b, const uint32_t *masks, const int64_t *pops, int64_t *costs,

@@ -49,6 +49,7 @@
 #include <cstdio>
 
 #include "pm_common.cuh"
+#include "scan_tile.cuh"
 #include "scan_walk.cuh"
 
 namespace {
@@ -188,17 +189,16 @@ __device__ __forceinline__ void apply_epilogue(const unsigned long long *acc_s, 
 // running at the same time walk the same clients for different tiles and
 // the rows they stream are shared through L2.
 // ---------------------------------------------------------------------------
-template <int G>
-__global__ void __launch_bounds__(1024) k_scan_columns(const pm_prob *__restrict__ probs, int K, pm_prob one,
-                                                       int64_t items, const uint32_t *__restrict__ colT,
-                                                       const uint32_t *__restrict__ active,
-                                                       unsigned long long *__restrict__ accum,
-                                                       int *__restrict__ tickets, int *__restrict__ err,
-                                                       ScanEpilogue ep, uint32_t stall)
+template <int G, bool kSliced>
+__global__ void __launch_bounds__(kSliced ? 512 : 1024)
+    k_scan_columns(const pm_prob *__restrict__ probs, int K, pm_prob one, int64_t items,
+                   const uint32_t *__restrict__ colT, const uint32_t *__restrict__ active,
+                   unsigned long long *__restrict__ accum, int *__restrict__ tickets, int *__restrict__ err,
+                   ScanEpilogue ep, uint32_t stall, int nb, uint32_t tab_off)
 {
     // the previous kernel of the stream may still run until pm_grid_dependency_wait(): before it only the
     // constant tables (Pi', Delta', the launch's problem table) are read
-    extern __shared__ __align__(128) uint32_t colbits[];  // [32W][G]
+    extern __shared__ __align__(128) uint32_t colbits[];  // [32W][G], then (kSliced, at tab_off) the warps' tables
     __shared__ unsigned long long acc_s[G * 32];
     __shared__ uint32_t a0_s[G], fin_s[G];
     __shared__ __align__(8) uint64_t bar;
@@ -216,6 +216,10 @@ __global__ void __launch_bounds__(1024) k_scan_columns(const pm_prob *__restrict
         mbar_init(&bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    [[maybe_unused]] TileWalk<G> walk;
+    const uint32_t my_tab = tab_off + (uint32_t)(warp * tile_table_words(nb, G));
+    if constexpr (kSliced)
+        TileWalk<G>::clear_table(colbits + my_tab, nb, lane);
     __syncthreads();
 
     uint32_t phase = 0;
@@ -240,7 +244,7 @@ __global__ void __launch_bounds__(1024) k_scan_columns(const pm_prob *__restrict
         // first steps of this warp's first two clients (constant tables), loaded while the tile lands
         const int64_t c_begin = split * pr.cps;
         const int64_t c_end = (c_begin + pr.cps < pr.n) ? c_begin + pr.cps : pr.n;
-        auto load = [&](int64_t cc, int base, uint32_t &j, int32_t &dl) {
+        [[maybe_unused]] auto load = [&](int64_t cc, int base, uint32_t &j, int32_t &dl) {
             const int r = base + lane;
             if (cc < c_end && r < L) {
                 j = __ldg(pi + cc * stride + r);
@@ -250,13 +254,18 @@ __global__ void __launch_bounds__(1024) k_scan_columns(const pm_prob *__restrict
                 dl = 0;
             }
         };
-        int64_t c = c_begin + warp;
-        uint32_t j_cur, j_nxt, j_nc, j_nc1;
-        int32_t d_cur, d_nxt, d_nc, d_nc1;
-        load(c, 0, j_cur, d_cur);
-        load(c, 32, j_nxt, d_nxt);
-        load(c + nwarps, 0, j_nc, d_nc);
-        load(c + nwarps, 32, j_nc1, d_nc1);
+        [[maybe_unused]] const int64_t c = c_begin + warp;
+        [[maybe_unused]] uint32_t j_cur, j_nxt, j_nc, j_nc1;
+        [[maybe_unused]] int32_t d_cur, d_nxt, d_nc, d_nc1;
+        const TileRows rows{pi, delta, stride, L, pr.cum != 0, pr.flush_units};
+        if constexpr (kSliced) {
+            walk.prefetch(rows, c_begin, c_end, warp, lane);
+        } else {
+            load(c, 0, j_cur, d_cur);
+            load(c, 32, j_nxt, d_nxt);
+            load(c + nwarps, 0, j_nc, d_nc);
+            load(c + nwarps, 32, j_nc1, d_nc1);
+        }
         if (!waited) {  // from here on: the columns, active bits and accumulators of the previous kernels
             pm_grid_dependency_wait();
             waited = true;
@@ -304,25 +313,34 @@ __global__ void __launch_bounds__(1024) k_scan_columns(const pm_prob *__restrict
         }
         __syncthreads();
 
-        uint32_t a0[G];
-        uint32_t any0 = 0;
+        if constexpr (kSliced) {
+            uint32_t any0 = 0;
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-            a0[g] = a0_s[g];
-            any0 |= a0[g];
-        }
-        unsigned long long acc[G];
+            for (int g = 0; g < G; ++g)
+                any0 |= a0_s[g];
+            if (any0 && c_begin < c_end)
+                walk.run(colbits, my_tab, nb, a0_s[lane % G], rows, c_begin, c_end, warp, nwarps, lane, acc_s);
+        } else {
+            uint32_t a0[G];
+            uint32_t any0 = 0;
 #pragma unroll
-        for (int g = 0; g < G; ++g)
-            acc[g] = 0ull;
+            for (int g = 0; g < G; ++g) {
+                a0[g] = a0_s[g];
+                any0 |= a0[g];
+            }
+            unsigned long long acc[G];
+#pragma unroll
+            for (int g = 0; g < G; ++g)
+                acc[g] = 0ull;
 
-        if (any0 && c < c_end)
-            scan_clients<G>(colbits, a0, c, c_end, nwarps, L, lane, pr.cum != 0, load, j_cur, d_cur, j_nxt, d_nxt, j_nc,
-                            d_nc, j_nc1, d_nc1, acc);
+            if (any0 && c < c_end)
+                scan_clients<G>(colbits, a0, c, c_end, nwarps, L, lane, pr.cum != 0, load, j_cur, d_cur, j_nxt, d_nxt,
+                                j_nc, d_nc, j_nc1, d_nc1, acc);
 #pragma unroll
-        for (int g = 0; g < G; ++g)
-            if (acc[g])
-                atomicAdd(&acc_s[g * 32 + lane], acc[g]);
+            for (int g = 0; g < G; ++g)
+                if (acc[g])
+                    atomicAdd(&acc_s[g * 32 + lane], acc[g]);
+        }
         __syncthreads();
 
         bool finish = true;
@@ -541,10 +559,14 @@ __global__ void k_wait_selftest(int *__restrict__ err, uint32_t limit)
     }
 }
 
-template <int G>
-const void *scan_fn()
+// The column kernel for G groups, with the bit-sliced walk or the client walk.
+using scan_kernel = void (*)(const pm_prob *, int, pm_prob, int64_t, const uint32_t *, const uint32_t *,
+                             unsigned long long *, int *, int *, ScanEpilogue, uint32_t, int, uint32_t);
+scan_kernel scan_fn(int G, bool sliced)
 {
-    return reinterpret_cast<const void *>(k_scan_columns<G>);
+    if (sliced)
+        return G == 4 ? k_scan_columns<4, true> : (G == 2 ? k_scan_columns<2, true> : k_scan_columns<1, true>);
+    return G == 4 ? k_scan_columns<4, false> : (G == 2 ? k_scan_columns<2, false> : k_scan_columns<1, false>);
 }
 
 }  // namespace
@@ -568,26 +590,54 @@ static pm_status allow_dynamic_smem(const pm_instance *inst, F *fn)
 
 pm_status pm_fitness_init(const pm_instance *inst)
 {
-    PM_TRY(allow_dynamic_smem(inst, k_scan_columns<1>));
-    PM_TRY(allow_dynamic_smem(inst, k_scan_columns<2>));
-    PM_TRY(allow_dynamic_smem(inst, k_scan_columns<4>));
+    for (int G : {1, 2, 4})
+        for (bool sliced : {false, true})
+            PM_TRY(allow_dynamic_smem(inst, scan_fn(G, sliced)));
     PM_TRY(allow_dynamic_smem(inst, k_scan_rows<false>));
     PM_TRY(allow_dynamic_smem(inst, k_scan_rows<true>));
     return PM_OK;
 }
 
 
-// Resident CTAs per SM of the column kernel for (G, warps) at this instance's W.
-static int column_ctas_per_sm(const pm_instance *inst, int G, int warps)
+size_t pm_scan_smem(int64_t W, int G, int warps, int nb)
 {
-    const size_t smem = column_smem_bytes(inst->W, G);
+    return column_smem_bytes(W, G) + (nb ? (size_t)warps * tile_table_words(nb, G) * 4 : 0);
+}
+
+void pm_walk_shape(const pm_instance *inst, int64_t W, int G, double depth, int &warps, int &nb)
+{
+    const size_t budget = inst->smem_optin > 4096 ? inst->smem_optin - 4096 : 0;
+    const int want = depth <= 32.0 ? 1 : (depth <= 160.0 ? 3 : 7);
+    for (int w = std::min(warps, 16); w >= 4 || w == std::min(warps, 16); w /= 2) {
+        for (int b : {7, 3, 1}) {
+            if (b <= want && pm_scan_smem(W, G, w, b) <= budget) {
+                warps = w;
+                nb = b;
+                return;
+            }
+        }
+        if (w <= 1)
+            break;
+    }
+    nb = 0;
+}
+
+// Resident CTAs per SM of the column kernel for a plan's (G, warps, nb) at this instance's W.
+static int column_ctas_per_sm(const pm_instance *inst, const pm_eval_plan &plan)
+{
     int nb = 0;
-    const void *fn = G == 4 ? scan_fn<4>() : (G == 2 ? scan_fn<2>() : scan_fn<1>());
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, warps * 32, smem) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &nb, reinterpret_cast<const void *>(scan_fn(plan.groups, plan.nb > 0)), plan.warps * 32,
+            pm_scan_smem(inst->W, plan.groups, plan.warps, plan.nb)) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     return nb;
+}
+
+static bool sliced_pays(const pm_instance *inst, int64_t pop)
+{
+    return pm_sliced_pays(inst, pm_ceil_div(pop, 32) * pm_ceil_div(inst->n, 32));
 }
 
 pm_eval_plan pm_plan_eval_with(const pm_instance *inst, int64_t pop, int G, int warps, int splits_hint)
@@ -595,23 +645,30 @@ pm_eval_plan pm_plan_eval_with(const pm_instance *inst, int64_t pop, int G, int 
     pm_eval_plan plan;
     const size_t budget = inst->smem_optin > 4096 ? inst->smem_optin - 4096 : 0;
     int64_t ctas_per_sm = 0;
-    if (G > 0 && column_smem_bytes(inst->W, G) <= budget)
-        ctas_per_sm = column_ctas_per_sm(inst, G, warps);
+    if (G > 0 && column_smem_bytes(inst->W, G) <= budget) {
+        plan.groups = G;
+        plan.warps = warps;
+        if (sliced_pays(inst, pop))
+            pm_walk_shape(inst, inst->W, G, pm_walk_depth(inst->m, inst->p, inst->L), plan.warps, plan.nb);
+        ctas_per_sm = column_ctas_per_sm(inst, plan);
+    }
     if (G <= 0 || ctas_per_sm <= 0) {
         plan.groups = 0;  // row kernel
+        plan.nb = 0;
         plan.warps = 8;
         plan.tiles = pm_ceil_div(pop, plan.warps);
         plan.bytes = (G < 0 && (size_t)plan.warps * inst->W * 32 + 1024 <= inst->smem_optin) ? 1 : 0;
         ctas_per_sm = 8;
     } else {
-        plan.groups = G;
-        plan.warps = warps;
         plan.tiles = pm_ceil_div(pop, 32 * G);
     }
     const int64_t slots = (int64_t)inst->sm_count * ctas_per_sm;
-    // default: about four work items per resident CTA slot; every warp gets at least one client
+    // default: about four work items per resident CTA slot; every warp gets at least one client (one unit of 32/G
+    // clients in the bit-sliced walk)
     const int64_t max_splits = std::max<int64_t>(1, inst->n / (plan.groups ? plan.warps : 1));
     int64_t splits = splits_hint > 0 ? splits_hint : pm_ceil_div(4 * slots, std::max<int64_t>(1, plan.tiles));
+    if (splits_hint <= 0 && plan.nb)
+        splits = std::min<int64_t>(splits, std::max<int64_t>(1, pm_ceil_div(inst->n * plan.groups, plan.warps * 32)));
     if (splits_hint <= 0 && splits > max_splits)  // too few clients for that: one item per slot instead
         splits = std::max<int64_t>(1, std::min<int64_t>(max_splits, slots / std::max<int64_t>(1, plan.tiles)));
     splits = std::min<int64_t>(std::max<int64_t>(1, splits), std::min<int64_t>(max_splits, 65535));
@@ -633,7 +690,7 @@ pm_eval_plan pm_plan_eval(const pm_instance *inst, int64_t pop)
     // fewer groups for small populations or when the tile does not fit: keep >= 8 tiles, or >= 16 where a
     // client's walk is short (expected first open rank (m+1)/(p+1) below 32: one or two steps, so the
     // launch's fixed costs weigh more than the per-step savings of wide tiles)
-    const int64_t min_tiles = (inst->m + 1) < 32 * (inst->p + 1) ? 16 : 8;
+    const int64_t min_tiles = sliced_pays(inst, pop) ? 1 : ((inst->m + 1) < 32 * (inst->p + 1) ? 16 : 8);
     while (G > 1 && (pop <= (int64_t)32 * (G / 2) * min_tiles || column_smem_bytes(inst->W, G) > budget))
         G /= 2;
     // 32 warps when only one CTA fits per SM, else 16
@@ -670,6 +727,7 @@ pm_prob pm_single_prob(const pm_instance *inst, const pm_eval_plan &plan, int64_
     pr.p = (int32_t)inst->p;
     pr.cum = inst->cum ? 1 : 0;
     pr.packed = pm_packed_reduction_ok(inst, plan.splits) ? 1 : 0;
+    pr.flush_units = plan.groups ? pm_flush_units(inst->max_d, plan.groups) : 0u;
     pr.pop = pop;
     pr.tiles = plan.tiles;
     pr.splits = plan.splits;
@@ -725,8 +783,7 @@ pm_status pm_launch_columns(const pm_instance *inst, const pm_eval_plan &plan, c
                             plan.groups, colT, stream);
 }
 
-pm_status pm_launch_scan(const pm_scan_launch &L, const pm_accept_args &acc, int64_t *costs, size_t smem,
-                         cudaStream_t stream)
+pm_status pm_launch_scan(const pm_scan_launch &L, const pm_accept_args &acc, int64_t *costs, cudaStream_t stream)
 {
     if (L.items <= 0)
         return PM_OK;
@@ -744,19 +801,9 @@ pm_status pm_launch_scan(const pm_scan_launch &L, const pm_accept_args &acc, int
     const unsigned grid = (unsigned)L.grid;
     unsigned long long *accum = reinterpret_cast<unsigned long long *>(L.accum);
     const uint32_t stall = take_stall() ? 1u : 0u;
-#define PM_SCAN_ARGS L.probs_dev, L.K, L.one, L.items, L.colT, L.active, accum, L.tickets, L.err, ep, stall
-    switch (G) {
-    case 1:
-        PM_CUDA(pm_launch(k_scan_columns<1>, grid, threads, smem, stream, PM_SCAN_ARGS));
-        break;
-    case 2:
-        PM_CUDA(pm_launch(k_scan_columns<2>, grid, threads, smem, stream, PM_SCAN_ARGS));
-        break;
-    default:
-        PM_CUDA(pm_launch(k_scan_columns<4>, grid, threads, smem, stream, PM_SCAN_ARGS));
-        break;
-    }
-#undef PM_SCAN_ARGS
+    const uint32_t tab_off = (uint32_t)(column_smem_bytes(L.Wmax, G) / 4);
+    PM_CUDA(pm_launch(scan_fn(G, L.nb > 0), grid, threads, pm_scan_smem(L.Wmax, G, L.warps, L.nb), stream, L.probs_dev,
+                      L.K, L.one, L.items, L.colT, L.active, accum, L.tickets, L.err, ep, stall, L.nb, tab_off));
     return PM_OK;
 }
 
@@ -771,6 +818,8 @@ pm_status pm_launch_eval(const pm_instance *inst, const pm_eval_plan &plan, cons
         pm_scan_launch L;
         L.groups = plan.groups;
         L.warps = plan.warps;
+        L.nb = plan.nb;
+        L.Wmax = inst->W;
         L.grid = plan.grid;
         L.K = 1;
         L.one = pm_single_prob(inst, plan, pop);
@@ -782,7 +831,7 @@ pm_status pm_launch_eval(const pm_instance *inst, const pm_eval_plan &plan, cons
         L.accum = partials_i64;
         L.tickets = tickets;
         L.err = err;
-        return pm_launch_scan(L, acc, costs, column_smem_bytes(inst->W, plan.groups), stream);
+        return pm_launch_scan(L, acc, costs, stream);
     }
     ScanEpilogue ep;
     ep.mode = acc.mode;

@@ -2207,7 +2207,7 @@ static pm_status ga_eval(pm_ga *ga, const uint32_t *masks, int64_t *costs, const
     L.accum = accum;
     L.tickets = tickets;
     L.err = err;
-    return pm_launch_scan(L, acc, costs, ga->plan.smem, s);
+    return pm_launch_scan(L, acc, costs, s);
 }
 
 // Enqueue one generation on `s`: under stream capture for the graph body
@@ -2327,7 +2327,7 @@ static pm_status enqueue_generation(pm_ga *ga, cudaStream_t s, cudaGraphConditio
         L.err = static_cast<int *>(ga->err.ptr);
         pm_accept_args store;
         store.columns_ready = true;
-        PM_TRY(pm_launch_scan(L, store, costQ, ga->spec_plan.smem, s));
+        PM_TRY(pm_launch_scan(L, store, costQ, s));
         PM_CUDA(pm_launch(k_ga_mutate_accept, (unsigned)pm_ceil_div(ga->plan.ind_total, 8), 256, 0, s, gps, gqs, K,
                           one, ga->gq, (int32_t)ga->Q, X, XQ, cost, costQ, improved, st));
     } else {

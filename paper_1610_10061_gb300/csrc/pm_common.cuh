@@ -75,6 +75,7 @@ struct pm_eval_plan {
     int64_t tiles = 0;    // ceil(pop / (32 G))
     int64_t grid = 0;     // CTAs launched (column kernel: persistent over tiles x splits items)
     int bytes = 0;        // row kernel only: each warp's bitset expanded to one byte per facility (byte masks)
+    int nb = 0;           // column kernel: blocks of 32 ranks per table of the bit-sliced walk; 0: the client walk
 };
 
 // One instance inside an evaluation launch (host and device).  Individuals
@@ -89,6 +90,7 @@ struct pm_prob {
     int32_t L, W, m, p;
     int32_t cum;
     int32_t packed;  // split sums and a split count share one 64-bit word (see pm_packed_reduction_ok)
+    uint32_t flush_units;  // bit-sliced walk: see pm_flush_units
     int64_t pop;
     int64_t ind_base;   // accumulators, active bits, GA per-individual arrays
     int64_t out_base;   // caller's cost array
@@ -199,6 +201,8 @@ struct pm_accept_args {
 // A scan launch over one or more instances.
 struct pm_scan_launch {
     int groups = 4, warps = 16;
+    int nb = 0;                          // as pm_eval_plan
+    int64_t Wmax = 0;                    // bitset words of the widest instance (sizes the shared memory)
     int64_t grid = 0;
     int K = 1;
     const pm_prob *probs_dev = nullptr;  // K > 1: device table
@@ -211,8 +215,32 @@ struct pm_scan_launch {
     int *tickets = nullptr;              // one per global tile, zero at rest
     int *err = nullptr;
 };
-pm_status pm_launch_scan(const pm_scan_launch &L, const pm_accept_args &acc, int64_t *costs, size_t smem,
-                         cudaStream_t stream);
+pm_status pm_launch_scan(const pm_scan_launch &L, const pm_accept_args &acc, int64_t *costs, cudaStream_t stream);
+// Shared-memory bytes of a column-kernel CTA: the tile and, with nb > 0, the warps' distance tables.
+size_t pm_scan_smem(int64_t W, int G, int warps, int nb);
+// Warps (at most `warps`) and table blocks of the bit-sliced walk for tiles of W words and walks whose deepest
+// rank is about `depth`; nb = 0 and warps unchanged where the tables do not fit beside the tile.
+void pm_walk_shape(const pm_instance *inst, int64_t W, int G, double depth, int &warps, int &nb);
+// Whether a launch has enough units of 1024 (client, individual) pairs for the bit-sliced walk: a unit is a chain
+// of about 1200 instructions of one warp, so with fewer than 12 per SM the SMs wait for single warps and the client
+// walk, which spreads one client over a warp, is the faster one (graph900 generation, 904 units per scan: 209 us
+// with the client walk, 270 us bit-sliced; 3001 x 2011, pop 777, 2350 units: 136 against 87 us).
+static inline bool pm_sliced_pays(const pm_instance *inst, int64_t units)
+{
+    return units >= (int64_t)inst->sm_count * 12;
+}
+// The deepest first open rank a unit of 1024 pairs is expected to meet: 1024 geometric draws of mean (m+1)/(p+1).
+static inline double pm_walk_depth(int64_t m, int64_t p, int64_t L)
+{
+    return std::min<double>((double)L, 7.5 * (double)(m + 1) / (double)(p + 1));
+}
+// Units of 32/G clients whose distances a warp may add up in 32 bits (all its lanes together) before it must add
+// the sums to the 64-bit ones; 0: not even one unit.
+static inline uint32_t pm_flush_units(int32_t max_d, int G)
+{
+    const uint64_t per = (uint64_t)std::max<int32_t>(max_d, 1) * (uint64_t)(32 / G);
+    return (uint32_t)std::min<uint64_t>(0xffffffffull / per, 0x7fffffffull);
+}
 // The single-instance launch of `plan` (K = 1, all bases 0).
 pm_prob pm_single_prob(const pm_instance *inst, const pm_eval_plan &plan, int64_t pop);
 
@@ -247,10 +275,10 @@ pm_status pm_launch_random_population(const pm_instance *inst, uint64_t seed, in
 // A scan plan over several instances (batch.cu): one tile shape for all,
 // per-instance splits, global numbering of individuals, rows, tiles.
 struct pm_multi_plan {
-    int groups = 4, warps = 16;
+    int groups = 4, warps = 16, nb = 0;
     int64_t grid = 0, items = 0, jobs = 0;
     int64_t tiles_total = 0, ind_total = 0, words_total = 0, cols_total = 0;
-    size_t smem = 0;  // tile bytes of the widest instance
+    int64_t Wmax = 0;  // bitset words of the widest instance
     std::vector<pm_prob> probs;
 };
 // Plan for `insts` with pops[k] individuals each; items_per_slot work items per
