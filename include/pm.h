@@ -81,7 +81,10 @@ typedef struct pm_instance pm_instance;
  * and the increments Delta'_i (Delta'_i0 = smallest distance, then
  * consecutive differences), both truncated to L = m - p + 1 columns.  The
  * tables stay resident on `device` (Pi' uint16, Delta' int32, rows padded to
- * a stride of round_up(L, 32) elements).
+ * a stride of round_up(L, 32) elements).  Where p is far below the expected
+ * first open rank (m + 1) / (p + 1) the instance also keeps the distances in
+ * 16 bits (up to 1 GiB; done without if they do not fit in memory): with few
+ * open facilities reading the p distances is cheaper than the scan.
  *   d       distance matrix; not retained.
  *   n, m, p 1 <= n, 1 <= p < m <= 65535.
  *   device  CUDA device ordinal; becomes the current device.
@@ -134,7 +137,8 @@ PM_API pm_status pm_instance_tables(const pm_instance *inst, uint16_t *pi_out, i
  * individual t and client i, walk Delta'_i in the order of Pi'_i, adding each
  * increment, and stop after the first rank whose facility is open in t; the
  * cost of t is the int64 sum over clients.  It equals the p-median objective
- * of Eqs. 1-3 for t's open set (Eq. 4 telescopes).
+ * of Eqs. 1-3 for t's open set (Eq. 4 telescopes); large populations with few
+ * open facilities are evaluated by that objective, with the same results.
  *   masks   pop x W bitsets (layout above), host or device memory.
  *   pop     number of individuals, >= 0 (0 is a no-op).
  *   costs   pop int64 results, host or device memory.

@@ -279,12 +279,20 @@ static pm_status create_impl(const int32_t *d, int64_t n, int64_t m, int64_t p, 
     PM_CUDA(cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
     inst->smem_optin = (size_t)v;
     const size_t tab = (size_t)n * (size_t)inst->stride;
-    pm_dbuf dbuf, pbuf;
+    const int64_t entries = pm_ceil_div(n, 8) * m;  // eight clients' 16-bit distances each
+    const bool dense = pm_direct_wanted(n, m, p, inst->smem_optin);
+    pm_dbuf dbuf, pbuf, ebuf;
     const pm_part parts[] = {{&inst->err, 256}, {&inst->flag, 256}, {&dbuf, tab * sizeof(int32_t)},
-                             {&pbuf, tab * sizeof(uint16_t)}};
-    PM_TRY(pm_carve(inst->tab_arena, parts, 4));
+                             {&pbuf, tab * sizeof(uint16_t)}, {&ebuf, (size_t)entries * 16}};
+    pm_status carved = pm_carve(inst->tab_arena, parts, dense ? 5 : 4);
+    // the 16-bit distances are optional (the scan needs only the tables): where they are large enough to be what did
+    // not fit, the instance does without them
+    if (carved == PM_ERR_OOM && dense && entries >= ((int64_t)1 << 22))
+        carved = pm_carve(inst->tab_arena, parts, 4);
+    PM_TRY(carved);
     inst->delta = static_cast<int32_t *>(dbuf.ptr);
     inst->pi = static_cast<uint16_t *>(pbuf.ptr);
+    inst->dense = static_cast<uint16_t *>(ebuf.ptr);
     PM_CUDA(cudaMemsetAsync(inst->err.ptr, 0, 256, stream));
     PM_TRY(pm_fitness_init(inst));
     const int32_t *d_dev = d;
@@ -437,9 +445,10 @@ extern "C" pm_status pm_eval_columns(pm_instance *inst, const uint32_t *cols, in
     std::lock_guard<std::mutex> guard(inst->lock);
     PM_CUDA(cudaSetDevice(inst->device));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const pm_eval_plan plan = pm_plan_eval(inst, pop);
+    pm_eval_plan plan = pm_plan_eval(inst, pop);
     if (!plan.groups)
         return PM_ERR_UNSUPPORTED;
+    plan.direct = pm_direct_plan();  // the caller's form is the scan's
     bool fresh = false;
     PM_TRY(inst->partials.reserve(pm_plan_partial_bytes(plan, pop), &fresh));
     if (fresh)  // accumulators start at zero; launches leave them zero

@@ -42,11 +42,27 @@ pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std
     if (pm_sliced_pays(i0, units))
         pm_walk_shape(i0, out.Wmax, G, depth, warps, out.nb);
     out.warps = warps;
+    // scan work estimate per instance: tiles x clients x expected 32-rank steps of a 128-individual tile
+    std::vector<double> work(K);
+    std::vector<pm_direct_plan> direct(K);
+    double total = 0.0;
+    for (int k = 0; k < K; ++k) {
+        const pm_instance *in = insts[k];
+        const double tiles = (double)pm_ceil_div(pops[k], 32 * G);
+        const double steps = 1.5 + pm_walk_depth(in->m, in->p, in->L) / 32.0;
+        work[k] = tiles * (double)in->n * steps;
+        if (out.nb) {  // in SM cycles per pair, the unit the two ways are compared in
+            work[k] = (double)pops[k] * (double)in->n *
+                      (direct[k].range ? pm_direct_cost(in->m, in->p, direct[k].range, direct[k].stages) : pm_scan_cost(in->m, in->p));
+            out.d_smem = std::max(out.d_smem, direct[k].smem);
+        }
+        total += work[k];
+    }
     int slots_per_sm = 0;
     // resident CTAs per SM for this shape and shared memory
     {
         const int by_smem = (int)std::max<size_t>(
-            1, i0->smem_optin / (pm_scan_smem(out.Wmax, G, warps, out.nb) + 3072));
+            1, i0->smem_optin / (std::max(pm_scan_smem(out.Wmax, G, warps, out.nb), out.d_smem) + 3072));
         const int by_threads = std::max(1, 2048 / (warps * 32));
         slots_per_sm = std::max(1, std::min(by_smem, by_threads));
         // register limit: 128 registers per thread in the bit-sliced walk, ~56 in the client walk
@@ -54,16 +70,6 @@ pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std
         slots_per_sm = std::min(slots_per_sm, by_regs);
     }
     const int64_t slots = (int64_t)i0->sm_count * slots_per_sm;
-    // scan work estimate per instance: tiles x clients x expected 32-rank steps of a 128-individual tile
-    std::vector<double> work(K);
-    double total = 0.0;
-    for (int k = 0; k < K; ++k) {
-        const pm_instance *in = insts[k];
-        const double tiles = (double)pm_ceil_div(pops[k], 32 * G);
-        const double steps = 1.5 + pm_walk_depth(in->m, in->p, in->L) / 32.0;
-        work[k] = tiles * (double)in->n * steps;
-        total += work[k];
-    }
     const double target_items = (double)slots * std::max(1, items_per_slot);
     int64_t ind = 0, words = 0, cols = 0, tiles_acc = 0, items = 0, jobs = 0;
     out.probs.resize(K);
@@ -90,6 +96,14 @@ pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std
         pr.cps = pm_ceil_div(in->n, splits);
         pr.packed = pm_packed_reduction_ok(in, splits) ? 1 : 0;
         pr.flush_units = pm_flush_units(in->max_d, G);
+        if (direct[k].range) {
+            pm_direct_splits(in, (int64_t)std::ceil(want_items / (double)pm_ceil_div(pops[k], direct[k].range)),
+                             direct[k]);
+            if (direct[k].range) {
+                pm_direct_prob(in, direct[k], pops[k], pr);
+                splits = pr.splits;
+            }
+        }
         pr.ind_base = ind;
         pr.out_base = 0;  // set by the caller for packed outputs
         pr.word_base = words;
@@ -99,10 +113,10 @@ pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std
         pr.job_base = jobs;
         ind += pm_round_up(std::max<int64_t>(pops[k], 1), 32);
         words += pops[k] * in->W;
-        cols += pr.tiles * in->W * 32 * G;
+        cols += pm_ceil_div(std::max<int64_t>(pops[k], 1), 32 * G) * in->W * 32 * G;
         tiles_acc += pr.tiles;
         items += pr.tiles * splits;
-        jobs += pr.tiles * G * in->W;
+        jobs += pr.d_range ? pops[k] : pr.tiles * G * in->W;
     }
     out.ind_total = ind;
     out.words_total = words;
@@ -120,10 +134,11 @@ pm_multi_plan pm_plan_from_single(const pm_instance *inst, const pm_eval_plan &p
     mp.groups = plan.groups;
     mp.warps = plan.warps;
     mp.nb = plan.nb;
-    mp.grid = plan.grid;
     mp.probs.push_back(pm_single_prob(inst, plan, pop));
-    mp.items = plan.tiles * plan.splits;
-    mp.jobs = plan.tiles * std::max(plan.groups, 1) * inst->W;
+    mp.items = mp.probs[0].tiles * mp.probs[0].splits;
+    mp.grid = plan.direct.range ? mp.items : plan.grid;
+    mp.jobs = plan.direct.range ? pop : plan.tiles * std::max(plan.groups, 1) * inst->W;
+    mp.d_smem = plan.direct.smem;
     mp.tiles_total = plan.tiles;
     mp.ind_total = pm_round_up(std::max<int64_t>(pop, 1), 32);
     mp.words_total = pop * inst->W;
@@ -138,6 +153,7 @@ void pm_scan_launch_from(const pm_multi_plan &mp, const pm_prob *probs_dev, pm_s
     L.warps = mp.warps;
     L.nb = mp.nb;
     L.Wmax = mp.Wmax;
+    L.d_smem = mp.d_smem;
     L.grid = mp.grid;
     L.K = (int)mp.probs.size();
     L.one = mp.probs[0];

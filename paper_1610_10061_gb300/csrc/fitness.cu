@@ -49,6 +49,7 @@
 #include <cstdio>
 
 #include "pm_common.cuh"
+#include "scan_direct.cuh"
 #include "scan_tile.cuh"
 #include "scan_walk.cuh"
 
@@ -58,44 +59,6 @@ constexpr int kMaxG = 4;
 constexpr uint32_t kSpinLimit = 1u << 22;  // bounded mbarrier wait (a few seconds at most)
 constexpr uint32_t kStallSpinLimit = 1u << 14;  // the poll limit of a launch armed by pm_debug_scan_timeout
 constexpr int kCountShift = 48;            // packed split reduction: count in bits 48..63, sum below
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p)
-{
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t phase)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(phase)
-        : "memory");
-    return ok != 0;
-}
-
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
-{
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(dst)),
-        "l"(src), "r"(bytes), "r"(smem_u32(bar))
-        : "memory");
-}
 
 // Largest k in [0, K) with base(k) <= x (bases ascending, base(0) = 0).
 template <typename F>
@@ -116,7 +79,8 @@ __device__ __forceinline__ int find_prob(int K, int64_t x, F base)
 // Row-major population -> facility-major tiles, for every instance of the
 // launch.  colT[col_base + (tile*32W + j)*G + g] (j < 32W) = bits over
 // individuals tile*32G + 32g + b of that instance.  One warp per (instance,
-// tile, g, w) job; grid-stride over the jobs.
+// tile, g, w) job; grid-stride over the jobs.  Instances evaluated by open
+// facilities get their individuals' lists instead (a job per individual).
 // ---------------------------------------------------------------------------
 __global__ void k_pop_to_columns(const uint32_t *__restrict__ masks, const pm_prob *__restrict__ probs, int K,
                                  pm_prob one, int64_t jobs, int32_t G, uint32_t *__restrict__ colT)
@@ -131,6 +95,11 @@ __global__ void k_pop_to_columns(const uint32_t *__restrict__ masks, const pm_pr
             pr = probs + find_prob(K, job, [&](int k) { return probs[k].job_base; });
         const int64_t lj = job - pr->job_base;
         const int32_t W = pr->W;
+        if (pr->d_range) {  // a list of open facilities per individual in place of the facility-major form
+            write_open_list(masks + pr->word_base + lj * W, W, pr->m, pr->p, colT + pr->col_base,
+                            (pr->pop + 31) / 32 * 32, lj, lane);
+            continue;
+        }
         const int32_t w = (int32_t)(lj % W);
         const int64_t tg = lj / W;
         const int32_t g = (int32_t)(tg % G);
@@ -155,12 +124,12 @@ struct ScanEpilogue {
 // one warp per individual: store the cost, or
 // accept the candidate (copy its bitset, cost and improved flag) when it is
 // strictly cheaper than the current individual.
-template <int G>
-__device__ __forceinline__ void apply_epilogue(const unsigned long long *acc_s, const uint32_t *fin_s, const pm_prob &pr,
-                                               int64_t ind0, int warp, int nwarps, int lane, const ScanEpilogue &ep)
+__device__ __forceinline__ void apply_epilogue(const unsigned long long *acc_s, const uint32_t *fin_s, int count,
+                                               const pm_prob &pr, int64_t ind0, int warp, int nwarps, int lane,
+                                               const ScanEpilogue &ep)
 {
     const int32_t W = pr.W;
-    for (int i = warp; i < G * 32; i += nwarps) {
+    for (int i = warp; i < count; i += nwarps) {
         const int64_t t = ind0 + i;
         if (t >= pr.pop)
             break;
@@ -182,6 +151,116 @@ __device__ __forceinline__ void apply_epilogue(const unsigned long long *acc_s, 
     }
 }
 
+// Bounded wait of every thread for the bulk copies of `bar`'s phase.
+__device__ __forceinline__ bool wait_copies(uint64_t *bar, uint32_t phase, bool stalled, int *err)
+{
+    const uint32_t limit = stalled ? kStallSpinLimit : kSpinLimit;
+    uint32_t spins = 0;
+    while (!mbar_try_wait(bar, phase)) {
+        if (++spins > limit) {
+            if (threadIdx.x == 0)
+                atomicExch(err, (int)PM_ERR_TIMEOUT);
+            uint32_t extra = 0;  // the copy may still land: wait once more, bounded, then leave
+            while (!mbar_try_wait(bar, phase) && ++extra < limit) {
+            }
+            return false;
+        }
+    }
+    return true;
+}
+
+// One work item of the evaluation by open facilities.
+struct DirectItem {
+    uint32_t *smem;                       // the entries (d_chunks per stage), then the sums and the bit words
+    const uint32_t *__restrict__ lists;   // of the instance
+    const uint32_t *__restrict__ masks;   // rows of the launch
+    int64_t ind0;                         // individuals ind0 .. ind0 + count - 1 of the instance
+    int count;
+    const uint32_t *a0;                   // the ones to evaluate
+    uint32_t *fast;                       // scratch, count / 32 words
+    uint32_t *sums;                       // count 64-bit sums, zero on entry
+    int64_t c_begin, c_end;
+    uint64_t *bar;                        // one per stage
+    int *err;
+    bool stalled;                         // failure-detection tests: no copy is issued
+};
+
+// The first copies of an item (constant data: before the launch's dependency wait).  One thread.
+__device__ __forceinline__ void direct_start(const pm_prob &pr, const DirectItem &it)
+{
+    const int64_t left = (it.c_end - it.c_begin + 7) / 8;
+    if (left > 0 && !it.stalled)
+        direct_fill(pr, it.smem, it.c_begin / 8, (int)min(left, (int64_t)pr.d_chunks), &it.bar[0]);
+}
+
+// The item, after direct_start and with sums and a0 in place; phases: bit s = the phase of stage s's next copies,
+// returned for the next item (0xffffffff when a wait gave up).
+__device__ __forceinline__ uint32_t direct_item(const pm_prob &pr, const DirectItem &it, uint32_t phases, int warp,
+                                                int nwarps, int lane)
+{
+    const int groups = (int)((min((int64_t)it.count, pr.pop - it.ind0) + 31) / 32);
+    const uint32_t pitch = (uint32_t)((pr.pop + 31) / 32 * 32);
+    const uint32_t *lists = it.lists + it.ind0;
+    bool mine = false;  // a bitset without a list among this warp's
+    for (int g = warp; g < groups; g += nwarps) {
+        const uint32_t a0 = it.a0[g];
+        const bool listed = ((a0 >> lane) & 1u) && __ldg(lists + 32 * g + lane) != kNoList;
+        const uint32_t b = __ballot_sync(PM_FULL_MASK, listed);
+        mine |= b != a0;
+        if (lane == 0)
+            it.fast[g] = b;
+    }
+    const bool unlisted = __syncthreads_or(mine) != 0;
+    const int64_t all = (it.c_end - it.c_begin + 7) / 8;  // chunks of the item
+    const uint32_t ent = smem_u32(it.smem), stage_bytes = (uint32_t)(pr.d_chunks * pr.m) * 16u;
+    int stage = 0;
+    for (int64_t c8 = 0; c8 < all; c8 += pr.d_chunks) {
+        const int64_t next = c8 + pr.d_chunks;
+        const int next_chunks = (int)min(all - next, (int64_t)pr.d_chunks);
+        if (pr.d_stages == 2 && next_chunks > 0 && threadIdx.x == 0 && !it.stalled)
+            direct_fill(pr, reinterpret_cast<char *>(it.smem) + (stage ^ 1) * stage_bytes, it.c_begin / 8 + next,
+                        next_chunks, &it.bar[stage ^ 1]);
+        if (!wait_copies(&it.bar[stage], (phases >> stage) & 1u, it.stalled, it.err))
+            return 0xffffffffu;
+        phases ^= 1u << stage;
+        const int chunks = (int)min(all - c8, (int64_t)pr.d_chunks);
+        if (chunks * groups >= 2 * nwarps)  // two individuals per lane as long as every warp has a task
+            direct_terms<2>(pr, ent + stage * stage_bytes, chunks, lists, pitch, groups, it.fast, it.sums, warp, nwarps,
+                            lane);
+        else
+            direct_terms<1>(pr, ent + stage * stage_bytes, chunks, lists, pitch, groups, it.fast, it.sums, warp, nwarps,
+                            lane);
+        __syncthreads();
+        if (pr.d_stages == 2)
+            stage ^= 1;
+        else if (next_chunks > 0 && threadIdx.x == 0 && !it.stalled)
+            direct_fill(pr, it.smem, it.c_begin / 8 + next, next_chunks, &it.bar[0]);
+    }
+    if (!unlisted)
+        return phases;
+    for (int i = 0; i < 32 * groups; ++i) {
+        if (!(((it.a0[i >> 5] & ~it.fast[i >> 5]) >> (i & 31)) & 1u))
+            continue;
+        unsigned long long sum = 0ull;
+        for (int64_t c = it.c_begin + warp; c < it.c_end; c += nwarps)
+            sum += row_term(pr, it.masks + pr.word_base + (it.ind0 + i) * pr.W, c, lane);
+        if (lane == 0 && sum)
+            atomicAdd(reinterpret_cast<unsigned long long *>(it.sums) + i, sum);
+    }
+    __syncthreads();
+    return phases;
+}
+
+// The same as a function of its own: beside the bit-sliced walk's registers in the kernel that does both.
+__device__ __noinline__ uint32_t direct_item_call(const pm_prob &pr, const DirectItem &it, uint32_t phases)
+{
+    return direct_item(pr, it, phases, threadIdx.x >> 5, blockDim.x >> 5, threadIdx.x & 31);
+}
+
+// What a launch's work items are: scanned client by client, scanned bit-sliced, evaluated by open facilities, or
+// (several instances) bit-sliced and by open facilities.
+enum class ScanKind { clients, sliced, direct, mixed };
+
 // ---------------------------------------------------------------------------
 // The column scan kernel (with the split reduction and epilogue fused), over
 // every instance of the launch.  Persistent: CTA b takes work items b, b +
@@ -189,19 +268,22 @@ __device__ __forceinline__ void apply_epilogue(const unsigned long long *acc_s, 
 // running at the same time walk the same clients for different tiles and
 // the rows they stream are shared through L2.
 // ---------------------------------------------------------------------------
-template <int G, bool kSliced>
-__global__ void __launch_bounds__(kSliced ? 512 : 1024)
+template <int G, ScanKind kKind>
+__global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
     k_scan_columns(const pm_prob *__restrict__ probs, int K, pm_prob one, int64_t items,
-                   const uint32_t *__restrict__ colT, const uint32_t *__restrict__ active,
-                   unsigned long long *__restrict__ accum, int *__restrict__ tickets, int *__restrict__ err,
-                   ScanEpilogue ep, uint32_t stall, int nb, uint32_t tab_off)
+                   const uint32_t *__restrict__ colT, const uint32_t *__restrict__ masks,
+                   const uint32_t *__restrict__ active, unsigned long long *__restrict__ accum,
+                   int *__restrict__ tickets, int *__restrict__ err, ScanEpilogue ep, uint32_t stall, int nb,
+                   uint32_t tab_off)
 {
     // the previous kernel of the stream may still run until pm_grid_dependency_wait(): before it only the
     // constant tables (Pi', Delta', the launch's problem table) are read
+    constexpr bool kSliced = kKind == ScanKind::sliced || kKind == ScanKind::mixed;
+    constexpr bool kDirect = kKind == ScanKind::direct || kKind == ScanKind::mixed;
     extern __shared__ __align__(128) uint32_t colbits[];  // [32W][G], then (kSliced, at tab_off) the warps' tables
-    __shared__ unsigned long long acc_s[G * 32];
-    __shared__ uint32_t a0_s[G], fin_s[G];
-    __shared__ __align__(8) uint64_t bar;
+    __shared__ unsigned long long tile_acc[G * 32];
+    __shared__ uint32_t tile_a0[G], tile_fin[G];
+    __shared__ __align__(8) uint64_t bar, d_bar[2];
     __shared__ int last_s;
     __shared__ pm_prob pr_s;
 
@@ -214,12 +296,13 @@ __global__ void __launch_bounds__(kSliced ? 512 : 1024)
 
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
+        mbar_init(&d_bar[0], 1);
+        mbar_init(&d_bar[1], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    [[maybe_unused]] uint32_t d_phases = 0;
     [[maybe_unused]] TileWalk<G> walk;
     const uint32_t my_tab = tab_off + (uint32_t)(warp * tile_table_words(nb, G));
-    if constexpr (kSliced)
-        TileWalk<G>::clear_table(colbits + my_tab, nb, lane);
     __syncthreads();
 
     uint32_t phase = 0;
@@ -234,12 +317,20 @@ __global__ void __launch_bounds__(kSliced ? 512 : 1024)
         const int64_t tile = li % pr.tiles;
         const int64_t split = li / pr.tiles;
         const int64_t gtile = pr.tile_base + tile;
-        const int64_t ind0 = tile * 32 * G;  // first individual of the tile, within the instance
         const int32_t W = pr.W, L = pr.L;
         const int64_t pop = pr.pop, stride = pr.stride;
         const uint16_t *__restrict__ pi = pr.pi;
         const int32_t *__restrict__ delta = pr.delta;
         const bool reload = gtile != loaded_tile;
+        const bool direct = kKind == ScanKind::direct || (kKind == ScanKind::mixed && pr.d_range != 0);
+        // the item's individuals: ind0 .. ind0 + count - 1 within the instance; their sums, the ones to evaluate
+        // and the ones whose epilogue this CTA applies (bit i of word i / 32)
+        const int count = direct ? pr.d_range : G * 32;
+        const int64_t ind0 = tile * count;
+        uint32_t *d_sums = colbits + (size_t)pr.d_stages * pr.d_chunks * pr.m * 4;
+        unsigned long long *acc_s = direct ? reinterpret_cast<unsigned long long *>(d_sums) : tile_acc;
+        uint32_t *a0_s = direct ? d_sums + 2 * count : tile_a0;
+        uint32_t *fin_s = direct ? a0_s + count / 32 : tile_fin;
 
         // first steps of this warp's first two clients (constant tables), loaded while the tile lands
         const int64_t c_begin = split * pr.cps;
@@ -258,9 +349,15 @@ __global__ void __launch_bounds__(kSliced ? 512 : 1024)
         [[maybe_unused]] uint32_t j_cur, j_nxt, j_nc, j_nc1;
         [[maybe_unused]] int32_t d_cur, d_nxt, d_nc, d_nc1;
         const TileRows rows{pi, delta, stride, L, pr.cum != 0, pr.flush_units};
+        [[maybe_unused]] const DirectItem d_item{colbits, colT + pr.col_base, masks, ind0, count, a0_s,  fin_s,
+                                                 d_sums,  c_begin,            c_end, d_bar, err,  stalled};
+        if constexpr (kDirect)
+            if (direct && threadIdx.x == 0)
+                direct_start(pr, d_item);
         if constexpr (kSliced) {
-            walk.prefetch(rows, c_begin, c_end, warp, lane);
-        } else {
+            if (!direct)
+                walk.prefetch(rows, c_begin, c_end, warp, lane);
+        } else if constexpr (kKind == ScanKind::clients) {
             load(c, 0, j_cur, d_cur);
             load(c, 32, j_nxt, d_nxt);
             load(c + nwarps, 0, j_nc, d_nc);
@@ -273,7 +370,9 @@ __global__ void __launch_bounds__(kSliced ? 512 : 1024)
 
         // stalled (failure-detection tests only): no copy is issued and nothing arrives on the barrier, so the
         // bounded wait below runs out with nothing in flight
-        if (reload && threadIdx.x == 0 && !stalled) {
+        if (reload && !direct && threadIdx.x == 0 && !stalled) {
+            // the tile's memory was read and (distance entries, tables) written by ordinary accesses before
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             const uint32_t tile_bytes = (uint32_t)W * 32u * G * 4u;
             mbar_arrive_expect_tx(&bar, tile_bytes);
             const char *src = reinterpret_cast<const char *>(colT + pr.col_base + tile * (int64_t)W * 32 * G);
@@ -283,44 +382,47 @@ __global__ void __launch_bounds__(kSliced ? 512 : 1024)
                 bulk_g2s(dst + off, src + off, sz, &bar);
             }
         }
-        if (warp < G) {
-            const int64_t t = ind0 + 32 * warp + lane;
+        for (int g = warp; g < count / 32; g += nwarps) {
+            const int64_t t = ind0 + 32 * g + lane;
             const int64_t tg = pr.ind_base + t;
             const bool on = (t < pop) && (active == nullptr || ((__ldg(active + (tg >> 5)) >> (tg & 31)) & 1u));
             const uint32_t b = __ballot_sync(PM_FULL_MASK, on);
             if (lane == 0)
-                a0_s[warp] = b;
+                a0_s[g] = b;
         }
-        for (int i = threadIdx.x; i < G * 32; i += blockDim.x)
+        for (int i = threadIdx.x; i < count; i += blockDim.x)
             acc_s[i] = 0ull;
+        if constexpr (kSliced)
+            if (!direct)
+                TileWalk<G>::clear_table(colbits + my_tab, nb, lane);
 
-        if (reload) {
-            // bounded wait for the tile (every thread waits)
-            const uint32_t limit = stalled ? kStallSpinLimit : kSpinLimit;
-            uint32_t spins = 0;
-            while (!mbar_try_wait(&bar, phase)) {
-                if (++spins > limit) {
-                    if (threadIdx.x == 0)
-                        atomicExch(err, (int)PM_ERR_TIMEOUT);
-                    uint32_t extra = 0;  // the copy may still land: wait once more, bounded, then leave
-                    while (!mbar_try_wait(&bar, phase) && ++extra < limit) {
-                    }
-                    return;
-                }
-            }
+        if (reload && !direct) {
+            if (!wait_copies(&bar, phase, stalled, err))
+                return;
             phase ^= 1u;
             loaded_tile = gtile;
         }
         __syncthreads();
 
-        if constexpr (kSliced) {
+        if constexpr (kDirect) {
+            if (direct) {
+                d_phases = kKind == ScanKind::direct ? direct_item(pr, d_item, d_phases, warp, nwarps, lane)
+                                                     : direct_item_call(pr, d_item, d_phases);
+                if (d_phases == 0xffffffffu)
+                    return;
+                loaded_tile = -1;  // the entries took the tile's place
+            }
+        }
+
+        if (kDirect && direct) {
+        } else if constexpr (kSliced) {
             uint32_t any0 = 0;
 #pragma unroll
             for (int g = 0; g < G; ++g)
                 any0 |= a0_s[g];
             if (any0 && c_begin < c_end)
                 walk.run(colbits, my_tab, nb, a0_s[lane % G], rows, c_begin, c_end, warp, nwarps, lane, acc_s);
-        } else {
+        } else if constexpr (kKind == ScanKind::clients) {
             uint32_t a0[G];
             uint32_t any0 = 0;
 #pragma unroll
@@ -349,28 +451,47 @@ __global__ void __launch_bounds__(kSliced ? 512 : 1024)
             // one atomic per individual carries the split's sum plus one count in the top 16 bits; the split
             // that brings the count to `splits` holds the total, applies that individual's epilogue and leaves
             // the word zero for the next launch -- no fences, no tile ticket
-            for (int i = threadIdx.x; i < G * 32; i += blockDim.x) {
-                const int64_t t = ind0 + i;
-                bool last = false;
-                if (t < pop && ((a0_s[i >> 5] >> (i & 31)) & 1u)) {
-                    const unsigned long long add = acc_s[i] + (1ull << kCountShift);
-                    const unsigned long long old = atomicAdd(accum + pr.ind_base + t, add);
-                    if ((old >> kCountShift) == (unsigned long long)(pr.splits - 1)) {
-                        acc_s[i] = (old + add) & ((1ull << kCountShift) - 1ull);
-                        accum[pr.ind_base + t] = 0ull;
-                        last = true;
+            // (four individuals per thread in flight, each CTA from another start: a wide item's atomics would
+            // otherwise wait one after another, and all CTAs' for the same words)
+            constexpr int kFlight = kDirect ? 4 : 1;
+            const int start = direct ? (int)((blockIdx.x * 352u) % (unsigned)count) : 0;
+            for (int i0 = threadIdx.x; i0 < count; i0 += kFlight * blockDim.x) {
+                unsigned long long add[kFlight], old[kFlight];
+#pragma unroll
+                for (int f = 0; f < kFlight; ++f) {
+                    int i = i0 + f * (int)blockDim.x;
+                    add[f] = 0ull;
+                    if (i < count) {
+                        i = i + start >= count ? i + start - count : i + start;
+                        if (ind0 + i < pop && ((a0_s[i >> 5] >> (i & 31)) & 1u)) {
+                            add[f] = acc_s[i] + (1ull << kCountShift);
+                            old[f] = atomicAdd(accum + pr.ind_base + ind0 + i, add[f]);
+                        }
                     }
                 }
-                const uint32_t b = __ballot_sync(PM_FULL_MASK, last);
-                if ((i & 31) == 0)
-                    fin_s[i >> 5] = b;
+#pragma unroll
+                for (int f = 0; f < kFlight; ++f) {
+                    int i = i0 + f * (int)blockDim.x;
+                    if (i >= count)
+                        break;
+                    i = i + start >= count ? i + start - count : i + start;
+                    const bool last = add[f] != 0ull &&
+                                      (old[f] >> kCountShift) == (unsigned long long)(pr.splits - 1);
+                    if (last) {
+                        acc_s[i] = (old[f] + add[f]) & ((1ull << kCountShift) - 1ull);
+                        accum[pr.ind_base + ind0 + i] = 0ull;
+                    }
+                    const uint32_t b = __ballot_sync(PM_FULL_MASK, last);
+                    if ((i & 31) == 0)
+                        fin_s[i >> 5] = b;
+                }
             }
             __syncthreads();
             fin = fin_s;
         } else if (pr.splits > 1) {
             // add this split's sums into the instance's accumulators; the last split of the tile
             // (atomic ticket) reads the totals and leaves the accumulators zero again
-            for (int i = threadIdx.x; i < G * 32; i += blockDim.x) {
+            for (int i = threadIdx.x; i < count; i += blockDim.x) {
                 const int64_t t = ind0 + i;
                 if (t < pop && acc_s[i] != 0ull)
                     atomicAdd(accum + pr.ind_base + t, acc_s[i]);
@@ -383,7 +504,7 @@ __global__ void __launch_bounds__(kSliced ? 512 : 1024)
             finish = last_s != 0;
             if (finish) {
                 __threadfence();
-                for (int i = threadIdx.x; i < G * 32; i += blockDim.x) {
+                for (int i = threadIdx.x; i < count; i += blockDim.x) {
                     const int64_t t = ind0 + i;
                     if (t < pop) {
                         acc_s[i] = __ldcg(accum + pr.ind_base + t);
@@ -396,7 +517,7 @@ __global__ void __launch_bounds__(kSliced ? 512 : 1024)
             }
         }
         if (finish)
-            apply_epilogue<G>(acc_s, fin, pr, ind0, warp, nwarps, lane, ep);
+            apply_epilogue(acc_s, fin, count, pr, ind0, warp, nwarps, lane, ep);
         __syncthreads();  // shared state (tile, acc_s, a0_s, pr_s) is reused by the next item
     }
 }
@@ -561,12 +682,24 @@ __global__ void k_wait_selftest(int *__restrict__ err, uint32_t limit)
 
 // The column kernel for G groups, with the bit-sliced walk or the client walk.
 using scan_kernel = void (*)(const pm_prob *, int, pm_prob, int64_t, const uint32_t *, const uint32_t *,
-                             unsigned long long *, int *, int *, ScanEpilogue, uint32_t, int, uint32_t);
-scan_kernel scan_fn(int G, bool sliced)
+                             const uint32_t *, unsigned long long *, int *, int *, ScanEpilogue, uint32_t, int, uint32_t);
+template <ScanKind kKind>
+scan_kernel scan_fn_of(int G)
 {
-    if (sliced)
-        return G == 4 ? k_scan_columns<4, true> : (G == 2 ? k_scan_columns<2, true> : k_scan_columns<1, true>);
-    return G == 4 ? k_scan_columns<4, false> : (G == 2 ? k_scan_columns<2, false> : k_scan_columns<1, false>);
+    return G == 4 ? k_scan_columns<4, kKind> : (G == 2 ? k_scan_columns<2, kKind> : k_scan_columns<1, kKind>);
+}
+scan_kernel scan_fn(int G, ScanKind kind)
+{
+    switch (kind) {
+    case ScanKind::sliced:
+        return scan_fn_of<ScanKind::sliced>(G);
+    case ScanKind::direct:
+        return k_scan_columns<1, ScanKind::direct>;
+    case ScanKind::mixed:
+        return scan_fn_of<ScanKind::mixed>(G);
+    default:
+        return scan_fn_of<ScanKind::clients>(G);
+    }
 }
 
 }  // namespace
@@ -591,8 +724,8 @@ static pm_status allow_dynamic_smem(const pm_instance *inst, F *fn)
 pm_status pm_fitness_init(const pm_instance *inst)
 {
     for (int G : {1, 2, 4})
-        for (bool sliced : {false, true})
-            PM_TRY(allow_dynamic_smem(inst, scan_fn(G, sliced)));
+        for (ScanKind kind : {ScanKind::clients, ScanKind::sliced, ScanKind::direct, ScanKind::mixed})
+            PM_TRY(allow_dynamic_smem(inst, scan_fn(G, kind)));
     PM_TRY(allow_dynamic_smem(inst, k_scan_rows<false>));
     PM_TRY(allow_dynamic_smem(inst, k_scan_rows<true>));
     return PM_OK;
@@ -622,12 +755,54 @@ void pm_walk_shape(const pm_instance *inst, int64_t W, int G, double depth, int 
     nb = 0;
 }
 
+size_t pm_direct_smem(int64_t m, int range, int chunks)  // chunks: of all stages
+{
+    return (size_t)chunks * m * 16 + (size_t)range * 8 + (size_t)(range / 32) * 8;
+}
+
+double pm_scan_cost(int64_t m, int64_t p) { return 0.35 + 0.037 * (double)(m + 1) / (double)(p + 1); }
+
+double pm_direct_cost(int64_t m, int64_t p, int64_t range, int stages)
+{
+    return 0.35 + 0.05 * (double)p + (stages == 2 ? 0.03 : 0.1) * (double)m / (double)range;
+}
+
+void pm_direct_shape(const pm_instance *inst, int64_t pop, size_t budget, int nwarps, pm_direct_plan &out)
+{
+    out = pm_direct_plan();
+    // the lists take the place of the facility-major form: p / 2 words per individual must not exceed its W
+    if (!inst->dense || (inst->p + 1) / 2 > inst->W || (int64_t)pm_round_up(pop, 32) * ((inst->p + 1) / 2) >= 1ll << 32)
+        return;
+    int r = (int)std::min<int64_t>(kDirectRange, pm_round_up(pop, 32));
+    while (r > 32 && pm_direct_smem(inst->m, r, 1) > budget)
+        r = (int)pm_round_up(r / 2, 32);
+    const int stages = pm_direct_smem(inst->m, r, 2) <= budget ? 2 : 1;
+    if (pm_direct_smem(inst->m, r, 1) > budget ||
+        pm_direct_cost(inst->m, inst->p, r, stages) >= pm_scan_cost(inst->m, inst->p))
+        return;
+    out.range = r;
+    out.chunks = 1;
+    out.stages = stages;
+    // enough (chunk, 32 individuals) tasks for every warp
+    while (out.chunks < 16 && out.chunks * (r / 32) < 2 * nwarps &&
+           pm_direct_smem(inst->m, r, 2 * out.chunks * out.stages) <= budget)
+        out.chunks *= 2;
+    out.smem = pm_direct_smem(inst->m, r, out.chunks * out.stages);
+}
+
+bool pm_direct_wanted(int64_t n, int64_t m, int64_t p, size_t smem_optin)
+{
+    // at most 1 GiB beside tables of three times that; the widest range a CTA takes
+    return n * m <= ((int64_t)1 << 29) && pm_direct_smem(m, 32, 1) + 4096 <= smem_optin &&
+           pm_direct_cost(m, p, kDirectRange, 1) < pm_scan_cost(m, p);
+}
+
 // Resident CTAs per SM of the column kernel for a plan's (G, warps, nb) at this instance's W.
 static int column_ctas_per_sm(const pm_instance *inst, const pm_eval_plan &plan)
 {
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &nb, reinterpret_cast<const void *>(scan_fn(plan.groups, plan.nb > 0)), plan.warps * 32,
+            &nb, reinterpret_cast<const void *>(scan_fn(plan.groups, plan.nb > 0 ? ScanKind::sliced : ScanKind::clients)), plan.warps * 32,
             pm_scan_smem(inst->W, plan.groups, plan.warps, plan.nb)) != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -695,7 +870,47 @@ pm_eval_plan pm_plan_eval(const pm_instance *inst, int64_t pop)
         G /= 2;
     // 32 warps when only one CTA fits per SM, else 16
     const int warps = 2 * column_smem_bytes(inst->W, G) + 8192 > inst->smem_optin ? 32 : 16;
-    return pm_plan_eval_with(inst, pop, G, warps, 0);
+    pm_eval_plan plan = pm_plan_eval_with(inst, pop, G, warps, 0);
+    pm_plan_direct(inst, pop, plan);
+    return plan;
+}
+
+bool pm_plan_direct(const pm_instance *inst, int64_t pop, pm_eval_plan &plan)
+{
+    const size_t budget = inst->smem_optin > 4096 ? inst->smem_optin - 4096 : 0;
+    if (!plan.nb)
+        return false;
+    pm_direct_shape(inst, pop, budget, plan.warps, plan.direct);
+    if (!plan.direct.range)
+        return false;
+    // one work item per resident CTA (one per SM: the entries take most of the shared memory), whole rounds of chunks
+    const int64_t ranges = pm_ceil_div(pop, plan.direct.range);
+    pm_direct_splits(inst, std::max<int64_t>(1, inst->sm_count / ranges), plan.direct);
+    return plan.direct.range != 0;
+}
+
+void pm_direct_splits(const pm_instance *inst, int64_t want, pm_direct_plan &d)
+{
+    // whole rounds of chunks where that leaves enough splits, else whole chunks; 32-bit sums allow 2^16 clients of
+    // distances below 2^16 an item
+    const int64_t cps = pm_ceil_div(inst->n, std::max<int64_t>(1, want));
+    const int64_t round = cps >= 8 * 8 * d.chunks ? 8 * d.chunks : 8;
+    d.cps = std::min<int64_t>(pm_round_up(cps, round), 65536 / round * round);
+    d.splits = pm_ceil_div(inst->n, d.cps);
+    if (d.splits >= 65536)
+        d = pm_direct_plan();
+}
+
+void pm_direct_prob(const pm_instance *inst, const pm_direct_plan &d, int64_t pop, pm_prob &pr)
+{
+    pr.d_range = d.range;
+    pr.d_chunks = d.chunks;
+    pr.d_stages = d.stages;
+    pr.dense = inst->dense;
+    pr.tiles = pm_ceil_div(pop, d.range);
+    pr.splits = d.splits;
+    pr.cps = d.cps;
+    pr.packed = pm_packed_reduction_ok(inst, d.splits) ? 1 : 0;
 }
 
 size_t pm_plan_partial_bytes(const pm_eval_plan &plan, int64_t pop)
@@ -732,6 +947,8 @@ pm_prob pm_single_prob(const pm_instance *inst, const pm_eval_plan &plan, int64_
     pr.tiles = plan.tiles;
     pr.splits = plan.splits;
     pr.cps = pm_ceil_div(inst->n, plan.splits);
+    if (plan.direct.range)
+        pm_direct_prob(inst, plan.direct, pop, pr);
     return pr;  // every base 0
 }
 
@@ -779,8 +996,10 @@ pm_status pm_launch_columns(const pm_instance *inst, const pm_eval_plan &plan, c
         return PM_OK;
     if (plan.groups == 0)
         return PM_ERR_UNSUPPORTED;
-    return launch_transpose(masks, nullptr, 1, pm_single_prob(inst, plan, pop), plan.tiles * plan.groups * inst->W,
-                            plan.groups, colT, stream);
+    pm_eval_plan columns = plan;
+    columns.direct = pm_direct_plan();
+    return launch_transpose(masks, nullptr, 1, pm_single_prob(inst, columns, pop),
+                            plan.tiles * plan.groups * inst->W, plan.groups, colT, stream);
 }
 
 pm_status pm_launch_scan(const pm_scan_launch &L, const pm_accept_args &acc, int64_t *costs, cudaStream_t stream)
@@ -802,8 +1021,11 @@ pm_status pm_launch_scan(const pm_scan_launch &L, const pm_accept_args &acc, int
     unsigned long long *accum = reinterpret_cast<unsigned long long *>(L.accum);
     const uint32_t stall = take_stall() ? 1u : 0u;
     const uint32_t tab_off = (uint32_t)(column_smem_bytes(L.Wmax, G) / 4);
-    PM_CUDA(pm_launch(scan_fn(G, L.nb > 0), grid, threads, pm_scan_smem(L.Wmax, G, L.warps, L.nb), stream, L.probs_dev,
-                      L.K, L.one, L.items, L.colT, L.active, accum, L.tickets, L.err, ep, stall, L.nb, tab_off));
+    const size_t smem = std::max(pm_scan_smem(L.Wmax, G, L.warps, L.nb), L.d_smem);
+    const ScanKind kind = L.d_smem == 0 ? (L.nb > 0 ? ScanKind::sliced : ScanKind::clients)
+                                        : (L.K == 1 ? ScanKind::direct : ScanKind::mixed);
+    PM_CUDA(pm_launch(scan_fn(G, kind), grid, threads, smem, stream, L.probs_dev, L.K, L.one, L.items, L.colT,
+                      L.masks, L.active, accum, L.tickets, L.err, ep, stall, L.nb, tab_off));
     return PM_OK;
 }
 
@@ -820,11 +1042,12 @@ pm_status pm_launch_eval(const pm_instance *inst, const pm_eval_plan &plan, cons
         L.warps = plan.warps;
         L.nb = plan.nb;
         L.Wmax = inst->W;
-        L.grid = plan.grid;
         L.K = 1;
         L.one = pm_single_prob(inst, plan, pop);
-        L.items = plan.tiles * plan.splits;
-        L.jobs = plan.tiles * plan.groups * inst->W;
+        L.items = L.one.tiles * L.one.splits;
+        L.grid = plan.direct.range ? L.items : plan.grid;
+        L.jobs = plan.direct.range ? pop : plan.tiles * plan.groups * inst->W;
+        L.d_smem = plan.direct.smem;
         L.masks = masks;
         L.colT = colT;
         L.active = active;

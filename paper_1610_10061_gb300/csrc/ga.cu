@@ -52,6 +52,7 @@
 
 #include "pm_alloc.h"
 #include "pm_common.cuh"
+#include "scan_direct.cuh"
 #include "scan_walk.cuh"
 
 // batch.cu
@@ -110,6 +111,7 @@ struct ga_prob {  // per instance layout of the GA arrays
     int64_t col_base;    // facility-major tiles
     uint32_t sid;
     uint32_t team;  // migration variant (ii): all deme bests into deme 0
+    uint32_t lists; // the scans evaluate this instance by open facilities: lists in place of the columns
 };
 
 // ----------------------------- Philox4x32-10 --------------------------------
@@ -213,13 +215,21 @@ struct ColumnsOut {
 
 // Transpose 32 rows (individuals t0 .. t0+31 of one instance, row r at
 // rows + r*rs) into that instance's tiles; rows of individuals >= pop read
-// as zero.  One warp, words w_begin, w_begin + w_step, ...
+// as zero.  One warp, words w_begin, w_begin + w_step, ...  Instances
+// evaluated by open facilities get the individuals' lists instead
+// (scan_direct.cuh), the warp taking rows w_begin, w_begin + w_step, ...
 __device__ __forceinline__ void write_columns(const uint32_t *rows, int64_t rs, int64_t t0, const ga_prob &gp,
                                               ColumnsOut co, int lane, int w_begin, int w_step)
 {
     if (co.colT == nullptr)
         return;
     const int32_t W = gp.W;
+    if (gp.lists) {
+        const int64_t pitch = (gp.pop + 31) / 32 * 32;
+        for (int r = w_begin; r < 32 && t0 + r < gp.pop; r += w_step)
+            write_open_list(rows + (int64_t)r * rs, W, gp.m, gp.p, co.colT + gp.col_base, pitch, t0 + r, lane);
+        return;
+    }
     const int64_t tile = t0 / (32 * co.G);
     const int32_t g = (int32_t)((t0 / 32) % co.G);
     for (int w = w_begin; w < W; w += w_step) {
@@ -2470,6 +2480,7 @@ static void ga_layout(pm_ga *ga)
         gp.best_base = bestw;
         gp.sid = ga->sid + (uint32_t)k;
         gp.team = ga->team ? 1u : 0u;
+        gp.lists = pr.d_range ? 1u : 0u;
         grp += pm_ceil_div(ga->P, 32);
         deme += ga->NB;
         dwords += ga->NB * in->W;
@@ -2500,6 +2511,7 @@ static void spec_layout(pm_ga *ga)
         gq.ind_base = pr.ind_base;
         gq.word_base = pr.word_base;
         gq.col_base = pr.col_base;
+        gq.lists = pr.d_range ? 1u : 0u;
         gq.grp_base = grp;
         grp += pm_ceil_div(QP, 32);
     }
@@ -2660,6 +2672,8 @@ static pm_status fused_prepare(pm_ga *ga, cudaStream_t s)
     const pm_instance *inst = ga->insts[0];
     const int G = ga->plan.groups;
     if (G != 1 && G != 2 && G != 4)
+        return PM_OK;
+    if (ga->gps[0].lists || ga->gq.lists)  // evaluated by open facilities: per-phase kernels only
         return PM_OK;
     int coop = 0;
     PM_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, inst->device));

@@ -67,6 +67,15 @@ struct pm_part {
 };
 pm_status pm_carve(pm_dbuf &arena, const pm_part *parts, int count);
 
+// The evaluation by open facilities (scan_direct.cuh): individuals per work item (0: not used), chunks of 8 clients
+// per stage of shared memory, stages (2: the next chunks' copies run under the present ones' work), client splits and
+// clients per split.
+struct pm_direct_plan {
+    int range = 0, chunks = 0, stages = 0;
+    int64_t splits = 0, cps = 0;
+    size_t smem = 0;
+};
+
 // Scratch for one fitness launch configuration (partial sums per client split).
 struct pm_eval_plan {
     int groups = 4;       // G: 32-individual groups per CTA
@@ -76,6 +85,9 @@ struct pm_eval_plan {
     int64_t grid = 0;     // CTAs launched (column kernel: persistent over tiles x splits items)
     int bytes = 0;        // row kernel only: each warp's bitset expanded to one byte per facility (byte masks)
     int nb = 0;           // column kernel: blocks of 32 ranks per table of the bit-sliced walk; 0: the client walk
+    // evaluation by open facilities in place of the scan, when direct.range > 0.  The column shape above stays the
+    // one the facility-major form and the scratch are laid out by.
+    pm_direct_plan direct;
 };
 
 // One instance inside an evaluation launch (host and device).  Individuals
@@ -91,6 +103,8 @@ struct pm_prob {
     int32_t cum;
     int32_t packed;  // split sums and a split count share one 64-bit word (see pm_packed_reduction_ok)
     uint32_t flush_units;  // bit-sliced walk: see pm_flush_units
+    int32_t d_range, d_chunks, d_stages;  // evaluation by open facilities (0: scan); tiles are d_range individuals
+    const uint16_t *dense;                // see pm_instance
     int64_t pop;
     int64_t ind_base;   // accumulators, active bits, GA per-individual arrays
     int64_t out_base;   // caller's cost array
@@ -99,7 +113,7 @@ struct pm_prob {
     int64_t tiles, tile_base;
     int64_t splits, cps;  // client splits and clients per split
     int64_t item_base;
-    int64_t job_base;     // transpose jobs (tiles * G * W per instance)
+    int64_t job_base;     // transpose jobs (tiles * G * W per instance; pop when its individuals get lists)
 };
 
 // Programmatic dependent launch.  Kernels of the GA generation and of the
@@ -146,6 +160,9 @@ struct pm_instance {
     bool cum = false;           // PM_TABLES_CUMULATIVE: delta holds D' (running sums of Delta') instead
     uint16_t *pi = nullptr;     // n x stride, Pi' (0-based facility ids)
     int32_t *delta = nullptr;   // n x stride, Delta'
+    // distances as 16 bits where the evaluation by open facilities may pay (else null): element ((c / 8) * m + j) * 8 +
+    // c % 8, ceil(n / 8) * m * 8 elements, zero for c >= n
+    uint16_t *dense = nullptr;
     int sm_count = 0;
     size_t smem_optin = 0;
     // staging and scratch for pm_eval_population
@@ -171,6 +188,8 @@ pm_eval_plan pm_plan_eval(const pm_instance *inst, int64_t pop);
 // A plan with explicit groups (0 = row kernel), warps per CTA and client
 // splits (0 = one full wave).
 pm_eval_plan pm_plan_eval_with(const pm_instance *inst, int64_t pop, int G, int warps, int splits_hint);
+// Evaluate by open facilities under this plan where that is the cheaper way (fills plan.direct).
+bool pm_plan_direct(const pm_instance *inst, int64_t pop, pm_eval_plan &plan);
 // Bytes of per-tile tickets the plan needs (zero before the first launch;
 // every launch leaves them zero, whatever the plan).
 size_t pm_plan_ticket_bytes(const pm_eval_plan &plan);
@@ -203,6 +222,7 @@ struct pm_scan_launch {
     int groups = 4, warps = 16;
     int nb = 0;                          // as pm_eval_plan
     int64_t Wmax = 0;                    // bitset words of the widest instance (sizes the shared memory)
+    size_t d_smem = 0;                   // bytes the evaluation by open facilities needs (0: no instance uses it)
     int64_t grid = 0;
     int K = 1;
     const pm_prob *probs_dev = nullptr;  // K > 1: device table
@@ -221,6 +241,21 @@ size_t pm_scan_smem(int64_t W, int G, int warps, int nb);
 // Warps (at most `warps`) and table blocks of the bit-sliced walk for tiles of W words and walks whose deepest
 // rank is about `depth`; nb = 0 and warps unchanged where the tables do not fit beside the tile.
 void pm_walk_shape(const pm_instance *inst, int64_t W, int G, double depth, int &warps, int &nb);
+// Evaluation by open facilities (scan_direct.cuh): shared-memory bytes of `chunks` resident chunks and `range`
+// individuals; the range, chunks and stages for `pop` individuals on inst (range 0: not to be used) within `budget`
+// bytes of shared memory and for `nwarps` warps; its client splits, about `want`; the launch's table entry.
+size_t pm_direct_smem(int64_t m, int range, int chunks);
+void pm_direct_shape(const pm_instance *inst, int64_t pop, size_t budget, int nwarps, pm_direct_plan &out);
+void pm_direct_splits(const pm_instance *inst, int64_t want, pm_direct_plan &d);
+void pm_direct_prob(const pm_instance *inst, const pm_direct_plan &d, int64_t pop, struct pm_prob &pr);
+// Estimated SM cycles per (individual, client) pair of the two ways, fitted to evaluations of 256 to 4096 subsets of
+// 300 to 10000 facilities, p = 3 to 1000: the scan's walk grows with the expected first open rank (1.76 cycles at m /
+// p = 33, 4.0 at 100, 12.7 at 322); p reads of 16 bytes for 8 pairs (1.05 cycles at p = 10, 3.4 at 60) plus the fill of
+// a chunk of m entries for `range` individuals, hidden but for its ends with two stages.
+double pm_scan_cost(int64_t m, int64_t p);
+double pm_direct_cost(int64_t m, int64_t p, int64_t range, int stages);
+// Whether an instance of these sizes should keep the 16-bit distances.
+bool pm_direct_wanted(int64_t n, int64_t m, int64_t p, size_t smem_optin);
 // Whether a launch has enough units of 1024 (client, individual) pairs for the bit-sliced walk: a unit is a chain
 // of about 1200 instructions of one warp, so with fewer than 12 per SM the SMs wait for single warps and the client
 // walk, which spreads one client over a warp, is the faster one (graph900 generation, 904 units per scan: 209 us
@@ -279,6 +314,7 @@ struct pm_multi_plan {
     int64_t grid = 0, items = 0, jobs = 0;
     int64_t tiles_total = 0, ind_total = 0, words_total = 0, cols_total = 0;
     int64_t Wmax = 0;  // bitset words of the widest instance
+    size_t d_smem = 0;
     std::vector<pm_prob> probs;
 };
 // Plan for `insts` with pops[k] individuals each; items_per_slot work items per

@@ -1,0 +1,195 @@
+// The evaluation by open facilities, for few of them: an individual's term at
+// a client is the smallest of its p open facilities' distances (the value the
+// scan of Section 4.2 stops at), so with p far below the (m + 1) / (p + 1)
+// ranks of a scan it is cheaper to read the p distances than to look for the
+// first open rank.
+//
+// The instance keeps its distances in 16 bits, in entries of eight clients:
+// entry (c / 8) * m + j holds facility j's distances to the clients c .. c + 7
+// in 16 bytes (built with the tables when every distance is below 2^16 and p
+// is small).  A CTA brings chunks (the m entries of eight clients) into shared
+// memory with bulk copies -- the next ones while it works on the present ones
+// where two sets fit -- and a lane owns an individual and reads one entry per
+// open facility (its id from the individual's list, two to a word, coalesced
+// over the individuals), taking the minimum of eight distances in four packed
+// instructions.  Sums are 32-bit in shared memory, for up to kDirectRange
+// individuals a CTA.
+//
+// Measured on GB300, 4096 subsets of 10000 x 10000 points: p = 3 / 10 / 30 /
+// 60 in 0.100 / 0.137 / 0.258 / 0.442 ms against 6.47 / 3.81 / 1.66 / 0.858
+// for the bit-sliced scan.  Bound by shared memory: 32 lanes' random entries
+// take about 11 wavefronts (0.047 SM cycles per pair and open facility), the
+// rest is the fill (200 MB of entries, 30 us of HBM time here, exposed where
+// only one stage fits).  Row-major distances with the entries put together by
+// the CTA (eight loads, eight permutations, two stores per pair of facilities)
+// took 0.21 ms at p = 10: the loads' latency was the CTA's critical path.
+//
+// A bitset without exactly p open facilities (unchecked calls only) has no
+// list; its terms come from a walk of the Pi' rows, as the scan defines them.
+#pragma once
+
+#include <cstdint>
+
+#include "bulk_copy.cuh"
+#include "pm_common.cuh"
+
+constexpr int kDirectRange = 4096;           // individuals of one work item, at most
+constexpr uint32_t kNoList = 0xffffffffu;    // first list word of a bitset without exactly p open facilities
+
+// The list of one individual's open facilities, by one warp: ids 2q and 2q+1
+// in word q of lists[q * pitch + t] (the last id twice when p is odd), or
+// kNoList in word 0.  row: the individual's W words (bits at or above m are
+// ignored, as the scan ignores them).
+__device__ __forceinline__ void write_open_list(const uint32_t *row, int32_t W, int32_t m, int32_t p, uint32_t *lists,
+                                                int64_t pitch, int64_t t, int lane)
+{
+    int count = 0;
+    for (int base = 0; base < W; base += 32) {
+        const int w = base + lane;
+        uint32_t x = w < W ? row[w] : 0u;
+        if (w == W - 1 && (m & 31))
+            x &= (1u << (m & 31)) - 1u;
+        const int n = __popc(x);
+        int incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(PM_FULL_MASK, incl, o);
+            if (lane >= o)
+                incl += y;
+        }
+        for (int pos = count + incl - n; x; ++pos) {
+            const uint16_t id = (uint16_t)(32 * w + __ffs(x) - 1);
+            x &= x - 1u;
+            if (pos < p)
+                reinterpret_cast<uint16_t *>(lists + (int64_t)(pos >> 1) * pitch + t)[pos & 1] = id;
+            if (pos == p - 1 && (p & 1))
+                reinterpret_cast<uint16_t *>(lists + (int64_t)(pos >> 1) * pitch + t)[1] = id;
+        }
+        count += __shfl_sync(PM_FULL_MASK, incl, 31);
+    }
+    __syncwarp();
+    if (count != p && lane == 0)
+        lists[t] = kNoList;
+}
+
+__device__ __forceinline__ uint32_t min_u16x2(uint32_t a, uint32_t b)
+{
+    uint32_t r;
+    asm("min.u16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
+// Copy the entries of `chunks` chunks from chunk c8 on to `dst` (shared), completing on `bar`.  One thread.
+__device__ __forceinline__ void direct_fill(const pm_prob &pr, void *dst, int64_t c8, int chunks, uint64_t *bar)
+{
+    const uint32_t bytes = (uint32_t)chunks * (uint32_t)pr.m * 16u;
+    const char *src = reinterpret_cast<const char *>(pr.dense) + c8 * (int64_t)pr.m * 16;
+    // the memory was read (and, for other kinds of items, written) by ordinary accesses before
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    mbar_arrive_expect_tx(bar, bytes);
+    for (uint32_t off = 0; off < bytes; off += 32768u)
+        bulk_g2s(static_cast<char *>(dst) + off, src + off, min(bytes - off, 32768u), bar);
+}
+
+// The resident chunks' terms of the individuals marked in fast[] (bit i of word i / 32, individual ind0 + i) into
+// sums[2 i] (the low words of the 64-bit sums).  One task = one chunk and 32 NI individuals, NI per lane.
+template <int NI>
+__device__ __forceinline__ void direct_terms(const pm_prob &pr, uint32_t ent, int chunks,
+                                             const uint32_t *__restrict__ lists, uint32_t pitch, int groups,
+                                             const uint32_t *fast, uint32_t *sums, int warp, int nwarps, int lane)
+{
+    const uint32_t words = (uint32_t)(pr.p + 1) / 2;
+    for (int k = 0, g0 = warp * NI; k < chunks;) {
+        if (g0 >= groups) {
+            g0 -= (groups + NI - 1) / NI * NI;
+            ++k;
+            continue;
+        }
+        const uint32_t base = ent + (uint32_t)(k * pr.m) * 16u;
+        bool on[NI];
+        uint32_t at[NI], v[NI][4];
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+            on[i] = g0 + i < groups && ((fast[g0 + i] >> lane) & 1u);
+            at[i] = 32u * (g0 + i) + lane;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                v[i][j] = ~0u;
+        }
+        auto use = [&](const uint32_t (&ids)[NI]) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int i = 0; i < NI; ++i) {
+                    uint32_t e[4];
+                    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(e[0]), "=r"(e[1]), "=r"(e[2]), "=r"(e[3])
+                                 : "r"(__dp2a_lo(ids[i], h ? 16u << 8 : 16u, base)));
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        v[i][j] = min_u16x2(v[i][j], e[j]);
+                }
+        };
+        uint32_t q = 0;
+        for (; q + 4 <= words; q += 4) {  // four words of every list in flight
+            uint32_t ids[4][NI];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int i = 0; i < NI; ++i) {
+                    ids[u][i] = on[i] ? __ldg(lists + at[i]) : 0u;
+                    at[i] += pitch;
+                }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                use(ids[u]);
+        }
+        if (q < words) {
+            uint32_t ids[3][NI];
+#pragma unroll
+            for (int u = 0; u < 3; ++u)
+                if (q + u < words)
+#pragma unroll
+                    for (int i = 0; i < NI; ++i) {
+                        ids[u][i] = on[i] ? __ldg(lists + at[i]) : 0u;
+                        at[i] += pitch;
+                    }
+#pragma unroll
+            for (int u = 0; u < 3; ++u)
+                if (q + u < words)
+                    use(ids[u]);
+        }
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+            uint32_t sum = 0u;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                sum = __dp2a_lo(v[i][j], 0x0101u, sum);
+            if (on[i])
+                atomicAdd(sums + 2 * (32 * (g0 + i) + lane), sum);
+        }
+        g0 += nwarps * NI;
+    }
+}
+
+// One client's term of a bitset by a walk of its Pi' row (one warp): the distance at the first open rank, 0 without one.
+__device__ __forceinline__ uint32_t row_term(const pm_prob &pr, const uint32_t *__restrict__ mask, int64_t c, int lane)
+{
+    const uint16_t *prow = pr.pi + c * pr.stride;
+    const int32_t *drow = pr.delta + c * pr.stride;
+    uint32_t carry = 0;
+    for (int base = 0; base < pr.L; base += 32) {
+        const int r = base + lane;
+        const uint32_t j = r < pr.L ? __ldg(prow + r) : 0u;
+        const uint32_t d = r < pr.L ? (uint32_t)__ldg(drow + r) : 0u;
+        const uint32_t hit = __ballot_sync(PM_FULL_MASK, r < pr.L && ((__ldg(mask + (j >> 5)) >> (j & 31)) & 1u));
+        if (hit) {
+            const int first = __ffs(hit) - 1;
+            return pr.cum ? __shfl_sync(PM_FULL_MASK, d, first)
+                          : carry + __reduce_add_sync(PM_FULL_MASK, lane <= first ? d : 0u);
+        }
+        if (!pr.cum)
+            carry += __reduce_add_sync(PM_FULL_MASK, d);
+    }
+    return 0u;
+}

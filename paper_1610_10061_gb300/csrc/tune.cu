@@ -24,7 +24,8 @@ static constexpr int kTuneChain = 8;
 namespace {
 bool same_shape(const pm_eval_plan &a, const pm_eval_plan &b)
 {
-    return a.groups == b.groups && a.warps == b.warps && a.splits == b.splits && a.bytes == b.bytes;
+    return a.groups == b.groups && a.warps == b.warps && a.splits == b.splits && a.bytes == b.bytes &&
+           a.direct.range == b.direct.range;
 }
 
 // The shape as the ABI reports it: groups -1 is the row kernel with byte masks.
@@ -51,6 +52,11 @@ extern "C" pm_status pm_tune_eval(pm_instance *inst, int64_t pop, void *stream, 
                 continue;
             for (int sp : {std::max(1, base.splits / 2), base.splits, base.splits * 2}) {
                 const pm_eval_plan pl = pm_plan_eval_with(inst, pop, G, warps, sp);
+                if (cands.empty()) {  // the heuristic's other way of evaluating, where it applies
+                    pm_eval_plan direct = pl;
+                    if (pm_plan_direct(inst, pop, direct))
+                        cands.push_back(direct);
+                }
                 bool dup = false;
                 for (const auto &c : cands)
                     dup = dup || same_shape(c, pl);
