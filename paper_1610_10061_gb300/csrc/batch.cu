@@ -9,6 +9,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <new>
 #include <vector>
 
@@ -18,6 +19,75 @@
 static constexpr int kTuneReps = 5;
 
 static size_t tile_bytes(int64_t W, int G) { return (size_t)W * 32 * G * 4; }
+
+// Divide the launch's tiles among at most `slots` CTAs of `warps` warps so that the longest CTA is as short as a
+// greedy walk over the tiles finds (bisection on its length).  A CTA takes the clients of one or more tiles in turn; a
+// share costs its walk (work[k] SM cycles for all of instance k) plus about kShareCycles for the tile's copy, the flush,
+// the atomics and the barriers.  Shares end on whole units of 32/G clients, a unit per warp where they are that long.
+static constexpr double kShareCycles = 8000.0;
+
+static void plan_shares(pm_multi_plan &out, const std::vector<double> &work, int64_t slots, int warps)
+{
+    const int K = (int)out.probs.size();
+    auto fill = [&](double cap, bool write) {
+        int64_t ctas = 0;
+        double load = 0.0;
+        if (write) {
+            out.shares.clear();
+            out.share_base.assign(1, 0);
+        }
+        for (int k = 0; k < K; ++k) {
+            const pm_prob &pr = out.probs[k];
+            const int64_t unit = pr.d_range ? 8 * pr.d_chunks : 32 / out.groups;
+            const int64_t units = pm_ceil_div(pr.n, unit), step = pr.d_range ? 1 : warps;
+            const double cost = work[k] / (double)(pr.tiles * units);
+            for (int64_t tile = 0; tile < pr.tiles; ++tile) {
+                const size_t first = out.shares.size();
+                for (int64_t u = 0; u < units;) {
+                    int64_t take = (int64_t)((cap - load - kShareCycles) / cost);
+                    if (load > 0.0 && take < std::min(step, units - u)) {  // this CTA is full
+                        load = 0.0;
+                        ++ctas;
+                        if (write)
+                            out.share_base.push_back((int32_t)out.shares.size());
+                        continue;
+                    }
+                    take = std::min(units - u, std::max<int64_t>(take / step, 1) * step);
+                    if (pr.d_range)  // 32-bit sums: 2^16 clients of distances below 2^16
+                        take = std::min<int64_t>(take, 65536 / unit);
+                    if (write)
+                        out.shares.push_back(pm_share{k, 0, tile, u * unit, std::min(pr.n, (u + take) * unit)});
+                    load += kShareCycles + cost * (double)take;
+                    u += take;
+                }
+                if (write)
+                    for (size_t i = first; i < out.shares.size(); ++i)
+                        out.shares[i].splits = (int32_t)(out.shares.size() - first);
+            }
+        }
+        if (load > 0.0) {
+            ++ctas;
+            if (write)
+                out.share_base.push_back((int32_t)out.shares.size());
+        }
+        return ctas;
+    };
+    double total = 0.0;
+    int64_t tiles = 0;
+    for (int k = 0; k < K; ++k) {
+        total += work[k];
+        tiles += out.probs[k].tiles;
+    }
+    double lo = total / (double)slots, hi = total + kShareCycles * (double)(tiles + 1) * 2.0 + 1.0;
+    for (int it = 0; it < 40 && hi > lo * 1.002; ++it) {
+        const double mid = 0.5 * (lo + hi);
+        if (fill(mid, false) <= slots)
+            hi = mid;
+        else
+            lo = mid;
+    }
+    fill(hi, true);
+}
 
 pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std::vector<int64_t> &pops, int G,
                         int warps, int items_per_slot, pm_multi_plan &out)
@@ -52,6 +122,11 @@ pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std
         const double steps = 1.5 + pm_walk_depth(in->m, in->p, in->L) / 32.0;
         work[k] = tiles * (double)in->n * steps;
         if (out.nb) {  // in SM cycles per pair, the unit the two ways are compared in
+            // few individuals do not pay for the lists (written by every GA operator) and the chunks' copies: 48
+            // uneven instances, pop 256: evaluation 131 us against 134 without, generation 2.67 against 2.53 ms; pop
+            // 1024: evaluation 352 against 460 us
+            if (pops[k] >= 512)
+                pm_direct_shape(in, pops[k], budget, warps, direct[k]);
             work[k] = (double)pops[k] * (double)in->n *
                       (direct[k].range ? pm_direct_cost(in->m, in->p, direct[k].range, direct[k].stages) : pm_scan_cost(in->m, in->p));
             out.d_smem = std::max(out.d_smem, direct[k].smem);
@@ -94,7 +169,7 @@ pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std
         splits = std::max<int64_t>(1, std::min<int64_t>(splits, pm_ceil_div(in->n, warps * per_warp)));
         pr.splits = splits;
         pr.cps = pm_ceil_div(in->n, splits);
-        pr.packed = pm_packed_reduction_ok(in, splits) ? 1 : 0;
+        pr.packed = pm_packed_reduction_ok(in, std::max(splits, slots)) ? 1 : 0;
         pr.flush_units = pm_flush_units(in->max_d, G);
         if (direct[k].range) {
             pm_direct_splits(in, (int64_t)std::ceil(want_items / (double)pm_ceil_div(pops[k], direct[k].range)),
@@ -118,14 +193,32 @@ pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std
         items += pr.tiles * splits;
         jobs += pr.d_range ? pops[k] : pr.tiles * G * in->W;
     }
+    if (out.nb && K > 1)
+        plan_shares(out, work, slots, warps);
     out.ind_total = ind;
     out.words_total = words;
     out.cols_total = cols;
     out.tiles_total = tiles_acc;
     out.items = items;
     out.jobs = jobs;
-    out.grid = std::min<int64_t>(items, slots);
+    out.grid = !out.shares.empty() ? (int64_t)out.share_base.size() - 1 : std::min<int64_t>(items, slots);
     return PM_OK;
+}
+
+size_t pm_multi_plan::table_bytes() const
+{
+    return probs.size() * sizeof(pm_prob) + shares.size() * sizeof(pm_share) + share_base.size() * sizeof(int32_t);
+}
+
+void pm_multi_plan::write_table(char *dst) const
+{
+    std::memcpy(dst, probs.data(), probs.size() * sizeof(pm_prob));
+    dst += probs.size() * sizeof(pm_prob);
+    if (shares.empty())
+        return;
+    std::memcpy(dst, shares.data(), shares.size() * sizeof(pm_share));
+    dst += shares.size() * sizeof(pm_share);
+    std::memcpy(dst, share_base.data(), share_base.size() * sizeof(int32_t));
 }
 
 pm_multi_plan pm_plan_from_single(const pm_instance *inst, const pm_eval_plan &plan, int64_t pop)
@@ -154,6 +247,7 @@ void pm_scan_launch_from(const pm_multi_plan &mp, const pm_prob *probs_dev, pm_s
     L.nb = mp.nb;
     L.Wmax = mp.Wmax;
     L.d_smem = mp.d_smem;
+    L.shares = L.K > 1 ? (int64_t)mp.shares.size() : 0;
     L.grid = mp.grid;
     L.K = (int)mp.probs.size();
     L.one = mp.probs[0];
@@ -189,9 +283,10 @@ static pm_status batch_plan(pm_batch *b, const std::vector<int64_t> &pops, int G
         pr.out_base = out;
         out += pr.pop;
     }
-    PM_TRY(b->probs.reserve(mp.probs.size() * sizeof(pm_prob)));
-    PM_CUDA(cudaMemcpyAsync(b->probs.ptr, mp.probs.data(), mp.probs.size() * sizeof(pm_prob), cudaMemcpyHostToDevice,
-                            s));
+    std::vector<char> table(mp.table_bytes());
+    mp.write_table(table.data());
+    PM_TRY(b->probs.reserve(table.size()));
+    PM_CUDA(cudaMemcpyAsync(b->probs.ptr, table.data(), table.size(), cudaMemcpyHostToDevice, s));
     bool fresh = false;
     PM_TRY(b->accum.reserve((size_t)mp.ind_total * 8, &fresh));
     if (fresh)

@@ -251,10 +251,22 @@ __device__ __forceinline__ uint32_t direct_item(const pm_prob &pr, const DirectI
     return phases;
 }
 
-// The same as a function of its own: beside the bit-sliced walk's registers in the kernel that does both.
+// The same as a function of its own, as the bit-sliced walk is.
 __device__ __noinline__ uint32_t direct_item_call(const pm_prob &pr, const DirectItem &it, uint32_t phases)
 {
     return direct_item(pr, it, phases, threadIdx.x >> 5, blockDim.x >> 5, threadIdx.x & 31);
+}
+
+// The bit-sliced walk as a function of its own: it needs all 128 registers, and inside the kernel's body every change
+// around it moved its speed by up to a tenth.
+template <int G>
+__device__ __noinline__ void tile_walk_call(const pm_prob &pr, uint32_t *smem, uint32_t tbl, int nb, uint32_t a0,
+                                            int64_t c_begin, int64_t c_end, unsigned long long *acc_s)
+{
+    const TileRows rows{pr.pi, pr.delta, pr.stride, pr.L, pr.cum != 0, pr.flush_units};
+    TileWalk<G> walk;
+    walk.prefetch(rows, c_begin, c_end, threadIdx.x >> 5, threadIdx.x & 31);
+    walk.run(smem, tbl, nb, a0, rows, c_begin, c_end, threadIdx.x >> 5, blockDim.x >> 5, threadIdx.x & 31, acc_s);
 }
 
 // What a launch's work items are: scanned client by client, scanned bit-sliced, evaluated by open facilities, or
@@ -263,10 +275,15 @@ enum class ScanKind { clients, sliced, direct, mixed };
 
 // ---------------------------------------------------------------------------
 // The column scan kernel (with the split reduction and epilogue fused), over
-// every instance of the launch.  Persistent: CTA b takes work items b, b +
-// gridDim.x, ...; within an instance item = split * tiles + tile, so the CTAs
-// running at the same time walk the same clients for different tiles and
-// the rows they stream are shared through L2.
+// every instance of the launch.  What a CTA takes, one after another:
+//  * client walk, pinned and tuned splits: work items b, b + gridDim.x, ...;
+//    within an instance item = split * tiles + tile, so the CTAs running at
+//    the same time walk the same clients for different tiles and the rows they
+//    stream are shared through L2;
+//  * bit-sliced walk of one instance: an even part of all tiles' units, so one
+//    or two tiles a CTA;
+//  * several instances, bit-sliced or by open facilities: the shares that the
+//    host divided the launch into (pm_share).
 // ---------------------------------------------------------------------------
 template <int G, ScanKind kKind>
 __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
@@ -274,7 +291,7 @@ __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
                    const uint32_t *__restrict__ colT, const uint32_t *__restrict__ masks,
                    const uint32_t *__restrict__ active, unsigned long long *__restrict__ accum,
                    int *__restrict__ tickets, int *__restrict__ err, ScanEpilogue ep, uint32_t stall, int nb,
-                   uint32_t tab_off)
+                   uint32_t tab_off, int64_t shares)
 {
     // the previous kernel of the stream may still run until pm_grid_dependency_wait(): before it only the
     // constant tables (Pi', Delta', the launch's problem table) are read
@@ -286,6 +303,8 @@ __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
     __shared__ __align__(8) uint64_t bar, d_bar[2];
     __shared__ int last_s;
     __shared__ pm_prob pr_s;
+    __shared__ pm_share share_s;
+    __shared__ int64_t next_s;
 
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -301,21 +320,57 @@ __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     [[maybe_unused]] uint32_t d_phases = 0;
-    [[maybe_unused]] TileWalk<G> walk;
     const uint32_t my_tab = tab_off + (uint32_t)(warp * tile_table_words(nb, G));
     __syncthreads();
 
     uint32_t phase = 0;
     int64_t loaded_tile = -1;  // global tile index of the tile in shared memory
     bool waited = false;
-    for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
-        if (threadIdx.x == 0)
-            pr_s = (K > 1) ? probs[find_prob(K, item, [&](int k) { return probs[k].item_base; })] : one;
+    // what this CTA takes, from pos on: shares of the launch's table, units of its only instance, or work items
+    int64_t pos = blockIdx.x, end = items;
+    const pm_share *share_tab = reinterpret_cast<const pm_share *>(probs + K);
+    if (kSliced && shares > 0) {
+        const int32_t *base = reinterpret_cast<const int32_t *>(share_tab + shares) + blockIdx.x;
+        pos = base[0];
+        end = base[1];
+    } else if (kKind == ScanKind::sliced && one.stream_units > 0) {
+        const int64_t units = one.tiles * one.stream_units;
+        pos = blockIdx.x * units / gridDim.x;
+        end = (blockIdx.x + 1) * units / gridDim.x;
+    }
+    while (pos < end) {
+        if (threadIdx.x == 0) {
+            if (kSliced && shares > 0) {
+                share_s = share_tab[pos];
+                pr_s = probs[share_s.prob];
+                next_s = pos + 1;
+            } else if (kKind == ScanKind::sliced && one.stream_units > 0) {
+                // the CTA that holds unit u is ((u + 1) grid - 1) / units, so the tile's shares are those of its
+                // first to its last unit
+                const int64_t units = one.tiles * one.stream_units, per = one.stream_units, g = gridDim.x;
+                const int64_t tile = pos / per, first = tile * per, stop = min(end, first + per);
+                pr_s = one;
+                share_s.tile = tile;
+                share_s.c_begin = (pos - first) * TileWalk<G>::kClients;
+                share_s.c_end = min(one.n, (stop - first) * TileWalk<G>::kClients);
+                share_s.splits = (int32_t)(((first + per) * g - 1) / units - ((first + 1) * g - 1) / units + 1);
+                next_s = stop;
+            } else {
+                pr_s = (K > 1) ? probs[find_prob(K, pos, [&](int k) { return probs[k].item_base; })] : one;
+                const int64_t li = pos - pr_s.item_base, split = li / pr_s.tiles;
+                share_s.tile = li - split * pr_s.tiles;
+                share_s.c_begin = split * pr_s.cps;
+                share_s.c_end = min(share_s.c_begin + pr_s.cps, pr_s.n);
+                share_s.splits = (int32_t)pr_s.splits;
+                next_s = pos + gridDim.x;
+            }
+        }
         __syncthreads();
         const pm_prob &pr = pr_s;
-        const int64_t li = item - pr.item_base;
-        const int64_t tile = li % pr.tiles;
-        const int64_t split = li / pr.tiles;
+        const int64_t tile = share_s.tile;
+        const int64_t c_begin = share_s.c_begin, c_end = share_s.c_end;
+        const int splits = share_s.splits;
+        pos = next_s;
         const int64_t gtile = pr.tile_base + tile;
         const int32_t W = pr.W, L = pr.L;
         const int64_t pop = pr.pop, stride = pr.stride;
@@ -333,8 +388,6 @@ __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
         uint32_t *fin_s = direct ? a0_s + count / 32 : tile_fin;
 
         // first steps of this warp's first two clients (constant tables), loaded while the tile lands
-        const int64_t c_begin = split * pr.cps;
-        const int64_t c_end = (c_begin + pr.cps < pr.n) ? c_begin + pr.cps : pr.n;
         [[maybe_unused]] auto load = [&](int64_t cc, int base, uint32_t &j, int32_t &dl) {
             const int r = base + lane;
             if (cc < c_end && r < L) {
@@ -348,16 +401,12 @@ __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
         [[maybe_unused]] const int64_t c = c_begin + warp;
         [[maybe_unused]] uint32_t j_cur, j_nxt, j_nc, j_nc1;
         [[maybe_unused]] int32_t d_cur, d_nxt, d_nc, d_nc1;
-        const TileRows rows{pi, delta, stride, L, pr.cum != 0, pr.flush_units};
         [[maybe_unused]] const DirectItem d_item{colbits, colT + pr.col_base, masks, ind0, count, a0_s,  fin_s,
                                                  d_sums,  c_begin,            c_end, d_bar, err,  stalled};
         if constexpr (kDirect)
             if (direct && threadIdx.x == 0)
                 direct_start(pr, d_item);
-        if constexpr (kSliced) {
-            if (!direct)
-                walk.prefetch(rows, c_begin, c_end, warp, lane);
-        } else if constexpr (kKind == ScanKind::clients) {
+        if constexpr (kKind == ScanKind::clients) {
             load(c, 0, j_cur, d_cur);
             load(c, 32, j_nxt, d_nxt);
             load(c + nwarps, 0, j_nc, d_nc);
@@ -406,8 +455,7 @@ __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
 
         if constexpr (kDirect) {
             if (direct) {
-                d_phases = kKind == ScanKind::direct ? direct_item(pr, d_item, d_phases, warp, nwarps, lane)
-                                                     : direct_item_call(pr, d_item, d_phases);
+                d_phases = direct_item_call(pr, d_item, d_phases);
                 if (d_phases == 0xffffffffu)
                     return;
                 loaded_tile = -1;  // the entries took the tile's place
@@ -421,7 +469,7 @@ __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
             for (int g = 0; g < G; ++g)
                 any0 |= a0_s[g];
             if (any0 && c_begin < c_end)
-                walk.run(colbits, my_tab, nb, a0_s[lane % G], rows, c_begin, c_end, warp, nwarps, lane, acc_s);
+                tile_walk_call<G>(pr, colbits, my_tab, nb, a0_s[lane % G], c_begin, c_end, acc_s);
         } else if constexpr (kKind == ScanKind::clients) {
             uint32_t a0[G];
             uint32_t any0 = 0;
@@ -447,7 +495,7 @@ __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
 
         bool finish = true;
         const uint32_t *fin = a0_s;  // individuals whose epilogue this CTA applies
-        if (pr.splits > 1 && pr.packed) {
+        if (splits > 1 && pr.packed) {
             // one atomic per individual carries the split's sum plus one count in the top 16 bits; the split
             // that brings the count to `splits` holds the total, applies that individual's epilogue and leaves
             // the word zero for the next launch -- no fences, no tile ticket
@@ -476,7 +524,7 @@ __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
                         break;
                     i = i + start >= count ? i + start - count : i + start;
                     const bool last = add[f] != 0ull &&
-                                      (old[f] >> kCountShift) == (unsigned long long)(pr.splits - 1);
+                                      (old[f] >> kCountShift) == (unsigned long long)(splits - 1);
                     if (last) {
                         acc_s[i] = (old[f] + add[f]) & ((1ull << kCountShift) - 1ull);
                         accum[pr.ind_base + ind0 + i] = 0ull;
@@ -488,7 +536,7 @@ __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
             }
             __syncthreads();
             fin = fin_s;
-        } else if (pr.splits > 1) {
+        } else if (splits > 1) {
             // add this split's sums into the instance's accumulators; the last split of the tile
             // (atomic ticket) reads the totals and leaves the accumulators zero again
             for (int i = threadIdx.x; i < count; i += blockDim.x) {
@@ -499,7 +547,7 @@ __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
             __threadfence();
             __syncthreads();
             if (threadIdx.x == 0)
-                last_s = (atomicAdd(tickets + gtile, 1) == (int)pr.splits - 1) ? 1 : 0;
+                last_s = (atomicAdd(tickets + gtile, 1) == splits - 1) ? 1 : 0;
             __syncthreads();
             finish = last_s != 0;
             if (finish) {
@@ -682,7 +730,8 @@ __global__ void k_wait_selftest(int *__restrict__ err, uint32_t limit)
 
 // The column kernel for G groups, with the bit-sliced walk or the client walk.
 using scan_kernel = void (*)(const pm_prob *, int, pm_prob, int64_t, const uint32_t *, const uint32_t *,
-                             const uint32_t *, unsigned long long *, int *, int *, ScanEpilogue, uint32_t, int, uint32_t);
+                             const uint32_t *, unsigned long long *, int *, int *, ScanEpilogue, uint32_t, int, uint32_t,
+                             int64_t);
 template <ScanKind kKind>
 scan_kernel scan_fn_of(int G)
 {
@@ -849,6 +898,15 @@ pm_eval_plan pm_plan_eval_with(const pm_instance *inst, int64_t pop, int G, int 
     splits = std::min<int64_t>(std::max<int64_t>(1, splits), std::min<int64_t>(max_splits, 65535));
     plan.splits = (int)splits;
     plan.grid = plan.groups ? std::min<int64_t>(plan.tiles * splits, slots) : plan.tiles;
+    if (plan.nb && splits_hint <= 0) {
+        // one wave of CTAs that share the units evenly: an item costs its CTA about 5 us beside the walk (the tile's
+        // copy, the flush, the atomics, two or three barriers), 4096 subsets of 10000 x 10000 at p = 1000 96 us in
+        // four items a CTA
+        const int64_t units = pm_ceil_div(inst->n * plan.groups, 32);
+        plan.stream = true;
+        plan.grid = std::min<int64_t>(slots, std::max<int64_t>(1, plan.tiles * units / 4));
+        plan.splits = (int)std::max<int64_t>(1, std::min<int64_t>(max_splits, plan.grid / plan.tiles));
+    }
     return plan;
 }
 
@@ -947,8 +1005,14 @@ pm_prob pm_single_prob(const pm_instance *inst, const pm_eval_plan &plan, int64_
     pr.tiles = plan.tiles;
     pr.splits = plan.splits;
     pr.cps = pm_ceil_div(inst->n, plan.splits);
-    if (plan.direct.range)
+    if (plan.stream) {
+        pr.stream_units = pm_ceil_div(inst->n * plan.groups, 32);
+        pr.packed = pm_packed_reduction_ok(inst, plan.grid) ? 1 : 0;
+    }
+    if (plan.direct.range) {
         pm_direct_prob(inst, plan.direct, pop, pr);
+        pr.stream_units = 0;
+    }
     return pr;  // every base 0
 }
 
@@ -1025,7 +1089,7 @@ pm_status pm_launch_scan(const pm_scan_launch &L, const pm_accept_args &acc, int
     const ScanKind kind = L.d_smem == 0 ? (L.nb > 0 ? ScanKind::sliced : ScanKind::clients)
                                         : (L.K == 1 ? ScanKind::direct : ScanKind::mixed);
     PM_CUDA(pm_launch(scan_fn(G, kind), grid, threads, smem, stream, L.probs_dev, L.K, L.one, L.items, L.colT,
-                      L.masks, L.active, accum, L.tickets, L.err, ep, stall, L.nb, tab_off));
+                      L.masks, L.active, accum, L.tickets, L.err, ep, stall, L.nb, tab_off, L.shares));
     return PM_OK;
 }
 

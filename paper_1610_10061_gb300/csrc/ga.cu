@@ -2554,11 +2554,11 @@ static pm_status ga_alloc(pm_ga *ga, cudaStream_t s, bool with_spec)
     const size_t n_zero = parts.size();
     parts.push_back({&ga->st, sizeof(ga_dev) * K});
     parts.push_back({&ga->glob, sizeof(ga_glob)});
-    parts.push_back({&ga->probs, sizeof(pm_prob) * K});
+    parts.push_back({&ga->probs, ga->plan.table_bytes()});
     parts.push_back({&ga->gprobs, sizeof(ga_prob) * K});
     if (with_spec) {
         parts.push_back({&ga->gqprobs, sizeof(ga_prob) * K});
-        parts.push_back({&ga->probsQ, sizeof(pm_prob) * K});
+        parts.push_back({&ga->probsQ, sp.table_bytes()});
     }
     PM_TRY(pm_carve(ga->arena, parts.data(), (int)parts.size()));
     char *base = static_cast<char *>(ga->arena.ptr);
@@ -2578,11 +2578,11 @@ static pm_status ga_alloc(pm_ga *ga, cudaStream_t s, bool with_spec)
     g.alive = K;
     put(ga->st, h.data(), sizeof(ga_dev) * K);
     put(ga->glob, &g, sizeof(g));
-    put(ga->probs, ga->plan.probs.data(), sizeof(pm_prob) * K);
+    ga->plan.write_table(host.data() + (static_cast<char *>(ga->probs.ptr) - base - host_off));
     put(ga->gprobs, ga->gps.data(), sizeof(ga_prob) * K);
     if (with_spec) {
         put(ga->gqprobs, ga->gqs.data(), sizeof(ga_prob) * K);
-        put(ga->probsQ, sp.probs.data(), sizeof(pm_prob) * K);
+        sp.write_table(host.data() + (static_cast<char *>(ga->probsQ.ptr) - base - host_off));
     }
     PM_CUDA(cudaMemcpyAsync(base + host_off, host.data(), host.size(), cudaMemcpyHostToDevice, s));
     PM_CUDA(cudaStreamSynchronize(s));

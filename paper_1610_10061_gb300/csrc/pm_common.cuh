@@ -85,6 +85,7 @@ struct pm_eval_plan {
     int64_t grid = 0;     // CTAs launched (column kernel: persistent over tiles x splits items)
     int bytes = 0;        // row kernel only: each warp's bitset expanded to one byte per facility (byte masks)
     int nb = 0;           // column kernel: blocks of 32 ranks per table of the bit-sliced walk; 0: the client walk
+    bool stream = false;  // bit-sliced walk: the CTAs share the units evenly (pm_prob::stream_units), not by `splits`
     // evaluation by open facilities in place of the scan, when direct.range > 0.  The column shape above stays the
     // one the facility-major form and the scratch are laid out by.
     pm_direct_plan direct;
@@ -113,7 +114,18 @@ struct pm_prob {
     int64_t tiles, tile_base;
     int64_t splits, cps;  // client splits and clients per split
     int64_t item_base;
+    // > 0 (one instance, bit-sliced walk): units per tile; CTA b takes units [b U / grid, (b + 1) U / grid) of the
+    // launch's U = tiles * stream_units, tile after tile, in place of work items
+    int64_t stream_units;
     int64_t job_base;     // transpose jobs (tiles * G * W per instance; pop when its individuals get lists)
+};
+
+// One CTA's share of a tile in a launch over several instances: clients [c_begin, c_end) of tile `tile` of instance
+// `prob`, one of `splits` shares of that tile.  The launch's table: the instances' pm_prob, then the shares in CTA
+// order, then (int32) the index of every CTA's first share and the number of shares.
+struct pm_share {
+    int32_t prob, splits;
+    int64_t tile, c_begin, c_end;
 };
 
 // Programmatic dependent launch.  Kernels of the GA generation and of the
@@ -223,6 +235,7 @@ struct pm_scan_launch {
     int nb = 0;                          // as pm_eval_plan
     int64_t Wmax = 0;                    // bitset words of the widest instance (sizes the shared memory)
     size_t d_smem = 0;                   // bytes the evaluation by open facilities needs (0: no instance uses it)
+    int64_t shares = 0;                  // > 0: the table behind probs_dev holds the CTAs' shares
     int64_t grid = 0;
     int K = 1;
     const pm_prob *probs_dev = nullptr;  // K > 1: device table
@@ -316,6 +329,11 @@ struct pm_multi_plan {
     int64_t Wmax = 0;  // bitset words of the widest instance
     size_t d_smem = 0;
     std::vector<pm_prob> probs;
+    std::vector<pm_share> shares;       // several instances, bit-sliced walk (else items)
+    std::vector<int32_t> share_base;    // grid + 1 entries
+    // the launch's device table (see pm_share)
+    size_t table_bytes() const;
+    void write_table(char *dst) const;
 };
 // Plan for `insts` with pops[k] individuals each; items_per_slot work items per
 // resident CTA (splits apportioned by an estimate of each instance's scan work).

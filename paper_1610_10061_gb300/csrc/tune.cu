@@ -25,7 +25,7 @@ namespace {
 bool same_shape(const pm_eval_plan &a, const pm_eval_plan &b)
 {
     return a.groups == b.groups && a.warps == b.warps && a.splits == b.splits && a.bytes == b.bytes &&
-           a.direct.range == b.direct.range;
+           a.direct.range == b.direct.range && a.stream == b.stream;
 }
 
 // The shape as the ABI reports it: groups -1 is the row kernel with byte masks.
@@ -42,6 +42,12 @@ extern "C" pm_status pm_tune_eval(pm_instance *inst, int64_t pop, void *stream, 
 
     // candidate shapes
     std::vector<pm_eval_plan> cands;
+    auto add = [&](const pm_eval_plan &pl) {
+        for (const auto &c : cands)
+            if (same_shape(c, pl))
+                return;
+        cands.push_back(pl);
+    };
     const size_t budget = inst->smem_optin > 4096 ? inst->smem_optin - 4096 : 0;
     for (int G : {4, 2, 1}) {
         if ((size_t)inst->W * 32 * G * 4 > budget)
@@ -50,6 +56,8 @@ extern "C" pm_status pm_tune_eval(pm_instance *inst, int64_t pop, void *stream, 
             const pm_eval_plan base = pm_plan_eval_with(inst, pop, G, warps, 0);
             if (base.groups != G)
                 continue;
+            if (base.stream)  // no fixed splits: the CTAs share the units evenly
+                add(base);
             for (int sp : {std::max(1, base.splits / 2), base.splits, base.splits * 2}) {
                 const pm_eval_plan pl = pm_plan_eval_with(inst, pop, G, warps, sp);
                 if (cands.empty()) {  // the heuristic's other way of evaluating, where it applies
@@ -57,11 +65,7 @@ extern "C" pm_status pm_tune_eval(pm_instance *inst, int64_t pop, void *stream, 
                     if (pm_plan_direct(inst, pop, direct))
                         cands.push_back(direct);
                 }
-                bool dup = false;
-                for (const auto &c : cands)
-                    dup = dup || same_shape(c, pl);
-                if (!dup)
-                    cands.push_back(pl);
+                add(pl);
             }
         }
     }
