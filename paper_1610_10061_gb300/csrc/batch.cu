@@ -111,6 +111,13 @@ pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std
         return PM_ERR_UNSUPPORTED;
     if (pm_sliced_pays(i0, units))
         pm_walk_shape(i0, out.Wmax, G, depth, warps, out.nb);
+    if (!out.nb) {
+        out.split = true;
+        for (const pm_instance *in : insts)
+            out.split = out.split && pm_split_fits(in, out.Wmax, G, warps);
+        if (out.split)
+            items_per_slot = 1;  // an item's fixed costs are most of a small launch
+    }
     out.warps = warps;
     // scan work estimate per instance: tiles x clients x expected 32-rank steps of a 128-individual tile
     std::vector<double> work(K);
@@ -137,7 +144,7 @@ pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std
     // resident CTAs per SM for this shape and shared memory
     {
         const int by_smem = (int)std::max<size_t>(
-            1, i0->smem_optin / (std::max(pm_scan_smem(out.Wmax, G, warps, out.nb), out.d_smem) + 3072));
+            1, i0->smem_optin / (std::max(pm_scan_smem(out.Wmax, G, warps, out.nb, out.split), out.d_smem) + 3072));
         const int by_threads = std::max(1, 2048 / (warps * 32));
         slots_per_sm = std::max(1, std::min(by_smem, by_threads));
         // register limit: 128 registers per thread in the bit-sliced walk, ~56 in the client walk
@@ -227,6 +234,7 @@ pm_multi_plan pm_plan_from_single(const pm_instance *inst, const pm_eval_plan &p
     mp.groups = plan.groups;
     mp.warps = plan.warps;
     mp.nb = plan.nb;
+    mp.split = plan.split;
     mp.probs.push_back(pm_single_prob(inst, plan, pop));
     mp.items = mp.probs[0].tiles * mp.probs[0].splits;
     mp.grid = plan.direct.range ? mp.items : plan.grid;
@@ -245,6 +253,7 @@ void pm_scan_launch_from(const pm_multi_plan &mp, const pm_prob *probs_dev, pm_s
     L.groups = mp.groups;
     L.warps = mp.warps;
     L.nb = mp.nb;
+    L.split = mp.split;
     L.Wmax = mp.Wmax;
     L.d_smem = mp.d_smem;
     L.shares = L.K > 1 ? (int64_t)mp.shares.size() : 0;

@@ -50,6 +50,7 @@
 
 #include "pm_common.cuh"
 #include "scan_direct.cuh"
+#include "scan_split.cuh"
 #include "scan_tile.cuh"
 #include "scan_walk.cuh"
 
@@ -269,9 +270,9 @@ __device__ __noinline__ void tile_walk_call(const pm_prob &pr, uint32_t *smem, u
     walk.run(smem, tbl, nb, a0, rows, c_begin, c_end, threadIdx.x >> 5, blockDim.x >> 5, threadIdx.x & 31, acc_s);
 }
 
-// What a launch's work items are: scanned client by client, scanned bit-sliced, evaluated by open facilities, or
+// What a launch's work items are: scanned client by client, rank-split or bit-sliced, evaluated by open facilities, or
 // (several instances) bit-sliced and by open facilities.
-enum class ScanKind { clients, sliced, direct, mixed };
+enum class ScanKind { clients, split, sliced, direct, mixed };
 
 // ---------------------------------------------------------------------------
 // The column scan kernel (with the split reduction and epilogue fused), over
@@ -286,7 +287,7 @@ enum class ScanKind { clients, sliced, direct, mixed };
 //    host divided the launch into (pm_share).
 // ---------------------------------------------------------------------------
 template <int G, ScanKind kKind>
-__global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
+__global__ void __launch_bounds__(kKind == ScanKind::clients || kKind == ScanKind::split ? 1024 : 512)
     k_scan_columns(const pm_prob *__restrict__ probs, int K, pm_prob one, int64_t items,
                    const uint32_t *__restrict__ colT, const uint32_t *__restrict__ masks,
                    const uint32_t *__restrict__ active, unsigned long long *__restrict__ accum,
@@ -320,7 +321,9 @@ __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     [[maybe_unused]] uint32_t d_phases = 0;
-    const uint32_t my_tab = tab_off + (uint32_t)(warp * tile_table_words(nb, G));
+    constexpr bool kSplit = kKind == ScanKind::split;
+    const uint32_t my_tab = tab_off + (uint32_t)(warp * (kSplit ? split_warp_words(G) : tile_table_words(nb, G)));
+    [[maybe_unused]] SplitWalk<G> split_walk;
     __syncthreads();
 
     uint32_t phase = 0;
@@ -406,6 +409,8 @@ __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
         if constexpr (kDirect)
             if (direct && threadIdx.x == 0)
                 direct_start(pr, d_item);
+        if constexpr (kSplit)
+            split_walk.prefetch(pr, c_begin, c_end, warp, nwarps, lane);
         if constexpr (kKind == ScanKind::clients) {
             load(c, 0, j_cur, d_cur);
             load(c, 32, j_nxt, d_nxt);
@@ -444,6 +449,8 @@ __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
         if constexpr (kSliced)
             if (!direct)
                 TileWalk<G>::clear_table(colbits + my_tab, nb, lane);
+        if constexpr (kSplit)
+            SplitWalk<G>::clear_table(colbits + my_tab, lane);
 
         if (reload && !direct) {
             if (!wait_copies(&bar, phase, stalled, err))
@@ -463,6 +470,22 @@ __global__ void __launch_bounds__(kKind != ScanKind::clients ? 512 : 1024)
         }
 
         if (kDirect && direct) {
+        } else if constexpr (kSplit) {
+            uint32_t acc[4] = {0u, 0u, 0u, 0u};
+            split_walk.run(colbits, colbits + my_tab, a0_s[(lane >> 3) & (G - 1)], pr, c_begin, c_end, warp, nwarps,
+                           lane, acc);
+            // the warps' sums side by side (over the warps' tables, which they have read), one thread per individual
+            *reinterpret_cast<uint4 *>(colbits + my_tab + 4 * lane) = make_uint4(acc[0], acc[1], acc[2], acc[3]);
+            __syncthreads();
+            for (int i = threadIdx.x; i < G * 32; i += blockDim.x) {
+                unsigned long long sum = 0ull;
+                const uint32_t *mine = colbits + tab_off + 8 * 4 * (i >> 5) + (i & 31);
+                for (int w = 0; w < nwarps; ++w, mine += split_warp_words(G))
+#pragma unroll
+                    for (int q = 0; q < 4 / G; ++q)
+                        sum += mine[q * G * 32];
+                acc_s[i] = sum;
+            }
         } else if constexpr (kSliced) {
             uint32_t any0 = 0;
 #pragma unroll
@@ -728,7 +751,13 @@ __global__ void k_wait_selftest(int *__restrict__ err, uint32_t limit)
     }
 }
 
-// The column kernel for G groups, with the bit-sliced walk or the client walk.
+// The walk of a column-kernel plan.
+ScanKind scan_kind(int nb, bool split)
+{
+    return nb > 0 ? ScanKind::sliced : (split ? ScanKind::split : ScanKind::clients);
+}
+
+// The column kernel for G groups and a kind of work items.
 using scan_kernel = void (*)(const pm_prob *, int, pm_prob, int64_t, const uint32_t *, const uint32_t *,
                              const uint32_t *, unsigned long long *, int *, int *, ScanEpilogue, uint32_t, int, uint32_t,
                              int64_t);
@@ -740,6 +769,8 @@ scan_kernel scan_fn_of(int G)
 scan_kernel scan_fn(int G, ScanKind kind)
 {
     switch (kind) {
+    case ScanKind::split:
+        return scan_fn_of<ScanKind::split>(G);
     case ScanKind::sliced:
         return scan_fn_of<ScanKind::sliced>(G);
     case ScanKind::direct:
@@ -773,7 +804,7 @@ static pm_status allow_dynamic_smem(const pm_instance *inst, F *fn)
 pm_status pm_fitness_init(const pm_instance *inst)
 {
     for (int G : {1, 2, 4})
-        for (ScanKind kind : {ScanKind::clients, ScanKind::sliced, ScanKind::direct, ScanKind::mixed})
+        for (ScanKind kind : {ScanKind::clients, ScanKind::split, ScanKind::sliced, ScanKind::direct, ScanKind::mixed})
             PM_TRY(allow_dynamic_smem(inst, scan_fn(G, kind)));
     PM_TRY(allow_dynamic_smem(inst, k_scan_rows<false>));
     PM_TRY(allow_dynamic_smem(inst, k_scan_rows<true>));
@@ -781,9 +812,10 @@ pm_status pm_fitness_init(const pm_instance *inst)
 }
 
 
-size_t pm_scan_smem(int64_t W, int G, int warps, int nb)
+size_t pm_scan_smem(int64_t W, int G, int warps, int nb, bool split)
 {
-    return column_smem_bytes(W, G) + (nb ? (size_t)warps * tile_table_words(nb, G) * 4 : 0);
+    const int words = split ? split_warp_words(G) : (nb ? tile_table_words(nb, G) : 0);
+    return column_smem_bytes(W, G) + (size_t)warps * words * 4;
 }
 
 void pm_walk_shape(const pm_instance *inst, int64_t W, int G, double depth, int &warps, int &nb)
@@ -792,7 +824,7 @@ void pm_walk_shape(const pm_instance *inst, int64_t W, int G, double depth, int 
     const int want = depth <= 32.0 ? 1 : (depth <= 160.0 ? 3 : 7);
     for (int w = std::min(warps, 16); w >= 4 || w == std::min(warps, 16); w /= 2) {
         for (int b : {7, 3, 1}) {
-            if (b <= want && pm_scan_smem(W, G, w, b) <= budget) {
+            if (b <= want && pm_scan_smem(W, G, w, b, false) <= budget) {
                 warps = w;
                 nb = b;
                 return;
@@ -851,8 +883,8 @@ static int column_ctas_per_sm(const pm_instance *inst, const pm_eval_plan &plan)
 {
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &nb, reinterpret_cast<const void *>(scan_fn(plan.groups, plan.nb > 0 ? ScanKind::sliced : ScanKind::clients)), plan.warps * 32,
-            pm_scan_smem(inst->W, plan.groups, plan.warps, plan.nb)) != cudaSuccess) {
+            &nb, reinterpret_cast<const void *>(scan_fn(plan.groups, scan_kind(plan.nb, plan.split))), plan.warps * 32,
+            pm_scan_smem(inst->W, plan.groups, plan.warps, plan.nb, plan.split)) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -862,6 +894,15 @@ static int column_ctas_per_sm(const pm_instance *inst, const pm_eval_plan &plan)
 static bool sliced_pays(const pm_instance *inst, int64_t pop)
 {
     return pm_sliced_pays(inst, pm_ceil_div(pop, 32) * pm_ceil_div(inst->n, 32));
+}
+
+bool pm_split_fits(const pm_instance *inst, int64_t W, int G, int warps)
+{
+    const size_t budget = inst->smem_optin > 4096 ? inst->smem_optin - 4096 : 0;
+    // a lane's 32-bit sums: its clients of one launch at most
+    const uint64_t clients = (uint64_t)(inst->n / (warps * (4 / G)) + 1);
+    return pm_scan_smem(W, G, warps, 0, true) <= budget &&
+           clients * (uint64_t)std::max<int32_t>(inst->max_d, 1) <= 0xffffffffull;
 }
 
 pm_eval_plan pm_plan_eval_with(const pm_instance *inst, int64_t pop, int G, int warps, int splits_hint)
@@ -874,11 +915,13 @@ pm_eval_plan pm_plan_eval_with(const pm_instance *inst, int64_t pop, int G, int 
         plan.warps = warps;
         if (sliced_pays(inst, pop))
             pm_walk_shape(inst, inst->W, G, pm_walk_depth(inst->m, inst->p, inst->L), plan.warps, plan.nb);
+        plan.split = !plan.nb && pm_split_fits(inst, inst->W, G, warps);
         ctas_per_sm = column_ctas_per_sm(inst, plan);
     }
     if (G <= 0 || ctas_per_sm <= 0) {
         plan.groups = 0;  // row kernel
         plan.nb = 0;
+        plan.split = false;
         plan.warps = 8;
         plan.tiles = pm_ceil_div(pop, plan.warps);
         plan.bytes = (G < 0 && (size_t)plan.warps * inst->W * 32 + 1024 <= inst->smem_optin) ? 1 : 0;
@@ -893,6 +936,12 @@ pm_eval_plan pm_plan_eval_with(const pm_instance *inst, int64_t pop, int G, int 
     int64_t splits = splits_hint > 0 ? splits_hint : pm_ceil_div(4 * slots, std::max<int64_t>(1, plan.tiles));
     if (splits_hint <= 0 && plan.nb)
         splits = std::min<int64_t>(splits, std::max<int64_t>(1, pm_ceil_div(inst->n * plan.groups, plan.warps * 32)));
+    if (splits_hint <= 0 && plan.split) {
+        // one wave, a CTA per SM at most, and no more CTAs than give every warp a round of 4/G clients
+        const int64_t each = (int64_t)plan.warps * (4 / plan.groups);
+        splits = std::max<int64_t>(1, std::min<int64_t>(inst->sm_count / std::max<int64_t>(1, plan.tiles),
+                                                        pm_ceil_div(inst->n, each)));
+    }
     if (splits_hint <= 0 && splits > max_splits)  // too few clients for that: one item per slot instead
         splits = std::max<int64_t>(1, std::min<int64_t>(max_splits, slots / std::max<int64_t>(1, plan.tiles)));
     splits = std::min<int64_t>(std::max<int64_t>(1, splits), std::min<int64_t>(max_splits, 65535));
@@ -919,15 +968,15 @@ pm_eval_plan pm_plan_eval(const pm_instance *inst, int64_t pop)
             return it->second;
     }
     const size_t budget = inst->smem_optin > 4096 ? inst->smem_optin - 4096 : 0;
-    int G = kMaxG;
-    // fewer groups for small populations or when the tile does not fit: keep >= 8 tiles, or >= 16 where a
-    // client's walk is short (expected first open rank (m+1)/(p+1) below 32: one or two steps, so the
-    // launch's fixed costs weigh more than the per-step savings of wide tiles)
-    const int64_t min_tiles = sliced_pays(inst, pop) ? 1 : ((inst->m + 1) < 32 * (inst->p + 1) ? 16 : 8);
-    while (G > 1 && (pop <= (int64_t)32 * (G / 2) * min_tiles || column_smem_bytes(inst->W, G) > budget))
+    // the bit-sliced walk: the widest tile the population fills.  Smaller launches (rank-split walk): 32 warps a CTA
+    // and tiles of 64 -- graph900's generation, pop 1024, 157 us against 162 with tiles of 128 -- or of 32 where one
+    // round of a CTA's warps then covers all clients, which saves the sums' way through global memory (graph100's
+    // generation 77 us against 82)
+    const bool sliced = sliced_pays(inst, pop);
+    int G = sliced ? kMaxG : (inst->n <= 128 ? 1 : 2);
+    while (G > 1 && (pop <= (int64_t)32 * (G / 2) || column_smem_bytes(inst->W, G) > budget))
         G /= 2;
-    // 32 warps when only one CTA fits per SM, else 16
-    const int warps = 2 * column_smem_bytes(inst->W, G) + 8192 > inst->smem_optin ? 32 : 16;
+    const int warps = sliced && 2 * column_smem_bytes(inst->W, G) + 8192 <= inst->smem_optin ? 16 : 32;
     pm_eval_plan plan = pm_plan_eval_with(inst, pop, G, warps, 0);
     pm_plan_direct(inst, pop, plan);
     return plan;
@@ -936,11 +985,14 @@ pm_eval_plan pm_plan_eval(const pm_instance *inst, int64_t pop)
 bool pm_plan_direct(const pm_instance *inst, int64_t pop, pm_eval_plan &plan)
 {
     const size_t budget = inst->smem_optin > 4096 ? inst->smem_optin - 4096 : 0;
-    if (!plan.nb)
+    // (below about 12 units of 1024 pairs per SM the chunks' copies and the lists are most of the time)
+    if (!plan.groups || pm_ceil_div(pop, 32) * pm_ceil_div(inst->n, 32) < (int64_t)inst->sm_count * 12)
         return false;
-    pm_direct_shape(inst, pop, budget, plan.warps, plan.direct);
+    const int warps = std::min(plan.warps, 16);
+    pm_direct_shape(inst, pop, budget, warps, plan.direct);
     if (!plan.direct.range)
         return false;
+    plan.warps = warps;
     // one work item per resident CTA (one per SM: the entries take most of the shared memory), whole rounds of chunks
     const int64_t ranges = pm_ceil_div(pop, plan.direct.range);
     pm_direct_splits(inst, std::max<int64_t>(1, inst->sm_count / ranges), plan.direct);
@@ -1085,8 +1137,8 @@ pm_status pm_launch_scan(const pm_scan_launch &L, const pm_accept_args &acc, int
     unsigned long long *accum = reinterpret_cast<unsigned long long *>(L.accum);
     const uint32_t stall = take_stall() ? 1u : 0u;
     const uint32_t tab_off = (uint32_t)(column_smem_bytes(L.Wmax, G) / 4);
-    const size_t smem = std::max(pm_scan_smem(L.Wmax, G, L.warps, L.nb), L.d_smem);
-    const ScanKind kind = L.d_smem == 0 ? (L.nb > 0 ? ScanKind::sliced : ScanKind::clients)
+    const size_t smem = std::max(pm_scan_smem(L.Wmax, G, L.warps, L.nb, L.split), L.d_smem);
+    const ScanKind kind = L.d_smem == 0 ? scan_kind(L.nb, L.split)
                                         : (L.K == 1 ? ScanKind::direct : ScanKind::mixed);
     PM_CUDA(pm_launch(scan_fn(G, kind), grid, threads, smem, stream, L.probs_dev, L.K, L.one, L.items, L.colT,
                       L.masks, L.active, accum, L.tickets, L.err, ep, stall, L.nb, tab_off, L.shares));
@@ -1105,6 +1157,7 @@ pm_status pm_launch_eval(const pm_instance *inst, const pm_eval_plan &plan, cons
         L.groups = plan.groups;
         L.warps = plan.warps;
         L.nb = plan.nb;
+        L.split = plan.split;
         L.Wmax = inst->W;
         L.K = 1;
         L.one = pm_single_prob(inst, plan, pop);

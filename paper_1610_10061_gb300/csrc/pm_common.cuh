@@ -85,6 +85,7 @@ struct pm_eval_plan {
     int64_t grid = 0;     // CTAs launched (column kernel: persistent over tiles x splits items)
     int bytes = 0;        // row kernel only: each warp's bitset expanded to one byte per facility (byte masks)
     int nb = 0;           // column kernel: blocks of 32 ranks per table of the bit-sliced walk; 0: the client walk
+    bool split = false;   // column kernel: the rank-split walk (nb = 0)
     bool stream = false;  // bit-sliced walk: the CTAs share the units evenly (pm_prob::stream_units), not by `splits`
     // evaluation by open facilities in place of the scan, when direct.range > 0.  The column shape above stays the
     // one the facility-major form and the scratch are laid out by.
@@ -233,6 +234,7 @@ struct pm_accept_args {
 struct pm_scan_launch {
     int groups = 4, warps = 16;
     int nb = 0;                          // as pm_eval_plan
+    bool split = false;
     int64_t Wmax = 0;                    // bitset words of the widest instance (sizes the shared memory)
     size_t d_smem = 0;                   // bytes the evaluation by open facilities needs (0: no instance uses it)
     int64_t shares = 0;                  // > 0: the table behind probs_dev holds the CTAs' shares
@@ -249,8 +251,8 @@ struct pm_scan_launch {
     int *err = nullptr;
 };
 pm_status pm_launch_scan(const pm_scan_launch &L, const pm_accept_args &acc, int64_t *costs, cudaStream_t stream);
-// Shared-memory bytes of a column-kernel CTA: the tile and, with nb > 0, the warps' distance tables.
-size_t pm_scan_smem(int64_t W, int G, int warps, int nb);
+// Shared-memory bytes of a column-kernel CTA: the tile and, with nb > 0 or split, the warps' distance tables.
+size_t pm_scan_smem(int64_t W, int G, int warps, int nb, bool split);
 // Warps (at most `warps`) and table blocks of the bit-sliced walk for tiles of W words and walks whose deepest
 // rank is about `depth`; nb = 0 and warps unchanged where the tables do not fit beside the tile.
 void pm_walk_shape(const pm_instance *inst, int64_t W, int G, double depth, int &warps, int &nb);
@@ -270,13 +272,16 @@ double pm_direct_cost(int64_t m, int64_t p, int64_t range, int stages);
 // Whether an instance of these sizes should keep the 16-bit distances.
 bool pm_direct_wanted(int64_t n, int64_t m, int64_t p, size_t smem_optin);
 // Whether a launch has enough units of 1024 (client, individual) pairs for the bit-sliced walk: a unit is a chain
-// of about 1200 instructions of one warp, so with fewer than 12 per SM the SMs wait for single warps and the client
-// walk, which spreads one client over a warp, is the faster one (graph900 generation, 904 units per scan: 209 us
-// with the client walk, 270 us bit-sliced; 3001 x 2011, pop 777, 2350 units: 136 against 87 us).
+// of about 1200 instructions of one warp, so with too few per SM the SMs wait for single warps and the rank-split
+// walk is the faster one.  GA generations whose scans have 16 to 23 units per SM (graph900 pop 2048; 5000 x 5000, p =
+// 500, pop 512): 213 and 303 us rank-split against 240 and 326 bit-sliced; 33 to 47 per SM (3000 x 3000, p = 30, pop
+// 256; graph900 pop 1024): 485 and 168 against 361 and 157.
 static inline bool pm_sliced_pays(const pm_instance *inst, int64_t units)
 {
-    return units >= (int64_t)inst->sm_count * 12;
+    return units >= (int64_t)inst->sm_count * 24;
 }
+// Whether the rank-split walk's tables fit beside tiles of W words and its 32-bit sums hold inst's distances.
+bool pm_split_fits(const pm_instance *inst, int64_t W, int G, int warps);
 // The deepest first open rank a unit of 1024 pairs is expected to meet: 1024 geometric draws of mean (m+1)/(p+1).
 static inline double pm_walk_depth(int64_t m, int64_t p, int64_t L)
 {
@@ -324,6 +329,7 @@ pm_status pm_launch_random_population(const pm_instance *inst, uint64_t seed, in
 // per-instance splits, global numbering of individuals, rows, tiles.
 struct pm_multi_plan {
     int groups = 4, warps = 16, nb = 0;
+    bool split = false;
     int64_t grid = 0, items = 0, jobs = 0;
     int64_t tiles_total = 0, ind_total = 0, words_total = 0, cols_total = 0;
     int64_t Wmax = 0;  // bitset words of the widest instance

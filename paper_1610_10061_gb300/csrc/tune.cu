@@ -25,7 +25,8 @@ namespace {
 bool same_shape(const pm_eval_plan &a, const pm_eval_plan &b)
 {
     return a.groups == b.groups && a.warps == b.warps && a.splits == b.splits && a.bytes == b.bytes &&
-           a.direct.range == b.direct.range && a.stream == b.stream;
+           a.direct.range == b.direct.range && a.stream == b.stream &&
+           a.split == b.split;
 }
 
 // The shape as the ABI reports it: groups -1 is the row kernel with byte masks.
