@@ -803,11 +803,20 @@ static pm_status allow_dynamic_smem(const pm_instance *inst, F *fn)
 
 pm_status pm_fitness_init(const pm_instance *inst)
 {
+    // once per device: the attributes stay with the loaded kernels (about 1 us each, 17 of them)
+    static std::mutex mu;
+    static bool done[64] = {};
+    const int dev = inst->device;
+    std::lock_guard<std::mutex> guard(mu);
+    if (dev >= 0 && dev < 64 && done[dev])
+        return PM_OK;
     for (int G : {1, 2, 4})
         for (ScanKind kind : {ScanKind::clients, ScanKind::split, ScanKind::sliced, ScanKind::direct, ScanKind::mixed})
             PM_TRY(allow_dynamic_smem(inst, scan_fn(G, kind)));
     PM_TRY(allow_dynamic_smem(inst, k_scan_rows<false>));
     PM_TRY(allow_dynamic_smem(inst, k_scan_rows<true>));
+    if (dev >= 0 && dev < 64)
+        done[dev] = true;
     return PM_OK;
 }
 

@@ -354,8 +354,8 @@ void pm_scan_launch_from(const pm_multi_plan &mp, const pm_prob *probs_dev, pm_s
 // Tables (tables.cu)
 // ---------------------------------------------------------------------------
 pm_status pm_build_tables(pm_instance *inst, const int32_t *d_dev, cudaStream_t stream);
-// Delta' of a cumulative instance (differences of its D' rows) into out (n x L, device).
-pm_status pm_launch_increments(const pm_instance *inst, int32_t *out, cudaStream_t stream);
+// Dense n x L copies of the tables on the device (Delta' also for cumulative instances); either output may be null.
+pm_status pm_launch_dense_rows(const pm_instance *inst, uint16_t *pi_out, int32_t *delta_out, cudaStream_t stream);
 
 // ---------------------------------------------------------------------------
 // Small helpers
