@@ -1110,8 +1110,8 @@ __device__ __forceinline__ bool cand_before(unsigned long long g, int32_t k, uns
 // The learned try's candidate moves straight from one individual's statistics
 // in shared memory (the fused form of k_candidates, which reads them back from
 // global memory): the open facilities in ascending order, the T closed
-// facilities of largest gain (ties: lower id) by T block-wide arg-max passes,
-// and the p * T feature rows (row a * T + b: the a-th open facility with the
+// facilities of largest gain (ties: lower id) -- with 32-bit gains in one pass,
+// else by T block-wide arg-max passes -- and the p * T feature rows (row a * T + b: the a-th open facility with the
 // b-th candidate; the first open one stands in past the open count), each
 // computed as k_candidates computes it.
 struct CandOut {
@@ -1123,20 +1123,78 @@ struct CandOut {
     int64_t n;
 };
 
+// The T <= N closed facilities of largest 32-bit gain -> top_k, in one pass: a facility's key (gain, then the lower id)
+// is 64 bits; every thread keeps its own N best, every warp takes T of them off its lanes' heads (red_top, kMaxCand per
+// warp), warp 0 the T best of those.  (T passes over all gains, each with a block-wide maximum, kept the CTA waiting
+// for about 25 us of a learned generation of 5000 x 5000 four waves of CTAs long.)
+template <int N>
+__device__ __forceinline__ void top_closed(const uint32_t *bits, const unsigned int *gains, int32_t m, int32_t T,
+                                           unsigned long long *red_top, int32_t *top_k)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    unsigned long long best[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+        best[q] = 0ull;  // behind every facility's key
+    for (int k = tid; k < m; k += blockDim.x) {
+        if ((bits[k >> 5] >> (k & 31)) & 1u)
+            continue;
+        unsigned long long key = ((unsigned long long)gains[k] << 17) | (unsigned long long)(0x1ffff - k);
+        if (key <= best[N - 1])
+            continue;
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            const unsigned long long hi = max(best[q], key);
+            key = min(best[q], key);
+            best[q] = hi;
+        }
+    }
+    auto pop_max = [&]() {  // the largest head of the warp's lanes, taken off its lane
+        const uint32_t hi = __reduce_max_sync(PM_FULL_MASK, (uint32_t)(best[0] >> 32));
+        const uint32_t lo = __reduce_max_sync(PM_FULL_MASK, (uint32_t)(best[0] >> 32) == hi ? (uint32_t)best[0] : 0u);
+        const unsigned long long top = ((unsigned long long)hi << 32) | lo;
+        if (best[0] == top)  // keys are distinct, but for the empty ones
+#pragma unroll
+            for (int q = 0; q < N; ++q)
+                best[q] = q + 1 < N ? best[q + 1] : 0ull;
+        return top;
+    };
+    for (int b = 0; b < T; ++b) {
+        const unsigned long long top = pop_max();
+        if (lane == 0)
+            red_top[warp * kMaxCand + b] = top;
+    }
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+        for (int q = 0; q < N; ++q)
+            best[q] = q < T && lane < nwarps ? red_top[lane * kMaxCand + q] : 0ull;
+        int32_t last = 0;
+        for (int b = 0; b < T; ++b) {
+            const unsigned long long top = pop_max();
+            last = top ? 0xffff - (int32_t)(top & 0xffffull) : last;  // fewer than T closed: repeat the previous one
+            if (lane == 0)
+                top_k[b] = last;
+        }
+    }
+    __syncthreads();
+}
+
 template <typename Acc>
 __device__ __forceinline__ void candidates_from_stats(const uint32_t *bits, const Acc *Gs, const Acc *Ls,
                                                       const int *Cs, const int *As, int32_t *open_s, int32_t W,
                                                       int32_t m, int64_t t, const CandOut &co)
 {
     constexpr int32_t kNone = 0x7fffffff;
+    const int32_t p = co.p, T = co.T;
     __shared__ int32_t top_k[kMaxCand];
     __shared__ unsigned long long top_g[kMaxCand];
     __shared__ float top_f1[kMaxCand], top_f3[kMaxCand], top_f6[kMaxCand];
     __shared__ unsigned long long red_g[32];
+    unsigned long long *red_top = reinterpret_cast<unsigned long long *>(open_s + ((p + 3) & ~3));
     __shared__ int32_t red_k[32];
     __shared__ int32_t nopen;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-    const int32_t p = co.p, T = co.T;
     for (int i = tid; i < p; i += blockDim.x)
         open_s[i] = 0;  // a bitset with fewer than p open facilities still yields valid ids
     __syncthreads();
@@ -1167,48 +1225,55 @@ __device__ __forceinline__ void candidates_from_stats(const uint32_t *bits, cons
         if (lane == 0)
             nopen = cnt < p ? cnt : p;
     }
-    for (int b = 0; b < T; ++b) {
-        unsigned long long bg = 0ull;
-        int32_t bk = kNone;
-        for (int k = tid; k < m; k += blockDim.x) {
-            if ((bits[k >> 5] >> (k & 31)) & 1u)
-                continue;
-            bool taken = false;
-            for (int q = 0; q < b; ++q)
-                taken = taken || (top_k[q] == k);
-            const unsigned long long gk = (unsigned long long)Gs[k];
-            if (!taken && cand_before(gk, k, bg, bk)) {
-                bg = gk;
-                bk = k;
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long og = __shfl_xor_sync(PM_FULL_MASK, bg, o);
-            const int32_t ok = __shfl_xor_sync(PM_FULL_MASK, bk, o);
-            if (cand_before(og, ok, bg, bk)) {
-                bg = og;
-                bk = ok;
-            }
-        }
-        if (lane == 0) {
-            red_g[warp] = bg;
-            red_k[warp] = bk;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            unsigned long long g0 = red_g[0];
-            int32_t k0 = red_k[0];
-            for (int w = 1; w < nwarps; ++w)
-                if (cand_before(red_g[w], red_k[w], g0, k0)) {
-                    g0 = red_g[w];
-                    k0 = red_k[w];
+    if constexpr (sizeof(Acc) == 4) {
+        if (T <= 4)
+            top_closed<4>(bits, Gs, m, T, red_top, top_k);
+        else
+            top_closed<kMaxCand>(bits, Gs, m, T, red_top, top_k);
+    } else {
+        for (int b = 0; b < T; ++b) {
+            unsigned long long bg = 0ull;
+            int32_t bk = kNone;
+            for (int k = tid; k < m; k += blockDim.x) {
+                if ((bits[k >> 5] >> (k & 31)) & 1u)
+                    continue;
+                bool taken = false;
+                for (int q = 0; q < b; ++q)
+                    taken = taken || (top_k[q] == k);
+                const unsigned long long gk = (unsigned long long)Gs[k];
+                if (!taken && cand_before(gk, k, bg, bk)) {
+                    bg = gk;
+                    bk = k;
                 }
-            if (k0 == kNone)  // fewer than T closed facilities: repeat the previous one
-                k0 = b > 0 ? top_k[b - 1] : 0;
-            top_k[b] = k0;
+            }
+    #pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long og = __shfl_xor_sync(PM_FULL_MASK, bg, o);
+                const int32_t ok = __shfl_xor_sync(PM_FULL_MASK, bk, o);
+                if (cand_before(og, ok, bg, bk)) {
+                    bg = og;
+                    bk = ok;
+                }
+            }
+            if (lane == 0) {
+                red_g[warp] = bg;
+                red_k[warp] = bk;
+            }
+            __syncthreads();
+            if (tid == 0) {
+                unsigned long long g0 = red_g[0];
+                int32_t k0 = red_k[0];
+                for (int w = 1; w < nwarps; ++w)
+                    if (cand_before(red_g[w], red_k[w], g0, k0)) {
+                        g0 = red_g[w];
+                        k0 = red_k[w];
+                    }
+                if (k0 == kNone)  // fewer than T closed facilities: repeat the previous one
+                    k0 = b > 0 ? top_k[b - 1] : 0;
+                top_k[b] = k0;
+            }
+            __syncthreads();
         }
-        __syncthreads();
     }
     const float Z = fmaxf((float)co.costs[t] / (float)p, 1.f);
     const float per = (float)co.n / (float)p, ratio = (float)p / (float)m;
@@ -2248,7 +2313,9 @@ pm_status pm_launch_learned_candidates(const pm_instance *inst, const uint32_t *
     const size_t bits = (size_t)pm_round_up(inst->W * 4, 16);
     const bool narrow = (double)inst->n * (double)std::max(inst->max_d, 1) < 4294967295.0;
     const size_t acc = (size_t)inst->m * (narrow ? 16 : 24);
-    const size_t smem = (size_t)pm_round_up(bits + acc, 16) + (size_t)pm_round_up(inst->p * 4, 16);
+    // ... + the open list + the warps' best candidates
+    const size_t smem = (size_t)pm_round_up(bits + acc, 16) + (size_t)pm_round_up(inst->p * 4, 16) +
+                        (size_t)32 * kMaxCand * 8;
     const int32_t *dist = inst->cum ? inst->delta : static_cast<const int32_t *>(inst->dsorted.ptr);
     const char *env = std::getenv("PM_LEARN_FUSED");  // PM_LEARN_FUSED=0: always the two kernels (for comparison)
     if (!dist || smem + 1024 > inst->smem_optin || (env && env[0] == '0')) {
