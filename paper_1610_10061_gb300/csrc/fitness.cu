@@ -124,7 +124,12 @@ struct ScanEpilogue {
 // The epilogue of one tile's individuals marked in fin_s (bit i of word i/32),
 // one warp per individual: store the cost, or
 // accept the candidate (copy its bitset, cost and improved flag) when it is
-// strictly cheaper than the current individual.
+// strictly cheaper than the current individual.  kFlight words of a row per
+// lane are copied at a time: with one, every 32 words of a long row wait for
+// memory, and the CTA that brings a tile's last share for most others (learned
+// generation of 5000 x 5000, p = 500: 1.09 ms, 1.05 with four; the short rows
+// of small launches are faster with one, graph900 0.163 against 0.164).
+template <int kFlight>
 __device__ __forceinline__ void apply_epilogue(const unsigned long long *acc_s, const uint32_t *fin_s, int count,
                                                const pm_prob &pr, int64_t ind0, int warp, int nwarps, int lane,
                                                const ScanEpilogue &ep)
@@ -141,8 +146,21 @@ __device__ __forceinline__ void apply_epilogue(const unsigned long long *acc_s, 
             ep.costs[pr.out_base + t] = sum;
         if (ep.mode == 1 && sum < ep.cur_cost[pr.ind_base + t]) {
             const int64_t row = pr.word_base + t * W;
-            for (int q = lane; q < W; q += 32)
-                ep.cur_masks[row + q] = ep.cand_masks[row + q];
+            if constexpr (kFlight == 1) {
+                for (int q = lane; q < W; q += 32)
+                    ep.cur_masks[row + q] = ep.cand_masks[row + q];
+            } else {
+                for (int q = lane; q < W; q += 32 * kFlight) {
+                    uint32_t v[kFlight];
+    #pragma unroll
+                    for (int f = 0; f < kFlight; ++f)
+                        v[f] = q + 32 * f < W ? __ldg(ep.cand_masks + row + q + 32 * f) : 0u;
+    #pragma unroll
+                    for (int f = 0; f < kFlight; ++f)
+                        if (q + 32 * f < W)
+                            ep.cur_masks[row + q + 32 * f] = v[f];
+                }
+            }
             if (lane == 0) {
                 ep.cur_cost[pr.ind_base + t] = sum;
                 if (ep.improved)
@@ -588,7 +606,7 @@ __global__ void __launch_bounds__(kKind == ScanKind::clients || kKind == ScanKin
             }
         }
         if (finish)
-            apply_epilogue(acc_s, fin, count, pr, ind0, warp, nwarps, lane, ep);
+            apply_epilogue<kSplit ? 1 : 4>(acc_s, fin, count, pr, ind0, warp, nwarps, lane, ep);
         __syncthreads();  // shared state (tile, acc_s, a0_s, pr_s) is reused by the next item
     }
 }
