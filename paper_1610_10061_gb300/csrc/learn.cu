@@ -152,6 +152,31 @@ __device__ __forceinline__ int core_idx(int row, int k, int K)
     return ((row >> 3) * (K >> 3) * 128 + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2) >> 1;
 }
 
+// The weights as the tensor-core kernels' B operands, kept beside the row-major BF16 copies (k_adam and k_refresh_bf16
+// write both), so that a CTA stages them with 16-byte copies: W1 (n = out, k = in), W2 (n = out, k = in), W2 (n = in,
+// k = out).
+constexpr int kTiledW1 = 0, kTiledW2T = kHid * kIn, kTiledW2 = kTiledW2T + kHid * kHid,
+              kTiledWords = kTiledW2 + kHid * kHid;  // elements
+
+__device__ __forceinline__ void store_tiled(__nv_bfloat16 *tiled, int i, __nv_bfloat16 w)  // parameter i of W1 or W2
+{
+    if (i < kOffB1) {
+        tiled[kTiledW1 + core_idx(i % kHid, i / kHid, kIn)] = w;
+    } else if (i >= kOffW2 && i < kOffB2) {
+        const int in = (i - kOffW2) / kHid, out = (i - kOffW2) % kHid;
+        tiled[kTiledW2T + core_idx(out, in, kHid)] = w;
+        tiled[kTiledW2 + core_idx(in, out, kHid)] = w;
+    }
+}
+
+// Copy `count` (a multiple of 8) elements into shared memory, 16 bytes a thread and step.
+__device__ __forceinline__ void stage16(__nv_bfloat16 *dst, const __nv_bfloat16 *src, int count)
+{
+#pragma unroll 4
+    for (int i = threadIdx.x; i < count / 8; i += blockDim.x)
+        reinterpret_cast<uint4 *>(dst)[i] = reinterpret_cast<const uint4 *>(src)[i];
+}
+
 struct TcSmem {
     __nv_bfloat16 A1[kTcRows * kIn];  // X tile
     __nv_bfloat16 B1[kHid * kIn];     // W1 as (n = out, k = in)
@@ -226,8 +251,7 @@ __device__ __forceinline__ void tc_sync_for_mma()
 }
 
 __global__ void __launch_bounds__(kTcThreads) k_mlp_fwd_tc(const __nv_bfloat16 *__restrict__ X, int64_t rows,
-                                                           const __nv_bfloat16 *__restrict__ W1b,
-                                                           const __nv_bfloat16 *__restrict__ W2b,
+                                                           const __nv_bfloat16 *__restrict__ tiled,
                                                            const __nv_bfloat16 *__restrict__ w3b,
                                                            const float *__restrict__ P, float *__restrict__ y_out,
                                                            int *__restrict__ err)
@@ -239,14 +263,8 @@ __global__ void __launch_bounds__(kTcThreads) k_mlp_fwd_tc(const __nv_bfloat16 *
     const int64_t tiles = (rows + kTcRows - 1) / kTcRows;
 
     // weights and biases, once per CTA
-    for (int i = tid; i < kIn * kHid; i += blockDim.x) {  // W1 [in][out]
-        const int in = i / kHid, out = i % kHid;
-        S.B1[core_idx(out, in, kIn)] = W1b[i];
-    }
-    for (int i = tid; i < kHid * kHid; i += blockDim.x) {  // W2 [in][out]
-        const int in = i / kHid, out = i % kHid;
-        S.B2[core_idx(out, in, kHid)] = W2b[i];
-    }
+    stage16(S.B1, tiled + kTiledW1, kHid * kIn);
+    stage16(S.B2, tiled + kTiledW2T, kHid * kHid);
     for (int i = tid; i < kHid; i += blockDim.x) {
         S.b1[i] = P[kOffB1 + i];
         S.b2[i] = P[kOffB2 + i];
@@ -746,10 +764,9 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
 }
 
 __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloat16 *__restrict__ X, int64_t rows,
-                                                                const __nv_bfloat16 *__restrict__ W1b,
-                                                                const __nv_bfloat16 *__restrict__ W2b,
-                                                                const __nv_bfloat16 *__restrict__ w3b,
-                                                                const float *__restrict__ P,
+                                                                const __nv_bfloat16 *tiled,
+                                                                const __nv_bfloat16 *w3b,
+                                                                const float *P,
                                                                 const float *__restrict__ t, float inv_batch,
                                                                 float *__restrict__ grads, float *__restrict__ loss,
                                                                 RowMap map, int tpc, int *__restrict__ err)
@@ -760,24 +777,8 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
     const int quad = warp & 3, half = warp >> 2;
     const int64_t tiles = (rows + kTcRows - 1) / kTcRows;
 
-    for (int i = tid; i < kIn * kHid; i += blockDim.x) {  // W1 [in][out]
-        const int in = i / kHid, out = i % kHid;
-        S.BW1[core_idx(out, in, kIn)] = W1b[i];
-    }
-    for (int i = tid; i < kHid * kHid; i += blockDim.x) {  // W2 [in][out]
-        const int in = i / kHid, out = i % kHid;
-        S.BW2T[core_idx(out, in, kHid)] = W2b[i];
-        S.BW2[core_idx(in, out, kHid)] = W2b[i];
-    }
-    for (int i = tid; i < kHid; i += blockDim.x) {
-        S.b1[i] = P[kOffB1 + i];
-        S.b2[i] = P[kOffB2 + i];
-        S.w3[i] = __bfloat162float(w3b[i]);
-        S.gb1[i] = 0.f;
-        S.gb2[i] = 0.f;
-        S.gw3[i] = 0.f;
-    }
-    const float b3 = P[kOffB3];
+    // Before the dependency wait (the previous step's k_adam may still run): the barrier, tensor memory and the first
+    // tile's rows, which no kernel of the training loop writes.
     if (tid == 0) {
         S.gb3 = 0.f;
         S.sq = 0.f;
@@ -791,12 +792,67 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    // a tile's rows: X (both layouts) and targets
+    auto stage_rows = [&](int64_t pos0) {
+        const int xr = tid >> 1, xh = tid & 1;
+        const bool valid = pos0 + xr < rows;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        int64_t src = 0;
+        if (valid) {
+            src = shuffled_row(map, map.pos0 + pos0 + xr);
+            v = __ldg(reinterpret_cast<const uint4 *>(X + src * kIn) + xh);
+        }
+        *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(S.AX) + (xr >> 3) * 256 + xh * 128 +
+                                   (xr & 7) * 16) = v;
+        const uint32_t wv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int f = 8 * xh + 2 * q;
+            reinterpret_cast<uint16_t *>(S.BXT)[core_idx(f, xr, kTcRows)] = (uint16_t)(wv[q] & 0xffffu);
+            reinterpret_cast<uint16_t *>(S.BXT)[core_idx(f + 1, xr, kTcRows)] = (uint16_t)(wv[q] >> 16);
+        }
+        if (xh == 0)
+            S.tgt[xr] = valid ? t[src] : 0.f;
+    };
+    stage_rows(blockIdx.x * (int64_t)tpc * kTcRows);
+    pm_grid_dependency_wait();
+    stage16(S.BW1, tiled + kTiledW1, kHid * kIn);
+    stage16(S.BW2T, tiled + kTiledW2T, kHid * kHid);
+    stage16(S.BW2, tiled + kTiledW2, kHid * kHid);
+    for (int i = tid; i < kHid; i += blockDim.x) {
+        S.b1[i] = P[kOffB1 + i];
+        S.b2[i] = P[kOffB2 + i];
+        S.w3[i] = __bfloat162float(w3b[i]);
+        S.gb1[i] = 0.f;
+        S.gb2[i] = 0.f;
+        S.gw3[i] = 0.f;
+    }
+    const float b3 = P[kOffB3];
     tc_sync_for_mma();
     const uint32_t tmem = S.tmem, C0 = tmem, C2 = tmem + 128u, C3 = tmem + 256u;
     const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
     const int r = quad * 32 + lane;  // this thread's row of the tile (its TMEM lane)
     const int c0 = half * 64;        // its first column
     constexpr uint32_t kSbo = (kHid / 8) * 128;
+    // Eight columns (four packed pairs) of this thread's row into a transposed tile (m or n = column, k = row).  The
+    // four groups of eight lanes lie 128 bytes apart, in the same banks, so each starts with another pair.
+    const int turn = (lane >> 3) & 3;
+    auto store_columns = [&](__nv_bfloat16 *tile, int col, const uint32_t (&pk)[4]) {
+        uint32_t a[4], b[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            a[i] = (turn & 1) ? pk[(i + 1) & 3] : pk[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            b[i] = (turn & 2) ? a[(i + 2) & 3] : a[i];
+        uint16_t *out = reinterpret_cast<uint16_t *>(tile) + core_idx(col, r, kTcRows);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int q = (i + turn) & 3;  // columns col + 2 q and the next, 16 bytes apart
+            out[16 * q] = (uint16_t)(b[i] & 0xffffu);
+            out[16 * q + 8] = (uint16_t)(b[i] >> 16);
+        }
+    };
 
     uint32_t phase = 0;
     bool ok = true, any = false;
@@ -810,28 +866,8 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
     const int64_t last = blockIdx.x * (int64_t)tpc + tpc;
     for (int64_t tile = blockIdx.x * (int64_t)tpc; tile < tiles && tile < last && ok; ++tile) {
         const int64_t pos0 = tile * kTcRows;
-        // ---- the tile's rows: X (both layouts) and targets ----
-        {
-            const int xr = tid >> 1, xh = tid & 1;
-            const bool valid = pos0 + xr < rows;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            int64_t src = 0;
-            if (valid) {
-                src = shuffled_row(map, map.pos0 + pos0 + xr);
-                v = __ldg(reinterpret_cast<const uint4 *>(X + src * kIn) + xh);
-            }
-            *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(S.AX) + (xr >> 3) * 256 + xh * 128 +
-                                       (xr & 7) * 16) = v;
-            const uint32_t wv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int f = 8 * xh + 2 * q;
-                reinterpret_cast<uint16_t *>(S.BXT)[core_idx(f, xr, kTcRows)] = (uint16_t)(wv[q] & 0xffffu);
-                reinterpret_cast<uint16_t *>(S.BXT)[core_idx(f + 1, xr, kTcRows)] = (uint16_t)(wv[q] >> 16);
-            }
-            if (xh == 0)
-                S.tgt[xr] = valid ? t[src] : 0.f;
-        }
+        if (tile > blockIdx.x * (int64_t)tpc)
+            stage_rows(pos0);
         const int nvalid = (int)((rows - pos0) < kTcRows ? (rows - pos0) : kTcRows);
         tc_sync_for_mma();
         if (tid == 0) {  // layer 1
@@ -856,9 +892,8 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
                     const float lo = bf16_lo(pk[q]), hi = bf16_hi(pk[q]);
                     bits |= (lo > 0.f ? 1u : 0u) << (8 * g + 2 * q);
                     bits |= (hi > 0.f ? 1u : 0u) << (8 * g + 2 * q + 1);
-                    reinterpret_cast<uint16_t *>(S.T1)[core_idx(col + 2 * q, r, kTcRows)] = (uint16_t)(pk[q] & 0xffffu);
-                    reinterpret_cast<uint16_t *>(S.T1)[core_idx(col + 2 * q + 1, r, kTcRows)] = (uint16_t)(pk[q] >> 16);
                 }
+                store_columns(S.T1, col, pk);
                 *reinterpret_cast<uint4 *>(S.R + core_idx(r, col, kHid)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
             }
             S.mask1[4 * r + (c0 + cc) / 32] = bits;
@@ -919,13 +954,13 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
                 const float g0 = bf16_lo(h2[q]) > 0.f ? dyr * S.w3[col] : 0.f;
                 const float g1 = bf16_hi(h2[q]) > 0.f ? dyr * S.w3[col + 1] : 0.f;
                 h2[q] = pack_bf16x2(g0, g1);  // dH2, packed
-                reinterpret_cast<uint16_t *>(S.T2)[core_idx(col, r, kTcRows)] = (uint16_t)(h2[q] & 0xffffu);
-                reinterpret_cast<uint16_t *>(S.T2)[core_idx(col + 1, r, kTcRows)] = (uint16_t)(h2[q] >> 16);
             }
 #pragma unroll
-            for (int g = 0; g < 8; ++g)
-                *reinterpret_cast<uint4 *>(S.R + core_idx(r, c0 + 8 * g, kHid)) =
-                    make_uint4(h2[4 * g], h2[4 * g + 1], h2[4 * g + 2], h2[4 * g + 3]);
+            for (int g = 0; g < 8; ++g) {
+                const uint32_t pk[4] = {h2[4 * g], h2[4 * g + 1], h2[4 * g + 2], h2[4 * g + 3]};
+                store_columns(S.T2, c0 + 8 * g, pk);
+                *reinterpret_cast<uint4 *>(S.R + core_idx(r, c0 + 8 * g, kHid)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            }
         }
         tc_sync_for_mma();
         if (tid == 0) {  // dH1 pre-activation, and dW2 += H1^T dH2
@@ -957,13 +992,16 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
             tc_ld32(C0 + lane_off + (uint32_t)(c0 + cc), v);
             const uint32_t bits = S.mask1[4 * r + (c0 + cc) / 32];
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const int col = c0 + cc + 2 * q;
-                const float g0 = ((bits >> (2 * q)) & 1u) ? __uint_as_float(v[2 * q]) : 0.f;
-                const float g1 = ((bits >> (2 * q + 1)) & 1u) ? __uint_as_float(v[2 * q + 1]) : 0.f;
-                const uint32_t pk = pack_bf16x2(g0, g1);
-                reinterpret_cast<uint16_t *>(S.T1)[core_idx(col, r, kTcRows)] = (uint16_t)(pk & 0xffffu);
-                reinterpret_cast<uint16_t *>(S.T1)[core_idx(col + 1, r, kTcRows)] = (uint16_t)(pk >> 16);
+            for (int g = 0; g < 4; ++g) {
+                uint32_t pk[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int k = 8 * g + 2 * q;
+                    const float g0 = ((bits >> k) & 1u) ? __uint_as_float(v[k]) : 0.f;
+                    const float g1 = ((bits >> (k + 1)) & 1u) ? __uint_as_float(v[k + 1]) : 0.f;
+                    pk[q] = pack_bf16x2(g0, g1);
+                }
+                store_columns(S.T1, c0 + cc + 8 * g, pk);
             }
         }
         tc_sync_for_mma();
@@ -991,8 +1029,12 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
             uint32_t v[32];
             tc_ld32(C2 + lane_off + (uint32_t)(c0 + cc), v);
 #pragma unroll
-            for (int q = 0; q < 32; ++q)
-                atomicAdd(grads + kOffW2 + r * kHid + c0 + cc + q, __uint_as_float(v[q]));
+            for (int q = 0; q < 32; q += 4)  // kOffW2 is a multiple of 4: 16-byte aligned
+                asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(
+                                 grads + kOffW2 + r * kHid + c0 + cc + q),
+                             "f"(__uint_as_float(v[q])), "f"(__uint_as_float(v[q + 1])),
+                             "f"(__uint_as_float(v[q + 2])), "f"(__uint_as_float(v[q + 3]))
+                             : "memory");
         }
         if (half == 0) {
             uint32_t v[16];
@@ -1025,12 +1067,15 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
 // Adam (Kingma & Ba 2015, Algorithm 1) on the FP32 masters; refreshes the BF16 copies.
 // The gradient buffer is left zero for the next step.  loss_word (nullable): the step's sum of squares, which
 // thread 0 moves (times inv_rows) into *loss_out and clears.
-__global__ void k_adam(float *__restrict__ P, float *__restrict__ M, float *__restrict__ V,
-                       float *__restrict__ G, int n, float lr, float bc1, float bc2,
-                       __nv_bfloat16 *__restrict__ W1b, __nv_bfloat16 *__restrict__ W2b,
-                       __nv_bfloat16 *__restrict__ w3b, float *__restrict__ loss_word, float *__restrict__ loss_out,
-                       float inv_rows)
+// What the kernel reads was written by the kernel that it may overlap (pm_launch): its pointers, and those of the
+// parameters in k_mlp_train_tc, are not __restrict__, so that no load moves above the dependency wait.
+__global__ void k_adam(float *P, float *M, float *V,
+                       float *G, int n, float lr, float bc1, float bc2,
+                       __nv_bfloat16 *W1b, __nv_bfloat16 *W2b,
+                       __nv_bfloat16 *w3b, __nv_bfloat16 *tiled,
+                       float *loss_word, float *loss_out, float inv_rows)
 {
+    pm_grid_dependency_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0 && loss_word != nullptr) {
         *loss_out = *loss_word * inv_rows;
@@ -1053,12 +1098,18 @@ __global__ void k_adam(float *__restrict__ P, float *__restrict__ M, float *__re
         W2b[i - kOffW2] = __float2bfloat16(w);
     else if (i >= kOffW3 && i < kOffB3)
         w3b[i - kOffW3] = __float2bfloat16(w);
+    store_tiled(tiled, i, __float2bfloat16(w));
 }
 
 __global__ void k_refresh_bf16(const float *__restrict__ P, __nv_bfloat16 *__restrict__ W1b,
-                               __nv_bfloat16 *__restrict__ W2b, __nv_bfloat16 *__restrict__ w3b)
+                               __nv_bfloat16 *__restrict__ W2b, __nv_bfloat16 *__restrict__ w3b,
+                               __nv_bfloat16 *__restrict__ tiled)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < kIn * kHid)
+        store_tiled(tiled, kOffW1 + i, __float2bfloat16(P[kOffW1 + i]));
+    if (i < kHid * kHid)
+        store_tiled(tiled, kOffW2 + i, __float2bfloat16(P[kOffW2 + i]));
     if (i < kIn * kHid)
         W1b[i] = __float2bfloat16(P[kOffW1 + i]);
     if (i < kHid * kHid)
@@ -1894,11 +1945,17 @@ static pm_status mlp_init_attrs()
     return PM_OK;
 }
 
+// The tiled weights lie behind the row-major copy of W2, in its buffer.
+static __nv_bfloat16 *tiled_weights(const pm_model *md)
+{
+    return static_cast<__nv_bfloat16 *>(md->W2b.ptr) + kHid * kHid;
+}
+
 static pm_status model_refresh(pm_model *md, cudaStream_t s)
 {
     k_refresh_bf16<<<(kHid * kHid + 255) / 256, 256, 0, s>>>(
         static_cast<const float *>(md->P.ptr), static_cast<__nv_bfloat16 *>(md->W1b.ptr),
-        static_cast<__nv_bfloat16 *>(md->W2b.ptr), static_cast<__nv_bfloat16 *>(md->w3b.ptr));
+        static_cast<__nv_bfloat16 *>(md->W2b.ptr), static_cast<__nv_bfloat16 *>(md->w3b.ptr), tiled_weights(md));
     PM_CUDA(cudaGetLastError());
     return PM_OK;
 }
@@ -1925,7 +1982,7 @@ extern "C" pm_status pm_model_create(int device, uint64_t seed, pm_model **out)
     if (st == PM_OK)
         st = md->W1b.reserve(kIn * kHid * 2);
     if (st == PM_OK)
-        st = md->W2b.reserve(kHid * kHid * 2);
+        st = md->W2b.reserve((kHid * kHid + kTiledWords) * 2);
     if (st == PM_OK)
         st = md->w3b.reserve(kHid * 2);
     if (st == PM_OK)
@@ -2012,7 +2069,7 @@ extern "C" pm_status pm_model_get_params(pm_model *md, float *params, void *stre
 }
 
 static pm_status mlp_launch(pm_model *md, bool train, const void *x, int64_t rows, float *y, const float *t,
-                            float inv_batch, cudaStream_t s, RowMap map = RowMap{})
+                            float inv_batch, cudaStream_t s, RowMap map = RowMap{}, bool chained = false)
 {
     const unsigned grid = (unsigned)pm_ceil_div(rows, kRows);
     const __nv_bfloat16 *X = static_cast<const __nv_bfloat16 *>(x);
@@ -2025,9 +2082,18 @@ static pm_status mlp_launch(pm_model *md, bool train, const void *x, int64_t row
         // gradient atomics: the weight gradients accumulate in tensor memory)
         const int64_t tiles = pm_ceil_div(rows, kTcRows);
         const int tpc = (int)std::max<int64_t>(1, pm_ceil_div(tiles, (int64_t)md->sm_count));
-        k_mlp_train_tc<<<(unsigned)pm_ceil_div(tiles, tpc), kTrThreads, sizeof(TrSmem), s>>>(
-            X, rows, W1b, W2b, w3b, P, t, inv_batch, static_cast<float *>(md->G.ptr),
-            static_cast<float *>(md->loss.ptr), map, tpc, static_cast<int *>(md->err.ptr));
+        const unsigned ctas = (unsigned)pm_ceil_div(tiles, tpc);
+        const __nv_bfloat16 *tiled = tiled_weights(md);
+        float *G = static_cast<float *>(md->G.ptr), *sq = static_cast<float *>(md->loss.ptr);
+        int *err = static_cast<int *>(md->err.ptr);
+        // a step of a training loop starts its first rows under the step before (chained), whose k_adam it waits for;
+        // the first one starts after whatever wrote the rows
+        if (chained)
+            PM_CUDA(pm_launch(k_mlp_train_tc, ctas, kTrThreads, sizeof(TrSmem), s, X, rows, tiled, w3b, P, t, inv_batch,
+                              G, sq, map, tpc, err));
+        else
+            k_mlp_train_tc<<<ctas, kTrThreads, sizeof(TrSmem), s>>>(X, rows, tiled, w3b, P, t, inv_batch, G, sq, map, tpc,
+                                                                    err);
     }
     else if (train)
         k_mlp<true><<<grid, 128, mlp_smem(true), s>>>(X, rows, W1b, W2b, w3b, P, y, t, inv_batch,
@@ -2035,7 +2101,7 @@ static pm_status mlp_launch(pm_model *md, bool train, const void *x, int64_t row
                                                       static_cast<float *>(md->loss.ptr), map);
     else
         k_mlp_fwd_tc<<<(unsigned)std::min<int64_t>(pm_ceil_div(rows, kTcRows), 3 * (int64_t)md->sm_count),
-                       kTcThreads, tc_smem(), s>>>(X, rows, W1b, W2b, w3b, P, y, static_cast<int *>(md->err.ptr));
+                       kTcThreads, tc_smem(), s>>>(X, rows, tiled_weights(md), w3b, P, y, static_cast<int *>(md->err.ptr));
     PM_CUDA(cudaGetLastError());
     return PM_OK;
 }
@@ -2115,8 +2181,8 @@ extern "C" pm_status pm_model_train_step(pm_model *md, const uint16_t *x, const 
     k_adam<<<(kParams + 255) / 256, 256, 0, s>>>(
         static_cast<float *>(md->P.ptr), static_cast<float *>(md->M.ptr), static_cast<float *>(md->V.ptr),
         static_cast<float *>(md->G.ptr), kParams, lr, bc1, bc2, static_cast<__nv_bfloat16 *>(md->W1b.ptr),
-        static_cast<__nv_bfloat16 *>(md->W2b.ptr), static_cast<__nv_bfloat16 *>(md->w3b.ptr), nullptr, nullptr,
-        0.f);
+        static_cast<__nv_bfloat16 *>(md->W2b.ptr), static_cast<__nv_bfloat16 *>(md->w3b.ptr), tiled_weights(md),
+        nullptr, nullptr, 0.f);
     PM_CUDA(cudaGetLastError());
     if (loss)
         PM_CUDA(cudaStreamSynchronize(s));
@@ -2185,16 +2251,16 @@ extern "C" pm_status pm_model_train(pm_model *md, const uint16_t *x, const float
         for (int64_t b0 = 0; b0 < rows; b0 += batch, ++k) {
             const int64_t nrow = std::min(batch, rows - b0);
             map.pos0 = b0;
-            PM_TRY(mlp_launch(md, true, x, nrow, y, t, 1.0f / (float)nrow, s, map));
+            PM_TRY(mlp_launch(md, true, x, nrow, y, t, 1.0f / (float)nrow, s, map, k > 0));
             md->step += 1;
             const float bc1 = 1.f - std::pow(0.9f, (float)md->step);
             const float bc2 = 1.f - std::pow(0.999f, (float)md->step);
-            k_adam<<<(kParams + 255) / 256, 256, 0, s>>>(
-                static_cast<float *>(md->P.ptr), static_cast<float *>(md->M.ptr), static_cast<float *>(md->V.ptr),
-                static_cast<float *>(md->G.ptr), kParams, lr, bc1, bc2, static_cast<__nv_bfloat16 *>(md->W1b.ptr),
-                static_cast<__nv_bfloat16 *>(md->W2b.ptr), static_cast<__nv_bfloat16 *>(md->w3b.ptr), loss_word,
-                step_loss + k, 1.0f / (float)nrow);
-            PM_CUDA(cudaGetLastError());
+            PM_CUDA(pm_launch(k_adam, (kParams + 255) / 256, 256, 0, s, static_cast<float *>(md->P.ptr),
+                              static_cast<float *>(md->M.ptr), static_cast<float *>(md->V.ptr),
+                              static_cast<float *>(md->G.ptr), (int)kParams, lr, bc1, bc2,
+                              static_cast<__nv_bfloat16 *>(md->W1b.ptr), static_cast<__nv_bfloat16 *>(md->W2b.ptr),
+                              static_cast<__nv_bfloat16 *>(md->w3b.ptr), tiled_weights(md), loss_word, step_loss + k,
+                              1.0f / (float)nrow));
         }
     }
     if (losses && !losses_dev) {
