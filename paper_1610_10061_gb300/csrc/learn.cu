@@ -42,6 +42,7 @@
 #include <vector>
 
 #include "pm_alloc.h"
+#include "bulk_copy.cuh"
 #include "pm_common.cuh"
 
 namespace {
@@ -716,13 +717,17 @@ __global__ void __launch_bounds__(128) k_mlp(const __nv_bfloat16 *__restrict__ X
 // arithmetic of the mma.sync kernel above and of the oracle with BF16
 // rounding.  The weight gradients accumulate in tensor memory over the CTA's
 // tiles and reach the global gradient with one atomic per parameter per CTA;
-// the bias and w3 gradients are column sums in shared memory.  Eight warps
-// read the accumulators (warps w and w + 4 share TMEM lanes 32 (w mod 4) and
-// take half the columns each); every wait on an MMA is bounded.
+// the bias and w3 gradients are column sums that the threads keep.
+//
+// A step of 4096 rows is 32 tiles, one to a CTA, each a chain of five MMA
+// rounds with a pass over the accumulators between them, so what counts is
+// the length of that chain.  Sixteen warps read the accumulators (those equal
+// mod 4 share TMEM lanes and take 32 columns each) and share each column sum
+// by rows; the weights arrive by bulk copies, in the layout that the MMA
+// reads, while the first layers run.  Every wait is bounded.  @MEASURED@
 // ---------------------------------------------------------------------------
-constexpr int kTrThreads = 256;
+constexpr int kTrThreads = 512, kTrParts = kTrThreads / kTcRows, kTrCols = kHid / kTrParts;
 constexpr uint32_t kTrTmemCols = 512;      // C0 [0,128), C2 [128,256), C3 [256,272)
-constexpr int kLdT = 130;                  // row stride (elements) of the plain H2^T copy: odd in words
 constexpr uint32_t kIdescN16 = (1u << 4) | (1u << 7) | (1u << 10) | ((16u >> 3) << 17) | ((128u >> 4) << 24);
 
 struct TrSmem {
@@ -734,23 +739,22 @@ struct TrSmem {
     __nv_bfloat16 R[kTcRows * kHid];    // H1 as (m = row, k = unit), then dH2
     __nv_bfloat16 T1[kHid * kTcRows];   // H1^T as (m = unit, k = row), then dH1^T
     __nv_bfloat16 T2[kHid * kTcRows];   // dH2^T as (n = unit, k = row)
-    __nv_bfloat16 H2T[kHid * kLdT];     // H2 as [unit][row] (plain), for the w3 gradient
+    __nv_bfloat16 H2T[kHid * kTcRows];  // H2^T, in the same layout, for the w3 gradient
     float b1[kHid], b2[kHid], w3[kHid];
-    float part[kTcRows], tgt[kTcRows], dy[kTcRows];
-    float gb1[kHid], gb2[kHid], gw3[kHid];  // this CTA's bias and w3 gradients
+    float part[kTrParts][kTcRows], tgt[kTcRows], dy[kTcRows];
+    float gb1[kTrParts][kHid], gb2[kTrParts][kHid], gw3[kTrParts][kHid];  // bias and w3 gradients by the tile's rows
     uint32_t mask1[kTcRows * 4];        // H1 > 0: row r, bit (unit & 31) of word 4 r + unit / 32
     float gb3, sq;
-    uint64_t bar;
+    uint64_t bar, staged[3];            // the MMAs; the copies of BW1, BW2T and BW2
     uint32_t tmem;
 };
+static_assert(sizeof(TrSmem) <= 227 * 1024, "one CTA's shared memory");
 
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&v)[16])
+__device__ __forceinline__ void tc_ld4(uint32_t taddr, uint32_t (&v)[4])
 {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr));
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                 : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
@@ -774,7 +778,7 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
     extern __shared__ __align__(1024) unsigned char tr_raw[];
     TrSmem &S = *reinterpret_cast<TrSmem *>(tr_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int quad = warp & 3, half = warp >> 2;
+    const int quad = warp & 3, part = warp >> 2;
     const int64_t tiles = (rows + kTcRows - 1) / kTcRows;
 
     // Before the dependency wait (the previous step's k_adam may still run): the barrier, tensor memory and the first
@@ -782,7 +786,9 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
     if (tid == 0) {
         S.gb3 = 0.f;
         S.sq = 0.f;
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32_learn(&S.bar)), "r"(1u) : "memory");
+        mbar_init(&S.bar, 1);
+        for (int i = 0; i < 3; ++i)
+            mbar_init(&S.staged[i], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
@@ -792,47 +798,48 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // a tile's rows: X (both layouts) and targets
+    // a tile's rows: X (both layouts) and targets, four features a thread
     auto stage_rows = [&](int64_t pos0) {
-        const int xr = tid >> 1, xh = tid & 1;
+        const int xr = tid >> 2, xq = tid & 3;
         const bool valid = pos0 + xr < rows;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        uint2 v = make_uint2(0u, 0u);
         int64_t src = 0;
         if (valid) {
             src = shuffled_row(map, map.pos0 + pos0 + xr);
-            v = __ldg(reinterpret_cast<const uint4 *>(X + src * kIn) + xh);
+            v = __ldg(reinterpret_cast<const uint2 *>(X + src * kIn) + xq);
         }
-        *reinterpret_cast<uint4 *>(reinterpret_cast<unsigned char *>(S.AX) + (xr >> 3) * 256 + xh * 128 +
-                                   (xr & 7) * 16) = v;
-        const uint32_t wv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int f = 8 * xh + 2 * q;
-            reinterpret_cast<uint16_t *>(S.BXT)[core_idx(f, xr, kTcRows)] = (uint16_t)(wv[q] & 0xffffu);
-            reinterpret_cast<uint16_t *>(S.BXT)[core_idx(f + 1, xr, kTcRows)] = (uint16_t)(wv[q] >> 16);
-        }
-        if (xh == 0)
+        *reinterpret_cast<uint2 *>(S.AX + core_idx(xr, 4 * xq, kIn)) = v;
+        uint16_t *xt = reinterpret_cast<uint16_t *>(S.BXT) + core_idx(4 * xq, xr, kTcRows);  // a feature on: 16 bytes
+        xt[0] = (uint16_t)(v.x & 0xffffu);
+        xt[8] = (uint16_t)(v.x >> 16);
+        xt[16] = (uint16_t)(v.y & 0xffffu);
+        xt[24] = (uint16_t)(v.y >> 16);
+        if (xq == 0)
             S.tgt[xr] = valid ? t[src] : 0.f;
     };
     stage_rows(blockIdx.x * (int64_t)tpc * kTcRows);
     pm_grid_dependency_wait();
-    stage16(S.BW1, tiled + kTiledW1, kHid * kIn);
-    stage16(S.BW2T, tiled + kTiledW2T, kHid * kHid);
-    stage16(S.BW2, tiled + kTiledW2, kHid * kHid);
-    for (int i = tid; i < kHid; i += blockDim.x) {
-        S.b1[i] = P[kOffB1 + i];
-        S.b2[i] = P[kOffB2 + i];
-        S.w3[i] = __bfloat162float(w3b[i]);
-        S.gb1[i] = 0.f;
-        S.gb2[i] = 0.f;
-        S.gw3[i] = 0.f;
+    if (tid == 0) {  // k_adam's ordinary stores, read by the copies
+        asm volatile("fence.proxy.async;" ::: "memory");
+        mbar_arrive_expect_tx(&S.staged[0], sizeof(S.BW1));
+        bulk_g2s(S.BW1, tiled + kTiledW1, sizeof(S.BW1), &S.staged[0]);
+        mbar_arrive_expect_tx(&S.staged[1], sizeof(S.BW2T));
+        bulk_g2s(S.BW2T, tiled + kTiledW2T, sizeof(S.BW2T), &S.staged[1]);
+        mbar_arrive_expect_tx(&S.staged[2], sizeof(S.BW2));
+        bulk_g2s(S.BW2, tiled + kTiledW2, sizeof(S.BW2), &S.staged[2]);
     }
+    if (tid < kHid)
+        S.b1[tid] = P[kOffB1 + tid];
+    else if (tid < 2 * kHid)
+        S.b2[tid - kHid] = P[kOffB2 + tid - kHid];
+    else if (tid < 3 * kHid)
+        S.w3[tid - 2 * kHid] = __bfloat162float(w3b[tid - 2 * kHid]);
     const float b3 = P[kOffB3];
     tc_sync_for_mma();
     const uint32_t tmem = S.tmem, C0 = tmem, C2 = tmem + 128u, C3 = tmem + 256u;
     const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
     const int r = quad * 32 + lane;  // this thread's row of the tile (its TMEM lane)
-    const int c0 = half * 64;        // its first column
+    const int c0 = part * kTrCols;   // its first column
     constexpr uint32_t kSbo = (kHid / 8) * 128;
     // Eight columns (four packed pairs) of this thread's row into a transposed tile (m or n = column, k = row).  The
     // four groups of eight lanes lie 128 bytes apart, in the same banks, so each starts with another pair.
@@ -855,9 +862,11 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
     };
 
     uint32_t phase = 0;
-    bool ok = true, any = false;
+    bool ok = true, any = false, staged = true;  // staged: of thread 0, the weights that it has waited for
+    float gw3 = 0.f, gb2 = 0.f, gb1 = 0.f;       // column tid mod 128 over the rows 32 part .. 32 part + 31 of the tiles
+    const int unit = tid & (kHid - 1), row0 = part * (kTcRows / kTrParts);
     auto wait_mma = [&]() {
-        bool w = tc_wait(&S.bar, phase);
+        bool w = tc_wait(&S.bar, phase) && staged;
         w = __syncthreads_and(w);
         phase ^= 1u;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -871,19 +880,21 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
         const int nvalid = (int)((rows - pos0) < kTcRows ? (rows - pos0) : kTcRows);
         tc_sync_for_mma();
         if (tid == 0) {  // layer 1
-            tc_mma(C0, umma_desc(S.AX, 128, (kIn / 8) * 128), umma_desc(S.BW1, 128, (kIn / 8) * 128), kIdesc, 0u);
+            staged = tc_wait(&S.staged[0], 0);
+            if (staged)
+                tc_mma(C0, umma_desc(S.AX, 128, (kIn / 8) * 128), umma_desc(S.BW1, 128, (kIn / 8) * 128), kIdesc, 0u);
             tc_commit(&S.bar);
         }
         if (!(ok = wait_mma()))
             break;
         // ---- H1 = bf16(relu(C0 + b1)) into R (rows) and T1 (transposed); its sign bits ----
-        for (int cc = 0; cc < 64; cc += 32) {
-            uint32_t v[32];
-            tc_ld32(C0 + lane_off + (uint32_t)(c0 + cc), v);
+        {
+            uint32_t v[kTrCols];
+            tc_ld32(C0 + lane_off + (uint32_t)c0, v);
             uint32_t bits = 0u;
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
-                const int col = c0 + cc + 8 * g;
+            for (int g = 0; g < kTrCols / 8; ++g) {
+                const int col = c0 + 8 * g;
                 uint32_t pk[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
@@ -896,12 +907,13 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
                 store_columns(S.T1, col, pk);
                 *reinterpret_cast<uint4 *>(S.R + core_idx(r, col, kHid)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
             }
-            S.mask1[4 * r + (c0 + cc) / 32] = bits;
+            S.mask1[kTrParts * r + part] = bits;
         }
         tc_sync_for_mma();
         if (tid == 0) {  // layer 2
+            staged = tc_wait(&S.staged[1], 0);
 #pragma unroll
-            for (int s = 0; s < kHid / 16; ++s)
+            for (int s = 0; s < kHid / 16 && staged; ++s)
                 tc_mma(C0, umma_desc(S.R + s * 128, 128, kSbo), umma_desc(S.BW2T + s * 128, 128, kSbo), kIdesc,
                        s > 0 ? 1u : 0u);
             tc_commit(&S.bar);
@@ -909,99 +921,105 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
         if (!(ok = wait_mma()))
             break;
         // ---- H2 = bf16(relu(C0 + b2)) (kept packed), y, dy, then dH2 into R and T2 ----
-        uint32_t h2[32];  // this thread's 64 columns of H2, packed pairs
-        float ysum = 0.f;
-        for (int cc = 0; cc < 64; cc += 32) {
-            uint32_t v[32];
-            tc_ld32(C0 + lane_off + (uint32_t)(c0 + cc), v);
-#pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const int col = c0 + cc + 2 * q;
-                const uint32_t hb = pack_relu_bf16x2(__uint_as_float(v[2 * q]) + S.b2[col],
-                                                     __uint_as_float(v[2 * q + 1]) + S.b2[col + 1]);
-                h2[cc / 2 + q] = hb;
-                ysum = fmaf(bf16_lo(hb), S.w3[col], ysum);
-                ysum = fmaf(bf16_hi(hb), S.w3[col + 1], ysum);
-                S.H2T[col * kLdT + r] = __ushort_as_bfloat16((unsigned short)(hb & 0xffffu));
-                S.H2T[(col + 1) * kLdT + r] = __ushort_as_bfloat16((unsigned short)(hb >> 16));
-            }
-        }
-        if (half == 1)
-            S.part[r] = ysum;
-        __syncthreads();
-        if (half == 0) {
-            const bool valid = r < nvalid;
-            const float e = valid ? (ysum + S.part[r] + b3 - S.tgt[r]) : 0.f;
-            const float dyv = valid ? 2.f * e * inv_batch : 0.f;
-            S.dy[r] = dyv;
-            float sq = e * e, d = dyv;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                sq += __shfl_xor_sync(PM_FULL_MASK, sq, o);
-                d += __shfl_xor_sync(PM_FULL_MASK, d, o);
-            }
-            if (lane == 0) {
-                atomicAdd(&S.sq, sq);
-                atomicAdd(&S.gb3, d);
-            }
-        }
-        __syncthreads();
         {
-            const float dyr = S.dy[r];
+            uint32_t h2[kTrCols / 2];  // this thread's columns of H2, packed pairs
+            float ysum = 0.f;
+            {
+                uint32_t v[kTrCols];
+                tc_ld32(C0 + lane_off + (uint32_t)c0, v);
 #pragma unroll
-            for (int q = 0; q < 32; ++q) {
-                const int col = c0 + 2 * q;
-                const float g0 = bf16_lo(h2[q]) > 0.f ? dyr * S.w3[col] : 0.f;
-                const float g1 = bf16_hi(h2[q]) > 0.f ? dyr * S.w3[col + 1] : 0.f;
-                h2[q] = pack_bf16x2(g0, g1);  // dH2, packed
+                for (int g = 0; g < kTrCols / 8; ++g) {
+                    uint32_t pk[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int col = c0 + 8 * g + 2 * q;
+                        pk[q] = pack_relu_bf16x2(__uint_as_float(v[8 * g + 2 * q]) + S.b2[col],
+                                                 __uint_as_float(v[8 * g + 2 * q + 1]) + S.b2[col + 1]);
+                        ysum = fmaf(bf16_lo(pk[q]), S.w3[col], ysum);
+                        ysum = fmaf(bf16_hi(pk[q]), S.w3[col + 1], ysum);
+                        h2[4 * g + q] = pk[q];
+                    }
+                    store_columns(S.H2T, c0 + 8 * g, pk);
+                }
+            }
+            S.part[part][r] = ysum;
+            __syncthreads();
+            float yr = S.part[0][r];
+#pragma unroll
+            for (int i = 1; i < kTrParts; ++i)
+                yr += S.part[i][r];
+            const float e = r < nvalid ? (yr + b3 - S.tgt[r]) : 0.f;
+            const float dyr = r < nvalid ? 2.f * e * inv_batch : 0.f;
+            if (part == 0) {
+                S.dy[r] = dyr;
+                float sq = e * e, d = dyr;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    sq += __shfl_xor_sync(PM_FULL_MASK, sq, o);
+                    d += __shfl_xor_sync(PM_FULL_MASK, d, o);
+                }
+                if (lane == 0) {
+                    atomicAdd(&S.sq, sq);
+                    atomicAdd(&S.gb3, d);
+                }
             }
 #pragma unroll
-            for (int g = 0; g < 8; ++g) {
-                const uint32_t pk[4] = {h2[4 * g], h2[4 * g + 1], h2[4 * g + 2], h2[4 * g + 3]};
+            for (int g = 0; g < kTrCols / 8; ++g) {
+                uint32_t pk[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int col = c0 + 8 * g + 2 * q;
+                    const uint32_t hb = h2[4 * g + q];
+                    pk[q] = pack_bf16x2(bf16_lo(hb) > 0.f ? dyr * S.w3[col] : 0.f,
+                                        bf16_hi(hb) > 0.f ? dyr * S.w3[col + 1] : 0.f);
+                }
                 store_columns(S.T2, c0 + 8 * g, pk);
                 *reinterpret_cast<uint4 *>(S.R + core_idx(r, c0 + 8 * g, kHid)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
             }
         }
         tc_sync_for_mma();
         if (tid == 0) {  // dH1 pre-activation, and dW2 += H1^T dH2
+            staged = tc_wait(&S.staged[2], 0);
 #pragma unroll
-            for (int s = 0; s < kHid / 16; ++s)
+            for (int s = 0; s < kHid / 16 && staged; ++s)
                 tc_mma(C0, umma_desc(S.R + s * 128, 128, kSbo), umma_desc(S.BW2 + s * 128, 128, kSbo), kIdesc,
                        s > 0 ? 1u : 0u);
 #pragma unroll
-            for (int s = 0; s < kTcRows / 16; ++s)
+            for (int s = 0; s < kTcRows / 16 && staged; ++s)
                 tc_mma(C2, umma_desc(S.T1 + s * 128, 128, kSbo), umma_desc(S.T2 + s * 128, 128, kSbo), kIdesc,
                        (any || s > 0) ? 1u : 0u);
             tc_commit(&S.bar);
         }
         // column sums of this tile while the tensor cores run: the w3 and layer-2 bias gradients
-        if (tid < kHid) {
-            float gw = 0.f, gb = 0.f;
-            for (int rr = 0; rr < nvalid; ++rr) {
-                gw = fmaf(__bfloat162float(S.H2T[tid * kLdT + rr]), S.dy[rr], gw);
-                gb += __bfloat162float(S.T2[core_idx(tid, rr, kTcRows)]);
+        for (int rr = row0; rr < row0 + kTcRows / kTrParts; rr += 8) {  // eight rows of a unit lie side by side
+            const uint4 hv = *reinterpret_cast<const uint4 *>(S.H2T + core_idx(unit, rr, kTcRows));
+            const uint4 gv = *reinterpret_cast<const uint4 *>(S.T2 + core_idx(unit, rr, kTcRows));
+            const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w}, gw[4] = {gv.x, gv.y, gv.z, gv.w};
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                if (rr + e < nvalid) {
+                    gw3 = fmaf((e & 1) ? bf16_hi(hw[e / 2]) : bf16_lo(hw[e / 2]), S.dy[rr + e], gw3);
+                    gb2 += (e & 1) ? bf16_hi(gw[e / 2]) : bf16_lo(gw[e / 2]);
+                }
             }
-            S.gw3[tid] += gw;
-            S.gb2[tid] += gb;
         }
         if (!(ok = wait_mma()))
             break;
         // ---- dH1 = bf16(C0 [H1 > 0]) into T1 (transposed) ----
-        for (int cc = 0; cc < 64; cc += 32) {
-            uint32_t v[32];
-            tc_ld32(C0 + lane_off + (uint32_t)(c0 + cc), v);
-            const uint32_t bits = S.mask1[4 * r + (c0 + cc) / 32];
+        {
+            uint32_t v[kTrCols];
+            tc_ld32(C0 + lane_off + (uint32_t)c0, v);
+            const uint32_t bits = S.mask1[kTrParts * r + part];
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
+            for (int g = 0; g < kTrCols / 8; ++g) {
                 uint32_t pk[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const int k = 8 * g + 2 * q;
-                    const float g0 = ((bits >> k) & 1u) ? __uint_as_float(v[k]) : 0.f;
-                    const float g1 = ((bits >> (k + 1)) & 1u) ? __uint_as_float(v[k + 1]) : 0.f;
-                    pk[q] = pack_bf16x2(g0, g1);
+                    pk[q] = pack_bf16x2(((bits >> k) & 1u) ? __uint_as_float(v[k]) : 0.f,
+                                        ((bits >> (k + 1)) & 1u) ? __uint_as_float(v[k + 1]) : 0.f);
                 }
-                store_columns(S.T1, c0 + cc + 8 * g, pk);
+                store_columns(S.T1, c0 + 8 * g, pk);
             }
         }
         tc_sync_for_mma();
@@ -1012,11 +1030,13 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
                        (any || s > 0) ? 1u : 0u);
             tc_commit(&S.bar);
         }
-        if (tid < kHid) {  // the layer-1 bias gradient: row sums of dH1^T
-            float gb = 0.f;
-            for (int rr = 0; rr < nvalid; ++rr)
-                gb += __bfloat162float(S.T1[core_idx(tid, rr, kTcRows)]);
-            S.gb1[tid] += gb;
+        for (int rr = row0; rr < row0 + kTcRows / kTrParts; rr += 8) {  // the layer-1 bias gradient
+            const uint4 gv = *reinterpret_cast<const uint4 *>(S.T1 + core_idx(unit, rr, kTcRows));
+            const uint32_t gw[4] = {gv.x, gv.y, gv.z, gv.w};
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (rr + e < nvalid)
+                    gb1 += (e & 1) ? bf16_hi(gw[e / 2]) : bf16_lo(gw[e / 2]);
         }
         if (!(ok = wait_mma()))
             break;
@@ -1025,28 +1045,35 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
     if (ok && any) {
         // this CTA's weight gradients from tensor memory: dW2 (lane = in, column = out), dW1^T (lane = out,
         // column = in feature)
-        for (int cc = 0; cc < 64; cc += 32) {
-            uint32_t v[32];
-            tc_ld32(C2 + lane_off + (uint32_t)(c0 + cc), v);
+        S.gw3[part][unit] = gw3;
+        S.gb2[part][unit] = gb2;
+        S.gb1[part][unit] = gb1;
+        {
+            uint32_t v[kTrCols];
+            tc_ld32(C2 + lane_off + (uint32_t)c0, v);
 #pragma unroll
-            for (int q = 0; q < 32; q += 4)  // kOffW2 is a multiple of 4: 16-byte aligned
-                asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(
-                                 grads + kOffW2 + r * kHid + c0 + cc + q),
+            for (int q = 0; q < kTrCols; q += 4)  // kOffW2 is a multiple of 4: 16-byte aligned
+                asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(grads + kOffW2 +
+                                                                                              r * kHid + c0 + q),
                              "f"(__uint_as_float(v[q])), "f"(__uint_as_float(v[q + 1])),
                              "f"(__uint_as_float(v[q + 2])), "f"(__uint_as_float(v[q + 3]))
                              : "memory");
         }
-        if (half == 0) {
-            uint32_t v[16];
-            tc_ld16(C3 + lane_off, v);
+        {
+            uint32_t v[kIn / kTrParts];
+            tc_ld4(C3 + lane_off + (uint32_t)(part * (kIn / kTrParts)), v);
 #pragma unroll
-            for (int f = 0; f < 16; ++f)
-                atomicAdd(grads + kOffW1 + f * kHid + r, __uint_as_float(v[f]));
+            for (int f = 0; f < kIn / kTrParts; ++f)
+                atomicAdd(grads + kOffW1 + (part * (kIn / kTrParts) + f) * kHid + r, __uint_as_float(v[f]));
         }
-        if (tid < kHid) {
-            atomicAdd(grads + kOffB1 + tid, S.gb1[tid]);
-            atomicAdd(grads + kOffB2 + tid, S.gb2[tid]);
-            atomicAdd(grads + kOffW3 + tid, S.gw3[tid]);
+        __syncthreads();
+        if (tid < 3 * kHid) {
+            const float(*sums)[kHid] = tid < kHid ? S.gb1 : tid < 2 * kHid ? S.gb2 : S.gw3;
+            float sum = sums[0][unit];
+#pragma unroll
+            for (int i = 1; i < kTrParts; ++i)
+                sum += sums[i][unit];
+            atomicAdd(grads + (tid < kHid ? kOffB1 : tid < 2 * kHid ? kOffB2 : kOffW3) + unit, sum);
         }
         if (tid == 0) {
             atomicAdd(grads + kOffB3, S.gb3);
@@ -1056,7 +1083,10 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
     if (!ok) {
         if (tid == 0)
             atomicExch(err, (int)PM_ERR_TIMEOUT);
-        (void)tc_wait(&S.bar, phase);  // let an MMA in flight finish (bounded) before its memory is released
+        // let an MMA and copies in flight finish (bounded) before their memory is released
+        (void)tc_wait(&S.bar, phase);
+        for (int i = 0; i < 3; ++i)
+            (void)tc_wait(&S.staged[i], 0);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
