@@ -739,16 +739,16 @@ struct TrSmem {
     __nv_bfloat16 R[kTcRows * kHid];    // H1 as (m = row, k = unit), then dH2
     __nv_bfloat16 T1[kHid * kTcRows];   // H1^T as (m = unit, k = row), then dH1^T
     __nv_bfloat16 T2[kHid * kTcRows];   // dH2^T as (n = unit, k = row)
-    __nv_bfloat16 H2T[kHid * kTcRows];  // H2^T, in the same layout, for the w3 gradient
     float b1[kHid], b2[kHid], w3[kHid];
-    float part[kTrParts][kTcRows], tgt[kTcRows], dy[kTcRows];
-    float gb1[kTrParts][kHid], gb2[kTrParts][kHid], gw3[kTrParts][kHid];  // bias and w3 gradients by the tile's rows
-    uint32_t mask1[kTcRows * 4];        // H1 > 0: row r, bit (unit & 31) of word 4 r + unit / 32
-    float gb3, sq;
+    float part[kTrParts][kTcRows], tgt[kTcRows];
+    float gb1[4][kHid], gb2[4][kHid], gw3[4][kHid];  // bias and w3 gradients of the tiles' rows 32 q .. 32 q + 31
     uint64_t bar, staged[3];            // the MMAs; the copies of BW1, BW2T and BW2
     uint32_t tmem;
 };
 static_assert(sizeof(TrSmem) <= 227 * 1024, "one CTA's shared memory");
+static_assert(kTrCols == 32 && kIn / kTrParts == 4, "the widths of tc_ld_fragments, tc_ld32 and tc_ld4");
+constexpr int kLdW2 = kHid + 4;  // row stride (floats) of the dW2 tile in R, T1 and T2: 16-byte stores of 8 rows in all banks
+static_assert(kHid * kLdW2 * 4 <= 3 * kHid * kHid * 2, "the dW2 tile lies in R, T1 and T2");
 
 __device__ __forceinline__ void tc_ld4(uint32_t taddr, uint32_t (&v)[4])
 {
@@ -756,6 +756,50 @@ __device__ __forceinline__ void tc_ld4(uint32_t taddr, uint32_t (&v)[4])
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
                  : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// The 32 accumulators of 32 lanes (rows) x 32 columns that a thread holds in the fragment layout of the 8 x 8 matrix
+// stores: v[g][i], i = 0..3, is the pair of columns 8 g + 2 (lane mod 4), + 1 of row 8 i + lane / 4.
+__device__ __forceinline__ void tc_ld_fragments(uint32_t taddr, float2 (&v)[4][4])
+{
+    uint32_t w[2][16];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        asm volatile("tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+                     "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                     : "=r"(w[h][0]), "=r"(w[h][1]), "=r"(w[h][2]), "=r"(w[h][3]), "=r"(w[h][4]), "=r"(w[h][5]),
+                       "=r"(w[h][6]), "=r"(w[h][7]), "=r"(w[h][8]), "=r"(w[h][9]), "=r"(w[h][10]), "=r"(w[h][11]),
+                       "=r"(w[h][12]), "=r"(w[h][13]), "=r"(w[h][14]), "=r"(w[h][15])
+                     : "r"(taddr + ((uint32_t)(16 * h) << 16)));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int g = 0; g < 4; ++g)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            v[g][i] = make_float2(__uint_as_float(w[i >> 1][4 * g + 2 * (i & 1)]),
+                                  __uint_as_float(w[i >> 1][4 * g + 2 * (i & 1) + 1]));
+}
+
+// Four 8 x 8 matrices of packed pairs, a row of a matrix (transposed: a column) to the 16 bytes at its lane's address.
+template <bool kTranspose>
+__device__ __forceinline__ void store_matrices(uint32_t addr, const uint32_t (&w)[4])
+{
+    if constexpr (kTranspose)
+        asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared::cta.b16 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(w[0]),
+                     "r"(w[1]), "r"(w[2]), "r"(w[3])
+                     : "memory");
+    else
+        asm volatile("stmatrix.sync.aligned.m8n8.x4.shared::cta.b16 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(w[0]),
+                     "r"(w[1]), "r"(w[2]), "r"(w[3])
+                     : "memory");
+}
+
+// 0xffff in each half whose BF16 is above zero.
+__device__ __forceinline__ uint32_t positive_mask(uint32_t p)
+{
+    __nv_bfloat162 h;
+    memcpy(&h, &p, 4);
+    return __hgt2_mask(h, __nv_bfloat162(__ushort_as_bfloat16(0), __ushort_as_bfloat16(0)));
 }
 
 __device__ __forceinline__ float bf16_lo(uint32_t p) { return __uint_as_float(p << 16); }
@@ -784,8 +828,6 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
     // Before the dependency wait (the previous step's k_adam may still run): the barrier, tensor memory and the first
     // tile's rows, which no kernel of the training loop writes.
     if (tid == 0) {
-        S.gb3 = 0.f;
-        S.sq = 0.f;
         mbar_init(&S.bar, 1);
         for (int i = 0; i < 3; ++i)
             mbar_init(&S.staged[i], 1);
@@ -818,8 +860,9 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
             S.tgt[xr] = valid ? t[src] : 0.f;
     };
     stage_rows(blockIdx.x * (int64_t)tpc * kTcRows);
+    __syncthreads();  // the barriers are ready
     pm_grid_dependency_wait();
-    if (tid == 0) {  // k_adam's ordinary stores, read by the copies
+    if (tid == 3 * kHid) {  // k_adam's ordinary stores, read by the copies
         asm volatile("fence.proxy.async;" ::: "memory");
         mbar_arrive_expect_tx(&S.staged[0], sizeof(S.BW1));
         bulk_g2s(S.BW1, tiled + kTiledW1, sizeof(S.BW1), &S.staged[0]);
@@ -841,30 +884,18 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
     const int r = quad * 32 + lane;  // this thread's row of the tile (its TMEM lane)
     const int c0 = part * kTrCols;   // its first column
     constexpr uint32_t kSbo = (kHid / 8) * 128;
-    // Eight columns (four packed pairs) of this thread's row into a transposed tile (m or n = column, k = row).  The
-    // four groups of eight lanes lie 128 bytes apart, in the same banks, so each starts with another pair.
-    const int turn = (lane >> 3) & 3;
-    auto store_columns = [&](__nv_bfloat16 *tile, int col, const uint32_t (&pk)[4]) {
-        uint32_t a[4], b[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            a[i] = (turn & 1) ? pk[(i + 1) & 3] : pk[i];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            b[i] = (turn & 2) ? a[(i + 2) & 3] : a[i];
-        uint16_t *out = reinterpret_cast<uint16_t *>(tile) + core_idx(col, r, kTcRows);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int q = (i + turn) & 3;  // columns col + 2 q and the next, 16 bytes apart
-            out[16 * q] = (uint16_t)(b[i] & 0xffffu);
-            out[16 * q + 8] = (uint16_t)(b[i] >> 16);
-        }
-    };
+    // in the fragment layout: rows 32 quad + 8 i + lane / 4, columns c0 + 8 g + pc and the next; where this lane's 16
+    // bytes of a matrix go, in the tiles by rows (R) and by units (T1, T2)
+    const int pr = quad * 32 + (lane >> 2), pc = 2 * (lane & 3);
+    const uint32_t by_row = smem_u32(S.R) + (quad * 4 + (lane >> 3)) * 2048 + (c0 / 8) * 128 + (lane & 7) * 16;
+    const uint32_t by_unit = (c0 / 8) * 2048 + (quad * 4 + (lane >> 3)) * 128 + (lane & 7) * 16;
+    const uint32_t T1a = smem_u32(S.T1) + by_unit, T2a = smem_u32(S.T2) + by_unit;
 
     uint32_t phase = 0;
     bool ok = true, any = false, staged = true;  // staged: of thread 0, the weights that it has waited for
-    float gw3 = 0.f, gb2 = 0.f, gb1 = 0.f;       // column tid mod 128 over the rows 32 part .. 32 part + 31 of the tiles
-    const int unit = tid & (kHid - 1), row0 = part * (kTcRows / kTrParts);
+    float gw3[8] = {}, gb2[8] = {}, gb1[8] = {};  // this thread's columns (2 g, 2 g + 1) over its rows of the tiles
+    float sq = 0.f, gb3 = 0.f;                    // of part 0: the rows that it turns into dy
+    const int unit = tid & (kHid - 1);
     auto wait_mma = [&]() {
         bool w = tc_wait(&S.bar, phase) && staged;
         w = __syncthreads_and(w);
@@ -888,26 +919,19 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
         if (!(ok = wait_mma()))
             break;
         // ---- H1 = bf16(relu(C0 + b1)) into R (rows) and T1 (transposed); its sign bits ----
+        uint32_t h1[4][4];
         {
-            uint32_t v[kTrCols];
-            tc_ld32(C0 + lane_off + (uint32_t)c0, v);
-            uint32_t bits = 0u;
+            float2 v[4][4];
+            tc_ld_fragments(C0 + lane_off + (uint32_t)c0, v);
 #pragma unroll
-            for (int g = 0; g < kTrCols / 8; ++g) {
-                const int col = c0 + 8 * g;
-                uint32_t pk[4];
+            for (int g = 0; g < 4; ++g) {
+                const float2 bias = *reinterpret_cast<const float2 *>(&S.b1[c0 + 8 * g + pc]);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    pk[q] = pack_relu_bf16x2(__uint_as_float(v[8 * g + 2 * q]) + S.b1[col + 2 * q],
-                                             __uint_as_float(v[8 * g + 2 * q + 1]) + S.b1[col + 2 * q + 1]);
-                    const float lo = bf16_lo(pk[q]), hi = bf16_hi(pk[q]);
-                    bits |= (lo > 0.f ? 1u : 0u) << (8 * g + 2 * q);
-                    bits |= (hi > 0.f ? 1u : 0u) << (8 * g + 2 * q + 1);
-                }
-                store_columns(S.T1, col, pk);
-                *reinterpret_cast<uint4 *>(S.R + core_idx(r, col, kHid)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                for (int i = 0; i < 4; ++i)
+                    h1[g][i] = pack_relu_bf16x2(v[g][i].x + bias.x, v[g][i].y + bias.y);
+                store_matrices<false>(by_row + 128 * g, h1[g]);
+                store_matrices<true>(T1a + 2048 * g, h1[g]);
             }
-            S.mask1[kTrParts * r + part] = bits;
         }
         tc_sync_for_mma();
         if (tid == 0) {  // layer 2
@@ -922,59 +946,65 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
             break;
         // ---- H2 = bf16(relu(C0 + b2)) (kept packed), y, dy, then dH2 into R and T2 ----
         {
-            uint32_t h2[kTrCols / 2];  // this thread's columns of H2, packed pairs
-            float ysum = 0.f;
+            uint32_t h2[4][4];
+            float y[4] = {};
             {
-                uint32_t v[kTrCols];
-                tc_ld32(C0 + lane_off + (uint32_t)c0, v);
+                float2 v[4][4];
+                tc_ld_fragments(C0 + lane_off + (uint32_t)c0, v);
 #pragma unroll
-                for (int g = 0; g < kTrCols / 8; ++g) {
-                    uint32_t pk[4];
+                for (int g = 0; g < 4; ++g) {
+                    const float2 bias = *reinterpret_cast<const float2 *>(&S.b2[c0 + 8 * g + pc]);
+                    const float2 w = *reinterpret_cast<const float2 *>(&S.w3[c0 + 8 * g + pc]);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int col = c0 + 8 * g + 2 * q;
-                        pk[q] = pack_relu_bf16x2(__uint_as_float(v[8 * g + 2 * q]) + S.b2[col],
-                                                 __uint_as_float(v[8 * g + 2 * q + 1]) + S.b2[col + 1]);
-                        ysum = fmaf(bf16_lo(pk[q]), S.w3[col], ysum);
-                        ysum = fmaf(bf16_hi(pk[q]), S.w3[col + 1], ysum);
-                        h2[4 * g + q] = pk[q];
+                    for (int i = 0; i < 4; ++i) {
+                        h2[g][i] = pack_relu_bf16x2(v[g][i].x + bias.x, v[g][i].y + bias.y);
+                        y[i] = fmaf(bf16_lo(h2[g][i]), w.x, y[i]);
+                        y[i] = fmaf(bf16_hi(h2[g][i]), w.y, y[i]);
                     }
-                    store_columns(S.H2T, c0 + 8 * g, pk);
                 }
             }
-            S.part[part][r] = ysum;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                y[i] += __shfl_xor_sync(PM_FULL_MASK, y[i], 1);
+                y[i] += __shfl_xor_sync(PM_FULL_MASK, y[i], 2);
+            }
+            if ((lane & 3) == 0) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    S.part[part][pr + 8 * i] = y[i];
+            }
             __syncthreads();
-            float yr = S.part[0][r];
+            float dy[4];  // of the rows of this thread: the four lanes that share them work out one each
+            {
+                const int row = pr + 8 * (lane & 3);
+                float yr = S.part[0][row];
 #pragma unroll
-            for (int i = 1; i < kTrParts; ++i)
-                yr += S.part[i][r];
-            const float e = r < nvalid ? (yr + b3 - S.tgt[r]) : 0.f;
-            const float dyr = r < nvalid ? 2.f * e * inv_batch : 0.f;
-            if (part == 0) {
-                S.dy[r] = dyr;
-                float sq = e * e, d = dyr;
+                for (int i = 1; i < kTrParts; ++i)
+                    yr += S.part[i][row];
+                const float e = row < nvalid ? (yr + b3 - S.tgt[row]) : 0.f;
+                const float d = row < nvalid ? 2.f * e * inv_batch : 0.f;
+                sq = fmaf(e, e, sq);
+                gb3 += d;
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    sq += __shfl_xor_sync(PM_FULL_MASK, sq, o);
-                    d += __shfl_xor_sync(PM_FULL_MASK, d, o);
-                }
-                if (lane == 0) {
-                    atomicAdd(&S.sq, sq);
-                    atomicAdd(&S.gb3, d);
-                }
+                for (int i = 0; i < 4; ++i)
+                    dy[i] = __shfl_sync(PM_FULL_MASK, d, (lane & ~3) | i);
             }
 #pragma unroll
-            for (int g = 0; g < kTrCols / 8; ++g) {
+            for (int g = 0; g < 4; ++g) {
+                const float2 w = *reinterpret_cast<const float2 *>(&S.w3[c0 + 8 * g + pc]);
                 uint32_t pk[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int col = c0 + 8 * g + 2 * q;
-                    const uint32_t hb = h2[4 * g + q];
-                    pk[q] = pack_bf16x2(bf16_lo(hb) > 0.f ? dyr * S.w3[col] : 0.f,
-                                        bf16_hi(hb) > 0.f ? dyr * S.w3[col + 1] : 0.f);
+                for (int i = 0; i < 4; ++i) {
+                    pk[i] = pack_bf16x2(dy[i] * w.x, dy[i] * w.y) & positive_mask(h2[g][i]);
+                    if (pr + 8 * i < nvalid) {
+                        gw3[2 * g] = fmaf(bf16_lo(h2[g][i]), dy[i], gw3[2 * g]);
+                        gw3[2 * g + 1] = fmaf(bf16_hi(h2[g][i]), dy[i], gw3[2 * g + 1]);
+                        gb2[2 * g] += bf16_lo(pk[i]);
+                        gb2[2 * g + 1] += bf16_hi(pk[i]);
+                    }
                 }
-                store_columns(S.T2, c0 + 8 * g, pk);
-                *reinterpret_cast<uint4 *>(S.R + core_idx(r, c0 + 8 * g, kHid)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                store_matrices<false>(by_row + 128 * g, pk);
+                store_matrices<true>(T2a + 2048 * g, pk);
             }
         }
         tc_sync_for_mma();
@@ -990,36 +1020,24 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
                        (any || s > 0) ? 1u : 0u);
             tc_commit(&S.bar);
         }
-        // column sums of this tile while the tensor cores run: the w3 and layer-2 bias gradients
-        for (int rr = row0; rr < row0 + kTcRows / kTrParts; rr += 8) {  // eight rows of a unit lie side by side
-            const uint4 hv = *reinterpret_cast<const uint4 *>(S.H2T + core_idx(unit, rr, kTcRows));
-            const uint4 gv = *reinterpret_cast<const uint4 *>(S.T2 + core_idx(unit, rr, kTcRows));
-            const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w}, gw[4] = {gv.x, gv.y, gv.z, gv.w};
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                if (rr + e < nvalid) {
-                    gw3 = fmaf((e & 1) ? bf16_hi(hw[e / 2]) : bf16_lo(hw[e / 2]), S.dy[rr + e], gw3);
-                    gb2 += (e & 1) ? bf16_hi(gw[e / 2]) : bf16_lo(gw[e / 2]);
-                }
-            }
-        }
         if (!(ok = wait_mma()))
             break;
         // ---- dH1 = bf16(C0 [H1 > 0]) into T1 (transposed) ----
         {
-            uint32_t v[kTrCols];
-            tc_ld32(C0 + lane_off + (uint32_t)c0, v);
-            const uint32_t bits = S.mask1[kTrParts * r + part];
+            float2 v[4][4];
+            tc_ld_fragments(C0 + lane_off + (uint32_t)c0, v);
 #pragma unroll
-            for (int g = 0; g < kTrCols / 8; ++g) {
+            for (int g = 0; g < 4; ++g) {
                 uint32_t pk[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int k = 8 * g + 2 * q;
-                    pk[q] = pack_bf16x2(((bits >> k) & 1u) ? __uint_as_float(v[k]) : 0.f,
-                                        ((bits >> (k + 1)) & 1u) ? __uint_as_float(v[k + 1]) : 0.f);
+                for (int i = 0; i < 4; ++i) {
+                    pk[i] = pack_bf16x2(v[g][i].x, v[g][i].y) & positive_mask(h1[g][i]);
+                    if (pr + 8 * i < nvalid) {
+                        gb1[2 * g] += bf16_lo(pk[i]);
+                        gb1[2 * g + 1] += bf16_hi(pk[i]);
+                    }
                 }
-                store_columns(S.T1, c0 + 8 * g, pk);
+                store_matrices<true>(T1a + 2048 * g, pk);
             }
         }
         tc_sync_for_mma();
@@ -1030,55 +1048,75 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
                        (any || s > 0) ? 1u : 0u);
             tc_commit(&S.bar);
         }
-        for (int rr = row0; rr < row0 + kTcRows / kTrParts; rr += 8) {  // the layer-1 bias gradient
-            const uint4 gv = *reinterpret_cast<const uint4 *>(S.T1 + core_idx(unit, rr, kTcRows));
-            const uint32_t gw[4] = {gv.x, gv.y, gv.z, gv.w};
-#pragma unroll
-            for (int e = 0; e < 8; ++e)
-                if (rr + e < nvalid)
-                    gb1 += (e & 1) ? bf16_hi(gw[e / 2]) : bf16_lo(gw[e / 2]);
-        }
         if (!(ok = wait_mma()))
             break;
         any = true;
     }
     if (ok && any) {
-        // this CTA's weight gradients from tensor memory: dW2 (lane = in, column = out), dW1^T (lane = out,
-        // column = in feature)
-        S.gw3[part][unit] = gw3;
-        S.gb2[part][unit] = gb2;
-        S.gb1[part][unit] = gb1;
+        // This CTA's weight gradients from tensor memory.  dW2 (lane = in, column = out) goes through shared memory and
+        // leaves as one bulk reduction per row; a lane's row is 512 bytes from the next one's, so reductions straight
+        // from the registers would each touch 32 sectors.
+        float *const tile2 = reinterpret_cast<float *>(S.R);
         {
             uint32_t v[kTrCols];
             tc_ld32(C2 + lane_off + (uint32_t)c0, v);
 #pragma unroll
-            for (int q = 0; q < kTrCols; q += 4)  // kOffW2 is a multiple of 4: 16-byte aligned
-                asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(grads + kOffW2 +
-                                                                                              r * kHid + c0 + q),
-                             "f"(__uint_as_float(v[q])), "f"(__uint_as_float(v[q + 1])),
-                             "f"(__uint_as_float(v[q + 2])), "f"(__uint_as_float(v[q + 3]))
-                             : "memory");
+            for (int q = 0; q < kTrCols; q += 4)
+                *reinterpret_cast<uint4 *>(tile2 + r * kLdW2 + c0 + q) = make_uint4(v[q], v[q + 1], v[q + 2], v[q + 3]);
         }
-        {
+        // the sums over the eight lanes that share the columns, each lane left with one of them
+        auto reduce8 = [&](const float (&x)[8]) {
+            float a[4], b[2];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                a[j] = ((lane & 16) ? x[4 + j] : x[j]) +
+                       __shfl_xor_sync(PM_FULL_MASK, (lane & 16) ? x[j] : x[4 + j], 16);
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                b[j] = ((lane & 8) ? a[2 + j] : a[j]) +
+                       __shfl_xor_sync(PM_FULL_MASK, (lane & 8) ? a[j] : a[2 + j], 8);
+            return ((lane & 4) ? b[1] : b[0]) + __shfl_xor_sync(PM_FULL_MASK, (lane & 4) ? b[0] : b[1], 4);
+        };
+        const int j = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+        const int col = c0 + 8 * (j >> 1) + pc + (j & 1);
+        S.gw3[quad][col] = reduce8(gw3);
+        S.gb2[quad][col] = reduce8(gb2);
+        S.gb1[quad][col] = reduce8(gb1);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncthreads();
+        if (tid < kHid) {  // kOffW2 is a multiple of 4: 16-byte aligned
+            asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(
+                             grads + kOffW2 + tid * kHid),
+                         "r"(smem_u32(tile2 + tid * kLdW2)), "r"((uint32_t)(kHid * sizeof(float)))
+                         : "memory");
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        }
+        {  // dW1^T (lane = out, column = in feature)
             uint32_t v[kIn / kTrParts];
             tc_ld4(C3 + lane_off + (uint32_t)(part * (kIn / kTrParts)), v);
 #pragma unroll
             for (int f = 0; f < kIn / kTrParts; ++f)
                 atomicAdd(grads + kOffW1 + (part * (kIn / kTrParts) + f) * kHid + r, __uint_as_float(v[f]));
         }
-        __syncthreads();
-        if (tid < 3 * kHid) {
-            const float(*sums)[kHid] = tid < kHid ? S.gb1 : tid < 2 * kHid ? S.gb2 : S.gw3;
-            float sum = sums[0][unit];
+        if (tid >= kHid) {
+            const int which = tid / kHid;
+            const float(*sums)[kHid] = which == 1 ? S.gb1 : which == 2 ? S.gb2 : S.gw3;
+            atomicAdd(grads + (which == 1 ? kOffB1 : which == 2 ? kOffB2 : kOffW3) + unit,
+                      (sums[0][unit] + sums[1][unit]) + (sums[2][unit] + sums[3][unit]));
+        }
+        if (part == 0) {
 #pragma unroll
-            for (int i = 1; i < kTrParts; ++i)
-                sum += sums[i][unit];
-            atomicAdd(grads + (tid < kHid ? kOffB1 : tid < 2 * kHid ? kOffB2 : kOffW3) + unit, sum);
+            for (int o = 16; o > 0; o >>= 1) {
+                sq += __shfl_xor_sync(PM_FULL_MASK, sq, o);
+                gb3 += __shfl_xor_sync(PM_FULL_MASK, gb3, o);
+            }
+            if (lane == 0) {
+                atomicAdd(grads + kOffB3, gb3);
+                atomicAdd(loss, sq);
+            }
         }
-        if (tid == 0) {
-            atomicAdd(grads + kOffB3, S.gb3);
-            atomicAdd(loss, S.sq);
-        }
+        if (tid < kHid)
+            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
     if (!ok) {
         if (tid == 0)
