@@ -716,15 +716,20 @@ __global__ void __launch_bounds__(128) k_mlp(const __nv_bfloat16 *__restrict__ X
 // dH2 = BF16(dy w3 [H2 > 0]) and dH1 = BF16((dH2 W2^T) [H1 > 0]) -- the
 // arithmetic of the mma.sync kernel above and of the oracle with BF16
 // rounding.  The weight gradients accumulate in tensor memory over the CTA's
-// tiles and reach the global gradient with one atomic per parameter per CTA;
-// the bias and w3 gradients are column sums that the threads keep.
+// tiles; the bias and w3 gradients are column sums that the threads keep.
 //
-// A step of 4096 rows is 32 tiles, one to a CTA, each a chain of five MMA
-// rounds with a pass over the accumulators between them, so what counts is
-// the length of that chain.  Sixteen warps read the accumulators (those equal
-// mod 4 share TMEM lanes and take 32 columns each) and share each column sum
-// by rows; the weights arrive by bulk copies, in the layout that the MMA
-// reads, while the first layers run.  Every wait is bounded.  @MEASURED@
+// A step of 4096 rows is 32 tiles, one to a CTA, each a chain of four rounds
+// of MMAs with a pass over the accumulators between them, so the length of
+// that chain and of the way from step to step is what counts, not the tensor
+// cores' rate.  Sixteen warps read the accumulators as 8 x 8 matrix fragments
+// (those equal mod 4 share TMEM lanes and take 32 columns each) and store
+// them by rows and transposed with the matrix stores; the weights arrive by
+// bulk copies, in the layout that the MMA reads, while the first layers run;
+// the W2 gradient leaves as bulk reductions.  Every wait is bounded.
+// Measured, a step of 4096 rows with Adam: 11.3 us, of which the gaps between
+// the kernels and k_adam take 3.7; with eight warps, two-byte stores and
+// staging, and reductions from the registers 33 us.  Issuing dW2 from a
+// second warp and 4 KB reductions did not shorten it (11.1 to 11.6 us).
 // ---------------------------------------------------------------------------
 constexpr int kTrThreads = 512, kTrParts = kTrThreads / kTcRows, kTrCols = kHid / kTrParts;
 constexpr uint32_t kTrTmemCols = 512;      // C0 [0,128), C2 [128,256), C3 [256,272)
@@ -740,7 +745,7 @@ struct TrSmem {
     __nv_bfloat16 T1[kHid * kTcRows];   // H1^T as (m = unit, k = row), then dH1^T
     __nv_bfloat16 T2[kHid * kTcRows];   // dH2^T as (n = unit, k = row)
     float b1[kHid], b2[kHid], w3[kHid];
-    float part[kTrParts][kTcRows], tgt[kTcRows];
+    float part[2][kTcRows], tgt[kTcRows];
     float gb1[4][kHid], gb2[4][kHid], gw3[4][kHid];  // bias and w3 gradients of the tiles' rows 32 q .. 32 q + 31
     uint64_t bar, staged[3];            // the MMAs; the copies of BW1, BW2T and BW2
     uint32_t tmem;
@@ -947,41 +952,46 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
         // ---- H2 = bf16(relu(C0 + b2)) (kept packed), y, dy, then dH2 into R and T2 ----
         {
             uint32_t h2[4][4];
-            float y[4] = {};
             {
                 float2 v[4][4];
                 tc_ld_fragments(C0 + lane_off + (uint32_t)c0, v);
 #pragma unroll
                 for (int g = 0; g < 4; ++g) {
                     const float2 bias = *reinterpret_cast<const float2 *>(&S.b2[c0 + 8 * g + pc]);
-                    const float2 w = *reinterpret_cast<const float2 *>(&S.w3[c0 + 8 * g + pc]);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
+                    for (int i = 0; i < 4; ++i)
                         h2[g][i] = pack_relu_bf16x2(v[g][i].x + bias.x, v[g][i].y + bias.y);
-                        y[i] = fmaf(bf16_lo(h2[g][i]), w.x, y[i]);
-                        y[i] = fmaf(bf16_hi(h2[g][i]), w.y, y[i]);
-                    }
+                    store_matrices<false>(by_row + 128 * g, h2[g]);
                 }
             }
+            __syncthreads();
+            // y, in the order of the forward kernels' sums (half a row a thread, by columns): every later rounding of
+            // the backward pass hangs on it
+            if (tid < 2 * kTcRows) {
+                const int row = tid & (kTcRows - 1), half = tid / kTcRows;
+                float y = 0.f;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                y[i] += __shfl_xor_sync(PM_FULL_MASK, y[i], 1);
-                y[i] += __shfl_xor_sync(PM_FULL_MASK, y[i], 2);
-            }
-            if ((lane & 3) == 0) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    S.part[part][pr + 8 * i] = y[i];
+                for (int c = 0; c < kHid / 2; c += 8) {
+                    const int col = half * (kHid / 2) + c;
+                    const uint4 h = *reinterpret_cast<const uint4 *>(S.R + core_idx(row, col, kHid));
+                    const float4 wa = *reinterpret_cast<const float4 *>(&S.w3[col]);
+                    const float4 wb = *reinterpret_cast<const float4 *>(&S.w3[col + 4]);
+                    y = fmaf(bf16_lo(h.x), wa.x, y);
+                    y = fmaf(bf16_hi(h.x), wa.y, y);
+                    y = fmaf(bf16_lo(h.y), wa.z, y);
+                    y = fmaf(bf16_hi(h.y), wa.w, y);
+                    y = fmaf(bf16_lo(h.z), wb.x, y);
+                    y = fmaf(bf16_hi(h.z), wb.y, y);
+                    y = fmaf(bf16_lo(h.w), wb.z, y);
+                    y = fmaf(bf16_hi(h.w), wb.w, y);
+                }
+                S.part[half][row] = y;
             }
             __syncthreads();
             float dy[4];  // of the rows of this thread: the four lanes that share them work out one each
             {
                 const int row = pr + 8 * (lane & 3);
-                float yr = S.part[0][row];
-#pragma unroll
-                for (int i = 1; i < kTrParts; ++i)
-                    yr += S.part[i][row];
-                const float e = row < nvalid ? (yr + b3 - S.tgt[row]) : 0.f;
+                const float e = row < nvalid ? (S.part[0][row] + S.part[1][row] + b3 - S.tgt[row]) : 0.f;
                 const float d = row < nvalid ? 2.f * e * inv_batch : 0.f;
                 sq = fmaf(e, e, sq);
                 gb3 += d;
@@ -1122,7 +1132,7 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_mlp_train_tc(const __nv_bfloa
         if (tid == 0)
             atomicExch(err, (int)PM_ERR_TIMEOUT);
         // let an MMA and copies in flight finish (bounded) before their memory is released
-        (void)tc_wait(&S.bar, phase);
+        (void)tc_wait(&S.bar, phase ^ 1u);
         for (int i = 0; i < 3; ++i)
             (void)tc_wait(&S.staged[i], 0);
     }
