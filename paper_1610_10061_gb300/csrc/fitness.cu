@@ -901,8 +901,9 @@ void pm_direct_shape(const pm_instance *inst, int64_t pop, size_t budget, int nw
 bool pm_direct_wanted(int64_t n, int64_t m, int64_t p, size_t smem_optin)
 {
     // at most 1 GiB beside tables of three times that; the widest range a CTA takes
-    return n * m <= ((int64_t)1 << 29) && pm_direct_smem(m, 32, 1) + 4096 <= smem_optin &&
-           pm_direct_cost(m, p, kDirectRange, 1) < pm_scan_cost(m, p);
+    return pm_deme_fits(n, m, p, smem_optin) ||
+           (n * m <= ((int64_t)1 << 29) && pm_direct_smem(m, 32, 1) + 4096 <= smem_optin &&
+            pm_direct_cost(m, p, kDirectRange, 1) < pm_scan_cost(m, p));
 }
 
 // Resident CTAs per SM of the column kernel for a plan's (G, warps, nb) at this instance's W.

@@ -30,6 +30,8 @@
 //                    counters; the last instance sets the loop condition
 //                    (k_ga_generation_end_one: the same for one instance in
 //                    one CTA).
+// For one instance that fits in shared memory all of it is one kernel, a
+// cluster of CTAs per deme (k_ga_deme).
 // The operators also write the facility-major copy of their output that the
 // scan reads, so no evaluation needs a separate transpose.  A call of several
 // generations is one CUDA graph: a gate kernel and a conditional while-node
@@ -171,10 +173,13 @@ __device__ __forceinline__ uint32_t ld_row(const uint32_t *p)
         return *p;
 }
 
-template <bool kCG>
+constexpr int kPlain = 2;  // ld_ro: rows in shared memory
+template <int kCG>
 __device__ __forceinline__ uint32_t ld_ro(const uint32_t *p)
 {
-    if constexpr (kCG)
+    if constexpr (kCG == kPlain)
+        return *p;
+    else if constexpr (kCG)
         return __ldcg(p);
     else
         return __ldg(p);
@@ -907,19 +912,19 @@ __global__ void __launch_bounds__(1024) k_ga_crossover(const ga_prob *__restrict
 
 // 32 bits of the bitset C starting at bit position s (s may be as low as
 // -31; bits read from below position 0 are zero).
-template <bool kCG>
-__device__ __forceinline__ uint32_t bits_from(const uint32_t *C, int32_t W, int64_t s)
+template <int kCG>
+__device__ __forceinline__ uint32_t bits_from(const uint32_t *C, int32_t W, int32_t s)
 {
     if (s < 0)
         return ld_ro<kCG>(C) << (uint32_t)(-s);
-    const int64_t q = s >> 5;
+    const int32_t q = s >> 5;
     const uint32_t r = (uint32_t)(s & 31);
     const uint32_t lo = ld_ro<kCG>(C + q);
     const uint32_t hi = (q + 1 < W) ? ld_ro<kCG>(C + q + 1) : 0u;
     return __funnelshift_r(lo, hi, r);
 }
 
-__device__ __forceinline__ uint32_t range_mask(int64_t lo, int64_t hi)  // bits [lo, hi) of a word, 0 <= lo <= hi <= 32
+__device__ __forceinline__ uint32_t range_mask(int32_t lo, int32_t hi)  // bits [lo, hi) of a word, 0 <= lo <= hi <= 32
 {
     const uint32_t upto = hi >= 32 ? 0xffffffffu : ((1u << hi) - 1u);
     const uint32_t below = lo >= 32 ? 0xffffffffu : ((1u << lo) - 1u);
@@ -932,8 +937,8 @@ __device__ __forceinline__ uint32_t range_mask(int64_t lo, int64_t hi)  // bits 
 // draw 4.  The mutant rotates bits [a, a+len) left by kl: F[a+i] =
 // C[a + (i+kl) mod len].  Depends on nothing a kernel of the generation
 // writes, so callers may take it before waiting for the previous kernel.
-struct MutantShift {
-    int64_t a, len, kl;
+struct MutantShift {  // m < 65536
+    int32_t a, len, kl;
 };
 
 __device__ __forceinline__ MutantShift mutant_shift(int32_t m, uint64_t seed, uint32_t gen, uint32_t t, uint32_t q,
@@ -942,7 +947,7 @@ __device__ __forceinline__ MutantShift mutant_shift(int32_t m, uint64_t seed, ui
     const uint4 v0 = draw_block(seed, gen, (uint32_t)t, OP_MUT + q, 0, sid);
     const uint32_t kind = uniform_below(v0.x, 2u);
     const uint32_t right = uniform_below(v0.y, 2u);
-    int64_t a, len, kk;
+    int32_t a, len, kk;
     if (kind == 0) {
         a = 0;
         len = m;
@@ -966,26 +971,26 @@ __device__ __forceinline__ MutantShift mutant_shift(int32_t m, uint64_t seed, ui
 }
 
 // The mutant F of the W-word row C for a shift, built by a warp (lanes over words).
-template <bool kCG = false>
+template <int kCG = 0>
 __device__ __forceinline__ void mutant_row_shift(const uint32_t *__restrict__ C, uint32_t *__restrict__ F, int32_t W,
                                                  const MutantShift &ms, int lane)
 {
-    const int64_t a = ms.a, len = ms.len, kl = ms.kl;
-    const int64_t pwrap = a + len - kl;  // positions >= pwrap wrap to the start of the block
+    const int32_t a = ms.a, len = ms.len, kl = ms.kl;
+    const int32_t pwrap = a + len - kl;  // positions >= pwrap wrap to the start of the block
     for (int w = lane; w < W; w += 32) {
-        const int64_t pos0 = (int64_t)w * 32;
-        const int64_t in_lo = a > pos0 ? a : pos0;
-        const int64_t in_hi = (a + len) < (pos0 + 32) ? (a + len) : (pos0 + 32);
+        const int32_t pos0 = w * 32;
+        const int32_t in_lo = a > pos0 ? a : pos0;
+        const int32_t in_hi = (a + len) < (pos0 + 32) ? (a + len) : (pos0 + 32);
         const uint32_t cw = ld_ro<kCG>(C + w);
         if (in_lo >= in_hi) {
             F[w] = cw;
             continue;
         }
         uint32_t out = cw & ~range_mask(in_lo - pos0, in_hi - pos0);
-        const int64_t e1 = in_hi < pwrap ? in_hi : pwrap;
+        const int32_t e1 = in_hi < pwrap ? in_hi : pwrap;
         if (in_lo < e1)
             out |= bits_from<kCG>(C, W, pos0 + kl) & range_mask(in_lo - pos0, e1 - pos0);
-        const int64_t s2 = in_lo > pwrap ? in_lo : pwrap;
+        const int32_t s2 = in_lo > pwrap ? in_lo : pwrap;
         if (s2 < in_hi)
             out |= bits_from<kCG>(C, W, pos0 + kl - len) & range_mask(s2 - pos0, in_hi - pos0);
         F[w] = out;
@@ -993,7 +998,7 @@ __device__ __forceinline__ void mutant_row_shift(const uint32_t *__restrict__ C,
 }
 
 // Try q's mutant F of the W-word row C (m bits) of individual t, built by a warp.
-template <bool kCG = false>
+template <int kCG = 0>
 __device__ __forceinline__ void mutant_row(const uint32_t *__restrict__ C, uint32_t *__restrict__ F, int32_t W,
                                            int32_t m, uint64_t seed, uint32_t gen, uint32_t t, uint32_t q,
                                            uint32_t sid, int lane)
@@ -2061,6 +2066,366 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_ga_fused(const __grid_cons
 }
 
 
+// ---------------------------------------------------------------------------
+// A whole generation in one kernel, for an instance whose 16-bit distances
+// fit in shared memory.  Individuals only meet others of their deme
+// (crossover partners), so a cluster of CTAs takes a deme (a CTA several small
+// ones) from its fresh population to its last mutation try: a
+// warp per individual builds each bitset (fresh_individual, crossover_child,
+// mutant_row, as the per-phase kernels do), evaluates it by its open
+// facilities and decides at once.  A crossover round writes its result into
+// the other of two copies of the rows, so one barrier per round is enough;
+// partners in other CTAs are read through distributed shared memory.  The
+// tries after an individual's first improvement are not evaluated.  The CTA
+// that finishes last takes the generation's end.
+//
+// What bounds it: the chain of 1 + R + Q warp-wide steps of about 1000 cycles
+// each (a bitset built, its facilities listed, two rounds of shared memory, a
+// sum) and R cluster barriers; the chip is mostly idle.  The per-phase kernels
+// need 2 R + 6 launches of 2.5 to 3.5 us for the same.  A generation of 64 /
+// 512 individuals of a 100-node graph, p = 5 / 10: 25 / 41 us against 73 / 91;
+// 200 nodes, p = 20, 512: 46 against 103.  The loop's body holds four
+// generations (kDemeUnroll; those past the budget return at once): an
+// iteration of the graph's loop costs about 4 us (28 us with one, 24.7 with
+// eight).
+// ---------------------------------------------------------------------------
+constexpr uint32_t kDemeSpinLimit = 1u << 22, kDemeStallLimit = 1u << 14;
+
+// The distances' entries (8 clients x facility, 16 bytes) lie at oct * deme_pitch(m) + facility: odd, so that eight lanes
+// (octets of clients) read all banks.
+__host__ __device__ __forceinline__ int64_t deme_pitch(int64_t m) { return m | 1; }
+
+// The cost of the bitset F (shared memory), by one warp: lanes over octets of clients, every open facility's distances.
+// list: room for p ids (16 bits, a multiple of eight of them).
+__device__ __forceinline__ uint32_t deme_eval(uint32_t ent, int pitch, int n8, const uint32_t *F, int W, int p,
+                                              uint16_t *list, int lane)
+{
+    // the ids of the open facilities, in any order: eight are read at a time and their entries are in flight together,
+    // so that the warp waits for shared memory twice per eight facilities
+    uint32_t x = lane < W ? F[lane] : 0u;
+    const int cnt = __popc(x);
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(PM_FULL_MASK, incl, o);
+        if (lane >= o)
+            incl += y;
+    }
+    const int total = __shfl_sync(PM_FULL_MASK, incl, 31);
+    const bool listed = W <= 32 && total == p;
+    if (listed) {
+        const uint32_t some = __ballot_sync(PM_FULL_MASK, x != 0u);
+        const int first = __ffs(some) - 1;
+        const int id0 = 32 * first + __shfl_sync(PM_FULL_MASK, __ffs(x) - 1, first);
+        for (int pos = incl - cnt; x; ++pos) {
+            list[pos] = (uint16_t)(32 * lane + __ffs(x) - 1);
+            x &= x - 1u;
+        }
+        if (lane < ((8 - (p & 7)) & 7))
+            list[p + lane] = (uint16_t)id0;  // the last eight: one of them again
+        __syncwarp();
+    }
+    uint32_t sum = 0u;
+    for (int o = 0; o < n8; o += 32) {
+        const bool on = o + lane < n8;
+        const uint32_t base = ent + (uint32_t)(on ? (o + lane) * pitch : 0) * 16u;
+        uint32_t v[4] = {~0u, ~0u, ~0u, ~0u}, any = 0u;
+        auto use = [&](uint32_t j) {
+            uint32_t e[4];
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(e[0]), "=r"(e[1]), "=r"(e[2]), "=r"(e[3])
+                         : "r"(base + 16u * j));
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                v[i] = min_u16x2(v[i], e[i]);
+        };
+        if (listed) {
+            any = 1u;
+            for (int q = 0; q < p; q += 8) {
+                const uint4 ids = *reinterpret_cast<const uint4 *>(list + q);
+                const uint32_t id[4] = {ids.x, ids.y, ids.z, ids.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    use(id[i] & 0xffffu);
+                    use(id[i] >> 16);
+                }
+            }
+        } else {  // more words than lanes, or (a population loaded with other bitsets) not p open facilities
+            for (int w = 0; w < W; ++w) {
+                uint32_t y = F[w];
+                any |= y;
+                while (y) {
+                    use(32u * (uint32_t)w + (uint32_t)__ffs(y) - 1u);
+                    y &= y - 1u;
+                }
+            }
+        }
+        if (on && any) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                sum = __dp2a_lo(v[i], 0x0101u, sum);
+        }
+    }
+    return __reduce_add_sync(PM_FULL_MASK, sum);
+}
+
+__device__ __forceinline__ void deme_advance(ga_glob *glob, int alive, cudaGraphConditionalHandle h, int in_graph)
+{
+    glob->alive = alive;
+    glob->step_gens += 1;
+    const long long left = glob->remaining - 1;
+    glob->remaining = left;
+    if (in_graph)
+        cudaGraphSetConditional(h, (left > 0 && alive) ? 1u : 0u);
+}
+
+__global__ void __launch_bounds__(1024, 1) k_ga_deme(ga_prob gp, const uint16_t *__restrict__ dense, int n8, int32_t R,
+                                                     int32_t Q, uint64_t seed, uint32_t *X, int64_t *cost,
+                                                     uint8_t *improved, uint32_t *deme_best, int64_t *deme_cost,
+                                                     uint32_t *best_row, ga_dev *st, ga_glob *glob, int *err,
+                                                     uint32_t stall, cudaGraphConditionalHandle h, int in_graph)
+{
+    extern __shared__ __align__(128) unsigned char dsm[];
+    __shared__ uint64_t bar;
+    __shared__ unsigned evals_s;
+    __shared__ int last_s;
+    __shared__ long long wc[32], wi[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, here = blockDim.x >> 5;  // here: a power of two
+    const int32_t W = gp.W, m = gp.m, p = gp.p;
+    const int pitch = (int)deme_pitch(m);
+    const int lp = (p + 7) & ~7;  // this warp's list of open facilities; then two copies of the CTA's rows
+    uint16_t *list = reinterpret_cast<uint16_t *>(dsm + (size_t)n8 * pitch * 16) + (int64_t)warp * lp;
+    uint32_t *rows = reinterpret_cast<uint32_t *>(dsm + (size_t)n8 * pitch * 16 + (size_t)here * lp * 2);
+    uint32_t *F = rows + (int64_t)(2 * here + warp) * W;                           // this warp's child or mutant
+    uint32_t *draws = rows + (int64_t)(3 * here) * W + (int64_t)warp * p;
+    const uint32_t ent = smem_u32(dsm);
+    const bool wide = gp.D > here;  // a deme is a cluster
+    const int64_t t = (int64_t)blockIdx.x * here + warp;
+    const bool live = t < gp.pop;
+    // the distances never change: their copies start before the previous kernel (the last generation's end) is done
+    if (warp == 0) {
+        if (lane == 0) {
+            evals_s = 0u;
+            mbar_init(&bar, 1);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            if (!stall)
+                mbar_arrive_expect_tx(&bar, (uint32_t)(n8 * m) * 16u);
+        }
+        __syncwarp();
+        if (!stall)  // a launch armed by pm_debug_scan_timeout issues none: the wait below runs out
+            for (int o = lane; o < n8; o += 32)
+                bulk_g2s(dsm + (size_t)o * pitch * 16, dense + (size_t)o * m * 8, (uint32_t)m * 16u, &bar);
+    }
+    __syncthreads();
+    pm_grid_dependency_wait();
+    const bool stopped = *reinterpret_cast<volatile int *>(&st->stop) != 0;  // the same for all CTAs
+    // past the call's last generation: the rest of the loop's body
+    const bool over = in_graph && *reinterpret_cast<volatile long long *>(&glob->remaining) <= 0;
+    const uint32_t gen = (uint32_t)*reinterpret_cast<volatile long long *>(&st->gen);
+    bool filled = false;
+    for (uint32_t spins = 0; !filled && spins < (stall ? kDemeStallLimit : kDemeSpinLimit); ++spins)
+        filled = mbar_try_wait(&bar, 0);
+    if (!filled) {
+        if (threadIdx.x == 0)
+            atomicExch(err, (int)PM_ERR_TIMEOUT);
+        for (uint32_t spins = 0; !stall && spins < kDemeSpinLimit && !mbar_try_wait(&bar, 0); ++spins)
+            ;  // copies in flight may still land
+    }
+    // a CTA without its distances keeps its cluster company (peers read its rows) but writes no result
+    const bool ok = __syncthreads_and(filled) != 0;
+    if (stopped || over) {
+        if (!in_graph && blockIdx.x == 0 && threadIdx.x == 0)
+            deme_advance(glob, 0, h, in_graph);
+        return;
+    }
+
+    uint32_t *row = rows + (int64_t)warp * W;
+    uint32_t c = 0u;
+    unsigned evals = 0u;
+    if (live) {
+        fresh_individual<true>(gp, t, gen, seed, deme_best, row, draws, lane);
+        c = deme_eval(ent, pitch, n8, row, W, p, list, lane);
+    }
+    int cur = 0;
+    if (p / 2 > 0) {
+        uint32_t my_r1 = 0u, my_i = 0u;
+        int step = 0;  // r mod lg D
+        for (int32_t r = 0; r < R; ++r, step = step + 1 == gp.lgD ? 0 : step + 1) {
+            const int64_t stride = gp.D >> (1 + step);
+            if ((r & 31) == 0 && r + lane < R) {  // the draws of 32 rounds, one a lane
+                const int64_t other = t ^ (gp.D >> (1 + ((r + lane) % gp.lgD)));
+                const uint4 v = draw_block(seed, gen, (uint32_t)(t < other ? t : other), OP_XOVER + (uint32_t)(r + lane),
+                                           0, gp.sid);
+                my_r1 = uniform_below(v.x, (uint32_t)m);
+                my_i = 1u + uniform_below(v.y, (uint32_t)(p / 2));
+            }
+            if (wide) {  // the round before is complete in every CTA of the deme
+                asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+                asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+            } else {
+                __syncthreads();
+            }
+            if (live) {
+                const int64_t partner = t ^ stride;
+                const uint32_t r1 = __shfl_sync(PM_FULL_MASK, my_r1, r & 31);
+                const int i = (int)__shfl_sync(PM_FULL_MASK, my_i, r & 31);
+                const uint32_t *C = rows + (int64_t)(here * cur + warp) * W;
+                const uint32_t *K = rows + (int64_t)(here * cur + (int)(partner & (here - 1))) * W;
+                if (stride >= here) {
+                    const uint32_t peer = (uint32_t)(partner & (gp.D - 1)) >> (__ffs(here) - 1);
+                    uint64_t at;
+                    asm("mapa.u64 %0, %1, %2;" : "=l"(at) : "l"(reinterpret_cast<uint64_t>(K)), "r"(peer));
+                    K = reinterpret_cast<const uint32_t *>(at);
+                }
+                const bool valid = crossover_child<false>(C, K, F, W, r1, i, lane);
+                __syncwarp();
+                const uint32_t *keep = C;
+                if (valid) {
+                    const uint32_t fc = deme_eval(ent, pitch, n8, F, W, p, list, lane);
+                    ++evals;
+                    if (fc < c) {
+                        c = fc;
+                        keep = F;
+                    }
+                }
+                uint32_t *next = rows + (int64_t)(here * (cur ^ 1) + warp) * W;
+                for (int w = lane; w < W; w += 32)
+                    next[w] = keep[w];
+                __syncwarp();
+            }
+            cur ^= 1;
+        }
+    }
+    if (wide)  // no rows of other CTAs are read from here on; waited for before the rows go away
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (live) {
+        const uint32_t *C = rows + (int64_t)(here * cur + warp) * W;
+        const uint32_t *best = C;
+        bool better = false;
+        int my_a = 0, my_len = 0, my_kl = 0;
+        for (int32_t q = 0; q < Q && !better; ++q) {
+            if ((q & 31) == 0 && q + lane < Q) {  // the shifts of 32 tries, one a lane
+                const MutantShift ms = mutant_shift(m, seed, gen, (uint32_t)t, (uint32_t)(q + lane), gp.sid);
+                my_a = (int)ms.a;
+                my_len = (int)ms.len;
+                my_kl = (int)ms.kl;
+            }
+            MutantShift ms;
+            ms.a = __shfl_sync(PM_FULL_MASK, my_a, q & 31);
+            ms.len = __shfl_sync(PM_FULL_MASK, my_len, q & 31);
+            ms.kl = __shfl_sync(PM_FULL_MASK, my_kl, q & 31);
+            mutant_row_shift<kPlain>(C, F, W, ms, lane);
+            __syncwarp();
+            const uint32_t fc = deme_eval(ent, pitch, n8, F, W, p, list, lane);
+            ++evals;
+            if (fc < c) {
+                c = fc;
+                best = F;
+                better = true;
+            }
+            __syncwarp();
+        }
+        if (ok) {
+            for (int w = lane; w < W; w += 32)
+                X[gp.word_base + t * W + w] = best[w];
+            if (lane == 0) {
+                cost[gp.ind_base + t] = (int64_t)c;
+                improved[gp.ind_base + t] = better ? 1 : 0;
+                atomicAdd(&evals_s, evals);
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (evals_s)
+            atomicAdd(reinterpret_cast<unsigned long long *>(&st->evals), (unsigned long long)evals_s);
+        __threadfence();
+        last_s = atomicAdd(&st->deme_ticket, 1) == (int)gridDim.x - 1 ? 1 : 0;
+    }
+    if (wide)
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    __syncthreads();
+    if (!last_s)
+        return;
+
+    // The generation's end (k_ga_generation_end_one's results) by the CTA that finishes last: a warp per deme, or per 32
+    // demes of fewer than 32 individuals, takes the lowest (cost, index); then the deme bests' rows and the global best.
+    __threadfence();
+    constexpr long long kNone = 0x7fffffffffffffffLL;
+    const long long *costs = reinterpret_cast<const long long *>(cost) + gp.ind_base;
+    const int D = (int)gp.D, NB = (int)gp.NB;
+    int *winner = reinterpret_cast<int *>(dsm);  // of each deme, where there is room (the distances are done with)
+    long long mc = kNone, mi = kNone;
+    auto take = [](long long &c0, long long &i0, long long c1, long long i1) {
+        if (c1 < c0 || (c1 == c0 && i1 < i0)) {
+            c0 = c1;
+            i0 = i1;
+        }
+    };
+    auto lowest = [&](long long &c0, long long &i0) {  // over the warp
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            take(c0, i0, __shfl_xor_sync(PM_FULL_MASK, c0, o), __shfl_xor_sync(PM_FULL_MASK, i0, o));
+    };
+    auto finish = [&](int d, long long c0, long long i0) {  // one lane: deme d's best
+        deme_cost[gp.deme_base + d] = c0;
+        winner[d] = (int)i0;
+        take(mc, mi, c0, i0);
+    };
+    if (D >= 32) {
+        for (int d = warp; d < NB; d += here) {
+            long long dc = kNone, di = kNone;
+            for (int x = lane; x < D; x += 32)
+                take(dc, di, __ldcg(costs + (int64_t)d * D + x), (long long)d * D + x);
+            lowest(dc, di);
+            if (lane == 0)
+                finish(d, dc, di);
+        }
+    } else {
+        for (int d = threadIdx.x; d < NB; d += blockDim.x) {
+            long long dc = kNone, di = kNone;
+            for (int x = 0; x < D; ++x)
+                take(dc, di, __ldcg(costs + (int64_t)d * D + x), (long long)d * D + x);
+            finish(d, dc, di);
+        }
+    }
+    lowest(mc, mi);
+    if (lane == 0) {
+        wc[warp] = mc;
+        wi[warp] = mi;
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < NB * W; x += blockDim.x) {
+        const int d = x / W, w = x - d * W;
+        deme_best[gp.dword_base + x] = __ldcg(X + gp.word_base + (int64_t)winner[d] * W + w);
+    }
+    if (warp == 0) {
+        mc = lane < here ? wc[lane] : kNone;
+        mi = lane < here ? wi[lane] : kNone;
+        lowest(mc, mi);
+        const long long prev = *reinterpret_cast<volatile long long *>(&st->best_cost);
+        const bool lower = prev < 0 || mc < prev;
+        if (lower)
+            for (int w = lane; w < W; w += 32)
+                best_row[gp.best_base + w] = __ldcg(X + gp.word_base + mi * W + w);
+        if (lane == 0) {
+            const long long sat = lower ? 0 : st->sat + 1;
+            if (lower)
+                st->best_cost = mc;
+            st->sat = sat;
+            if (st->trace)
+                st->trace[glob->step_gens] = lower ? mc : prev;
+            atomicAdd(reinterpret_cast<unsigned long long *>(&st->evals), (unsigned long long)gp.pop);
+            st->gen = (long long)gen + 1;
+            st->total_gens += 1;
+            st->deme_ticket = 0;
+            const int stop = (st->saturation > 0 && sat >= st->saturation) ? 1 : 0;
+            st->stop = stop;
+            deme_advance(glob, stop ? 0 : 1, h, in_graph);
+        }
+    }
+}
+
 // Uniform random p-subsets (Floyd sampling, generation 0, no migration), one
 // thread per individual, bitsets written in place.
 __global__ void k_random_population(uint32_t *__restrict__ X, int64_t P, int32_t W, int32_t m, int32_t p,
@@ -2086,6 +2451,22 @@ __global__ void k_random_population(uint32_t *__restrict__ X, int64_t P, int32_t
 }  // namespace
 
 // ------------------------------- host side ---------------------------------
+
+constexpr int64_t kDemeChain = 96, kDemeWork = 100 * 1024;  // see deme_prepare
+constexpr int kDemeUnroll = 4;                               // generations in the body of the graph's loop
+
+static int64_t deme_chain(int64_t n, int64_t p) { return p * pm_ceil_div(pm_ceil_div(n, 8), 32); }
+
+static size_t deme_smem(int64_t n, int64_t m, int64_t p, int64_t warps)
+{
+    return (size_t)(pm_ceil_div(n, 8) * deme_pitch(m) * 16 +
+                    warps * ((3 * pm_ceil_div(m, 32) + p) * 4 + pm_round_up(p, 8) * 2));
+}
+
+bool pm_deme_fits(int64_t n, int64_t m, int64_t p, size_t smem_optin)
+{
+    return deme_smem(n, m, p, 32) + 2048 <= smem_optin && deme_chain(n, p) <= kDemeChain;
+}
 
 pm_status pm_launch_random_population(const pm_instance *inst, uint64_t seed, int64_t pop, uint32_t *masks,
                                       cudaStream_t s)
@@ -2135,6 +2516,10 @@ struct pm_ga {
     size_t fused_smem = 0;
     int64_t f_tiles = 0, f_splits = 1, f_cps = 0, f_tilesQ = 0, f_splitsQ = 1, f_cpsQ = 0;
     pm_dbuf bar;
+    // the kernel over whole demes in place of a generation's phases when the GA qualifies
+    bool deme = false;
+    int deme_warps = 32;
+    size_t deme_smem = 0;
     // learned swap proposal (single-instance GAs)
     pm_model *model = nullptr;
     int T = 4;
@@ -2220,10 +2605,84 @@ static pm_status ga_eval(pm_ga *ga, const uint32_t *masks, int64_t *costs, const
     return pm_launch_scan(L, acc, costs, s);
 }
 
+static cudaLaunchConfig_t deme_config(const pm_ga *ga, cudaStream_t s, cudaLaunchAttribute (&attr)[2])
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)pm_ceil_div(ga->P, ga->deme_warps));
+    cfg.blockDim = dim3((unsigned)ga->deme_warps * 32u);
+    cfg.dynamicSmemBytes = ga->deme_smem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)std::max<int64_t>(1, ga->D / ga->deme_warps);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pm_pdl_enabled() ? 2 : 1;
+    return cfg;
+}
+
+// The rule for the kernel over whole demes (k_ga_deme): one instance with Floyd generation and no learned try, whose
+// distances fit beside the CTA's rows, and demes of at most a cluster of 16 CTAs.  kDemeChain bounds an evaluation's chain
+// (p facilities for each 32 octets of clients) and kDemeWork what the population adds to it, where the phases' launches
+// are the cheaper way: us a generation, demes of 256, this kernel and the phases: chain 64 (256 nodes, p = 64), 512
+// individuals: 72 / 109; chain 120 (330 nodes, p = 60): 107 / 107; chain 200 (300 nodes, p = 100): 163 / 112; 4096
+// individuals, chain 25 (250 nodes): 140 / 178; chain 50 (100 nodes): 183 / 145.
+// PM_GA_DEME=0 and PM_GA_SPEC=0 in the environment keep the per-phase kernels (identical results; for comparison).
+static pm_status deme_prepare(pm_ga *ga)
+{
+    ga->deme = false;
+    const pm_instance *inst = ga->insts[0];
+    const char *v = std::getenv("PM_GA_DEME");
+    if ((v && v[0] == '0') || !spec_allowed() || ga->K != 1 || ga->model || ga->comb || !inst->dense || ga->D > 512 ||
+        ga->P > 4096 || ga->P * deme_chain(inst->n, inst->p) > kDemeWork || inst->n > 65536 ||
+        !pm_deme_fits(inst->n, inst->m, inst->p, inst->smem_optin))
+        return PM_OK;
+    // as few warps a CTA as a deme's cluster and two CTAs per SM allow: what a generation waits for is each warp's
+    // chain, and warps that share a scheduler stretch it.  Demes of 256: 44.5 us a generation with 16 CTAs of 16 warps,
+    // 58.7 with eight of 32 (100 x 100, p = 10).
+    int64_t warps = std::max<int64_t>(4, ga->D / 16);
+    while (warps < 16 && pm_ceil_div(ga->P, warps) > 2 * inst->sm_count)
+        warps *= 2;
+    PM_CUDA(cudaFuncSetAttribute(k_ga_deme, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inst->smem_optin - 2048));
+    PM_CUDA(cudaFuncSetAttribute(k_ga_deme, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    for (; warps <= 32; warps *= 2) {
+        ga->deme_warps = (int)warps;
+        ga->deme_smem = std::max<size_t>(deme_smem(inst->n, inst->m, inst->p, warps), (size_t)ga->NB * 4);
+        cudaLaunchAttribute attr[2];
+        const cudaLaunchConfig_t cfg = deme_config(ga, nullptr, attr);
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, k_ga_deme, &cfg) == cudaSuccess && clusters > 0) {
+            ga->deme = true;
+            return PM_OK;
+        }
+        cudaGetLastError();
+    }
+    return PM_OK;
+}
+
+static pm_status deme_launch(pm_ga *ga, cudaStream_t s, cudaGraphConditionalHandle h, int in_graph)
+{
+    const pm_instance *inst = ga->insts[0];
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = deme_config(ga, s, attr);
+    PM_CUDA(cudaLaunchKernelEx(&cfg, k_ga_deme, ga->gps[0], (const uint16_t *)inst->dense, (int)pm_ceil_div(inst->n, 8),
+                               (int32_t)ga->R, (int32_t)ga->Q, ga->seed, static_cast<uint32_t *>(ga->X.ptr),
+                               static_cast<int64_t *>(ga->cost.ptr), static_cast<uint8_t *>(ga->improved.ptr),
+                               static_cast<uint32_t *>(ga->deme_best.ptr), static_cast<int64_t *>(ga->deme_cost.ptr),
+                               static_cast<uint32_t *>(ga->best.ptr), static_cast<ga_dev *>(ga->st.ptr),
+                               static_cast<ga_glob *>(ga->glob.ptr), static_cast<int *>(ga->err.ptr),
+                               pm_take_scan_stall() ? 1u : 0u, h, in_graph));
+    return PM_OK;
+}
+
 // Enqueue one generation on `s`: under stream capture for the graph body
 // (in_graph = 1), or directly on the stream (in_graph = 0).
 static pm_status enqueue_generation(pm_ga *ga, cudaStream_t s, cudaGraphConditionalHandle h, int in_graph)
 {
+    if (ga->deme)
+        return deme_launch(ga, s, h, in_graph);
     const ga_prob *gps = static_cast<const ga_prob *>(ga->gprobs.ptr);
     const ga_prob one = ga->gps[0];
     const int K = ga->K;
@@ -2445,6 +2904,8 @@ static pm_status build_graph(pm_ga *ga)
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     PM_CUDA(cudaStreamBeginCaptureToGraph(ga->cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     pm_status st_gen = enqueue_generation(ga, ga->cap, h, 1);
+    for (int i = 1; ga->deme && i < kDemeUnroll && st_gen == PM_OK; ++i)
+        st_gen = enqueue_generation(ga, ga->cap, h, 1);
     cudaGraph_t captured = nullptr;
     cudaError_t e = cudaStreamEndCapture(ga->cap, &captured);
     PM_TRY(st_gen);
@@ -2805,6 +3266,8 @@ static pm_status ga_create_common(pm_ga *ga, cudaStream_t s)
         st = ga_make_stream(ga);
     if (st == PM_OK)
         st = fused_prepare(ga, s);
+    if (st == PM_OK)
+        st = deme_prepare(ga);
     if (st == PM_OK)
         st = build_graph(ga);
     return st;
@@ -3229,7 +3692,9 @@ extern "C" pm_status pm_ga_info(const pm_ga *ga, int64_t *pop, int64_t *deme, in
             *kernels_per_step_call = 2;
         return PM_OK;
     }
-    if (kernels_per_generation)
+    if (kernels_per_generation && ga->deme)
+        *kernels_per_generation = 1;
+    else if (kernels_per_generation)
         *kernels_per_generation = 1 + per_eval + rounds * (1 + per_eval) +
                                   (ga->spec ? 3 : ga->Q * (1 + per_eval)) + 1 + (ga->model ? 4 + per_eval : 0);
     if (kernels_per_step_call)

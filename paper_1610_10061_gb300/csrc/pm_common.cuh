@@ -271,6 +271,8 @@ double pm_scan_cost(int64_t m, int64_t p);
 double pm_direct_cost(int64_t m, int64_t p, int64_t range, int stages);
 // Whether an instance of these sizes should keep the 16-bit distances.
 bool pm_direct_wanted(int64_t n, int64_t m, int64_t p, size_t smem_optin);
+// Whether a GA's CTA can hold all of them and evaluate an individual by them in a short chain (k_ga_deme).
+bool pm_deme_fits(int64_t n, int64_t m, int64_t p, size_t smem_optin);
 // Whether a launch has enough units of 1024 (client, individual) pairs for the bit-sliced walk: a unit is a chain
 // of about 1200 instructions of one warp, so with too few per SM the SMs wait for single warps and the rank-split
 // walk is the faster one.  GA generations whose scans have 16 to 23 units per SM (graph900 pop 2048; 5000 x 5000, p =
