@@ -13,6 +13,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import sys
 
 import numpy as np
 
@@ -132,16 +133,22 @@ def _check(status: int, where: str):
         raise PMError(status, where)
 
 
+# An evaluation of a small population is about 5 us in the library, so what the marshalling costs counts: addresses go as
+# plain integers (the signatures above convert them) and the current stream is asked for by its raw handle, which needs
+# no stream object and no availability check.  Instance.eval of 64 subsets of a 100-node graph: 19 -> 13 us a call.
+
 def _stream(stream):
     if stream is not None:
-        return ctypes.c_void_p(int(stream))
+        return int(stream)
+    torch = sys.modules.get("torch")  # a program that has not imported it has no current stream
+    if torch is None:
+        return 0
     try:
-        import torch
-        if torch.cuda.is_available() and torch.cuda.is_initialized():
-            return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     except Exception:
         pass
-    return ctypes.c_void_p(0)
+    return 0
 
 
 def _addr(a):
@@ -151,11 +158,11 @@ def _addr(a):
     if isinstance(a, np.ndarray):
         if not a.flags["C_CONTIGUOUS"]:
             raise ValueError("array must be C-contiguous")
-        return ctypes.c_void_p(a.ctypes.data)
+        return a.ctypes.data
     if hasattr(a, "data_ptr"):
         if not a.is_contiguous():
             raise ValueError("tensor must be contiguous")
-        return ctypes.c_void_p(a.data_ptr())
+        return a.data_ptr()
     raise TypeError(f"unsupported buffer type {type(a)}")
 
 
@@ -580,7 +587,8 @@ class Instance:
 
     def eval(self, masks, costs=None, checked: bool = False, stream=None):
         """Costs of a population; numpy in -> numpy out, CUDA tensor in -> CUDA tensor out."""
-        pop = int(masks.shape[0]) if masks.ndim == 2 else int(masks.shape[0] // self.W)
+        shape = masks.shape
+        pop = int(shape[0]) if len(shape) == 2 else int(shape[0] // self.W)
         if costs is None:
             if isinstance(masks, np.ndarray):
                 costs = np.zeros(pop, dtype=np.int64)
