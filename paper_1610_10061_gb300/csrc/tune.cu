@@ -5,8 +5,10 @@
 // client and wants many small CTAs; for long scans it is issue-bound and
 // wants large tiles that share each staged row chunk among 128 individuals.
 // The candidates cover both mask layouts: facility-major bit columns (the
-// column kernel, G x 32 individuals per shared-memory load) and
-// individual-major bitsets (the row kernel, one individual per warp).
+// column kernel, G x 32 individuals per shared-memory load, in whichever walk
+// the launch's size asks for) and individual-major bitsets (the row kernel,
+// one individual per warp), and the evaluation by open facilities where the
+// instance has the distances for it.
 // Rather than model that, the tuner times the candidate shapes on the
 // instance itself and keeps the fastest per population size.
 
@@ -50,6 +52,7 @@ extern "C" pm_status pm_tune_eval(pm_instance *inst, int64_t pop, void *stream, 
         cands.push_back(pl);
     };
     const size_t budget = inst->smem_optin > 4096 ? inst->smem_optin - 4096 : 0;
+    bool direct_asked = false;
     for (int G : {4, 2, 1}) {
         if ((size_t)inst->W * 32 * G * 4 > budget)
             continue;
@@ -61,7 +64,8 @@ extern "C" pm_status pm_tune_eval(pm_instance *inst, int64_t pop, void *stream, 
                 add(base);
             for (int sp : {std::max(1, base.splits / 2), base.splits, base.splits * 2}) {
                 const pm_eval_plan pl = pm_plan_eval_with(inst, pop, G, warps, sp);
-                if (cands.empty()) {  // the heuristic's other way of evaluating, where it applies
+                if (warps == 16 && !direct_asked) {  // the heuristic's other way of evaluating, where it applies
+                    direct_asked = true;
                     pm_eval_plan direct = pl;
                     if (pm_plan_direct(inst, pop, direct))
                         cands.push_back(direct);
