@@ -81,8 +81,11 @@ __device__ __forceinline__ int find_prob(int K, int64_t x, F base)
 // launch.  colT[col_base + (tile*32W + j)*G + g] (j < 32W) = bits over
 // individuals tile*32G + 32g + b of that instance.  One warp per (instance,
 // tile, g, w) job; grid-stride over the jobs.  Instances evaluated by open
-// facilities get their individuals' lists instead (a job per individual).
+// facilities get their individuals' lists instead (a job per individual;
+// kLists: some instance of the launch does -- the lists' registers cost the
+// transposition 2 us at 4096 x 10000).
 // ---------------------------------------------------------------------------
+template <bool kLists>
 __global__ void k_pop_to_columns(const uint32_t *__restrict__ masks, const pm_prob *__restrict__ probs, int K,
                                  pm_prob one, int64_t jobs, int32_t G, uint32_t *__restrict__ colT)
 {
@@ -96,7 +99,7 @@ __global__ void k_pop_to_columns(const uint32_t *__restrict__ masks, const pm_pr
             pr = probs + find_prob(K, job, [&](int k) { return probs[k].job_base; });
         const int64_t lj = job - pr->job_base;
         const int32_t W = pr->W;
-        if (pr->d_range) {  // a list of open facilities per individual in place of the facility-major form
+        if (kLists && pr->d_range) {  // a list of open facilities per individual in place of the facility-major form
             write_open_list(masks + pr->word_base + lj * W, W, pr->m, pr->p, colT + pr->col_base,
                             (pr->pop + 31) / 32 * 32, lj, lane);
             continue;
@@ -872,7 +875,8 @@ double pm_scan_cost(int64_t m, int64_t p) { return 0.35 + 0.037 * (double)(m + 1
 
 double pm_direct_cost(int64_t m, int64_t p, int64_t range, int stages)
 {
-    return 0.35 + 0.05 * (double)p + (stages == 2 ? 0.03 : 0.1) * (double)m / (double)range;
+    const double walk = p < kOrderedList ? 0.35 + 0.05 * (double)p : 0.75 + 0.03 * (double)p;
+    return walk + (stages == 2 ? 0.03 : 0.1) * (double)m / (double)range;
 }
 
 void pm_direct_shape(const pm_instance *inst, int64_t pop, size_t budget, int nwarps, pm_direct_plan &out)
@@ -1129,7 +1133,8 @@ static pm_status launch_transpose(const uint32_t *masks, const pm_prob *probs, i
 {
     const int threads = 256;
     const int64_t blocks = std::min<int64_t>(pm_ceil_div(jobs, threads / 32), (int64_t)2048);
-    PM_CUDA(pm_launch(k_pop_to_columns, (unsigned)blocks, threads, 0, stream, masks, probs, K, one, jobs, G, colT));
+    PM_CUDA(pm_launch(K > 1 || one.d_range ? k_pop_to_columns<true> : k_pop_to_columns<false>, (unsigned)blocks, threads,
+                      0, stream, masks, probs, K, one, jobs, G, colT));
     return PM_OK;
 }
 

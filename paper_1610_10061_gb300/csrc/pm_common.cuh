@@ -265,8 +265,10 @@ void pm_direct_splits(const pm_instance *inst, int64_t want, pm_direct_plan &d);
 void pm_direct_prob(const pm_instance *inst, const pm_direct_plan &d, int64_t pop, struct pm_prob &pr);
 // Estimated SM cycles per (individual, client) pair of the two ways, fitted to evaluations of 256 to 4096 subsets of
 // 300 to 10000 facilities, p = 3 to 1000: the scan's walk grows with the expected first open rank (1.76 cycles at m /
-// p = 33, 4.0 at 100, 12.7 at 322); p reads of 16 bytes for 8 pairs (1.05 cycles at p = 10, 3.4 at 60) plus the fill of
-// a chunk of m entries for `range` individuals, hidden but for its ends with two stages.
+// p = 33, 4.0 at 100, 12.7 at 322); p reads of 16 bytes for 8 pairs (1.05 cycles at p = 10; with the lists ordered for
+// the banks, from p = 16 on, 1.35 at 20, 1.89 at 40, 3.37 at 100; for fewer facilities than thousands up to 0.3 more, and
+// the line lies on their side: 1000 facilities, p = 40, 117 us against the scan's 63, estimated 1.95 against 1.25)
+// plus the fill of a chunk of m entries for `range` individuals, hidden but for its ends with two stages.
 double pm_scan_cost(int64_t m, int64_t p);
 double pm_direct_cost(int64_t m, int64_t p, int64_t range, int stages);
 // Whether an instance of these sizes should keep the 16-bit distances.

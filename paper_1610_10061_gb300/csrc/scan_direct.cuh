@@ -15,13 +15,15 @@
 // instructions.  Sums are 32-bit in shared memory, for up to kDirectRange
 // individuals a CTA.
 //
-// Measured on GB300, 4096 subsets of 10000 x 10000 points: p = 3 / 10 / 30 /
-// 60 in 0.100 / 0.137 / 0.258 / 0.442 ms against 6.47 / 3.81 / 1.66 / 0.858
-// for the bit-sliced scan.  Bound by shared memory: 32 lanes' random entries
-// take about 11 wavefronts (0.047 SM cycles per pair and open facility), the
-// rest is the fill (200 MB of entries, 30 us of HBM time here, exposed where
-// only one stage fits).  Row-major distances with the entries put together by
-// the CTA (eight loads, eight permutations, two stores per pair of facilities)
+// Measured on GB300, 4096 subsets of 10000 x 10000 points: p = 3 / 10 / 20 /
+// 40 / 80 / 100 in 0.100 / 0.133 / 0.176 / 0.246 / 0.375 / 0.438 ms against
+// 6.28 / 4.29 / 2.28 / 1.22 / 0.696 / 0.530 for the bit-sliced scan.  Bound by
+// shared memory: 32 lanes' random entries take about 11 wavefronts (0.047 SM
+// cycles per pair and open facility), half of that with lists in an order that
+// suits the banks (write_open_list); the rest is the fill (200 MB of entries,
+// 30 us of HBM time here, exposed where only one stage fits).  Row-major
+// distances with the entries put together by the CTA (eight loads, eight
+// permutations, two stores per pair of facilities)
 // took 0.21 ms at p = 10: the loads' latency was the CTA's critical path.
 //
 // A bitset without exactly p open facilities (unchecked calls only) has no
@@ -35,41 +37,171 @@
 
 constexpr int kDirectRange = 4096;           // individuals of one work item, at most
 constexpr uint32_t kNoList = 0xffffffffu;    // first list word of a bitset without exactly p open facilities
+constexpr int kOrderedList = 16;             // open facilities from which the lists are ordered for the banks
 
 // The list of one individual's open facilities, by one warp: ids 2q and 2q+1
 // in word q of lists[q * pitch + t] (the last id twice when p is odd), or
 // kNoList in word 0.  row: the individual's W words (bits at or above m are
 // ignored, as the scan ignores them).
+//
+// Eight lanes read their 16-byte entries in one wavefront if the entries lie
+// in different eighths of the banks, that is if the ids differ mod 8.  So from
+// kOrderedList facilities on the list is not in the order of the ids: position
+// s of individual t takes an id of class (s + t) mod 8 while it has one (the
+// k-th id of class c goes to position 8 k + (c - t) mod 8), and the ids that
+// find no such position fill the holes that other classes leave, most of them
+// near the end.  Wavefronts per eight lanes at p = 10 / 30 / 100: 2.14 / 1.72 /
+// 1.42 against 2.6; below kOrderedList the list costs more than that saves
+// (p = 3, 4096 subsets of 10000 x 10000: 108 us against 100; p = 10: 136, 133).
 __device__ __forceinline__ void write_open_list(const uint32_t *row, int32_t W, int32_t m, int32_t p, uint32_t *lists,
                                                 int64_t pitch, int64_t t, int lane)
 {
-    int count = 0;
-    for (int base = 0; base < W; base += 32) {
-        const int w = base + lane;
+    auto word = [&](int w) {
         uint32_t x = w < W ? row[w] : 0u;
         if (w == W - 1 && (m & 31))
             x &= (1u << (m & 31)) - 1u;
-        const int n = __popc(x);
-        int incl = n;
+        return x;
+    };
+    auto by_class = [](uint32_t x, uint32_t (&c)[2]) {  // class 4 h + i in byte i of c[h]
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            c[h] = 0u;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                c[h] |= __popc(x & (0x01010101u << (4 * h + i))) << (8 * i);
+        }
+    };
+    if (p < kOrderedList) {
+        int count = 0;
+        for (int base = 0; base < W; base += 32) {
+            uint32_t x = word(base + lane);
+            const int n = __popc(x);
+            int incl = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(PM_FULL_MASK, incl, o);
+                if (lane >= o)
+                    incl += y;
+            }
+            for (int pos = count + incl - n; x; ++pos) {
+                const uint16_t id = (uint16_t)(32 * (base + lane) + __ffs(x) - 1);
+                x &= x - 1u;
+                if (pos < p)
+                    reinterpret_cast<uint16_t *>(lists + (int64_t)(pos >> 1) * pitch + t)[pos & 1] = id;
+                if (pos == p - 1 && (p & 1))
+                    reinterpret_cast<uint16_t *>(lists + (int64_t)(pos >> 1) * pitch + t)[1] = id;
+            }
+            count += __shfl_sync(PM_FULL_MASK, incl, 31);
+        }
+        __syncwarp();
+        if (count != p && lane == 0)
+            lists[t] = kNoList;
+        return;
+    }
+    // how many ids of each class there are: n in lane c
+    uint32_t tot[4] = {};  // 16-bit halves: classes 0, 2 | 1, 3 | 4, 6 | 5, 7
+    for (int base = 0; base < W; base += 32) {
+        uint32_t c[2];
+        by_class(word(base + lane), c);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            tot[2 * h] += c[h] & 0x00ff00ffu;
+            tot[2 * h + 1] += (c[h] >> 8) & 0x00ff00ffu;
+        }
+    }
+    int count = 0, n = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        tot[i] = __reduce_add_sync(PM_FULL_MASK, tot[i]);
+        count += (int)(tot[i] & 0xffffu) + (int)(tot[i] >> 16);
+        const int c = 4 * (i >> 1) + (i & 1);  // in the low half; c + 2 in the high one
+        if (lane == c)
+            n = (int)(tot[i] & 0xffffu);
+        if (lane == c + 2)
+            n = (int)(tot[i] >> 16);
+    }
+    if (count != p) {
+        if (lane == 0)
+            lists[t] = kNoList;
+        return;
+    }
+    const int turn = (int)(t & 7);
+    auto first = [&](int c) { return (c - turn) & 7; };             // class c's first position
+    auto places = [&](int c) { return (p - first(c) + 7) >> 3; };   // and how many it has below p
+    const int surplus = lane < 8 ? n - places(lane) : 0;
+    int over = max(surplus, 0), hole = max(-surplus, 0);  // then: of the classes before this lane's
+    const int holes = hole;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        const int a = __shfl_up_sync(PM_FULL_MASK, over, o), b = __shfl_up_sync(PM_FULL_MASK, hole, o);
+        if (lane >= o) {
+            over += a;
+            hole += b;
+        }
+    }
+    over -= max(surplus, 0);
+    hole -= holes;
+    // the position of hole x (x below the number of holes), all lanes together
+    auto hole_at = [&](int x) {
+        int pos = 0;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const int b = __shfl_sync(PM_FULL_MASK, hole, c), h = __shfl_sync(PM_FULL_MASK, holes, c);
+            const int k = __shfl_sync(PM_FULL_MASK, n, c) + x - b;
+            if (x >= b && x < b + h)
+                pos = 8 * k + first(c);
+        }
+        return pos;
+    };
+    const int near = hole_at(lane);  // the first 32 holes
+    int before = 0;                  // lane c: ids of class c in the words before
+    for (int base = 0; base < W; base += 32) {
+        uint32_t x = word(base + lane);
+        if (!__any_sync(PM_FULL_MASK, x != 0u))
+            continue;
+        const uint32_t all = x;
+        uint32_t c[2], incl[2];
+        by_class(x, c);  // at most 128 a class over the warp: bytes do
+        incl[0] = c[0];
+        incl[1] = c[1];
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(PM_FULL_MASK, incl, o);
-            if (lane >= o)
-                incl += y;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t y = __shfl_up_sync(PM_FULL_MASK, incl[h], o);
+                if (lane >= o)
+                    incl[h] += y;
+            }
         }
-        for (int pos = count + incl - n; x; ++pos) {
-            const uint16_t id = (uint16_t)(32 * w + __ffs(x) - 1);
-            x &= x - 1u;
-            if (pos < p)
+        while (__any_sync(PM_FULL_MASK, x != 0u)) {  // an id a lane
+            const int b = x ? __ffs(x) - 1 : 0, cl = b & 7;
+            const int sh = 8 * (cl & 3);
+            int k = __shfl_sync(PM_FULL_MASK, before, cl);
+            k += (int)((((cl & 4) ? incl[1] - c[1] : incl[0] - c[0]) >> sh) & 0xffu);
+            k += __popc(all & (0x01010101u << cl) & ((1u << b) - 1u));
+            int pos = 8 * k + first(cl);
+            const int extra = k - places(cl) + __shfl_sync(PM_FULL_MASK, over, cl);
+            const bool late = pos >= p;
+            const int to = __shfl_sync(PM_FULL_MASK, near, extra & 31);
+            if (late)
+                pos = to;
+            if (__any_sync(PM_FULL_MASK, x != 0u && late && extra >= 32)) {
+                const int far = hole_at(late ? extra : 0);
+                if (late)
+                    pos = far;
+            }
+            if (x) {
+                const uint16_t id = (uint16_t)(32 * (base + lane) + b);
                 reinterpret_cast<uint16_t *>(lists + (int64_t)(pos >> 1) * pitch + t)[pos & 1] = id;
-            if (pos == p - 1 && (p & 1))
-                reinterpret_cast<uint16_t *>(lists + (int64_t)(pos >> 1) * pitch + t)[1] = id;
+                if (pos == p - 1 && (p & 1))
+                    reinterpret_cast<uint16_t *>(lists + (int64_t)(pos >> 1) * pitch + t)[1] = id;
+                x &= x - 1u;
+            }
         }
-        count += __shfl_sync(PM_FULL_MASK, incl, 31);
+        const uint32_t t0 = __shfl_sync(PM_FULL_MASK, incl[0], 31), t1 = __shfl_sync(PM_FULL_MASK, incl[1], 31);
+        if (lane < 8)
+            before += (int)(((lane & 4 ? t1 : t0) >> (8 * (lane & 3))) & 0xffu);
     }
-    __syncwarp();
-    if (count != p && lane == 0)
-        lists[t] = kNoList;
 }
 
 __device__ __forceinline__ uint32_t min_u16x2(uint32_t a, uint32_t b)

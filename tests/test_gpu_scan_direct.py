@@ -155,3 +155,22 @@ def test_batches_of_both_ways(pm, monkeypatch, spec):
         alone.close()
     ga.close()
     batch.close()
+
+
+@pytest.mark.parametrize("m,p,ids", [(1500, 16, None), (1500, 17, None), (4000, 33, None), (4001, 60, None),
+                                     (4000, 33, "one class"), (4000, 45, "two classes"), (4000, 40, "last words")])
+def test_lists_ordered_for_the_banks(pm, m, p, ids):
+    """From 16 open facilities on the lists are ordered by the ids mod 8: random subsets, and subsets whose ids crowd a
+    class (most of them then fill holes) or a few words."""
+    n, pop = 700, 1100
+    rng = np.random.default_rng(m + p)
+    pool = {None: np.arange(m), "one class": np.arange(5, m, 8), "two classes": np.arange(m)[np.arange(m) % 8 < 2],
+            "last words": np.arange(m - 64, m)}[ids]
+    masks = np.zeros((pop, (m + 31) // 32), dtype=np.uint32)
+    for t in range(pop):
+        for j in rng.choice(pool if t % 3 else np.arange(m), size=p, replace=False):
+            masks[t, j >> 5] |= np.uint32(1) << np.uint32(j & 31)
+    d = _distances(n, m, 65535, seed=p)
+    inst = pm.Instance(d, p)
+    np.testing.assert_array_equal(inst.eval(masks), oracle.eval_direct(d, masks))
+    inst.close()
