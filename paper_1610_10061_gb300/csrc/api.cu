@@ -418,7 +418,7 @@ extern "C" pm_status pm_columns_layout(pm_instance *inst, int64_t pop, int32_t *
     if (!inst || pop < 1)
         return PM_ERR_INVALID_ARG;
     std::lock_guard<std::mutex> guard(inst->lock);
-    const pm_eval_plan plan = pm_plan_eval(inst, pop);
+    const pm_eval_plan plan = pm_plan_columns(inst, pop);
     if (groups)
         *groups = plan.groups;
     if (words)
@@ -434,7 +434,7 @@ extern "C" pm_status pm_population_columns(pm_instance *inst, const uint32_t *ma
         return PM_ERR_INVALID_ARG;
     std::lock_guard<std::mutex> guard(inst->lock);
     PM_CUDA(cudaSetDevice(inst->device));
-    return pm_launch_columns(inst, pm_plan_eval(inst, pop), masks, pop, cols, static_cast<cudaStream_t>(stream));
+    return pm_launch_columns(inst, pm_plan_columns(inst, pop), masks, pop, cols, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" pm_status pm_eval_columns(pm_instance *inst, const uint32_t *cols, int64_t pop, int64_t *costs,
@@ -446,10 +446,9 @@ extern "C" pm_status pm_eval_columns(pm_instance *inst, const uint32_t *cols, in
     std::lock_guard<std::mutex> guard(inst->lock);
     PM_CUDA(cudaSetDevice(inst->device));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    pm_eval_plan plan = pm_plan_eval(inst, pop);
+    const pm_eval_plan plan = pm_plan_columns(inst, pop);
     if (!plan.groups)
         return PM_ERR_UNSUPPORTED;
-    plan.direct = pm_direct_plan();  // the caller's form is the scan's
     bool fresh = false;
     PM_TRY(inst->partials.reserve(pm_plan_partial_bytes(plan, pop), &fresh));
     if (fresh)  // accumulators start at zero; launches leave them zero

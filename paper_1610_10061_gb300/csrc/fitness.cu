@@ -13,22 +13,22 @@
 //    G words of facility j (128 bits for G = 4) tests 32G individuals.
 //  * Work items are (client split, tile) pairs, split-major, walked by a
 //    persistent grid so that CTAs running at the same time stream the same
-//    rows through L2.  A CTA brings its tile's 32W x G words into shared
-//    memory with TMA bulk copies (cp.async.bulk + mbarrier, bounded wait)
-//    and keeps them while consecutive items share the tile.
-//  * A warp takes one client at a time and walks its row 32 ranks per step:
-//    lane r holds Pi'[r] and Delta'[r] (coalesced loads, the next step and
-//    the next client's first step prefetched into registers).  If no still
-//    active individual of the tile has facility Pi'[r] open at any lane, the
-//    step only adds the 32 increments to a running carry (one warp
-//    reduction).  Otherwise a warp scan turns the increments into running
-//    sums (the sum of Delta' up to rank r), and each group with hits
-//    resolves its individuals' first open ranks: with few hit lanes by
-//    walking those lanes in rank order, else by transposing the 32 x 32 bit
-//    block (rank x individual) with five shuffles so lane b finds its
-//    individual's first open rank with one find-first-set.  Resolved
-//    individuals leave the active set; the walk ends when none is left.
-//  * Per-lane int64 sums are combined in shared memory.  With one client
+//    rows through L2; large launches give every CTA an even share of the
+//    units of 1024 (individual, client) pairs instead, in one wave.  A CTA
+//    brings its tile's 32W x G words into shared memory with TMA bulk copies
+//    (cp.async.bulk + mbarrier, bounded wait) and keeps them while
+//    consecutive items share the tile.
+//  * A client's first open ranks are found in one of four ways (ScanKind):
+//      sliced   a lane per client, the 32 individuals of a word at once
+//               (scan_tile.cuh): large launches;
+//      split    eight lanes share a client's ranks (scan_split.cuh): launches
+//               too small to fill the chip with units;
+//      direct   the smallest of the open facilities' distances in place of
+//               the ranks (scan_direct.cuh): few open facilities;
+//      clients  a warp per client, 32 ranks a step (scan_walk.cuh): where the
+//               others' tables or 32-bit sums do not fit.
+//    mixed: a batch whose instances take sliced and direct.
+//  * The lanes' sums are combined in shared memory.  With one client
 //    split the CTA applies the epilogue itself.  Otherwise each split adds
 //    its sum and a count of one into a single 64-bit word per individual
 //    (sum in bits 0..47, count above); the split whose atomic completes the
@@ -991,6 +991,12 @@ pm_eval_plan pm_plan_eval_with(const pm_instance *inst, int64_t pop, int G, int 
     return plan;
 }
 
+// The heuristic's warps per CTA for tiles of G groups: two CTAs per SM where the bit-sliced walk's tiles leave room.
+static int column_warps(const pm_instance *inst, int64_t pop, int G)
+{
+    return sliced_pays(inst, pop) && 2 * column_smem_bytes(inst->W, G) + 8192 <= inst->smem_optin ? 16 : 32;
+}
+
 pm_eval_plan pm_plan_eval(const pm_instance *inst, int64_t pop)
 {
     {
@@ -1008,10 +1014,15 @@ pm_eval_plan pm_plan_eval(const pm_instance *inst, int64_t pop)
     int G = sliced ? kMaxG : (inst->n <= 128 ? 1 : 2);
     while (G > 1 && (pop <= (int64_t)32 * (G / 2) || column_smem_bytes(inst->W, G) > budget))
         G /= 2;
-    const int warps = sliced && 2 * column_smem_bytes(inst->W, G) + 8192 <= inst->smem_optin ? 16 : 32;
-    pm_eval_plan plan = pm_plan_eval_with(inst, pop, G, warps, 0);
+    pm_eval_plan plan = pm_plan_eval_with(inst, pop, G, column_warps(inst, pop, G), 0);
     pm_plan_direct(inst, pop, plan);
     return plan;
+}
+
+pm_eval_plan pm_plan_columns(const pm_instance *inst, int64_t pop)
+{
+    const pm_eval_plan plan = pm_plan_eval(inst, pop);
+    return plan.direct.range ? pm_plan_eval_with(inst, pop, plan.groups, column_warps(inst, pop, plan.groups), 0) : plan;
 }
 
 bool pm_plan_direct(const pm_instance *inst, int64_t pop, pm_eval_plan &plan)
@@ -1145,9 +1156,7 @@ pm_status pm_launch_columns(const pm_instance *inst, const pm_eval_plan &plan, c
         return PM_OK;
     if (plan.groups == 0)
         return PM_ERR_UNSUPPORTED;
-    pm_eval_plan columns = plan;
-    columns.direct = pm_direct_plan();
-    return launch_transpose(masks, nullptr, 1, pm_single_prob(inst, columns, pop),
+    return launch_transpose(masks, nullptr, 1, pm_single_prob(inst, plan, pop),
                             plan.tiles * plan.groups * inst->W, plan.groups, colT, stream);
 }
 

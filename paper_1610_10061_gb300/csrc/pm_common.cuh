@@ -198,6 +198,8 @@ struct pm_instance {
 // Choose the tile configuration for `pop` individuals on `inst` (the tuned
 // plan if the autotuner has run for this size, else a heuristic).
 pm_eval_plan pm_plan_eval(const pm_instance *inst, int64_t pop);
+// The plan of an evaluation from the facility-major form: pm_plan_eval's tiles, never by open facilities.
+pm_eval_plan pm_plan_columns(const pm_instance *inst, int64_t pop);
 // A plan with explicit groups (0 = row kernel), warps per CTA and client
 // splits (0 = one full wave).
 pm_eval_plan pm_plan_eval_with(const pm_instance *inst, int64_t pop, int G, int warps, int splits_hint);
