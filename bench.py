@@ -208,10 +208,11 @@ def measured_bf16_peak():
 
 def scan_source_text(read):
     """The code of the scan kernel k_scan_columns: its region of fitness.cu (from the epilogue arguments to the row
-    kernel), the client walk (scan_walk.cuh) and the bit transpose of pm_common.cuh.  read(name) returns a source
-    file's text."""
+    kernel), the walks (scan_walk.cuh, scan_tile.cuh, scan_split.cuh, scan_direct.cuh) and the bit transpose of
+    pm_common.cuh.  read(name) returns a source file's text."""
     fit = read("fitness.cu")
-    parts = [fit[fit.index("struct ScanEpilogue {"):fit.index("// Row kernel (fallback")], read("scan_walk.cuh")]
+    parts = [fit[fit.index("struct ScanEpilogue {"):fit.index("// Row kernel (fallback")]]
+    parts += [read(f"scan_{walk}.cuh") for walk in ("walk", "tile", "split", "direct")]
     common = read("pm_common.cuh")
     i = common.index("__device__ __forceinline__ uint32_t pm_transpose32")
     parts.append(common[i:common.index("\n}\n", i) + 3])
@@ -832,7 +833,8 @@ def eval_pass_record(pm, torch, name, tables="delta", steps=None, warmup=3, budg
     alg_bytes = pop * (n * ek * 6 + W * 4 + 8)
     peak, peak_kind = measured_peaks()
     scan_ms = time_scan_alone(pm, torch, inst, dmask, pop, dcost, flush, stream, 20)
-    kernel_ms = scan_ms if scan_ms is not None else mean_ms
+    # a pass shorter than the scan of the facility-major form evaluates by open facilities: its launch is not timed apart
+    kernel_ms = scan_ms if scan_ms is not None and scan_ms <= mean_ms else mean_ms
     achieved = alg_bytes / (kernel_ms / 1000) / 1e9
     traffic = profiled_traffic(name)
     inst.close()
@@ -847,10 +849,10 @@ def eval_pass_record(pm, torch, name, tables="delta", steps=None, warmup=3, budg
                         "launch_ms": kernel_ms, "pass_ms": mean_ms, "alg_bytes_per_launch": alg_bytes,
                         "peak_source": f"{peak_kind} burst copy bandwidth",
                         "note": "achieved = algorithmic bytes (pop * (n*(m+1)/(p+1)*6 + 4W + 8), the Pi'/Delta' "
-                                "prefix every evaluation scans) / the scan kernel's live launch time; each row "
-                                "chunk a CTA stages serves 128 individuals, so this exceeds the DRAM bytes moved "
-                                "(traffic, ncu, committed summary of this source), whose own fraction of the peak "
-                                "is traffic_frac"},
+                                "prefix every evaluation scans) / the scan kernel's live launch time (the pass's where it "
+                                "is evaluated by open facilities); what a CTA stages serves its whole tile or "
+                                "range of individuals, so this exceeds the DRAM bytes moved (traffic, ncu, committed "
+                                "summary of this source), whose own fraction of the peak is traffic_frac"},
            "roofline_issue": issue_roofline(name, kernel_ms), "clocks": clk, "l2": "flushed between timed steps"}
     if tables_rec is not None:
         rec["tables_build"] = tables_rec

@@ -237,7 +237,9 @@ PM_API pm_status pm_eval_columns(pm_instance *inst, const uint32_t *cols, int64_
  * runs one thread per chromosome).  Candidates: facility-major tiles of
  * 32, 64 or 128 individuals per CTA (groups = 1, 2, 4; those whose tile fits
  * in shared memory), 8, 16 or 32 warps per CTA, and client splits around the
- * one-wave default (x1/2, x1, x2); the row kernel with bitsets and with byte
+ * one-wave default (x1/2, x1, x2) as well as the default's even shares; the
+ * evaluation by open facilities where the instance keeps its distances in 16
+ * bits (reported with the shape it stands beside); the row kernel with bitsets and with byte
  * masks (one byte per facility, where 8 warps' masks fit in shared memory).  Each
  * candidate evaluates a uniformly random population (Floyd sampling, fixed
  * seed) once untimed, then five times eight back-to-back evaluations timed
@@ -287,9 +289,11 @@ PM_API pm_status pm_selftest_bounded_wait(int device, void *stream);
  * paper).  After `after` more successful device allocations by this library,
  * the next one fails on the host, without calling CUDA, and the call that
  * made it returns PM_ERR_OOM having launched nothing on that memory and
- * freed what it had obtained (one exception: a GA that cannot get the
- * buffers of the speculative mutation cycle runs the cycle try by try, with
- * the same results, instead of failing); the injection then disarms itself.
+ * freed what it had obtained (two exceptions: a GA that cannot get the
+ * buffers of the speculative mutation cycle runs the cycle try by try, and a
+ * large instance that cannot get the room of its optional 16-bit distances
+ * does without them, both with the same results, instead of failing); the
+ * injection then disarms itself.
  * A negative `after` disarms it (the default).  pending (host, nullable)
  * receives the allocations that were still to succeed before the failure
  * armed until now, or -1 if none was armed or it has happened.
@@ -409,7 +413,11 @@ typedef struct pm_model pm_model;
  * environment, such a GA with Floyd generation and no model runs all the
  * generations of a pm_ga_step call in one cooperative persistent launch,
  * its phases separated by grid-wide barriers (bounded: PM_ERR_TIMEOUT after
- * 4 s); the populations are the same.
+ * 4 s); the populations are the same.  A small instance (n x m up to about
+ * 100,000 with few open facilities, distances below 2^16) with Floyd
+ * generation, no model and demes of at most 512 runs a generation as one
+ * kernel, a cluster of CTAs per deme (PM_GA_DEME=0 or PM_GA_SPEC=0 in the
+ * environment keep the phases; the populations are the same).
  * Errors: PM_ERR_INVALID_ARG, PM_ERR_OOM, PM_ERR_CUDA; PM_ERR_UNSUPPORTED for
  * PM_GA_INIT_COMBINADIC beyond its limits.
  */
