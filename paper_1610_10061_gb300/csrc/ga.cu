@@ -2214,7 +2214,9 @@ __global__ void __launch_bounds__(1024, 1) k_ga_deme(ga_prob gp, const uint16_t 
         __syncwarp();
         if (!stall)  // a launch armed by pm_debug_scan_timeout issues none: the wait below runs out
             for (int o = lane; o < n8; o += 32)
-                bulk_g2s(dsm + (size_t)o * pitch * 16, dense + (size_t)o * m * 8, (uint32_t)m * 16u, &bar);
+                for (int j = 0; j < m; j += 2048)  // at most 32 KB a copy
+                    bulk_g2s(dsm + ((size_t)o * pitch + j) * 16, dense + ((size_t)o * m + j) * 8,
+                             (uint32_t)min(m - j, 2048) * 16u, &bar);
     }
     __syncthreads();
     pm_grid_dependency_wait();

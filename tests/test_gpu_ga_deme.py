@@ -32,6 +32,7 @@ CASES = [  # n x m, p, GA parameters
     (100, 100, 8, dict(pop=1024, deme=512)),
     (264, 65, 2, dict(pop=6, deme=2)),
     (8, 4, 1, dict(pop=4096, deme=2)),
+    (5, 7001, 3, dict(pop=64, deme=64)),
 ]
 
 
