@@ -1006,15 +1006,28 @@ pm_eval_plan pm_plan_eval(const pm_instance *inst, int64_t pop)
             return it->second;
     }
     const size_t budget = inst->smem_optin > 4096 ? inst->smem_optin - 4096 : 0;
-    // the bit-sliced walk: the widest tile the population fills.  Smaller launches (rank-split walk): 32 warps a CTA
-    // and tiles of 64 -- graph900's generation, pop 1024, 157 us against 162 with tiles of 128 -- or of 32 where one
-    // round of a CTA's warps then covers all clients, which saves the sums' way through global memory (graph100's
-    // generation 77 us against 82)
+    // the bit-sliced walk: the widest tile the population fills
     const bool sliced = sliced_pays(inst, pop);
     int G = sliced ? kMaxG : (inst->n <= 128 ? 1 : 2);
     while (G > 1 && (pop <= (int64_t)32 * (G / 2) || column_smem_bytes(inst->W, G) > budget))
         G /= 2;
-    pm_eval_plan plan = pm_plan_eval_with(inst, pop, G, column_warps(inst, pop, G), 0);
+    int warps = column_warps(inst, pop, G);
+    if (!sliced && inst->n > 128) {
+        // The rank-split walk: one round of four clients a warp (tiles of 32), by as few warps a CTA as leave at most a
+        // CTA per SM, since a warp's chain is shorter with fewer beside it; 16 where walks are short, so that the CTAs'
+        // fixed parts are fewer.  Scans alone, us, with 8 / 16 warps and with tiles of 64 and 32: 496 nodes, p = 7, 256
+        // individuals 7.3 / 8.9 / 11.7; 2000 points, p = 20, 64 individuals 12.2 / 14.2 / 18.0.  Generations: 496 nodes, p =
+        // 40, 256 individuals 110 / 106 / 116; graph900, 256 individuals 130 / 116 / 123.  Launches of more than a round for
+        // every SM take 32 warps and tiles of 64: graph900, 1024 individuals, 7.8 us a scan, 9.0 with 16.
+        auto one_wave = [&](int w) { return pm_ceil_div(pop, 32) * pm_ceil_div(inst->n, (int64_t)w * 4) <= inst->sm_count; };
+        const bool deep = inst->m + 1 > 20 * (inst->p + 1);
+        if (one_wave(16)) {
+            G = 1;
+            warps = deep && one_wave(8) ? 8 : 16;
+        }
+    }
+    // (up to 128 clients one round of 32 warps covers them all, which saves the sums' way through global memory)
+    pm_eval_plan plan = pm_plan_eval_with(inst, pop, G, warps, 0);
     pm_plan_direct(inst, pop, plan);
     return plan;
 }
