@@ -318,6 +318,20 @@ PM_API pm_status pm_debug_fail_alloc(int64_t after, int64_t *pending);
  */
 PM_API pm_status pm_debug_scan_timeout(int64_t launches, int64_t *pending);
 
+/*
+ * pm_debug_scan_launches -- which way the scan launches took (for tests; no
+ * counterpart in the paper): every way gives the same costs, so results alone
+ * do not show it.  counts (host, PM_SCAN_COUNTS values) receives the launches
+ * enqueued since the library was loaded, by any call (those captured into a
+ * GA's graph count once): the row kernel, the client walk, the rank-split
+ * walk, the bit-sliced walk, the evaluation by open facilities, a batch of
+ * both of the last two, and, of all these, the ones whose CTAs took the shares
+ * a batch was divided into.  Always PM_OK (PM_ERR_INVALID_ARG for a null
+ * pointer).
+ */
+#define PM_SCAN_COUNTS 7
+PM_API pm_status pm_debug_scan_launches(int64_t *counts);
+
 /* ------------------------------------------------------------------------
  * The Hammer-Beresnev polynomial (Section 2.1, Eq. 6, Example 1): a second
  * evaluator of the same costs, for small instances and for checking.

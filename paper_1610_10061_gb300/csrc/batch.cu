@@ -256,9 +256,9 @@ void pm_scan_launch_from(const pm_multi_plan &mp, const pm_prob *probs_dev, pm_s
     L.split = mp.split;
     L.Wmax = mp.Wmax;
     L.d_smem = mp.d_smem;
-    L.shares = L.K > 1 ? (int64_t)mp.shares.size() : 0;
     L.grid = mp.grid;
     L.K = (int)mp.probs.size();
+    L.shares = L.K > 1 ? (int64_t)mp.shares.size() : 0;
     L.one = mp.probs[0];
     L.probs_dev = L.K > 1 ? probs_dev : nullptr;
     L.items = mp.items;

@@ -293,7 +293,7 @@ __device__ __noinline__ void tile_walk_call(const pm_prob &pr, uint32_t *smem, u
 
 // What a launch's work items are: scanned client by client, rank-split or bit-sliced, evaluated by open facilities, or
 // (several instances) bit-sliced and by open facilities.
-enum class ScanKind { clients, split, sliced, direct, mixed };
+enum class ScanKind { clients, split, sliced, direct, mixed };  // in the order of pm_debug_scan_launches
 
 // ---------------------------------------------------------------------------
 // The column scan kernel (with the split reduction and epilogue fused), over
@@ -1150,6 +1150,20 @@ extern "C" pm_status pm_debug_scan_timeout(int64_t launches, int64_t *pending)
     return PM_OK;
 }
 
+// Scan launches enqueued so far (pm_debug_scan_launches): the row kernel, then by ScanKind, then those over shares.
+static std::atomic<long long> g_scan_launches[PM_SCAN_COUNTS];
+
+static void count_launch(int slot) { g_scan_launches[slot].fetch_add(1, std::memory_order_relaxed); }
+
+extern "C" pm_status pm_debug_scan_launches(int64_t *counts)
+{
+    if (!counts)
+        return PM_ERR_INVALID_ARG;
+    for (int k = 0; k < PM_SCAN_COUNTS; ++k)
+        counts[k] = (int64_t)g_scan_launches[k].load();
+    return PM_OK;
+}
+
 // Enqueue the transpose (unless the caller wrote the columns) and the column
 // scan of a launch; smem = the tile bytes of the launch's widest instance.
 static pm_status launch_transpose(const uint32_t *masks, const pm_prob *probs, int K, const pm_prob &one, int64_t jobs,
@@ -1197,6 +1211,9 @@ pm_status pm_launch_scan(const pm_scan_launch &L, const pm_accept_args &acc, int
                                         : (L.K == 1 ? ScanKind::direct : ScanKind::mixed);
     PM_CUDA(pm_launch(scan_fn(G, kind), grid, threads, smem, stream, L.probs_dev, L.K, L.one, L.items, L.colT,
                       L.masks, L.active, accum, L.tickets, L.err, ep, stall, L.nb, tab_off, L.shares));
+    count_launch(1 + (int)kind);
+    if (L.shares > 0)
+        count_launch(PM_SCAN_COUNTS - 1);
     return PM_OK;
 }
 
@@ -1235,6 +1252,7 @@ pm_status pm_launch_eval(const pm_instance *inst, const pm_eval_plan &plan, cons
     ep.cur_masks = acc.cur_masks;
     ep.cand_masks = acc.cand_masks;
     ep.improved = acc.improved;
+    count_launch(0);
     const int64_t cps = pm_ceil_div(inst->n, plan.splits);
     const size_t smem = (size_t)plan.warps * inst->W * 4 * (plan.bytes ? 8 : 1);
     dim3 grid((unsigned)plan.tiles, (unsigned)plan.splits);

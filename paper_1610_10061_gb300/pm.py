@@ -73,6 +73,7 @@ _SIGS = {
     "pm_selftest_bounded_wait": ([ctypes.c_int, _P], _S),
     "pm_debug_fail_alloc": ([_I64, _P], _S),
     "pm_debug_scan_timeout": ([_I64, _P], _S),
+    "pm_debug_scan_launches": ([_P], _S),
     "pm_eval_status": ([_P, _P], _S),
     "pm_columns_layout": ([_P, _I64, _P, _P], _S),
     "pm_population_columns": ([_P, _P, _I64, _P, _P], _S),
@@ -234,6 +235,14 @@ def pm_debug_scan_timeout(launches: int) -> int:
     pending = ctypes.c_int64(0)
     _check(_lib.pm_debug_scan_timeout(int(launches), ctypes.byref(pending)), "pm_debug_scan_timeout")
     return int(pending.value)
+
+
+def pm_debug_scan_launches() -> dict:
+    """Scan launches enqueued since the library was loaded, by the way they took."""
+    names = ("rows", "clients", "split", "sliced", "direct", "mixed", "shares")
+    counts = (ctypes.c_int64 * len(names))()
+    _check(_lib.pm_debug_scan_launches(counts), "pm_debug_scan_launches")
+    return dict(zip(names, counts))
 
 
 def pm_eval_status(inst, stream=None) -> int:
