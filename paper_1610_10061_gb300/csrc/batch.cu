@@ -41,7 +41,18 @@ static void plan_shares(pm_multi_plan &out, const std::vector<double> &work, int
             const int64_t unit = pr.d_range ? 8 * pr.d_chunks : 32 / out.groups;
             const int64_t units = pm_ceil_div(pr.n, unit), step = pr.d_range ? 1 : warps;
             const double cost = work[k] / (double)(pr.tiles * units);
-            for (int64_t tile = 0; tile < pr.tiles; ++tile) {
+            const int64_t most = pr.d_range ? 65536 / unit : units;  // 32-bit sums: 2^16 clients of distances below 2^16
+            const double whole = kShareCycles + cost * (double)units;
+            for (int64_t tile = 0; tile < pr.tiles;) {
+                // the tiles that this CTA takes whole, all at once: a launch has many more tiles than CTAs
+                const int64_t run = most < units ? 0 : std::min(pr.tiles - tile, (int64_t)std::max(0.0, (cap - load) / whole));
+                if (run > 0) {
+                    for (int64_t i = 0; write && i < run; ++i)
+                        out.shares.push_back(pm_share{k, 1, tile + i, 0, pr.n});
+                    load += whole * (double)run;
+                    tile += run;
+                    continue;
+                }
                 const size_t first = out.shares.size();
                 for (int64_t u = 0; u < units;) {
                     int64_t take = (int64_t)((cap - load - kShareCycles) / cost);
@@ -52,9 +63,7 @@ static void plan_shares(pm_multi_plan &out, const std::vector<double> &work, int
                             out.share_base.push_back((int32_t)out.shares.size());
                         continue;
                     }
-                    take = std::min(units - u, std::max<int64_t>(take / step, 1) * step);
-                    if (pr.d_range)  // 32-bit sums: 2^16 clients of distances below 2^16
-                        take = std::min<int64_t>(take, 65536 / unit);
+                    take = std::min({units - u, std::max<int64_t>(take / step, 1) * step, most});
                     if (write)
                         out.shares.push_back(pm_share{k, 0, tile, u * unit, std::min(pr.n, (u + take) * unit)});
                     load += kShareCycles + cost * (double)take;
@@ -63,6 +72,7 @@ static void plan_shares(pm_multi_plan &out, const std::vector<double> &work, int
                 if (write)
                     for (size_t i = first; i < out.shares.size(); ++i)
                         out.shares[i].splits = (int32_t)(out.shares.size() - first);
+                ++tile;
             }
         }
         if (load > 0.0) {
