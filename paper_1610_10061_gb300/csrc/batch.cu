@@ -108,30 +108,54 @@ pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std
     out = pm_multi_plan();
     out.groups = G;
     const pm_instance *i0 = insts[0];
-    double depth = 0.0;
-    int64_t units = 0;  // units of 1024 pairs
+    const size_t budget = i0->smem_optin > 4096 ? i0->smem_optin - 4096 : 0;
+    // the instances that are evaluated by open facilities where the launch is divided into shares.  Few individuals do not
+    // pay for the lists (written by every GA operator) and the chunks' copies: 48 uneven instances, pop 256: evaluation
+    // 131 us against 134 without, generation 2.67 against 2.53 ms; pop 1024: evaluation 352 against 460 us
+    std::vector<pm_direct_plan> direct(K);
+    int64_t units = 0;              // units of 1024 pairs
+    double depth = 0.0, ranks = 0.0;  // deepest walk; ranks of all units' walks (by open facilities: what takes as long)
     for (int k = 0; k < K; ++k) {
         const pm_instance *in = insts[k];
         out.Wmax = std::max(out.Wmax, in->W);
-        depth = std::max(depth, pm_walk_depth(in->m, in->p, in->L));
-        units += pm_ceil_div(pops[k], 32) * pm_ceil_div(in->n, 32);
+        if (pops[k] >= 512)
+            pm_direct_shape(in, pops[k], budget, std::min(warps, 16), direct[k]);
+        const int64_t u = pm_ceil_div(pops[k], 32) * pm_ceil_div(in->n, 32);
+        double walk = pm_walk_depth(in->m, in->p, in->L);
+        if (direct[k].range)
+            walk *= std::min(1.0, pm_direct_cost(in->m, in->p, direct[k].range, direct[k].stages) / pm_scan_cost(in->m, in->p));
+        else
+            depth = std::max(depth, walk);
+        units += u;
+        ranks += (double)u * walk;
     }
-    const size_t budget = i0->smem_optin > 4096 ? i0->smem_optin - 4096 : 0;
     if (tile_bytes(out.Wmax, G) > budget)
         return PM_ERR_UNSUPPORTED;
-    if (pm_sliced_pays(i0, units))
+    // The bit-sliced walk and the evaluation by open facilities, in shares of equal cost: from half as many units per SM
+    // on as one instance needs (pm_sliced_pays), if the shares' walks are not much shorter than the longest walk of one
+    // unit, a warp's chain that nothing shortens.  Evaluations, us, sliced and rank-split: 512 individuals of 2000 x 2000, p =
+    // 12, and 3000 x 1000, p = 5 (16 units per SM) 19 / 100; 256 of nine 900 x 900, p = 90 (13) 16 / 24; the shares' walks
+    // 0.37 of the longest 76 / 106; 0.26 of it 252 / 190; 40 of 900 x 900, p = 90, and one of 300 x 7000, p = 3 (31 units
+    // per SM, 0.04 of the longest) 253 / 148.
+    const bool sliced = K == 1 ? pm_sliced_pays(i0, units)
+                               : units >= (int64_t)i0->sm_count * 12 && ranks >= 0.35 * depth * 16.0 * i0->sm_count;
+    if (sliced)
         pm_walk_shape(i0, out.Wmax, G, depth, warps, out.nb);
     if (!out.nb) {
-        out.split = true;
-        for (const pm_instance *in : insts)
-            out.split = out.split && pm_split_fits(in, out.Wmax, G, warps);
-        if (out.split)
+        auto split_fits = [&](int w) {
+            return std::all_of(insts.begin(), insts.end(),
+                               [&](const pm_instance *in) { return pm_split_fits(in, out.Wmax, G, w); });
+        };
+        out.split = split_fits(warps);
+        if (out.split) {
             items_per_slot = 1;  // an item's fixed costs are most of a small launch
+            if (warps == 16 && 2 * (pm_scan_smem(out.Wmax, G, 16, 0, true) + 3072) > i0->smem_optin && split_fits(32))
+                warps = 32;  // the walk's tables leave room for one CTA per SM only
+        }
     }
     out.warps = warps;
     // scan work estimate per instance: tiles x clients x expected 32-rank steps of a 128-individual tile
     std::vector<double> work(K);
-    std::vector<pm_direct_plan> direct(K);
     double total = 0.0;
     for (int k = 0; k < K; ++k) {
         const pm_instance *in = insts[k];
@@ -139,14 +163,13 @@ pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std
         const double steps = 1.5 + pm_walk_depth(in->m, in->p, in->L) / 32.0;
         work[k] = tiles * (double)in->n * steps;
         if (out.nb) {  // in SM cycles per pair, the unit the two ways are compared in
-            // few individuals do not pay for the lists (written by every GA operator) and the chunks' copies: 48
-            // uneven instances, pop 256: evaluation 131 us against 134 without, generation 2.67 against 2.53 ms; pop
-            // 1024: evaluation 352 against 460 us
-            if (pops[k] >= 512)
-                pm_direct_shape(in, pops[k], budget, warps, direct[k]);
+            // (a scan's walk as pm_scan_cost has it, but never deeper than the rows)
+            const double mean = std::min((double)(in->m + 1) / (double)(in->p + 1), (double)in->L / 7.5);
             work[k] = (double)pops[k] * (double)in->n *
-                      (direct[k].range ? pm_direct_cost(in->m, in->p, direct[k].range, direct[k].stages) : pm_scan_cost(in->m, in->p));
+                      (direct[k].range ? pm_direct_cost(in->m, in->p, direct[k].range, direct[k].stages) : 0.35 + 0.037 * mean);
             out.d_smem = std::max(out.d_smem, direct[k].smem);
+        } else {
+            direct[k] = pm_direct_plan();
         }
         total += work[k];
     }
@@ -162,6 +185,17 @@ pm_status pm_plan_multi(const std::vector<const pm_instance *> &insts, const std
         slots_per_sm = std::min(slots_per_sm, by_regs);
     }
     const int64_t slots = (int64_t)i0->sm_count * slots_per_sm;
+    if (out.split) {
+        // One item a CTA, or two where the instance with the most work has deep walks and more than a round of them an item:
+        // they even out the walks' different lengths.  Evaluations, us, with one and two: 300 individuals of 2848 x 2848, p
+        // = 4, among four instances 137 / 114; 128 of 4832 x 6749, p = 4, among seven 264 / 191; but 256 of four 2000 x
+        // 2000, p = 20, and 100 x 6000, p = 6 84 / 102.
+        const int k = (int)(std::max_element(work.begin(), work.end()) - work.begin());
+        const double tiles = (double)pm_ceil_div(pops[k], 32 * G);
+        const double splits = std::max(1.0, std::ceil((double)slots * work[k] / total / tiles));
+        if ((double)insts[k]->n / splits > (double)(warps * (4 / G)) && pm_walk_depth(insts[k]->m, insts[k]->p, insts[k]->L) > 2048.0)
+            items_per_slot = 2;
+    }
     const double target_items = (double)slots * std::max(1, items_per_slot);
     int64_t ind = 0, words = 0, cols = 0, tiles_acc = 0, items = 0, jobs = 0;
     out.probs.resize(K);
@@ -322,14 +356,16 @@ static pm_status batch_plan(pm_batch *b, const std::vector<int64_t> &pops, int G
     return PM_OK;
 }
 
-static void default_shape(const pm_batch *b, int &G, int &warps, int &ips)
+// The shape for populations of at most `pop`: the widest tile that one of them fills more than half (lanes of empty
+// groups have no other work), two CTAs per SM where the tiles leave room.
+static void default_shape(const pm_batch *b, int64_t pop, int &G, int &warps, int &ips)
 {
     const size_t budget = b->insts[0]->smem_optin > 4096 ? b->insts[0]->smem_optin - 4096 : 0;
     int64_t Wmax = 0;
     for (auto *in : b->insts)
         Wmax = std::max<int64_t>(Wmax, in->W);
     G = 4;
-    while (G > 1 && tile_bytes(Wmax, G) > budget)
+    while (G > 1 && (tile_bytes(Wmax, G) > budget || pop <= 16 * G))
         G /= 2;
     warps = 2 * tile_bytes(Wmax, G) + 8192 > b->insts[0]->smem_optin ? 32 : 16;
     ips = 4;
@@ -377,7 +413,7 @@ static pm_status batch_eval_impl(pm_batch *b, const uint32_t *masks, const std::
         warps = b->tuned_warps;
         ips = b->tuned_ips;
     } else {
-        default_shape(b, G, warps, ips);
+        default_shape(b, *std::max_element(pops.begin(), pops.end()), G, warps, ips);
     }
     if (!b->have_plan || b->plan_pops != pops || b->plan_G != G || b->plan_warps != warps)
         PM_TRY(batch_plan(b, pops, G, warps, ips, s));
@@ -533,7 +569,7 @@ pm_status pm_batch_ga_plan(pm_batch *b, int64_t pop, pm_multi_plan &out)
         warps = b->tuned_warps;
         ips = b->tuned_ips;
     } else {
-        default_shape(b, G, warps, ips);
+        default_shape(b, pop, G, warps, ips);
     }
     PM_TRY(pm_plan_multi(b->insts, pv, G, warps, ips, out));
     for (auto &pr : out.probs)
@@ -542,7 +578,7 @@ pm_status pm_batch_ga_plan(pm_batch *b, int64_t pop, pm_multi_plan &out)
 }
 
 // The speculative mutation cycle's candidates of a batched GA: popQ = Q x pop per instance, planned with the
-// tile shape the GA's own scans use (tuned for pop, or the default); costs indexed like the GA's.
+// tile shape tuned for pop, or the default for theirs; costs indexed like the GA's.
 pm_status pm_batch_ga_plan_candidates(pm_batch *b, int64_t pop, int64_t popQ, pm_multi_plan &out)
 {
     std::vector<int64_t> pv(b->insts.size(), pop), pq(b->insts.size(), popQ);
@@ -552,7 +588,7 @@ pm_status pm_batch_ga_plan_candidates(pm_batch *b, int64_t pop, int64_t popQ, pm
         warps = b->tuned_warps;
         ips = b->tuned_ips;
     } else {
-        default_shape(b, G, warps, ips);
+        default_shape(b, popQ, G, warps, ips);
     }
     PM_TRY(pm_plan_multi(b->insts, pq, G, warps, ips, out));
     for (auto &pr : out.probs)
