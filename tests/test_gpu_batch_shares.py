@@ -65,6 +65,34 @@ def test_costs_equal_the_oracle(pm, name):
         inst.close()
 
 
+RULES = {  # shapes, individuals of each, the kind of launch, whether in shares
+    "from 12 units per SM on": ([(900, 850, 85, 3000)] * 9, 256, "sliced", 1),
+    "one deep walk among short ones": ([(700, 300, 30, 3000)] * 40 + [(290, 6000, 3, 3000)], 128, "split", 0),
+    "few units": ([(1000, 1000, 8, 60000), (400, 300, 9, 3000)], 64, "split", 0),
+    "populations of one word": ([(700, 200, 20, 500)] * 120, 32, "sliced", 1),
+}
+
+
+@pytest.mark.parametrize("name", RULES)
+def test_rule_for_the_way(pm, name):
+    shapes, pop, kind, shares = RULES[name]
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    units = sum(-(-pop // 32) * -(-s[0] // 32) for s in shapes)
+    assert units < 24 * sm and (units >= 12 * sm) == (name != "few units")
+    data = {s: _distances(s[0], s[1], s[3], seed=k) for k, s in enumerate(dict.fromkeys(shapes))}
+    insts = {s: pm.Instance(d, s[2]) for s, d in data.items()}
+    batch = pm.Batch([insts[s] for s in shapes])
+    masks = [random_masks(pop, s[1], s[2], seed=k) for k, s in enumerate(shapes)]
+    dev = torch.from_numpy(np.concatenate([mk.reshape(-1) for mk in masks]).view(np.int32)).cuda()
+    before = _routes(pm)
+    got = batch.eval(dev, [pop] * len(shapes)).cpu().numpy().reshape(len(shapes), pop)
+    taken = _routes(pm, before)
+    assert taken[kind] == 1 and taken["shares"] == shares, taken
+    for k in {0, 1, len(shapes) // 2, len(shapes) - 1}:
+        np.testing.assert_array_equal(got[k], oracle.eval_direct(data[shapes[k]], masks[k]))
+    batch.close()
+
+
 @pytest.mark.parametrize("spec", ["0", "1"])
 def test_ga_with_individuals_left_out(pm, monkeypatch, spec):
     """Children that are not evaluated (failed crossovers, mutation after an improvement) and instances that stop."""
