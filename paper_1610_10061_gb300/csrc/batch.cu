@@ -11,6 +11,7 @@
 #include <cmath>
 #include <cstring>
 #include <new>
+#include <numeric>
 #include <vector>
 
 #include "pm_common.cuh"
@@ -29,11 +30,15 @@ static constexpr double kShareCycles = 8000.0;
 static void plan_shares(pm_multi_plan &out, const std::vector<double> &work, int64_t slots, int warps)
 {
     const int K = (int)out.probs.size();
+    int64_t tiles = 0;
+    for (const pm_prob &pr : out.probs)
+        tiles += pr.tiles;
     auto fill = [&](double cap, bool write) {
         int64_t ctas = 0;
         double load = 0.0;
         if (write) {
             out.shares.clear();
+            out.shares.reserve((size_t)(tiles + 2 * slots));
             out.share_base.assign(1, 0);
         }
         for (int k = 0; k < K; ++k) {
@@ -48,7 +53,7 @@ static void plan_shares(pm_multi_plan &out, const std::vector<double> &work, int
                 const int64_t run = most < units ? 0 : std::min(pr.tiles - tile, (int64_t)std::max(0.0, (cap - load) / whole));
                 if (run > 0) {
                     for (int64_t i = 0; write && i < run; ++i)
-                        out.shares.push_back(pm_share{k, 1, tile + i, 0, pr.n});
+                        out.shares.push_back(pm_share{k, 1, tile + i, 0, pr.n, 0});
                     load += whole * (double)run;
                     tile += run;
                     continue;
@@ -65,7 +70,8 @@ static void plan_shares(pm_multi_plan &out, const std::vector<double> &work, int
                     }
                     take = std::min({units - u, std::max<int64_t>(take / step, 1) * step, most});
                     if (write)
-                        out.shares.push_back(pm_share{k, 0, tile, u * unit, std::min(pr.n, (u + take) * unit)});
+                        out.shares.push_back(pm_share{k, 0, tile, u * unit, std::min(pr.n, (u + take) * unit),
+                                                      (int64_t)(out.shares.size() - first)});
                     load += kShareCycles + cost * (double)take;
                     u += take;
                 }
@@ -82,12 +88,7 @@ static void plan_shares(pm_multi_plan &out, const std::vector<double> &work, int
         }
         return ctas;
     };
-    double total = 0.0;
-    int64_t tiles = 0;
-    for (int k = 0; k < K; ++k) {
-        total += work[k];
-        tiles += out.probs[k].tiles;
-    }
+    const double total = std::accumulate(work.begin(), work.end(), 0.0);
     double lo = total / (double)slots, hi = total + kShareCycles * (double)(tiles + 1) * 2.0 + 1.0;
     for (int it = 0; it < 40 && hi > lo * 1.002; ++it) {
         const double mid = 0.5 * (lo + hi);
@@ -275,10 +276,11 @@ void pm_multi_plan::write_table(char *dst) const
 pm_multi_plan pm_plan_from_single(const pm_instance *inst, const pm_eval_plan &plan, int64_t pop)
 {
     pm_multi_plan mp;
-    mp.groups = plan.groups;
+    const bool direct = plan.direct.range != 0;
+    mp.groups = direct ? plan.direct.groups : plan.groups;
     mp.warps = plan.warps;
-    mp.nb = plan.nb;
-    mp.split = plan.split;
+    mp.nb = direct ? plan.direct.nb : plan.nb;
+    mp.split = !direct && plan.split;
     mp.probs.push_back(pm_single_prob(inst, plan, pop));
     mp.items = mp.probs[0].tiles * mp.probs[0].splits;
     mp.grid = plan.direct.range ? mp.items : plan.grid;

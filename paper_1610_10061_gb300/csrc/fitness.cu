@@ -191,15 +191,155 @@ __device__ __forceinline__ bool wait_copies(uint64_t *bar, uint32_t phase, bool 
     return true;
 }
 
+// The bit-sliced walk as a function of its own: it needs all 128 registers, and inside the kernel's body every change
+// around it moved its speed by up to a tenth.
+template <int G>
+__device__ __noinline__ void tile_walk_call(const pm_prob &pr, uint32_t *smem, uint32_t tbl, int nb, uint32_t a0,
+                                            int64_t c_begin, int64_t c_end, unsigned long long *acc_s)
+{
+    const TileRows rows{pr.pi, pr.delta, pr.stride, pr.L, pr.cum != 0, pr.flush_units};
+    TileWalk<G> walk;
+    walk.prefetch(rows, c_begin, c_end, threadIdx.x >> 5, threadIdx.x & 31);
+    walk.run(smem, tbl, nb, a0, rows, c_begin, c_end, threadIdx.x >> 5, blockDim.x >> 5, threadIdx.x & 31, acc_s);
+}
+
+// What direct_left needs of its launch (the kernel's arguments).
+struct LeftLaunch {
+    const pm_prob *probs;
+    int K;
+    const pm_prob *one;
+    int64_t items;
+    const uint32_t *colT, *masks, *active;
+    unsigned long long *accum;
+    ScanEpilogue ep;
+    int nb;
+    uint32_t tab_off;
+    int64_t shares;
+};
+
+// The individuals without lists of the CTA's items by open facilities, after those: gathered 32 G at a time into a
+// facility-major tile that the bit-sliced walk is taken over, so that sets of other sizes than p cost what the scan costs
+// them.  The CTAs that share an item's individuals (each has other clients of them) divide the units of all these tiles
+// and clients evenly, as a bit-sliced launch does: an item's own clients would be far fewer than its warps walk at a time.
+// 4096 sets of 11 of 10000 x 10000, p = 10: 4.3 ms (the scan of all with a client a warp 5.1; a walk of its own for every
+// set and client 287).  Apart from the items' loop, where its registers would cost sets of p two to seven percent.
+// smem: all of the CTA's (at tab_off the walk's tables); acc, ids: 32 G; left: kDirectRange / 32.
+template <int G>
+__device__ __noinline__ void direct_left(const LeftLaunch &L, uint32_t *smem, unsigned long long *acc, uint32_t *left,
+                                         uint16_t *ids, pm_prob *pr_s, pm_share *share_s)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    constexpr uint16_t kOpenSum = 0x8000;  // in ids: the sum is not complete
+    const uint32_t tbl = L.tab_off + (uint32_t)(warp * tile_table_words(L.nb, G));
+    const pm_share *share_tab = reinterpret_cast<const pm_share *>(L.probs + L.K);
+    const bool shared = L.shares > 0;
+    const int32_t *base = reinterpret_cast<const int32_t *>(share_tab + L.shares) + blockIdx.x;
+    const int64_t last = shared ? base[1] : L.items, step = shared ? 1 : gridDim.x;
+    for (int64_t item = shared ? base[0] : blockIdx.x; item < last; item += step) {
+        __syncthreads();  // everybody is done with the item before
+        if (threadIdx.x == 0) {
+            if (shared) {
+                *share_s = share_tab[item];
+                *pr_s = L.probs[share_s->prob];
+            } else {
+                *pr_s = *L.one;
+                share_s->index = item / pr_s->tiles;
+                share_s->tile = item - share_s->index * pr_s->tiles;
+                share_s->splits = (int32_t)pr_s->splits;
+            }
+        }
+        __syncthreads();
+        const pm_prob &pr = *pr_s;
+        if (!pr.d_range)
+            continue;
+        const int W = pr.W, groups = pr.d_range / 32;
+        const int64_t ind0 = share_s->tile * pr.d_range;
+        int all = 0;
+        for (int g = warp; g < groups; g += nwarps) {
+            const int64_t t = ind0 + 32 * g + lane, tg = pr.ind_base + t;
+            const bool on = t < pr.pop && (L.active == nullptr || ((__ldg(L.active + (tg >> 5)) >> (tg & 31)) & 1u)) &&
+                            __ldg(L.colT + pr.col_base + t) == kNoList;
+            const uint32_t b = __ballot_sync(PM_FULL_MASK, on);
+            if (lane == 0)
+                left[g] = b;
+        }
+        __syncthreads();
+        for (int g = lane; g < groups; g += 32)
+            all += __popc(left[g]);
+        all = __reduce_add_sync(PM_FULL_MASK, all);
+        const int64_t per = (pr.n * G + 31) / 32, units = (all + 32 * G - 1) / (32 * G) * per;  // of a tile, of all
+        const int64_t ctas = max((int64_t)1, min((int64_t)share_s->splits, units / 4)), index = share_s->index;
+        const int64_t end = index < ctas ? (index + 1) * units / ctas : 0;
+        for (int64_t pos = index * units / ctas; pos < end;) {
+            const int64_t tile = pos / per, first = tile * per, stop = min(end, first + per);
+            const int shares = (int)(((first + per) * ctas - 1) / units - ((first + 1) * ctas - 1) / units + 1);
+            const int count = min(all - (int)tile * 32 * G, 32 * G);
+            if (warp == 0) {
+                int rank = -(int)tile * 32 * G;  // among the tile's individuals
+                for (int g = 0; g < groups && rank < count; ++g) {
+                    const uint32_t w = left[g];
+                    const int r = rank + __popc(w & ((1u << lane) - 1u));
+                    if (((w >> lane) & 1u) && r >= 0 && r < count)
+                        ids[r] = (uint16_t)(32 * g + lane);
+                    rank += __popc(w);
+                }
+            }
+            __syncthreads();
+            for (int job = warp; job < G * W; job += nwarps) {
+                const int g = job / W, w = job - g * W, i = 32 * g + lane;
+                const uint32_t x = i < count ? __ldg(L.masks + pr.word_base + (ind0 + ids[i]) * W + w) : 0u;
+                smem[(32 * w + lane) * G + g] = pm_transpose32(x, lane);
+            }
+            TileWalk<G>::clear_table(smem + tbl, L.nb, lane);
+            for (int i = threadIdx.x; i < 32 * G; i += blockDim.x)
+                acc[i] = 0ull;
+            __syncthreads();
+            const int mine = count - 32 * (lane % G);  // individuals of the lane's group
+            const uint32_t a0 = mine >= 32 ? ~0u : (mine > 0 ? (1u << mine) - 1u : 0u);
+            tile_walk_call<G>(pr, smem, tbl, L.nb, a0, (pos - first) * TileWalk<G>::kClients,
+                              min(pr.n, (stop - first) * TileWalk<G>::kClients), acc);
+            __syncthreads();
+            for (int i = threadIdx.x; shares > 1 && i < count; i += blockDim.x) {
+                unsigned long long *sum = L.accum + pr.ind_base + ind0 + ids[i];
+                const unsigned long long add = acc[i] + (1ull << kCountShift), old = atomicAdd(sum, add);
+                if ((old >> kCountShift) == (unsigned long long)(shares - 1)) {
+                    acc[i] = (old + add) & ((1ull << kCountShift) - 1ull);
+                    *sum = 0ull;
+                } else {
+                    ids[i] |= kOpenSum;
+                }
+            }
+            __syncthreads();
+            for (int i = warp; i < count; i += nwarps) {
+                if (ids[i] & kOpenSum)
+                    continue;
+                const int64_t t = ind0 + ids[i], sum = (int64_t)acc[i];
+                if (L.ep.costs != nullptr && lane == 0)
+                    L.ep.costs[pr.out_base + t] = sum;
+                if (L.ep.mode == 1 && sum < L.ep.cur_cost[pr.ind_base + t]) {
+                    for (int w = lane; w < W; w += 32)
+                        L.ep.cur_masks[pr.word_base + t * W + w] = L.ep.cand_masks[pr.word_base + t * W + w];
+                    if (lane == 0) {
+                        L.ep.cur_cost[pr.ind_base + t] = sum;
+                        if (L.ep.improved)
+                            L.ep.improved[pr.ind_base + t] = 1;
+                    }
+                }
+            }
+            __syncthreads();
+            pos = stop;
+        }
+    }
+}
+
 // One work item of the evaluation by open facilities.
 struct DirectItem {
     uint32_t *smem;                       // the entries (d_chunks per stage), then the sums and the bit words
     const uint32_t *__restrict__ lists;   // of the instance
-    const uint32_t *__restrict__ masks;   // rows of the launch
     int64_t ind0;                         // individuals ind0 .. ind0 + count - 1 of the instance
     int count;
-    const uint32_t *a0;                   // the ones to evaluate
-    uint32_t *fast;                       // scratch, count / 32 words
+    uint32_t *a0;                         // the ones to evaluate; direct_item leaves the ones with lists
+    int *left;                            // set to 1 when there were others (direct_left evaluates them)
     uint32_t *sums;                       // count 64-bit sums, zero on entry
     int64_t c_begin, c_end;
     uint64_t *bar;                        // one per stage
@@ -223,16 +363,16 @@ __device__ __forceinline__ uint32_t direct_item(const pm_prob &pr, const DirectI
     const int groups = (int)((min((int64_t)it.count, pr.pop - it.ind0) + 31) / 32);
     const uint32_t pitch = (uint32_t)((pr.pop + 31) / 32 * 32);
     const uint32_t *lists = it.lists + it.ind0;
-    bool mine = false;  // a bitset without a list among this warp's
     for (int g = warp; g < groups; g += nwarps) {
         const uint32_t a0 = it.a0[g];
         const bool listed = ((a0 >> lane) & 1u) && __ldg(lists + 32 * g + lane) != kNoList;
         const uint32_t b = __ballot_sync(PM_FULL_MASK, listed);
-        mine |= b != a0;
-        if (lane == 0)
-            it.fast[g] = b;
+        if (lane == 0 && b != a0) {
+            it.a0[g] = b;
+            *it.left = 1;
+        }
     }
-    const bool unlisted = __syncthreads_or(mine) != 0;
+    __syncthreads();
     const int64_t all = (it.c_end - it.c_begin + 7) / 8;  // chunks of the item
     const uint32_t ent = smem_u32(it.smem), stage_bytes = (uint32_t)(pr.d_chunks * pr.m) * 16u;
     int stage = 0;
@@ -247,10 +387,10 @@ __device__ __forceinline__ uint32_t direct_item(const pm_prob &pr, const DirectI
         phases ^= 1u << stage;
         const int chunks = (int)min(all - c8, (int64_t)pr.d_chunks);
         if (chunks * groups >= 2 * nwarps)  // two individuals per lane as long as every warp has a task
-            direct_terms<2>(pr, ent + stage * stage_bytes, chunks, lists, pitch, groups, it.fast, it.sums, warp, nwarps,
+            direct_terms<2>(pr, ent + stage * stage_bytes, chunks, lists, pitch, groups, it.a0, it.sums, warp, nwarps,
                             lane);
         else
-            direct_terms<1>(pr, ent + stage * stage_bytes, chunks, lists, pitch, groups, it.fast, it.sums, warp, nwarps,
+            direct_terms<1>(pr, ent + stage * stage_bytes, chunks, lists, pitch, groups, it.a0, it.sums, warp, nwarps,
                             lane);
         __syncthreads();
         if (pr.d_stages == 2)
@@ -258,18 +398,6 @@ __device__ __forceinline__ uint32_t direct_item(const pm_prob &pr, const DirectI
         else if (next_chunks > 0 && threadIdx.x == 0 && !it.stalled)
             direct_fill(pr, it.smem, it.c_begin / 8 + next, next_chunks, &it.bar[0]);
     }
-    if (!unlisted)
-        return phases;
-    for (int i = 0; i < 32 * groups; ++i) {
-        if (!(((it.a0[i >> 5] & ~it.fast[i >> 5]) >> (i & 31)) & 1u))
-            continue;
-        unsigned long long sum = 0ull;
-        for (int64_t c = it.c_begin + warp; c < it.c_end; c += nwarps)
-            sum += row_term(pr, it.masks + pr.word_base + (it.ind0 + i) * pr.W, c, lane);
-        if (lane == 0 && sum)
-            atomicAdd(reinterpret_cast<unsigned long long *>(it.sums) + i, sum);
-    }
-    __syncthreads();
     return phases;
 }
 
@@ -277,18 +405,6 @@ __device__ __forceinline__ uint32_t direct_item(const pm_prob &pr, const DirectI
 __device__ __noinline__ uint32_t direct_item_call(const pm_prob &pr, const DirectItem &it, uint32_t phases)
 {
     return direct_item(pr, it, phases, threadIdx.x >> 5, blockDim.x >> 5, threadIdx.x & 31);
-}
-
-// The bit-sliced walk as a function of its own: it needs all 128 registers, and inside the kernel's body every change
-// around it moved its speed by up to a tenth.
-template <int G>
-__device__ __noinline__ void tile_walk_call(const pm_prob &pr, uint32_t *smem, uint32_t tbl, int nb, uint32_t a0,
-                                            int64_t c_begin, int64_t c_end, unsigned long long *acc_s)
-{
-    const TileRows rows{pr.pi, pr.delta, pr.stride, pr.L, pr.cum != 0, pr.flush_units};
-    TileWalk<G> walk;
-    walk.prefetch(rows, c_begin, c_end, threadIdx.x >> 5, threadIdx.x & 31);
-    walk.run(smem, tbl, nb, a0, rows, c_begin, c_end, threadIdx.x >> 5, blockDim.x >> 5, threadIdx.x & 31, acc_s);
 }
 
 // What a launch's work items are: scanned client by client, rank-split or bit-sliced, evaluated by open facilities, or
@@ -309,7 +425,7 @@ enum class ScanKind { clients, split, sliced, direct, mixed };  // in the order 
 // ---------------------------------------------------------------------------
 template <int G, ScanKind kKind>
 __global__ void __launch_bounds__(kKind == ScanKind::clients || kKind == ScanKind::split ? 1024 : 512)
-    k_scan_columns(const pm_prob *__restrict__ probs, int K, pm_prob one, int64_t items,
+    k_scan_columns(const pm_prob *__restrict__ probs, int K, const __grid_constant__ pm_prob one, int64_t items,
                    const uint32_t *__restrict__ colT, const uint32_t *__restrict__ masks,
                    const uint32_t *__restrict__ active, unsigned long long *__restrict__ accum,
                    int *__restrict__ tickets, int *__restrict__ err, ScanEpilogue ep, uint32_t stall, int nb,
@@ -342,6 +458,12 @@ __global__ void __launch_bounds__(kKind == ScanKind::clients || kKind == ScanKin
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     [[maybe_unused]] uint32_t d_phases = 0;
+    // by open facilities: whether some individual has no list; an item's, and a tile of them (direct_left)
+    __shared__ int left_seen;
+    __shared__ uint32_t left_s[kDirect ? kDirectRange / 32 : 1];
+    __shared__ uint16_t left_ids[kDirect ? G * 32 : 1];
+    if (kDirect && threadIdx.x == 0)
+        left_seen = 0;
     constexpr bool kSplit = kKind == ScanKind::split;
     const uint32_t my_tab = tab_off + (uint32_t)(warp * (kSplit ? split_warp_words(G) : tile_table_words(nb, G)));
     [[maybe_unused]] SplitWalk<G> split_walk;
@@ -385,6 +507,7 @@ __global__ void __launch_bounds__(kKind == ScanKind::clients || kKind == ScanKin
                 share_s.tile = li - split * pr_s.tiles;
                 share_s.c_begin = split * pr_s.cps;
                 share_s.c_end = min(share_s.c_begin + pr_s.cps, pr_s.n);
+                share_s.index = split;
                 share_s.splits = (int32_t)pr_s.splits;
                 next_s = pos + gridDim.x;
             }
@@ -425,7 +548,7 @@ __global__ void __launch_bounds__(kKind == ScanKind::clients || kKind == ScanKin
         [[maybe_unused]] const int64_t c = c_begin + warp;
         [[maybe_unused]] uint32_t j_cur, j_nxt, j_nc, j_nc1;
         [[maybe_unused]] int32_t d_cur, d_nxt, d_nc, d_nc1;
-        [[maybe_unused]] const DirectItem d_item{colbits, colT + pr.col_base, masks, ind0, count, a0_s,  fin_s,
+        [[maybe_unused]] const DirectItem d_item{colbits, colT + pr.col_base, ind0, count, a0_s,  &left_seen,
                                                  d_sums,  c_begin,            c_end, d_bar, err,  stalled};
         if constexpr (kDirect)
             if (direct && threadIdx.x == 0)
@@ -612,6 +735,10 @@ __global__ void __launch_bounds__(kKind == ScanKind::clients || kKind == ScanKin
             apply_epilogue<kSplit ? 1 : 4>(acc_s, fin, count, pr, ind0, warp, nwarps, lane, ep);
         __syncthreads();  // shared state (tile, acc_s, a0_s, pr_s) is reused by the next item
     }
+    if constexpr (kDirect)
+        if (left_seen)
+            direct_left<G>(LeftLaunch{probs, K, &one, items, colT, masks, active, accum, ep, nb, tab_off, shares}, colbits,
+                           tile_acc, left_s, left_ids, &pr_s, &share_s);
 }
 
 // ---------------------------------------------------------------------------
@@ -795,7 +922,7 @@ scan_kernel scan_fn(int G, ScanKind kind)
     case ScanKind::sliced:
         return scan_fn_of<ScanKind::sliced>(G);
     case ScanKind::direct:
-        return k_scan_columns<1, ScanKind::direct>;
+        return scan_fn_of<ScanKind::direct>(G);
     case ScanKind::mixed:
         return scan_fn_of<ScanKind::mixed>(G);
     default:
@@ -900,6 +1027,18 @@ void pm_direct_shape(const pm_instance *inst, int64_t pop, size_t budget, int nw
            pm_direct_smem(inst->m, r, 2 * out.chunks * out.stages) <= budget)
         out.chunks *= 2;
     out.smem = pm_direct_smem(inst->m, r, out.chunks * out.stages);
+    // individuals without lists: the widest tile with the walk's tables (of as many blocks as need no more memory)
+    for (int G = 4; G > 0; G /= 2)
+        for (int nb : {7, 3, 1}) {
+            const size_t need = pm_scan_smem(inst->W, G, nwarps, nb, false);
+            if (need > (nb == 1 ? budget : out.smem))
+                continue;
+            out.groups = G;
+            out.nb = nb;
+            out.smem = std::max(out.smem, need);
+            return;
+        }
+    out = pm_direct_plan();
 }
 
 bool pm_direct_wanted(int64_t n, int64_t m, int64_t p, size_t smem_optin)
@@ -1119,6 +1258,7 @@ pm_prob pm_single_prob(const pm_instance *inst, const pm_eval_plan &plan, int64_
     }
     if (plan.direct.range) {
         pm_direct_prob(inst, plan.direct, pop, pr);
+        pr.flush_units = pm_flush_units(inst->max_d, plan.direct.groups);
         pr.stream_units = 0;
     }
     return pr;  // every base 0
@@ -1226,10 +1366,10 @@ pm_status pm_launch_eval(const pm_instance *inst, const pm_eval_plan &plan, cons
     unsigned long long *partials = reinterpret_cast<unsigned long long *>(partials_i64);
     if (plan.groups) {
         pm_scan_launch L;
-        L.groups = plan.groups;
+        L.groups = plan.direct.range ? plan.direct.groups : plan.groups;
         L.warps = plan.warps;
-        L.nb = plan.nb;
-        L.split = plan.split;
+        L.nb = plan.direct.range ? plan.direct.nb : plan.nb;
+        L.split = !plan.direct.range && plan.split;
         L.Wmax = inst->W;
         L.K = 1;
         L.one = pm_single_prob(inst, plan, pop);

@@ -68,10 +68,10 @@ struct pm_part {
 pm_status pm_carve(pm_dbuf &arena, const pm_part *parts, int count);
 
 // The evaluation by open facilities (scan_direct.cuh): individuals per work item (0: not used), chunks of 8 clients
-// per stage of shared memory, stages (2: the next chunks' copies run under the present ones' work), client splits and
-// clients per split.
+// per stage of shared memory, stages (2: the next chunks' copies run under the present ones' work), groups of a tile and
+// table blocks of the bit-sliced walk for individuals without lists, client splits and clients per split.
 struct pm_direct_plan {
-    int range = 0, chunks = 0, stages = 0;
+    int range = 0, chunks = 0, stages = 0, groups = 0, nb = 0;
     int64_t splits = 0, cps = 0;
     size_t smem = 0;
 };
@@ -122,11 +122,11 @@ struct pm_prob {
 };
 
 // One CTA's share of a tile in a launch over several instances: clients [c_begin, c_end) of tile `tile` of instance
-// `prob`, one of `splits` shares of that tile.  The launch's table: the instances' pm_prob, then the shares in CTA
+// `prob`, share `index` of `splits` of that tile.  The launch's table: the instances' pm_prob, then the shares in CTA
 // order, then (int32) the index of every CTA's first share and the number of shares.
 struct pm_share {
     int32_t prob, splits;
-    int64_t tile, c_begin, c_end;
+    int64_t tile, c_begin, c_end, index;
 };
 
 // Programmatic dependent launch.  Kernels of the GA generation and of the

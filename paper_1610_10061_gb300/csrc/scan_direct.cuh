@@ -27,7 +27,8 @@
 // took 0.21 ms at p = 10: the loads' latency was the CTA's critical path.
 //
 // A bitset without exactly p open facilities (unchecked calls only) has no
-// list; its terms come from a walk of the Pi' rows, as the scan defines them.
+// list: such individuals are gathered into facility-major tiles and scanned
+// (direct_left in fitness.cu).
 #pragma once
 
 #include <cstdint>
@@ -302,26 +303,4 @@ __device__ __forceinline__ void direct_terms(const pm_prob &pr, uint32_t ent, in
         }
         g0 += nwarps * NI;
     }
-}
-
-// One client's term of a bitset by a walk of its Pi' row (one warp): the distance at the first open rank, 0 without one.
-__device__ __forceinline__ uint32_t row_term(const pm_prob &pr, const uint32_t *__restrict__ mask, int64_t c, int lane)
-{
-    const uint16_t *prow = pr.pi + c * pr.stride;
-    const int32_t *drow = pr.delta + c * pr.stride;
-    uint32_t carry = 0;
-    for (int base = 0; base < pr.L; base += 32) {
-        const int r = base + lane;
-        const uint32_t j = r < pr.L ? __ldg(prow + r) : 0u;
-        const uint32_t d = r < pr.L ? (uint32_t)__ldg(drow + r) : 0u;
-        const uint32_t hit = __ballot_sync(PM_FULL_MASK, r < pr.L && ((__ldg(mask + (j >> 5)) >> (j & 31)) & 1u));
-        if (hit) {
-            const int first = __ffs(hit) - 1;
-            return pr.cum ? __shfl_sync(PM_FULL_MASK, d, first)
-                          : carry + __reduce_add_sync(PM_FULL_MASK, lane <= first ? d : 0u);
-        }
-        if (!pr.cum)
-            carry += __reduce_add_sync(PM_FULL_MASK, d);
-    }
-    return 0u;
 }
