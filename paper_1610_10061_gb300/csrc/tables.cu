@@ -671,6 +671,31 @@ static int bits_needed(uint32_t v)
     return b;
 }
 
+// One-time per-device attributes: all the shared memory that the kernels' own leaves.  Not set to what an instance needs
+// just before its launch: another thread's instance may set less in between.
+static pm_status tables_init(const pm_instance *inst)
+{
+    static std::mutex mu;
+    static bool done[64] = {};
+    const int dev = inst->device;
+    std::lock_guard<std::mutex> guard(mu);
+    if (dev < 64 && done[dev])
+        return PM_OK;
+    auto allow = [&](auto *fn) -> pm_status {
+        cudaFuncAttributes fa;
+        PM_CUDA(cudaFuncGetAttributes(&fa, fn));
+        PM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(inst->smem_optin - fa.sharedSizeBytes)));
+        return PM_OK;
+    };
+    PM_TRY(allow(k_tables_buckets));
+    PM_TRY(allow(k_tables<true>));
+    PM_TRY(allow(k_tables<false>));
+    if (dev < 64)
+        done[dev] = true;
+    return PM_OK;
+}
+
 // The bucket sort of every row: buckets, threads and shared memory for rows of m, false where a row does not fit.
 static bool bucket_shape(const pm_instance *inst, int &nb_log, int &threads, size_t &smem)
 {
@@ -686,6 +711,7 @@ static bool bucket_shape(const pm_instance *inst, int &nb_log, int &threads, siz
 pm_status pm_build_tables(pm_instance *inst, const int32_t *d_dev, cudaStream_t stream)
 {
     const int64_t count = inst->n * inst->m;
+    PM_TRY(tables_init(inst));
     PM_TRY(inst->flag.reserve(64));
     int *mm = reinterpret_cast<int *>(inst->flag.ptr);
     k_minmax_init<<<1, 1, 0, stream>>>(mm);
@@ -697,7 +723,6 @@ pm_status pm_build_tables(pm_instance *inst, const int32_t *d_dev, cudaStream_t 
     size_t bsmem = 0;
     const bool buckets = bucket_shape(inst, nb_log, threads, bsmem);
     if (buckets) {
-        PM_CUDA(cudaFuncSetAttribute(k_tables_buckets, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsmem));
         int per_sm = 1;
         PM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tables_buckets, threads, bsmem));
         const int64_t grid = std::min<int64_t>(inst->n, (int64_t)inst->sm_count * std::max(per_sm, 1));
@@ -730,8 +755,6 @@ pm_status pm_build_tables(pm_instance *inst, const int32_t *d_dev, cudaStream_t 
     size_t dyn = 0;
     if (in_smem) {
         dyn = row_bytes;
-        PM_CUDA(cudaFuncSetAttribute(packed ? k_tables<true> : k_tables<false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
         const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(4, (int64_t)(inst->smem_optin / (dyn + static_bytes))));
         grid = std::min<int64_t>(inst->n, (int64_t)inst->sm_count * per_sm);
     } else {
