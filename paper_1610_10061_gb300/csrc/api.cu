@@ -90,6 +90,33 @@ static DevicePool *device_pool()
     return &dp;
 }
 
+cudaError_t pm_device_malloc_beside(void **ptr, size_t bytes, void **second, size_t second_bytes)
+{
+    *second = nullptr;
+    DevicePool *dp = device_pool();
+    const bool pool = dp && dp->pool;
+    if (injected_failure()) {
+        *ptr = nullptr;
+        return cudaErrorMemoryAllocation;
+    }
+    cudaError_t e = pool ? cudaMallocFromPoolAsync(ptr, bytes, dp->pool, dp->stream) : cudaMalloc(ptr, bytes);
+    if (e != cudaSuccess)
+        return e;
+    if (injected_failure() || (pool ? cudaMallocFromPoolAsync(second, second_bytes, dp->pool, dp->stream)
+                                    : cudaMalloc(second, second_bytes)) != cudaSuccess) {
+        *second = nullptr;
+        pm_clear_stale_error();
+    }
+    e = pool ? cudaStreamSynchronize(dp->stream) : cudaSuccess;
+    if (e != cudaSuccess) {
+        (void)cudaFreeAsync(*ptr, dp->stream);
+        if (*second)
+            (void)cudaFreeAsync(*second, dp->stream);
+        *ptr = *second = nullptr;
+    }
+    return e;
+}
+
 cudaError_t pm_device_malloc(void **ptr, size_t bytes)
 {
     if (injected_failure()) {
@@ -111,8 +138,10 @@ cudaError_t pm_device_malloc(void **ptr, size_t bytes)
     return e;
 }
 
-void pm_device_free(void *ptr)
+void pm_device_free(void *ptr, void *second)
 {
+    if (!ptr)
+        std::swap(ptr, second);
     if (!ptr)
         return;
     int cur = 0, dev = 0;
@@ -129,10 +158,14 @@ void pm_device_free(void *ptr)
     DevicePool *dp = device_pool();
     if (!dp || !dp->pool) {
         pm_clear_error(cudaFree(ptr));
+        if (second)
+            pm_clear_error(cudaFree(second));
     } else {
         // as cudaFree does, wait for every launch that may still use the memory, then return it to the pool
         pm_clear_error(cudaDeviceSynchronize());
         pm_clear_error(cudaFreeAsync(ptr, dp->stream));
+        if (second)
+            pm_clear_error(cudaFreeAsync(second, dp->stream));
     }
     if (dev != cur)
         pm_clear_error(cudaSetDevice(cur));
@@ -188,7 +221,7 @@ void pm_dbuf::release()
     borrowed = false;
 }
 
-pm_status pm_carve(pm_dbuf &arena, const pm_part *parts, int count)
+pm_status pm_carve(pm_dbuf &arena, const pm_part *parts, int count, pm_dbuf *second, size_t second_bytes)
 {
     size_t total = 0;
     for (int k = 0; k < count; ++k) {
@@ -196,7 +229,14 @@ pm_status pm_carve(pm_dbuf &arena, const pm_part *parts, int count)
         total += (std::max<size_t>(parts[k].bytes, 256) + 255) & ~size_t(255);
     }
     arena.release();
-    PM_TRY(arena.reserve(total));
+    if (second) {
+        second->release();
+        PM_CUDA(pm_device_malloc_beside(&arena.ptr, total, &second->ptr, second_bytes));
+        arena.bytes = total;
+        second->bytes = second->ptr ? second_bytes : 0;
+    } else {
+        PM_TRY(arena.reserve(total));
+    }
     char *base = static_cast<char *>(arena.ptr);
     size_t off = 0;
     for (int k = 0; k < count; ++k) {
@@ -257,9 +297,15 @@ static void destroy_instance(pm_instance *inst)
     inst->columns.release();
     inst->flag.release();
     inst->err.release();
-    inst->tab_arena.release();  // the tables, err and flag
+    pm_device_free(inst->tab_arena.ptr, inst->entries.ptr);  // the tables, err and flag; the 16-bit distances
     inst->dsorted.release();
     delete inst;
+}
+
+void pm_drop_entries(pm_instance *inst)
+{
+    inst->dense = nullptr;
+    inst->entries.release();
 }
 
 static pm_status create_impl(const int32_t *d, int64_t n, int64_t m, int64_t p, int device, cudaStream_t stream,
@@ -279,20 +325,18 @@ static pm_status create_impl(const int32_t *d, int64_t n, int64_t m, int64_t p, 
     PM_CUDA(cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
     inst->smem_optin = (size_t)v;
     const size_t tab = (size_t)n * (size_t)inst->stride;
-    const int64_t entries = pm_ceil_div(n, 8) * m;  // eight clients' 16-bit distances each
-    const bool dense = pm_direct_wanted(n, m, p, inst->smem_optin);
+    // The 16-bit distances are optional (the scan needs only the tables).  Small ones lie beside the tables; larger ones are an
+    // allocation of their own, which is given back when the distances turn out not to fit and done without when there is
+    // no room for it.
+    const size_t entries = (size_t)pm_ceil_div(n, 8) * (size_t)m * 16;  // eight clients' distances each
+    const bool dense = pm_direct_wanted(n, m, p, inst->smem_optin), own = dense && entries >= ((size_t)4 << 20);
     pm_dbuf dbuf, pbuf, ebuf;
     const pm_part parts[] = {{&inst->err, 256}, {&inst->flag, 256}, {&dbuf, tab * sizeof(int32_t)},
-                             {&pbuf, tab * sizeof(uint16_t)}, {&ebuf, (size_t)entries * 16}};
-    pm_status carved = pm_carve(inst->tab_arena, parts, dense ? 5 : 4);
-    // the 16-bit distances are optional (the scan needs only the tables): where they are large enough to be what did
-    // not fit, the instance does without them
-    if (carved == PM_ERR_OOM && dense && entries >= ((int64_t)1 << 22))
-        carved = pm_carve(inst->tab_arena, parts, 4);
-    PM_TRY(carved);
+                             {&pbuf, tab * sizeof(uint16_t)}, {&ebuf, entries}};
+    PM_TRY(pm_carve(inst->tab_arena, parts, dense && !own ? 5 : 4, own ? &inst->entries : nullptr, entries));
     inst->delta = static_cast<int32_t *>(dbuf.ptr);
     inst->pi = static_cast<uint16_t *>(pbuf.ptr);
-    inst->dense = static_cast<uint16_t *>(ebuf.ptr);
+    inst->dense = static_cast<uint16_t *>(own ? inst->entries.ptr : ebuf.ptr);
     PM_CUDA(cudaMemsetAsync(inst->err.ptr, 0, 256, stream));
     PM_TRY(pm_fitness_init(inst));
     const int32_t *d_dev = d;

@@ -14,9 +14,13 @@
 // without calling CUDA when the armed failure is due.
 cudaError_t pm_device_malloc(void **ptr, size_t bytes);
 
+// The same, and with the one wait a second allocation that may fail (null).
+cudaError_t pm_device_malloc_beside(void **ptr, size_t bytes, void **second, size_t second_bytes);
+
 // Releases memory of pm_device_malloc after every launch on its device has
 // finished (as cudaFree waits); the pool keeps it for later allocations.
-void pm_device_free(void *ptr);
+// second: another allocation on the same device, released after the same wait.
+void pm_device_free(void *ptr, void *second = nullptr);
 
 // Stream-ordered memory from the same pool on stream s (released with
 // cudaFreeAsync on s), with the same injected failure.

@@ -65,7 +65,8 @@ struct pm_part {
     pm_dbuf *buf;
     size_t bytes;
 };
-pm_status pm_carve(pm_dbuf &arena, const pm_part *parts, int count);
+// second (optional): a buffer of its own that is allocated with the arena in one wait, and left empty if there is no room.
+pm_status pm_carve(pm_dbuf &arena, const pm_part *parts, int count, pm_dbuf *second = nullptr, size_t second_bytes = 0);
 
 // The evaluation by open facilities (scan_direct.cuh): individuals per work item (0: not used), chunks of 8 clients
 // per stage of shared memory, stages (2: the next chunks' copies run under the present ones' work), groups of a tile and
@@ -181,6 +182,7 @@ struct pm_instance {
     // staging and scratch for pm_eval_population
     pm_dbuf stage_masks, stage_costs, partials, tickets, columns, flag, err;
     pm_dbuf tab_arena;  // one allocation holding delta, pi, err and flag
+    pm_dbuf entries;    // the memory of dense (empty when it is small and lies in tab_arena)
     // Delta' instances: the running sums D' (the sorted distances), built once on the first request for swap
     // statistics, which then read distances directly instead of re-summing increments
     mutable pm_dbuf dsorted;
@@ -359,6 +361,8 @@ void pm_scan_launch_from(const pm_multi_plan &mp, const pm_prob *probs_dev, pm_s
 // ---------------------------------------------------------------------------
 // Tables (tables.cu)
 // ---------------------------------------------------------------------------
+// Give the memory of the 16-bit distances back (api.cu).
+void pm_drop_entries(pm_instance *inst);
 pm_status pm_build_tables(pm_instance *inst, const int32_t *d_dev, cudaStream_t stream);
 // Dense n x L copies of the tables on the device (Delta' also for cumulative instances); either output may be null.
 pm_status pm_launch_dense_rows(const pm_instance *inst, uint16_t *pi_out, int32_t *delta_out, cudaStream_t stream);

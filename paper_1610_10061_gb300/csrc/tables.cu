@@ -742,7 +742,7 @@ pm_status pm_build_tables(pm_instance *inst, const int32_t *d_dev, cudaStream_t 
     const int passes = (bits_needed((uint32_t)host_mm[1]) + 7) / 8;
     const bool packed = host_mm[1] < 65536;  // distance and facility id in one 32-bit word
     if (!packed)
-        inst->dense = nullptr;
+        pm_drop_entries(inst);  // the 16-bit distances cannot be used
     if (buckets && host_mm[2] == 0)
         return PM_OK;
     const int only_marked = buckets ? 1 : 0;  // the rows the bucket sort left
