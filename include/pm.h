@@ -83,8 +83,9 @@ typedef struct pm_instance pm_instance;
  * tables stay resident on `device` (Pi' uint16, Delta' int32, rows padded to
  * a stride of round_up(L, 32) elements).  Where p is far below the expected
  * first open rank (m + 1) / (p + 1) the instance also keeps the distances in
- * 16 bits (up to 1 GiB; done without if they do not fit in memory): with few
- * open facilities reading the p distances is cheaper than the scan.
+ * 16 bits (up to 1 GiB; done without if one of them does not fit in 16 bits or
+ * all do not in memory): with few open facilities reading the p distances is
+ * cheaper than the scan.
  *   d       distance matrix; not retained.
  *   n, m, p 1 <= n, 1 <= p < m <= 65535.
  *   device  CUDA device ordinal; becomes the current device.

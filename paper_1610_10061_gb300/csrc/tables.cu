@@ -26,7 +26,9 @@
 // neither 24 nor 48 warps per SM nor twice the buckets change it by more than
 // 3 %.  A row with a fuller bucket (distances crowded in a small part of their
 // range) or a distance of 2^16 or more is left to the radix sort, marked by a
-// first increment of -1.
+// first increment of -1.  Once one row in kLeftOf is, the CTAs give up and the
+// radix sort takes all rows: creating 5000 x 5000, p = 5, crowded 440 us, 495
+// with every row tried (the radix sort alone 415), up to 10^6 614, 650 (628).
 //
 // k_tables (those rows): a stable LSD radix sort of the distances with 8-bit
 // digits.  The row starts in facility order, so a stable sort on the distance
@@ -75,11 +77,16 @@ __global__ void k_minmax(const int32_t *__restrict__ d, int64_t count, int *__re
 }
 
 // The same, leaving the distances as 16 bits in entries of eight clients (scan_direct.cuh), from the one read of d
-// the check needs anyway: thread = entry, eight rows' loads coalesced over the facilities.  (Distances that do not
-// fit are cut off; the entries are then not used.)
+// the check needs anyway: thread = entry, eight rows' loads coalesced over the facilities.  A CTA stops writing entries
+// once it sees, or another one has reported, a distance that does not fit (they are then not used).
 __global__ void __launch_bounds__(256) k_minmax_entries(const int32_t *__restrict__ d, int64_t n, int32_t m,
                                                         int *__restrict__ out, uint4 *__restrict__ entries)
 {
+    __shared__ volatile int past;  // no barriers: a late look costs some writes
+    if (threadIdx.x == 0)
+        past = 0;
+    __syncthreads();
+    bool reported = false;  // of thread 0
     int lo = 0x7fffffff, hi = (int)0x80000000;
     const int64_t step = (int64_t)gridDim.x * blockDim.x, chunks = (n + 7) / 8;
     const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -92,6 +99,7 @@ __global__ void __launch_bounds__(256) k_minmax_entries(const int32_t *__restric
 #pragma unroll
         for (int i = 0; i < 8; ++i)
             v[i] = 8 * c + i < n ? __ldg(d + (8 * c + i) * m + j) : -1;
+        const int seen = threadIdx.x == 0 ? *reinterpret_cast<volatile int *>(out + 1) : 0;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             if (8 * c + i < n) {
@@ -101,8 +109,15 @@ __global__ void __launch_bounds__(256) k_minmax_entries(const int32_t *__restric
                 v[i] = 0;
             }
         }
-        entries[c * m + j] = make_uint4(__byte_perm(v[0], v[1], 0x5410), __byte_perm(v[2], v[3], 0x5410),
-                                        __byte_perm(v[4], v[5], 0x5410), __byte_perm(v[6], v[7], 0x5410));
+        if (max(seen, hi) > 0xffff)
+            past = 1;
+        if (!past) {
+            entries[c * m + j] = make_uint4(__byte_perm(v[0], v[1], 0x5410), __byte_perm(v[2], v[3], 0x5410),
+                                            __byte_perm(v[4], v[5], 0x5410), __byte_perm(v[6], v[7], 0x5410));
+        } else if (threadIdx.x == 0 && !reported) {
+            reported = true;
+            atomicMax(out + 1, 0x10000);
+        }
         c += step_c;
         j += step_j;
         if (j >= m) {
@@ -118,15 +133,17 @@ __global__ void __launch_bounds__(256) k_minmax_entries(const int32_t *__restric
     }
 }
 
-// Smallest and largest distance, and the number of rows left to the radix sort.
+// Smallest and largest distance, the number of rows left to the radix sort, whether the bucket sort gave up.
 __global__ void k_minmax_init(int *out)
 {
     out[0] = 0x7fffffff;
     out[1] = (int)0x80000000;
     out[2] = 0;
+    out[3] = 0;
 }
 
 constexpr int kBucketMost = 48;
+constexpr int kLeftOf = 32;
 
 // Batcher's odd-even merge sort of v[LO .. LO + N) in registers (N a power of two).
 template <int LO, int N, int R>
@@ -190,13 +207,13 @@ __device__ __forceinline__ void sort_windows(uint32_t *B, int m)
 __global__ void __launch_bounds__(512, 2) k_tables_buckets(const int32_t *__restrict__ d, int64_t n, int32_t m, int32_t L,
                                                         int64_t stride, int nb_log, int cum,
                                                         uint16_t *__restrict__ pi, int32_t *__restrict__ delta,
-                                                        int *__restrict__ out)
+                                                        int *out, int most_left, int check)
 {
     extern __shared__ __align__(16) uint32_t words[];
     __shared__ uint32_t warp_sum[16];
     __shared__ int row_lo[16], row_hi[16];
     __shared__ uint32_t scale_s;
-    __shared__ int bad_s, most_s;
+    __shared__ int bad_s, most_s, stop_s;
     const int32_t mp = (m + 15) / 16 * 16 + 48;
     uint32_t *A = words + 4, *B = A + mp + 4, *ends = B + bucket_at(mp) + 4;
     const int nb = 1 << nb_log, T = blockDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = T >> 5;
@@ -211,6 +228,7 @@ __global__ void __launch_bounds__(512, 2) k_tables_buckets(const int32_t *__rest
         for (int i = threadIdx.x; i < nb / 4; i += T)
             reinterpret_cast<uint4 *>(ends)[i] = make_uint4(0u, 0u, 0u, 0u);
         int lo = 0x7fffffff, hi = (int)0x80000000;
+        const int given = threadIdx.x == 0 ? *reinterpret_cast<volatile int *>(out + 2) : 0;  // rows left so far
         if (wide) {
             for (int i0 = 4 * threadIdx.x; i0 < m; i0 += 16 * T) {
                 int4 v[4];
@@ -261,11 +279,32 @@ __global__ void __launch_bounds__(512, 2) k_tables_buckets(const int32_t *__rest
             all_hi = max(all_hi, hi);
             bad_s = lo < 0 || hi > 0xffff;
             most_s = 0;
+            stop_s = given > most_left;
             // the map of [0, X) onto the buckets: floor(x scale / 2^32), scale = floor(nb 2^32 / X)
             const uint64_t X = max(((uint64_t)(uint32_t)hi + 1) * (uint64_t)m, (uint64_t)nb + 1);
             scale_s = (uint32_t)(((uint64_t)nb << 32) / X);
         }
         __syncthreads();
+        if (stop_s) {  // too many rows for the radix sort already: it takes them all
+            if (threadIdx.x == 0)
+                out[3] = 1;
+            if (check) {  // ... and what is left to do here is the check of the distances
+                int l = 0x7fffffff, h = (int)0x80000000;
+                for (row += gridDim.x; row < n; row += gridDim.x)
+                    for (int i = threadIdx.x; i < m; i += T) {
+                        const int v = __ldg(d + row * (int64_t)m + i);
+                        l = min(l, v);
+                        h = max(h, v);
+                    }
+                l = __reduce_min_sync(PM_FULL_MASK, l);
+                h = __reduce_max_sync(PM_FULL_MASK, h);
+                if (lane == 0) {
+                    atomicMin(out + 0, l);
+                    atomicMax(out + 1, h);
+                }
+            }
+            break;
+        }
         const uint32_t scale = scale_s;
         auto bucket = [&](uint32_t word) { return __umulhi((word >> 16) * (uint32_t)m + (word & 0xffffu), scale); };
         if (!bad_s) {
@@ -708,46 +747,12 @@ static bool bucket_shape(const pm_instance *inst, int &nb_log, int &threads, siz
     return smem + 2048 <= inst->smem_optin;
 }
 
-pm_status pm_build_tables(pm_instance *inst, const int32_t *d_dev, cudaStream_t stream)
+// The radix sort of every row, or of the marked ones.
+static pm_status radix_sort(const pm_instance *inst, const int32_t *d_dev, bool packed, int passes, bool marked,
+                            cudaStream_t stream)
 {
-    const int64_t count = inst->n * inst->m;
-    PM_TRY(tables_init(inst));
-    PM_TRY(inst->flag.reserve(64));
-    int *mm = reinterpret_cast<int *>(inst->flag.ptr);
-    k_minmax_init<<<1, 1, 0, stream>>>(mm);
-    const int64_t blocks = std::min<int64_t>(pm_ceil_div(count, 256), (int64_t)inst->sm_count * 8);
-    if (inst->dense)
-        k_minmax_entries<<<(unsigned)blocks, 256, 0, stream>>>(d_dev, inst->n, (int32_t)inst->m, mm,
-                                                               reinterpret_cast<uint4 *>(inst->dense));
-    int nb_log = 0, threads = 0;
-    size_t bsmem = 0;
-    const bool buckets = bucket_shape(inst, nb_log, threads, bsmem);
-    if (buckets) {
-        int per_sm = 1;
-        PM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tables_buckets, threads, bsmem));
-        const int64_t grid = std::min<int64_t>(inst->n, (int64_t)inst->sm_count * std::max(per_sm, 1));
-        k_tables_buckets<<<(unsigned)grid, threads, bsmem, stream>>>(d_dev, inst->n, (int32_t)inst->m,
-                                                                     (int32_t)inst->L, inst->stride, nb_log,
-                                                                     inst->cum ? 1 : 0, inst->pi, inst->delta, mm);
-    } else if (!inst->dense) {
-        k_minmax<<<(unsigned)blocks, 256, 0, stream>>>(d_dev, count, mm);
-    }
-    PM_CUDA(cudaGetLastError());
-    int host_mm[3];
-    PM_CUDA(cudaMemcpyAsync(host_mm, mm, sizeof(host_mm), cudaMemcpyDeviceToHost, stream));
-    PM_CUDA(cudaStreamSynchronize(stream));
-    if (host_mm[0] < 0)
-        return PM_ERR_NEGATIVE_DIST;
-    inst->max_d = host_mm[1];
-    const int passes = (bits_needed((uint32_t)host_mm[1]) + 7) / 8;
-    const bool packed = host_mm[1] < 65536;  // distance and facility id in one 32-bit word
-    if (!packed)
-        pm_drop_entries(inst);  // the 16-bit distances cannot be used
-    if (buckets && host_mm[2] == 0)
-        return PM_OK;
-    const int only_marked = buckets ? 1 : 0;  // the rows the bucket sort left
-
     const size_t row_bytes = (size_t)inst->m * (packed ? 8 : 12);
+    const int only_marked = marked ? 1 : 0;
     const size_t static_bytes = sizeof(uint32_t) * (kSortWarps * 256 + 256 + 8) + 1024;
     const bool in_smem = row_bytes + static_bytes <= inst->smem_optin;
     unsigned char *gscratch = nullptr;
@@ -776,4 +781,48 @@ pm_status pm_build_tables(pm_instance *inst, const int32_t *d_dev, cudaStream_t 
         cudaFreeAsync(gscratch, stream);
     PM_CUDA(le);
     return PM_OK;
+}
+
+pm_status pm_build_tables(pm_instance *inst, const int32_t *d_dev, cudaStream_t stream)
+{
+    const int64_t count = inst->n * inst->m;
+    PM_TRY(tables_init(inst));
+    PM_TRY(inst->flag.reserve(64));
+    int *mm = reinterpret_cast<int *>(inst->flag.ptr);
+    k_minmax_init<<<1, 1, 0, stream>>>(mm);
+    const int64_t blocks = std::min<int64_t>(pm_ceil_div(count, 256), (int64_t)inst->sm_count * 8);
+    if (inst->dense)
+        k_minmax_entries<<<(unsigned)blocks, 256, 0, stream>>>(d_dev, inst->n, (int32_t)inst->m, mm,
+                                                               reinterpret_cast<uint4 *>(inst->dense));
+    int nb_log = 0, threads = 0;
+    size_t bsmem = 0;
+    bool buckets = bucket_shape(inst, nb_log, threads, bsmem);
+    if (buckets) {
+        int per_sm = 1;
+        PM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tables_buckets, threads, bsmem));
+        const int64_t grid = std::min<int64_t>(inst->n, (int64_t)inst->sm_count * std::max(per_sm, 1));
+        const int64_t most_left = std::min<int64_t>(inst->n / kLeftOf, 0x7fffffff);
+        k_tables_buckets<<<(unsigned)grid, threads, bsmem, stream>>>(d_dev, inst->n, (int32_t)inst->m,
+                                                                     (int32_t)inst->L, inst->stride, nb_log,
+                                                                     inst->cum ? 1 : 0, inst->pi, inst->delta, mm,
+                                                                     (int)most_left, inst->dense ? 0 : 1);
+    } else if (!inst->dense) {
+        k_minmax<<<(unsigned)blocks, 256, 0, stream>>>(d_dev, count, mm);
+    }
+    PM_CUDA(cudaGetLastError());
+    int host_mm[4];
+    PM_CUDA(cudaMemcpyAsync(host_mm, mm, sizeof(host_mm), cudaMemcpyDeviceToHost, stream));
+    PM_CUDA(cudaStreamSynchronize(stream));
+    if (host_mm[3])  // the bucket sort gave up
+        buckets = false;
+    if (host_mm[0] < 0)
+        return PM_ERR_NEGATIVE_DIST;
+    inst->max_d = host_mm[1];
+    const int passes = (bits_needed((uint32_t)host_mm[1]) + 7) / 8;
+    const bool packed = host_mm[1] < 65536;  // distance and facility id in one 32-bit word
+    if (!packed)
+        pm_drop_entries(inst);  // the 16-bit distances cannot be used
+    if (buckets && host_mm[2] == 0)
+        return PM_OK;
+    return radix_sort(inst, d_dev, packed, passes, buckets, stream);
 }

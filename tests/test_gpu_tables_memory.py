@@ -32,6 +32,8 @@ for x in (d, big, many):
 
 def test_unused_entries_are_given_back():
     """In a child process without the memory pool, where free memory shows what an instance holds."""
+    from paper_1610_10061_gb300 import build
+    build.build()
     env = dict(os.environ, PM_POOL="0", PYTHONPATH=ROOT)
     out = subprocess.run([sys.executable, "-c", CHILD], capture_output=True, text=True, env=env, cwd=ROOT, timeout=300)
     assert out.returncode == 0, out.stderr
