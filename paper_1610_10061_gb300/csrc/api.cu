@@ -10,6 +10,7 @@
 
 #include "pm_alloc.h"
 #include "pm_common.cuh"
+#include "pm_reach.h"
 
 void pm_note_cuda_error(cudaError_t e, const char *what, const char *file, int line)
 {
@@ -430,10 +431,18 @@ extern "C" pm_status pm_instance_tables(const pm_instance *inst, uint16_t *pi_ou
         return PM_ERR_INVALID_ARG;
     PM_CUDA(cudaSetDevice(inst->device));
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // device outputs are written by one kernel (5000 x 4951: the call takes 70 us, strided device copies 180); host
-    // outputs go through a strided copy, by way of a dense device copy where Delta' has to be formed first
-    uint16_t *pi_dev = pi_out && pm_is_device_ptr(pi_out) ? pi_out : nullptr;
-    int32_t *delta_dev = delta_out && pm_is_device_ptr(delta_out) ? delta_out : nullptr;
+    // outputs on the instance's device are written by one kernel (5000 x 4951: the call takes 70 us, strided device copies
+    // 180); others go through a strided copy, by way of a dense device copy where Delta' has to be formed first
+    auto by_kernel = [&](const void *out) {
+        cudaPointerAttributes a;
+        if (!out || cudaPointerGetAttributes(&a, out) != cudaSuccess) {
+            pm_clear_stale_error();
+            return false;
+        }
+        return pm_kernel_may_store(a, out, inst->device);
+    };
+    uint16_t *pi_dev = by_kernel(pi_out) ? pi_out : nullptr;
+    int32_t *delta_dev = by_kernel(delta_out) ? delta_out : nullptr;
     if (pi_dev || delta_dev)
         PM_TRY(pm_launch_dense_rows(inst, pi_dev, delta_dev, s));
     if (pi_out && !pi_dev)
@@ -448,7 +457,7 @@ extern "C" pm_status pm_instance_tables(const pm_instance *inst, uint16_t *pi_ou
         int32_t *tmp = nullptr;
         PM_CUDA(pm_device_malloc_async(reinterpret_cast<void **>(&tmp), bytes, s));
         pm_status st = pm_launch_dense_rows(inst, nullptr, tmp, s);
-        cudaError_t e = st == PM_OK ? cudaMemcpyAsync(delta_out, tmp, bytes, cudaMemcpyDeviceToHost, s) : cudaSuccess;
+        cudaError_t e = st == PM_OK ? cudaMemcpyAsync(delta_out, tmp, bytes, cudaMemcpyDefault, s) : cudaSuccess;
         cudaFreeAsync(tmp, s);
         PM_TRY(st);
         PM_CUDA(e);
