@@ -2095,7 +2095,8 @@ constexpr uint32_t kDemeSpinLimit = 1u << 22, kDemeStallLimit = 1u << 14;
 // (octets of clients) read all banks.
 __host__ __device__ __forceinline__ int64_t deme_pitch(int64_t m) { return m | 1; }
 
-// The cost of the bitset F (shared memory), by one warp: lanes over octets of clients, every open facility's distances.
+// The cost of the bitset F (shared memory; exactly p open facilities, no bits from m on), by one warp: lanes over octets of
+// clients, every open facility's distances.
 // list: room for p ids (16 bits, a multiple of eight of them).
 __device__ __forceinline__ uint32_t deme_eval(uint32_t ent, int pitch, int n8, const uint32_t *F, int W, int p,
                                               uint16_t *list, int lane)
@@ -2150,7 +2151,7 @@ __device__ __forceinline__ uint32_t deme_eval(uint32_t ent, int pitch, int n8, c
                     use(id[i] >> 16);
                 }
             }
-        } else {  // more words than lanes, or (a population loaded with other bitsets) not p open facilities
+        } else {  // more words than lanes
             for (int w = 0; w < W; ++w) {
                 uint32_t y = F[w];
                 any |= y;
@@ -2520,6 +2521,7 @@ struct pm_ga {
     pm_dbuf bar;
     // the kernel over whole demes in place of a generation's phases when the GA qualifies
     bool deme = false;
+    bool p_subsets = true;  // see ga_create_single
     int deme_warps = 32;
     size_t deme_smem = 0;
     // learned swap proposal (single-instance GAs)
@@ -2625,8 +2627,8 @@ static cudaLaunchConfig_t deme_config(const pm_ga *ga, cudaStream_t s, cudaLaunc
     return cfg;
 }
 
-// The rule for the kernel over whole demes (k_ga_deme): one instance with Floyd generation and no learned try, whose
-// distances fit beside the CTA's rows, and demes of at most a cluster of 16 CTAs.  kDemeChain bounds an evaluation's chain
+// The rule for the kernel over whole demes (k_ga_deme): one instance with Floyd generation and no learned try, p-subsets
+// only (a loaded state may hold others, which the scans bound by the row's end), whose distances fit beside the CTA's rows, and demes of at most a cluster of 16 CTAs.  kDemeChain bounds an evaluation's chain
 // (p facilities for each 32 octets of clients) and kDemeWork what the population adds to it, where the phases' launches
 // are the cheaper way: us a generation, demes of 256, this kernel and the phases: chain 64 (256 nodes, p = 64), 512
 // individuals: 72 / 109; chain 120 (330 nodes, p = 60): 107 / 107; chain 200 (300 nodes, p = 100): 163 / 112; 4096
@@ -2637,7 +2639,7 @@ static pm_status deme_prepare(pm_ga *ga)
     ga->deme = false;
     const pm_instance *inst = ga->insts[0];
     const char *v = std::getenv("PM_GA_DEME");
-    if ((v && v[0] == '0') || !spec_allowed() || ga->K != 1 || ga->model || ga->comb || !inst->dense || ga->D > 512 ||
+    if ((v && v[0] == '0') || !spec_allowed() || ga->K != 1 || ga->model || ga->comb || !ga->p_subsets || !inst->dense || ga->D > 512 ||
         ga->P > 4096 || ga->P * deme_chain(inst->n, inst->p) > kDemeWork || inst->n > 65536 ||
         !pm_deme_fits(inst->n, inst->m, inst->p, inst->smem_optin))
         return PM_OK;
@@ -3315,8 +3317,9 @@ static pm_status comb_prepare(pm_ga *ga, const pm_instance *inst, cudaStream_t s
     return overflow ? PM_ERR_UNSUPPORTED : PM_OK;
 }
 
+// p_subsets: whether every bitset that the GA will meet has exactly p open facilities (its own always have).
 static pm_status ga_create_single(pm_instance *inst, uint64_t seed, int64_t pop, const pm_ga_params *params,
-                                  void *stream, int graphs, pm_ga **out)
+                                  void *stream, int graphs, bool p_subsets, pm_ga **out)
 {
     if (!out || !inst)
         return PM_ERR_INVALID_ARG;
@@ -3325,6 +3328,7 @@ static pm_status ga_create_single(pm_instance *inst, uint64_t seed, int64_t pop,
     if (!ga)
         return PM_ERR_OOM;
     ga->graphs = graphs;
+    ga->p_subsets = p_subsets;
     ga->insts.push_back(inst);
     ga->device = inst->device;
     ga->K = 1;
@@ -3375,7 +3379,7 @@ static pm_status ga_create_single(pm_instance *inst, uint64_t seed, int64_t pop,
 extern "C" pm_status pm_ga_create(pm_instance *inst, uint64_t seed, int64_t pop, const pm_ga_params *params,
                                   void *stream, pm_ga **out)
 {
-    return ga_create_single(inst, seed, pop, params, stream, 3, out);
+    return ga_create_single(inst, seed, pop, params, stream, 3, true, out);
 }
 
 extern "C" pm_status pm_batch_ga_create(pm_batch *b, uint64_t seed, int64_t pop, const pm_ga_params *params,
@@ -3638,8 +3642,21 @@ extern "C" pm_status pm_ga_load(pm_instance *inst, const void *buf, size_t len, 
     prm.saturation = h.S;
     prm.stream_id = h.sid;
     prm.flags = h.flags & (PM_GA_MIGRATE_TEAM | PM_GA_INIT_COMBINADIC);
+    // the deme bests migrate into the next generation: whether all of them have exactly p open facilities
+    bool p_subsets = true;
+    const size_t demes = h.D > 0 && h.P >= h.D ? (size_t)(h.P / h.D) : 0;
+    if (demes <= (len - sizeof(h)) / ((size_t)inst->W * 4)) {
+        std::vector<uint32_t> row((size_t)inst->W);
+        for (size_t b = 0; b < demes && p_subsets; ++b) {
+            std::memcpy(row.data(), static_cast<const char *>(buf) + sizeof(h) + b * row.size() * 4, row.size() * 4);
+            int64_t open = 0;
+            for (uint32_t w : row)
+                open += __builtin_popcount(w);
+            p_subsets = open == inst->p && !((inst->m & 31) && row.back() >> (inst->m & 31));
+        }
+    }
     pm_ga *ga = nullptr;
-    PM_TRY(pm_ga_create(inst, h.seed, h.P, &prm, stream, &ga));
+    PM_TRY(ga_create_single(inst, h.seed, h.P, &prm, stream, 3, p_subsets, &ga));
     if (len < ga_blob_size(ga)) {
         ga_free(ga);
         return PM_ERR_INVALID_ARG;
@@ -3718,7 +3735,7 @@ extern "C" pm_status pm_ga_run(pm_instance *inst, uint64_t seed, int64_t pop, in
         return PM_ERR_INVALID_ARG;
     pm_ga *ga = nullptr;
     // one job of `gens` generations: only the graph that runs them is built
-    PM_TRY(ga_create_single(inst, seed, pop, params, stream, gens == 1 ? 2 : 1, &ga));
+    PM_TRY(ga_create_single(inst, seed, pop, params, stream, gens == 1 ? 2 : 1, true, &ga));
     pm_status st = pm_ga_step(ga, gens, trace, stream);
     if (st == PM_OK)
         st = pm_ga_result(ga, best_cost, best_mask, gens_run, evals, stream);
