@@ -382,8 +382,14 @@ __device__ __forceinline__ uint32_t direct_item(const pm_prob &pr, const DirectI
         if (pr.d_stages == 2 && next_chunks > 0 && threadIdx.x == 0 && !it.stalled)
             direct_fill(pr, reinterpret_cast<char *>(it.smem) + (stage ^ 1) * stage_bytes, it.c_begin / 8 + next,
                         next_chunks, &it.bar[stage ^ 1]);
-        if (!wait_copies(&it.bar[stage], (phases >> stage) & 1u, it.stalled, it.err))
+        if (!wait_copies(&it.bar[stage], (phases >> stage) & 1u, it.stalled, it.err)) {
+            // the next chunks' copies may be under way, too: they must not land after the CTA has left (bounded)
+            for (uint32_t spins = 0; pr.d_stages == 2 && next_chunks > 0 && !it.stalled && spins < kSpinLimit &&
+                                     !mbar_try_wait(&it.bar[stage ^ 1], (phases >> (stage ^ 1)) & 1u);
+                 ++spins) {
+            }
             return 0xffffffffu;
+        }
         phases ^= 1u << stage;
         const int chunks = (int)min(all - c8, (int64_t)pr.d_chunks);
         if (chunks * groups >= 2 * nwarps)  // two individuals per lane as long as every warp has a task
