@@ -1142,6 +1142,12 @@ static int column_warps(const pm_instance *inst, int64_t pop, int G)
     return sliced_pays(inst, pop) && 2 * column_smem_bytes(inst->W, G) + 8192 <= inst->smem_optin ? 16 : 32;
 }
 
+static bool is_tuned(const pm_instance *inst, int64_t pop)
+{
+    std::lock_guard<std::mutex> g(inst->plan_mu);
+    return inst->tuned.count(pop) != 0;
+}
+
 pm_eval_plan pm_plan_eval(const pm_instance *inst, int64_t pop)
 {
     {
@@ -1472,12 +1478,31 @@ extern "C" pm_status pm_eval_population_noalloc(pm_instance *inst, const uint32_
         return PM_OK;
     if (!masks || !costs || !pm_is_device_ptr(masks) || !pm_is_device_ptr(costs))
         return PM_ERR_INVALID_ARG;
-    const pm_eval_plan plan = pm_plan_eval(inst, pop);
+    auto need = [&](const pm_eval_plan &pl) {
+        return 256 + pm_plan_ticket_bytes(pl) + (size_t)pm_round_up((int64_t)pm_plan_column_bytes(inst, pl), 256) +
+               pm_plan_partial_bytes(pl, pop);
+    };
+    pm_eval_plan plan = pm_plan_eval(inst, pop);
+    if (plan.groups && (size_t)(pop + 128) * (size_t)(4 * inst->W + 9) + 1024 > kNoAllocScratchBytes && !is_tuned(inst, pop)) {
+        // Near the limit: which populations fit is decided by a fixed layout, tiles of up to 128 individuals and 8 of them at
+        // least (16 where walks are short), and does not change with the way an evaluation takes.  A plan that needs more
+        // (narrower tiles have more tickets) gives way to one of that layout.
+        const size_t budget = inst->smem_optin > 4096 ? inst->smem_optin - 4096 : 0;
+        const int64_t min_tiles = (inst->m + 1) < 32 * (inst->p + 1) ? 16 : 8;
+        int G = kMaxG;
+        while (G > 1 && (pop <= (int64_t)32 * (G / 2) * min_tiles || column_smem_bytes(inst->W, G) > budget))
+            G /= 2;
+        const pm_eval_plan wide = pm_plan_eval_with(inst, pop, G, 16, 0);
+        if (need(wide) > kNoAllocScratchBytes)
+            return PM_ERR_INVALID_ARG;
+        if (need(plan) > kNoAllocScratchBytes)
+            plan = wide;
+    }
+    if (need(plan) > kNoAllocScratchBytes)
+        return PM_ERR_INVALID_ARG;
     const size_t tick = pm_plan_ticket_bytes(plan);
     const size_t cols = (size_t)pm_round_up((int64_t)pm_plan_column_bytes(inst, plan), 256);
     const size_t part = pm_plan_partial_bytes(plan, pop);
-    if (256 + tick + cols + part > kNoAllocScratchBytes)
-        return PM_ERR_INVALID_ARG;
     PM_CUDA(cudaSetDevice(inst->device));
     unsigned char *base = nullptr;
     PM_TRY(noalloc_scratch(inst->device, &base));
