@@ -142,14 +142,15 @@ def _stream(stream):
     if stream is not None:
         return int(stream)
     torch = sys.modules.get("torch")  # a program that has not imported it has no current stream
-    if torch is None:
+    try:
+        if torch is None or not torch.cuda.is_initialized():
+            return 0
+    except AttributeError:  # it is being imported
         return 0
     try:
-        if torch.cuda.is_initialized():
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
-    except Exception:
-        pass
-    return 0
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    except Exception:  # private names: without them the public call, never another stream than the current one
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _addr(a):
