@@ -1159,10 +1159,12 @@ pm_eval_plan pm_plan_eval(const pm_instance *inst, int64_t pop)
     const size_t budget = inst->smem_optin > 4096 ? inst->smem_optin - 4096 : 0;
     // the bit-sliced walk: the widest tile the population fills
     const bool sliced = sliced_pays(inst, pop);
-    int G = sliced ? kMaxG : (inst->n <= 128 ? 1 : 2);
+    int G = sliced ? kMaxG : 2;
     while (G > 1 && (pop <= (int64_t)32 * (G / 2) || column_smem_bytes(inst->W, G) > budget))
         G /= 2;
     int warps = column_warps(inst, pop, G);
+    int splits = 0;
+    auto one_wave = [&](int w) { return pm_ceil_div(pop, 32) * pm_ceil_div(inst->n, (int64_t)w * 4) <= inst->sm_count; };
     if (!sliced && inst->n > 128) {
         // The rank-split walk: one round of four clients a warp (tiles of 32), by as few warps a CTA as leave at most a
         // CTA per SM, since a warp's chain is shorter with fewer beside it; 16 where walks are short, so that the CTAs'
@@ -1170,15 +1172,33 @@ pm_eval_plan pm_plan_eval(const pm_instance *inst, int64_t pop)
         // individuals 7.3 / 8.9 / 11.7; 2000 points, p = 20, 64 individuals 12.2 / 14.2 / 18.0.  Generations: 496 nodes, p =
         // 40, 256 individuals 110 / 106 / 116; graph900, 256 individuals 130 / 116 / 123.  Launches of more than a round for
         // every SM take 32 warps and tiles of 64: graph900, 1024 individuals, 7.8 us a scan, 9.0 with 16.
-        auto one_wave = [&](int w) { return pm_ceil_div(pop, 32) * pm_ceil_div(inst->n, (int64_t)w * 4) <= inst->sm_count; };
         const bool deep = inst->m + 1 > 20 * (inst->p + 1);
         if (one_wave(16)) {
             G = 1;
             warps = deep && one_wave(8) ? 8 : 16;
         }
+    } else if (!sliced) {
+        // Up to 128 clients: one round of a CTA's 32 warps covers them, which saves the sums' way through global memory, but
+        // crowds the walks on the few SMs that a CTA per tile takes.  So 8 warps a CTA while that is at most a CTA per SM, for
+        // more than 64 clients, deep walks or few individuals: 128 clients, 1000 facilities, p = 4, 512 individuals 16 us, 27
+        // with 32 warps (a client a warp 21); 9000, p = 9 73, 135 (77); generations of 64 on 128 x 3000, p = 100 132, 148
+        // (129); but of 512 on 64 x 100, p = 3 116, 109 (113).  And several CTAs with tiles of 64 for deep walks of more
+        // tiles than SMs (64 x 9000, p = 31, 8192 individuals 65, 87 (66)) and the deepest of more clients (128 x 9000, p =
+        // 9, 2048 of them 87, 138 (106); 4096 129, 141 (109)).
+        const double mean = (double)(inst->m + 1) / (double)(inst->p + 1);
+        if (inst->n > 32 && one_wave(8) &&
+            (inst->n > 64 || (mean > 200.0 && pop <= 1024) || (inst->m <= 1024 && pop <= 128))) {
+            G = 1;
+            warps = 8;
+        } else if (mean > 60.0 && (pm_ceil_div(pop, 32) > inst->sm_count || (inst->n > 112 && mean > 200.0))) {
+            const int64_t each = 4 / G, ctas = pm_ceil_div(pop, 32 * G) * pm_ceil_div(inst->n, 8 * each);
+            warps = ctas <= 2 * inst->sm_count ? 8 : 16;
+        } else {
+            G = 1;
+        }
+        splits = (int)pm_ceil_div(inst->n, warps * (4 / G));
     }
-    // (up to 128 clients one round of 32 warps covers them all, which saves the sums' way through global memory)
-    pm_eval_plan plan = pm_plan_eval_with(inst, pop, G, warps, 0);
+    pm_eval_plan plan = pm_plan_eval_with(inst, pop, G, warps, splits);
     pm_plan_direct(inst, pop, plan);
     return plan;
 }
