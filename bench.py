@@ -738,9 +738,37 @@ def run_ours(args):
         }
         if world == 1 and not args.no_extra:
             line.update(extra_records(pm, torch, args))
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)  # every record in full
+        print(json.dumps(headline(line)), flush=True)
     if world > 1:
         torch.distributed.destroy_process_group()
+
+
+def headline(line):
+    """The default run's line with its records cut to their figures: a line of a few kilobytes, which a reader that
+    keeps the end of the output has whole.  (The full line goes to standard error.)"""
+    def cut(rec, keys):
+        return None if rec is None else {k: rec[k] for k in keys if k in rec}
+
+    roof = ("bound", "achieved", "peak", "unit", "frac", "traffic", "kernel", "peak_source", "launch_ms",
+            "instructions_per_launch", "launch_ms_alone", "frac_alone", "chain")
+    out = {k: v for k, v in line.items() if k not in ("eval_euclid10000", "learned", "batched256")}
+    out["roofline"] = cut(line.get("roofline"), roof)
+    out["roofline_alg_bytes"] = cut(line.get("roofline_alg_bytes"), ("bound", "achieved", "peak", "unit", "frac",
+                                                                     "traffic", "l2_bytes", "launch_ms", "pass_ms"))
+    out["e2e"] = cut(line.get("e2e"), ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"))
+    if "eval_euclid10000" in line:
+        out["eval_euclid10000"] = [
+            dict(cut(r, ("p", "pop", "steps", "ms_per_pass", "evals_per_s")),
+                 roofline=cut(r.get("roofline"), ("bound", "frac", "traffic", "traffic_frac")))
+            for r in line["eval_euclid10000"]]
+    if "learned" in line:
+        out["learned"] = {name: cut(r, ("plain_time_s", "learned_time_s", "speedup_amortised", "reached",
+                                        "plain_ms_per_gen", "learned_ms_per_gen"))
+                          for name, r in line["learned"].items()}
+    if "batched256" in line:
+        out["batched256"] = cut(line["batched256"], ("value", "unit", "ms_per_step", "steps"))
+    return out
 
 
 def extra_records(pm, torch, args):
