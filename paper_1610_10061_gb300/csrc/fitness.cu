@@ -155,10 +155,10 @@ __device__ __forceinline__ void apply_epilogue(const unsigned long long *acc_s, 
             } else {
                 for (int q = lane; q < W; q += 32 * kFlight) {
                     uint32_t v[kFlight];
-    #pragma unroll
+#pragma unroll
                     for (int f = 0; f < kFlight; ++f)
                         v[f] = q + 32 * f < W ? __ldg(ep.cand_masks + row + q + 32 * f) : 0u;
-    #pragma unroll
+#pragma unroll
                     for (int f = 0; f < kFlight; ++f)
                         if (q + 32 * f < W)
                             ep.cur_masks[row + q + 32 * f] = v[f];
@@ -1299,11 +1299,6 @@ pm_prob pm_single_prob(const pm_instance *inst, const pm_eval_plan &plan, int64_
 // Scan launches still to be armed by pm_debug_scan_timeout.
 static std::atomic<long long> g_scan_stall{0};
 
-static bool take_stall()
-{
-    return pm_take_scan_stall();
-}
-
 bool pm_take_scan_stall()
 {
     long long k = g_scan_stall.load();
@@ -1376,7 +1371,7 @@ pm_status pm_launch_scan(const pm_scan_launch &L, const pm_accept_args &acc, int
     const int threads = L.warps * 32;
     const unsigned grid = (unsigned)L.grid;
     unsigned long long *accum = reinterpret_cast<unsigned long long *>(L.accum);
-    const uint32_t stall = take_stall() ? 1u : 0u;
+    const uint32_t stall = pm_take_scan_stall() ? 1u : 0u;
     const uint32_t tab_off = (uint32_t)(column_smem_bytes(L.Wmax, G) / 4);
     const size_t smem = std::max(pm_scan_smem(L.Wmax, G, L.warps, L.nb, L.split), L.d_smem);
     const ScanKind kind = L.d_smem == 0 ? scan_kind(L.nb, L.split)

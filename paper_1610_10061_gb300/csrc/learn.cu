@@ -1375,7 +1375,7 @@ __device__ __forceinline__ void candidates_from_stats(const uint32_t *bits, cons
                     bk = k;
                 }
             }
-    #pragma unroll
+#pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 const unsigned long long og = __shfl_xor_sync(PM_FULL_MASK, bg, o);
                 const int32_t ok = __shfl_xor_sync(PM_FULL_MASK, bk, o);
