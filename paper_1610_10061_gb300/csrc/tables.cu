@@ -27,8 +27,8 @@
 // 3 %.  A row with a fuller bucket (distances crowded in a small part of their
 // range) or a distance of 2^16 or more is left to the radix sort, marked by a
 // first increment of -1.  Once one row in kLeftOf is, the CTAs give up and the
-// radix sort takes all rows: creating 5000 x 5000, p = 5, crowded 440 us, 495
-// with every row tried (the radix sort alone 415), up to 10^6 614, 650 (628).
+// radix sort takes all rows: creating 5000 x 5000, p = 5, crowded 430 us, 495
+// with every row tried (the radix sort alone 415), up to 10^6 608, 650 (628).
 //
 // k_tables (those rows): a stable LSD radix sort of the distances with 8-bit
 // digits.  The row starts in facility order, so a stable sort on the distance
@@ -77,16 +77,12 @@ __global__ void k_minmax(const int32_t *__restrict__ d, int64_t count, int *__re
 }
 
 // The same, leaving the distances as 16 bits in entries of eight clients (scan_direct.cuh), from the one read of d
-// the check needs anyway: thread = entry, eight rows' loads coalesced over the facilities.  A CTA stops writing entries
-// once it sees, or another one has reported, a distance that does not fit (they are then not used).
+// the check needs anyway: thread = entry, eight rows' loads coalesced over the facilities.  A thread that has seen a
+// distance that does not fit writes no more entries (they are then not used).  Asking the other threads, too, takes 8 of
+// the kernel's 38 us (5000 x 5000) where all fit.
 __global__ void __launch_bounds__(256) k_minmax_entries(const int32_t *__restrict__ d, int64_t n, int32_t m,
                                                         int *__restrict__ out, uint4 *__restrict__ entries)
 {
-    __shared__ volatile int past;  // no barriers: a late look costs some writes
-    if (threadIdx.x == 0)
-        past = 0;
-    __syncthreads();
-    bool reported = false;  // of thread 0
     int lo = 0x7fffffff, hi = (int)0x80000000;
     const int64_t step = (int64_t)gridDim.x * blockDim.x, chunks = (n + 7) / 8;
     const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -99,7 +95,6 @@ __global__ void __launch_bounds__(256) k_minmax_entries(const int32_t *__restric
 #pragma unroll
         for (int i = 0; i < 8; ++i)
             v[i] = 8 * c + i < n ? __ldg(d + (8 * c + i) * m + j) : -1;
-        const int seen = threadIdx.x == 0 ? *reinterpret_cast<volatile int *>(out + 1) : 0;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             if (8 * c + i < n) {
@@ -109,15 +104,9 @@ __global__ void __launch_bounds__(256) k_minmax_entries(const int32_t *__restric
                 v[i] = 0;
             }
         }
-        if (max(seen, hi) > 0xffff)
-            past = 1;
-        if (!past) {
+        if (hi <= 0xffff)
             entries[c * m + j] = make_uint4(__byte_perm(v[0], v[1], 0x5410), __byte_perm(v[2], v[3], 0x5410),
                                             __byte_perm(v[4], v[5], 0x5410), __byte_perm(v[6], v[7], 0x5410));
-        } else if (threadIdx.x == 0 && !reported) {
-            reported = true;
-            atomicMax(out + 1, 0x10000);
-        }
         c += step_c;
         j += step_j;
         if (j >= m) {
