@@ -831,8 +831,10 @@ def eval_pass_record(pm, torch, name, tables="delta", steps=None, warmup=3, budg
     dmask = torch.from_numpy(masks.view(np.int32)).cuda()
     dcost = torch.empty(pop, dtype=torch.int64, device="cuda")
     flush = torch.empty(512 << 20, dtype=torch.uint8, device="cuda")
+    before = pm.pm_debug_scan_launches()["direct"]
     for _ in range(warmup):
         pm.pm_eval_population(inst.handle, dmask, pop, dcost, 0, stream.cuda_stream)
+    direct = pm.pm_debug_scan_launches()["direct"] > before  # evaluated by open facilities, not by the scan
     if steps is None:  # about budget_s of passes, so that clock samples fall inside the timed region
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         e0.record(stream)
@@ -858,11 +860,22 @@ def eval_pass_record(pm, torch, name, tables="delta", steps=None, warmup=3, budg
     ms = [a.elapsed_time(b) for a, b in zip(es, ee)]
     mean_ms = statistics.mean(ms)
     ek = (m + 1) / (p + 1)
-    alg_bytes = pop * (n * ek * 6 + W * 4 + 8)
     peak, peak_kind = measured_peaks()
-    scan_ms = time_scan_alone(pm, torch, inst, dmask, pop, dcost, flush, stream, 20)
-    # a pass shorter than the scan of the facility-major form evaluates by open facilities: its launch is not timed apart
-    kernel_ms = scan_ms if scan_ms is not None and scan_ms <= mean_ms else mean_ms
+    if direct:  # its launch is not timed apart from the lists'
+        alg_bytes = (n + 7) // 8 * m * 16 + pop * (W * 4 + 8)
+        scan_ms, kernel_ms = None, mean_ms
+        kernel = "lists of open facilities + k_scan_columns (by open facilities)"
+        note = ("achieved = the 16-bit distances, the bitsets and the costs, each once, / the pass's time; bound by "
+                "shared memory (p entries of 16 bytes for every eight pairs), not by these bytes")
+    else:
+        alg_bytes = pop * (n * ek * 6 + W * 4 + 8)
+        scan_ms = time_scan_alone(pm, torch, inst, dmask, pop, dcost, flush, stream, 20)
+        kernel_ms = scan_ms if scan_ms is not None else mean_ms
+        kernel = "k_scan_columns" if scan_ms is not None else "row kernel + reduction"
+        note = ("achieved = algorithmic bytes (pop * (n*(m+1)/(p+1)*6 + 4W + 8), the Pi'/Delta' prefix every "
+                "evaluation scans) / the scan kernel's live launch time; what a CTA stages serves its whole tile "
+                "of individuals, so this exceeds the DRAM bytes moved (traffic, ncu, committed summary of this "
+                "source), whose own fraction of the peak is traffic_frac")
     achieved = alg_bytes / (kernel_ms / 1000) / 1e9
     traffic = profiled_traffic(name)
     inst.close()
@@ -873,14 +886,9 @@ def eval_pass_record(pm, torch, name, tables="delta", steps=None, warmup=3, budg
            "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                         "frac": achieved / peak, "traffic": traffic,
                         "traffic_frac": (traffic / (kernel_ms / 1000) / 1e9 / peak) if traffic else None,
-                        "kernel": "k_scan_columns" if scan_ms is not None else "row kernel + reduction",
+                        "kernel": kernel,
                         "launch_ms": kernel_ms, "pass_ms": mean_ms, "alg_bytes_per_launch": alg_bytes,
-                        "peak_source": f"{peak_kind} burst copy bandwidth",
-                        "note": "achieved = algorithmic bytes (pop * (n*(m+1)/(p+1)*6 + 4W + 8), the Pi'/Delta' "
-                                "prefix every evaluation scans) / the scan kernel's live launch time (the pass's where it "
-                                "is evaluated by open facilities); what a CTA stages serves its whole tile or "
-                                "range of individuals, so this exceeds the DRAM bytes moved (traffic, ncu, committed "
-                                "summary of this source), whose own fraction of the peak is traffic_frac"},
+                        "peak_source": f"{peak_kind} burst copy bandwidth", "note": note},
            "roofline_issue": issue_roofline(name, kernel_ms), "clocks": clk, "l2": "flushed between timed steps"}
     if tables_rec is not None:
         rec["tables_build"] = tables_rec
